@@ -1,13 +1,13 @@
 // Fixed-length bucket mode: the gradient is cut into buckets of d elements and every bucket is
 // quantized on its own (the setting of all the paper's experiments, d = 128 ... 32768).
 //
-// One CTA takes one bucket at a time and does the whole path on it from a single read: the bucket's
-// keys are sorted in shared memory, the levels follow from the definitions applied to the sorted
-// keys (Algorithm 1 with Q* for ORQ, optionally followed by refinement sweeps; the sign change of g
-// for BinGrad-pb; the conditional means for BinGrad-b), then the bucket is read once more (from L2)
-// to be quantized and packed.  Results are those of the per-tensor entry points called with tensor
-// offsets j * d: same level definitions, same Philox counters (tensor index = bucket index), same
-// packed layout.
+// One team of threads (a warp for buckets of up to 512 elements, a CTA for longer ones) takes one
+// bucket at a time and does the whole path on it: the bucket's values are sorted in shared memory, the
+// levels follow from the definitions applied to the sorted values (Algorithm 1 with Q* for ORQ,
+// optionally followed by refinement sweeps; the sign change of g for BinGrad-pb; the conditional means
+// for BinGrad-b), then the values are quantized and packed.  Results are those of the per-tensor entry
+// points called with tensor offsets j * d: same level definitions, same Philox counters (tensor index =
+// bucket index), same packed layout.
 #include <math.h>
 
 #include <atomic>
@@ -18,11 +18,12 @@
 
 namespace ogq {
 
-constexpr int kBktMaxD = 32768;        // longest bucket (its keys take 128 KB of shared memory)
-constexpr int kBktPrefixMaxD = 4096;   // buckets up to this length also keep fp64 prefix sums of the sorted values
-constexpr int kBktMaxThreads = 1024;
-static_assert(kBktMaxD * sizeof(uint32_t) <= 160 * 1024, "the keys of the longest bucket must fit the shared-memory limit set at launch");
-constexpr int kBktMaxWarps = kBktMaxThreads / 32;
+constexpr int kBktWarpD = 512;         // buckets up to this length are worked on by one warp each
+constexpr int kBktWarpsPerCta = 4;     // ... this many to a CTA, independent of one another
+constexpr int kBktPrefixMaxD = 4096;   // buckets up to this length keep the prefix sum of every sorted value,
+                                       // longer ones that of every thread's first value
+constexpr int kBktMaxWarps = 32;
+constexpr int kBktLevels = 17;         // most levels of a bucket
 
 struct BktArgs {
     const float* grad;
@@ -37,27 +38,118 @@ struct BktArgs {
     int64_t words_per_bucket;
 };
 
-// Ascending bitonic sort of P = KPT * blockDim.x keys held in registers, KPT per thread: thread t
-// owns positions t * KPT ... t * KPT + KPT - 1 of the sequence.  The network is the variant whose
-// merges start with a "flip" (position i against i ^ (k - 1)) followed by halvings (i against
-// i ^ j): every compare-exchange then puts the smaller key at the lower position, so no direction
-// has to be computed.  Distances inside a thread's registers cost a min and a max; distances up to
-// 16 * KPT cross lanes by shuffle; only the larger ones (a few stages, none when the CTA is one
-// warp) go through shared memory with a barrier.  xch: P words of shared memory.
-__device__ __forceinline__ void bkt_cmpx(uint32_t& a, uint32_t& b)
+// ---------------------------------------------------------------------------
+// Teams: a warp (WARP) or the whole CTA.
+// ---------------------------------------------------------------------------
+template <bool WARP>
+__device__ __forceinline__ void team_sync()
 {
-    const uint32_t lo = min(a, b), hi = max(a, b);
+    if constexpr (WARP) __syncwarp();
+    else __syncthreads();
+}
+
+// Sums of N doubles over the team, in a fixed order, valid in every thread.  scratch: N * kBktMaxWarps
+// doubles (CTA teams only).
+template <bool WARP, int N>
+__device__ __forceinline__ void team_sum(double (&v)[N], double* scratch)
+{
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = warp_sum(v[i]);
+    if constexpr (!WARP) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        __syncthreads();
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < N; ++i) scratch[i * kBktMaxWarps + warp] = v[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = warp_sum(lane < nw ? scratch[i * kBktMaxWarps + lane] : 0.0);
+    }
+}
+
+// Maximum of a and sum of b over the team, valid in every thread.
+template <bool WARP>
+__device__ __forceinline__ void team_max_sum(uint32_t& a, uint32_t& b, uint32_t* scratch)
+{
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    if constexpr (!WARP) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        __syncthreads();
+        if (lane == 0) { scratch[warp] = a; scratch[kBktMaxWarps + warp] = b; }
+        __syncthreads();
+        a = __reduce_max_sync(0xffffffffu, lane < nw ? scratch[lane] : 0u);
+        b = __reduce_add_sync(0xffffffffu, lane < nw ? scratch[kBktMaxWarps + lane] : 0u);
+    }
+}
+
+// Exclusive sum of v over the team's threads (warps in order); total over the team in tot.
+template <bool WARP, class Tv>
+__device__ __forceinline__ Tv team_excl_scan(Tv v, Tv* scratch, Tv& tot)
+{
+    const int lane = threadIdx.x & 31;
+    Tv inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const Tv nb = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc = nb + inc;
+    }
+    const Tv up = __shfl_up_sync(0xffffffffu, inc, 1);
+    const Tv own = lane == 0 ? (Tv)0 : up;
+    if constexpr (WARP) {
+        tot = __shfl_sync(0xffffffffu, inc, 31);
+        return own;
+    } else {
+        const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+        __syncthreads();
+        if (lane == 31) scratch[warp] = inc;
+        __syncthreads();
+        Tv w = lane < nw ? scratch[lane] : (Tv)0;
+        Tv winc = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const Tv nb = __shfl_up_sync(0xffffffffu, winc, o);
+            if (lane >= o) winc = nb + winc;
+        }
+        tot = __shfl_sync(0xffffffffu, winc, 31);
+        const Tv wbase = __shfl_sync(0xffffffffu, winc, warp > 0 ? warp - 1 : 0);
+        return warp > 0 ? wbase + own : own;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Sorting
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void bkt_cmpx(float& a, float& b)
+{
+    const float lo = fminf(a, b), hi = fmaxf(a, b);
     a = lo;
     b = hi;
 }
 
+// Batcher's odd-even merge sort of a thread's N registers, written out at compile time (N = 16: 63
+// compare-exchanges).
+template <int N>
+__device__ __forceinline__ void bkt_sort_thread(float (&r)[N])
+{
+#pragma unroll
+    for (int p = 1; p < N; p <<= 1) {
+#pragma unroll
+        for (int k = p; k >= 1; k >>= 1) {
+#pragma unroll
+            for (int i = 0; i + k < N; ++i)
+                if (i >= k % p && ((i - k % p) / k) % 2 == 0 && i / (2 * p) == (i + k) / (2 * p)) bkt_cmpx(r[i], r[i + k]);
+        }
+    }
+}
+
 // Exchange with thread t ^ m: this thread's register e against the partner's register e (REV false)
-// or KPT - 1 - e (REV true); the thread on the lower side keeps the smaller keys.
+// or KPT - 1 - e (REV true); the thread on the lower side keeps the smaller values.
 template <int KPT, bool REV>
-__device__ __forceinline__ void bkt_cross(uint32_t (&r)[KPT], uint32_t* xch, int m, bool keep_min)
+__device__ __forceinline__ void bkt_cross(float (&r)[KPT], float* xch, int m, bool keep_min)
 {
     const int t = threadIdx.x, nt = blockDim.x;
-    uint32_t o[KPT];
+    float o[KPT];
     if (m < 32) {
 #pragma unroll
         for (int e = 0; e < KPT; ++e) o[e] = __shfl_xor_sync(0xffffffffu, r[REV ? KPT - 1 - e : e], m);
@@ -69,286 +161,421 @@ __device__ __forceinline__ void bkt_cross(uint32_t (&r)[KPT], uint32_t* xch, int
 #pragma unroll
         for (int e = 0; e < KPT; ++e) o[e] = xch[(REV ? KPT - 1 - e : e) * nt + (t ^ m)];
     }
-    // the side of the exchange decides once whether this thread keeps minima or maxima: one predicated
-    // instruction pair per key instead of a minimum, a maximum and a select
 #pragma unroll
-    for (int e = 0; e < KPT; ++e)
-        asm("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p min.u32 %0, %0, %1; @!p max.u32 %0, %0, %1; }"
-            : "+r"(r[e]) : "r"(o[e]), "r"((uint32_t)keep_min));
+    for (int e = 0; e < KPT; ++e) r[e] = keep_min ? fminf(r[e], o[e]) : fmaxf(r[e], o[e]);
 }
 
-// The stages of a merge that stay inside a warp, written out at compile time (no run-time dispatch on
-// the merge size, so the registers never have to be moved between code paths): halvings at lane
-// distances 16 ... 1 (FROM_LANES) or only those inside a thread's registers.
-template <int KPT, bool FROM_LANES>
-__device__ __forceinline__ void bkt_merge_tail(uint32_t (&r)[KPT], uint32_t* xch)
+// Ascending bitonic sort of the KPT * (team threads) values held in registers, thread t owning positions
+// t * KPT ... of the sequence.  Merges start with a "flip" (position i against i ^ (k - 1)) followed by
+// halvings (i against i ^ j), so every compare-exchange puts the smaller value at the lower position.
+// Only buckets whose values the cells of bkt_sort cannot separate come here.  xch: one float per position
+// (CTA teams only).
+template <int KPT, bool WARP>
+__device__ __noinline__ void bkt_bitonic(float (&r)[KPT], float* xch)
 {
-    const int t = threadIdx.x;
-    if constexpr (FROM_LANES) {
-#pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) bkt_cross<KPT, false>(r, xch, m, (t & m) == 0);
-    }
-#pragma unroll
-    for (int j = KPT / 2; j >= 1; j >>= 1) {
-#pragma unroll
-        for (int e = 0; e < KPT; ++e)
-            if ((e & j) == 0) bkt_cmpx(r[e], r[e | j]);
-    }
-}
-
-// Sorts the 32 * KPT keys of every warp ascending: the whole network unrolled at compile time.
-template <int KPT>
-__device__ __forceinline__ void bkt_sort_warp(uint32_t (&r)[KPT], uint32_t* xch)
-{
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int k = 2; k <= 32 * KPT; k <<= 1) {
-        if (k <= KPT) {
-#pragma unroll
-            for (int e = 0; e < KPT; ++e)
-                if ((e & (k >> 1)) == 0) bkt_cmpx(r[e], r[e ^ (k - 1)]);
-#pragma unroll
-            for (int j = k >> 2; j >= 1; j >>= 1) {
-#pragma unroll
-                for (int e = 0; e < KPT; ++e)
-                    if ((e & j) == 0) bkt_cmpx(r[e], r[e | j]);
-            }
-        } else {
-            const int m = k / KPT - 1;  // flip: lane t against t ^ m, registers reversed
-            bkt_cross<KPT, true>(r, xch, m, (t & ((m + 1) >> 1)) == 0);
-#pragma unroll
-            for (int j = k >> 2; j >= KPT; j >>= 1) bkt_cross<KPT, false>(r, xch, j / KPT, (t & (j / KPT)) == 0);
-            bkt_merge_tail<KPT, false>(r, xch);
-        }
-    }
-}
-
-template <int KPT>
-__device__ __forceinline__ void bkt_sort_regs(uint32_t (&r)[KPT], uint32_t* xch, int P)
-{
-    const int t = threadIdx.x;
-    bkt_sort_warp<KPT>(r, xch);
-    // merges across warps: the flip and the halvings at 32 threads or more go through shared memory
-    for (int k = 64 * KPT; k <= P; k <<= 1) {
+    const int t = WARP ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+    const int P = KPT * (WARP ? 32 : (int)blockDim.x);
+    bkt_sort_thread<KPT>(r);
+    for (int k = 2 * KPT; k <= P; k <<= 1) {
         const int m = k / KPT - 1;
         bkt_cross<KPT, true>(r, xch, m, (t & ((m + 1) >> 1)) == 0);
-        for (int j = k >> 2; j >= 32 * KPT; j >>= 1) bkt_cross<KPT, false>(r, xch, j / KPT, (t & (j / KPT)) == 0);
-        bkt_merge_tail<KPT, true>(r, xch);
-    }
-}
-
-__device__ __forceinline__ int bkt_lower(const uint32_t* a, int n, uint32_t k)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) { const int mid = (lo + hi) >> 1; if (a[mid] < k) lo = mid + 1; else hi = mid; }
-    return lo;
-}
-
-__device__ __forceinline__ int bkt_upper(const uint32_t* a, int n, uint32_t k)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) { const int mid = (lo + hi) >> 1; if (a[mid] <= k) lo = mid + 1; else hi = mid; }
-    return lo;
-}
-
-// Sum of a double over the CTA, valid in every thread.  scratch: kBktMaxWarps + 1 doubles.
-__device__ __forceinline__ double bkt_block_sum(double x, double* scratch)
-{
+        for (int j = k >> 2; j >= KPT; j >>= 1) bkt_cross<KPT, false>(r, xch, j / KPT, (t & (j / KPT)) == 0);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = x;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = 0.0;
-        const int nw = (blockDim.x + 31) >> 5;
-        for (int i = 0; i < nw; ++i) r += scratch[i];
-        scratch[kBktMaxWarps] = r;
+        for (int j = KPT / 2; j >= 1; j >>= 1) {
+#pragma unroll
+            for (int e = 0; e < KPT; ++e)
+                if ((e & j) == 0) bkt_cmpx(r[e], r[e | j]);
+        }
     }
-    __syncthreads();
-    return scratch[kBktMaxWarps];
+    if constexpr (!WARP) __syncthreads();
 }
 
-// Q*(L, R) on sorted keys with prefix sums (pre[i] = sum of the values of keys[0..i)): called by one
-// thread.  With T = sum_{L <= v <= R} (v - L) / (R - L) the result is the (floor(T) + 1)-th largest
-// element of the segment.
-__device__ __forceinline__ uint32_t bkt_qstar_prefix(const uint32_t* keys, const double* pre, int n, uint32_t kl,
-                                                     uint32_t kr)
-{
-    if (kr <= kl) return kl;
-    const int i0 = bkt_lower(keys, n, kl), i1 = bkt_upper(keys, n, kr);
-    const double Lv = (double)key_to_float(kl), Rv = (double)key_to_float(kr);
-    const int m = i1 - i0;
-    const double A = (pre[i1] - pre[i0]) - Lv * (double)m;
-    long long k = (long long)floor(A / (Rv - Lv));
-    if (k < 0) k = 0;
-    if (k > m - 1) k = m - 1;
-    return keys[i1 - 1 - (int)k];
-}
-
-// One depth of Algorithm 1 for a bucket held by ONE warp, called by all its lanes with the sorted keys
-// still in their registers.  The positions of the brackets come from counting (a compare per key and
-// one warp reduction per bracket) instead of binary searches in shared memory, whose dependent loads
-// are what a lone lane spends its time on; the levels of the depth are counted one after the other,
-// then lane i finishes level i (the fp64 division of every level of the depth at the same time).
-// Positions past n hold the largest key, which no bracket reaches.  lvkey: the level keys in shared
-// memory, the brackets of this depth already in place.
+// Index of sorted position i in shared memory: four words of padding after every thread's KPT values, so
+// that the 128-bit accesses of neighbouring threads fall into different banks.
 template <int KPT>
-__device__ __forceinline__ void bkt_depth_warp(const uint32_t (&r)[KPT], const uint32_t* keys, const double* pre,
-                                               uint32_t* lvkey, int s, int stride, int lane)
+__device__ __forceinline__ int bkt_at(int i)
 {
-    int my_i0 = 0, my_i1 = 0, my_q = -1;
-    uint32_t my_kl = 0u, my_kr = 0u;
-    int idx = 0;
-    for (int q = stride; q < s - 1; q += 2 * stride, ++idx) {
-        const uint32_t kl = lvkey[q - stride], kr = lvkey[q + stride];
-        int i0 = 0, i1 = 0;
-        if (kr > kl) {
-            uint32_t below = 0u, upto = 0u;
+    return KPT >= 8 ? i + i / KPT * 4 : i;
+}
+// The same for the fp64 prefix sums (one double of padding).
+template <int KPT>
+__device__ __forceinline__ int bkt_pre_at(int i)
+{
+    return i + i / KPT;
+}
+
+// Cells per thread of the sort.  Two to four cells per value where shared memory allows it.
+template <int KPT>
+constexpr int kBktCellsPerThread = KPT <= 8 ? 16 : 32;
+
+// Sorts the team's n values into sv (position i at bkt_at<KPT>(i); positions n .. P hold +Inf) and leaves
+// thread t the KPT values at positions t * KPT ... in r.  fetch(e) returns the e-th of the thread's own
+// values (any arrangement), have(e) whether there is one.
+//
+// A counting sort into cells, then a repair of the order inside the cells.  The cell of a value v is a
+// monotone function of it that spreads the usual gradient distributions (one peak around 0, tails of any
+// weight) almost evenly: the leading bits of the float 1 + k |v|, which are a piecewise linear log2, with
+// k = 2 / (geometric mean of the magnitudes), scaled so that the bucket's largest magnitude falls into the
+// last cell, negative values mirrored.  The counts are added up over the cells in order and every value
+// goes to the next free position of its cell.  Each value is then at most a cell's width from its place,
+// and a few passes of odd-even transposition (KPT - 1 exchanges in registers, one with the next thread)
+// put it there; a comparison of all neighbours tells when.  Values that the cells do not separate (a
+// narrow peak far from 0) are left to the bitonic network after kRepairs rounds.
+//   What bounds it: instruction issue on the integer / min-max pipe.  About 25 instructions per value,
+// whatever the length, against 60 (one warp) to 130 (32 warps, plus their exchanges through shared
+// memory) of the bitonic network that did the whole sort before: with it the launch for 25.6 M values,
+// ORQ s = 9, took 351 us at d = 512, 384 at 2048, 694 at 32768; now 153, 168 and 242.
+//   mean_bits: mean of (magnitude bits >> 16), maxabs: largest magnitude, signed_values: false when all
+// values are magnitudes (BinGrad-pb).  cells: NC + padding words; sv may share their memory (a barrier lies between).
+template <int KPT, bool WARP, class Fetch, class Have>
+__device__ __forceinline__ void bkt_sort(float (&r)[KPT], float* sv, uint32_t* cells, float* edge, uint32_t* scan_scratch,
+                                         int n, uint32_t mean_bits, float maxabs, bool signed_values, Fetch fetch, Have have)
+{
+    constexpr int CPT = kBktCellsPerThread<KPT>;
+    constexpr int kPasses = 3, kRepairs = 3;
+    const int lane = threadIdx.x & 31;
+    const int t = WARP ? lane : (int)threadIdx.x, nt = WARP ? 32 : (int)blockDim.x;
+    const int P = KPT * nt;
+    auto cell_at = [](uint32_t c) -> uint32_t { return c + c / CPT * 4; };
+
+    uint4* mine = reinterpret_cast<uint4*>(cells + t * (CPT + 4));
 #pragma unroll
-            for (int e = 0; e < KPT; ++e) {
-                below += (r[e] < kl) ? 1u : 0u;
-                upto += (r[e] <= kr) ? 1u : 0u;
+    for (int q = 0; q < CPT / 4; ++q) mine[q] = make_uint4(0u, 0u, 0u, 0u);
+    // the map's constants: the same in every thread
+    float geo = __uint_as_float(mean_bits << 16);
+    geo = fmaxf(geo, fmaxf(maxabs * 0x1p-20f, 1e-37f));
+    const float k = __fdividef(2.0f, geo);
+    const uint32_t one = 0x3f800000u;
+    const uint32_t range = __float_as_uint(fmaf(maxabs, k, 1.0f)) - one;
+    const uint32_t nc = (uint32_t)(nt * CPT);
+    const uint32_t side = signed_values ? nc / 2 : nc, base = signed_values ? nc / 2 : 0u;
+    // floor((side - 2) * 2^32 / (range + 1)), a little less: umulhi(x, mul) < side - 2 for every x <= range.
+    // Zeros get the first cell and the values of the largest magnitude (all the clipped ones) the last:
+    // those two values may be there in any number, and equal values need no order among themselves.
+    const uint32_t mul = range > 2 * side ? (uint32_t)((float)(side - 2) * 0.99999f * (4294967296.0f / ((float)range + 1.0f))) : 0u;
+    team_sync<WARP>();
+    uint32_t at[KPT];  // cell of every value
+#pragma unroll
+    for (int e = 0; e < KPT; ++e) {
+        at[e] = 0u;
+        if (have(e)) {
+            const float v = fetch(e);
+            const uint32_t x = __float_as_uint(fmaf(fabsf(v), k, 1.0f)) - one;
+            at[e] = cell_at(base + ((__umulhi(x, mul) + min(x, 1u) + (x == range ? 1u : 0u)) ^ (uint32_t)((int)__float_as_uint(v) >> 31)));
+            atomicAdd(cells + at[e], 1u);
+        }
+    }
+    team_sync<WARP>();
+    {
+        // exclusive sums over the cells, in place: this thread's CPT consecutive ones
+        uint32_t sum = 0u;
+#pragma unroll
+        for (int q = 0; q < CPT / 4; ++q) {
+            const uint4 w = mine[q];
+            sum += (w.x + w.y) + (w.z + w.w);
+        }
+        uint32_t tot;
+        uint32_t run = team_excl_scan<WARP>(sum, scan_scratch, tot);
+#pragma unroll
+        for (int q = 0; q < CPT / 4; ++q) {
+            const uint4 w = mine[q];
+            uint4 o;
+            o.x = run; o.y = o.x + w.x; o.z = o.y + w.y; o.w = o.z + w.z;
+            run = o.w + w.w;
+            mine[q] = o;
+        }
+    }
+    team_sync<WARP>();
+    // the next free position of the value's cell
+#pragma unroll
+    for (int e = 0; e < KPT; ++e)
+        if (have(e)) at[e] = atomicAdd(cells + at[e], 1u);
+    team_sync<WARP>();  // the cells are dead: sv may lie over them
+#pragma unroll
+    for (int e = 0; e < KPT; ++e)
+        if (have(e)) sv[bkt_at<KPT>((int)at[e])] = fetch(e);
+    for (int i = n + t; i < P; i += nt) sv[bkt_at<KPT>(i)] = __int_as_float(0x7f800000);
+    team_sync<WARP>();
+    float4* own = reinterpret_cast<float4*>(sv + bkt_at<KPT>(t * KPT));
+#pragma unroll
+    for (int q = 0; q < KPT / 4; ++q) {
+        const float4 w = own[q];
+        r[4 * q] = w.x; r[4 * q + 1] = w.y; r[4 * q + 2] = w.z; r[4 * q + 3] = w.w;
+    }
+    for (int round = 0;; ++round) {
+#pragma unroll
+        for (int pass = 0; pass < kPasses; ++pass) {
+#pragma unroll
+            for (int e = 0; e + 1 < KPT; e += 2) bkt_cmpx(r[e], r[e + 1]);
+#pragma unroll
+            for (int e = 1; e + 1 < KPT; e += 2) bkt_cmpx(r[e], r[e + 1]);
+            // the pair that two threads share
+            float nx = __shfl_down_sync(0xffffffffu, r[0], 1), pv = __shfl_up_sync(0xffffffffu, r[KPT - 1], 1);
+            if constexpr (WARP) {
+                if (lane == 31) nx = r[KPT - 1];
+                if (lane == 0) pv = r[0];
+            } else {
+                const int warp = threadIdx.x >> 5;
+                float* ed = edge + (pass & 1) * 2 * kBktMaxWarps;
+                if (lane == 0) ed[2 * warp] = r[0];
+                if (lane == 31) ed[2 * warp + 1] = r[KPT - 1];
+                __syncthreads();
+                if (lane == 31) nx = t + 1 < nt ? ed[2 * warp + 2] : r[KPT - 1];
+                if (lane == 0) pv = t > 0 ? ed[2 * warp - 1] : r[0];
             }
-            i0 = (int)__reduce_add_sync(0xffffffffu, below);
-            i1 = (int)__reduce_add_sync(0xffffffffu, upto);
+            r[KPT - 1] = fminf(r[KPT - 1], nx);
+            r[0] = fmaxf(r[0], pv);
         }
-        if (lane == idx) { my_i0 = i0; my_i1 = i1; my_kl = kl; my_kr = kr; my_q = q; }
-    }
-    __syncwarp();
-    if (my_q >= 0) {
-        uint32_t res = my_kl;
-        if (my_kr > my_kl) {
-            const double Lv = (double)key_to_float(my_kl), Rv = (double)key_to_float(my_kr);
-            const int m = my_i1 - my_i0;
-            const double A = (pre[my_i1] - pre[my_i0]) - Lv * (double)m;
-            long long k = (long long)floor(A / (Rv - Lv));
-            if (k < 0) k = 0;
-            if (k > m - 1) k = m - 1;
-            res = keys[my_i1 - 1 - (int)k];
+        // (the pairs that two threads share are in order: the exchange above came last)
+        bool ok = true;
+#pragma unroll
+        for (int e = 0; e + 1 < KPT; ++e) ok = ok && r[e] <= r[e + 1];
+        if (WARP ? __all_sync(0xffffffffu, ok) : __syncthreads_and(ok)) break;
+        if (round >= kRepairs) {
+            float tmp[KPT];
+#pragma unroll
+            for (int e = 0; e < KPT; ++e) tmp[e] = r[e];
+            bkt_bitonic<KPT, WARP>(tmp, sv);
+#pragma unroll
+            for (int e = 0; e < KPT; ++e) r[e] = tmp[e];
+            break;
         }
-        lvkey[my_q] = res;
     }
-    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < KPT / 4; ++q) own[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+    team_sync<WARP>();
 }
 
-// The same without prefix sums: called by every thread of the CTA, the segment's sum is a block sum.
-__device__ __forceinline__ uint32_t bkt_qstar_block(const uint32_t* keys, int n, uint32_t kl, uint32_t kr,
-                                                    double* scratch)
+// ---------------------------------------------------------------------------
+// Levels from the sorted values
+// ---------------------------------------------------------------------------
+struct BktLevel {
+    float v;
+    int i_lt, i_le;      // #{values < v}, #{values <= v}
+    double s_lt, s_le;   // sums of those
+};
+
+// Sorted values of a bucket with prefix sums.  FULL: pre holds the sum before every position, else the
+// sum before every thread's first position and the rest is added up from the values.
+template <int KPT, bool FULL>
+struct BktSorted {
+    const float* sv;
+    const double* pre;
+    int n;
+
+    __device__ __forceinline__ float at(int i) const { return sv[bkt_at<KPT>(i)]; }
+
+    __device__ __forceinline__ double before(int i) const
+    {
+        if constexpr (FULL) {
+            return pre[bkt_pre_at<KPT>(i)];
+        } else {
+            const int t = i / KPT;
+            double a = pre[t];
+            for (int q = t * KPT; q < i; ++q) a += (double)at(q);
+            return a;
+        }
+    }
+    __device__ __forceinline__ int lower(float v, int hi) const  // first position in [0, hi) that holds a value >= v
+    {
+        int lo = 0;
+        while (lo < hi) { const int mid = (lo + hi) >> 1; if (at(mid) < v) lo = mid + 1; else hi = mid; }
+        return lo;
+    }
+    __device__ __forceinline__ int upper(float v, int lo) const  // first position in [lo, n) that holds a value > v
+    {
+        int hi = n;
+        while (lo < hi) { const int mid = (lo + hi) >> 1; if (at(mid) <= v) lo = mid + 1; else hi = mid; }
+        return lo;
+    }
+    // first and last-plus-one position of the run of values equal to at(p) (usually p alone)
+    __device__ __forceinline__ int run_begin(int p, float v) const { return (p > 0 && at(p - 1) == v) ? lower(v, p) : p; }
+    __device__ __forceinline__ int run_end(int p, float v) const { return (p + 1 < n && at(p + 1) == v) ? upper(v, p + 1) : p + 1; }
+
+    __device__ __forceinline__ BktLevel level_at(int p) const
+    {
+        BktLevel l;
+        l.v = at(p);
+        l.i_lt = run_begin(p, l.v);
+        l.i_le = run_end(p, l.v);
+        l.s_lt = before(l.i_lt);
+        l.s_le = FULL ? before(l.i_le) : l.s_lt + (double)l.v * (double)(l.i_le - l.i_lt);
+        return l;
+    }
+    // Q*(L, R): with T = sum_{L <= v <= R} (v - L) / (R - L) the (floor(T) + 1)-th largest value of the segment
+    __device__ __forceinline__ BktLevel qstar(const BktLevel& L, const BktLevel& R) const
+    {
+        if (!(R.v > L.v)) return L;
+        const double Lv = (double)L.v, Rv = (double)R.v;
+        const int m = R.i_le - L.i_lt;
+        const double A = (R.s_le - L.s_lt) - Lv * (double)m;
+        const int k = __double2int_rd(A / (Rv - Lv));  // floor
+        return level_at(R.i_le - 1 - min(max(k, 0), m - 1));
+    }
+};
+
+// Thread t's part of the prefix sums; base: the sum before its first value.
+template <int KPT, bool FULL>
+__device__ __forceinline__ void bkt_prefix(const float (&r)[KPT], double* pre, int t, double base)
 {
-    if (kr <= kl) return kl;
-    const int i0 = bkt_lower(keys, n, kl), i1 = bkt_upper(keys, n, kr);
-    const double Lv = (double)key_to_float(kl), Rv = (double)key_to_float(kr);
-    double a = 0.0;
-    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) a += (double)key_to_float(keys[i]) - Lv;
-    a = bkt_block_sum(a, scratch);
-    const int m = i1 - i0;
-    long long k = (long long)floor(a / (Rv - Lv));
-    if (k < 0) k = 0;
-    if (k > m - 1) k = m - 1;
-    return keys[i1 - 1 - (int)k];
-}
-
-template <int BITS, int KPT>
-__global__ void __launch_bounds__(kBktMaxThreads)
-k_bucket_encode(BktArgs A, const __grid_constant__ PhiloxKeys pk)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double sh_d[kBktMaxWarps + 1];
-    __shared__ uint32_t sh_lvkey[kMaxLevels];
-    __shared__ float sh_lv[kMaxLevels];
-    __shared__ float sh_w[kMaxLevels];
-    __shared__ float2 sh_tab[kMaxLevels];
-    __shared__ uint32_t sh_words[kBktMaxWarps][(BITS == 3 || BITS == 5) ? 4 * BITS : 1];
-    __shared__ int sh_flag, sh_changed;
-    __shared__ float sh_b0;
-
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
-    const int s = A.s;
-    const bool orq = A.scheme == OGQ_ORQ, pbs = A.scheme == OGQ_BINGRAD_PB;
-    uint32_t* keys = reinterpret_cast<uint32_t*>(smem);
-    const int Pmax = KPT * blockDim.x;
-    double* pre = (A.d <= kBktPrefixMaxD) ? reinterpret_cast<double*>(smem + (size_t)Pmax * sizeof(uint32_t)) : nullptr;
-    if ((BITS == 3 || BITS == 5) && lane < 4 * BITS) sh_words[warp][lane] = 0u;
-
-    for (int j = blockIdx.x; j < A.nb; j += gridDim.x) {
-        const int64_t base_i = (int64_t)j * A.d;
-        const int n = (int)((A.total - base_i < (int64_t)A.d) ? A.total - base_i : (int64_t)A.d);
-        const float* src = A.grad + base_i;
-        int stbits = 0;
-        __syncthreads();
-        if (threadIdx.x == 0) { sh_flag = 0; sh_b0 = 0.f; }
-        __syncthreads();
-        // The bucket's values, KPT per thread (element e * blockDim.x + threadIdx.x: coalesced), all loads
-        // issued before the first use; positions past n read element 0 and are not used.  Every later
-        // pass over the bucket but the quantizer's runs from these registers.
-        float rawv[KPT];
+    if constexpr (FULL) {
+        double run = base;
+        double* p = pre + bkt_pre_at<KPT>(t * KPT);
 #pragma unroll
         for (int e = 0; e < KPT; ++e) {
-            const int i = e * blockDim.x + threadIdx.x;
-            rawv[e] = __ldg(src + (i < n ? i : 0));
+            p[e] = run;
+            run += (double)r[e];  // +Inf past the end: those positions are never asked for
         }
-        // clipping threshold of this bucket: c times the standard deviation about the mean (none: +Inf)
-        float tau = __int_as_float(0x7f800000);
-        if (A.clip_c > 0.f) {
-            const double v0 = (double)__ldg(src);
-            double s1 = 0.0, s2 = 0.0;
-#pragma unroll
-            for (int e = 0; e < KPT; ++e) {
-                if (e * (int)blockDim.x + (int)threadIdx.x < n) {
-                    const double dv = (double)rawv[e] - v0;
-                    s1 += dv;
-                    s2 += dv * dv;
-                }
-            }
-            s1 = bkt_block_sum(s1, sh_d);
-            s2 = bkt_block_sum(s2, sh_d);
-            double var = (s2 - s1 * s1 / (double)n) / (double)n;
-            if (!(var > 0.0)) var = 0.0;  // also a non-finite bucket: everything clips to 0
-            tau = (float)((double)A.clip_c * sqrt(var));
-        }
+    } else {
+        pre[t] = base;
+    }
+}
 
-        if (A.scheme == OGQ_BINGRAD_B) {
-            // ---- BinGrad-b: b_0 = mean, b_{-1}, b_1 = conditional means, optional Lloyd updates
-            double sum = 0.0;
-            int bad = 0;
+// Shared memory of one team besides the sort's: level records and the quantizer's table.
+struct BktShared {
+    BktLevel lv[kBktLevels];
+    float2 tab[kMaxLevels];  // {level k, width of the segment above it}
+};
+
+// Scratch of a CTA team's block-wide sums and scans, and of the pairs its warps share in the sort.
+template <bool WARP>
+struct BktScratch {
+    double d[WARP ? 1 : 3 * kBktMaxWarps];
+    uint32_t u[WARP ? 1 : 2 * kBktMaxWarps];
+    float edge[WARP ? 1 : 4 * kBktMaxWarps];
+};
+
+// The whole path on bucket j.  EXACT: the bucket fills the team, KPT values for every thread (every full
+// bucket whose length is a power of two); otherwise positions are compared with the bucket's length.
+template <int BITS, int KPT, bool WARP, bool FULL, bool EXACT>
+__device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKeys& pk, int j, int next_j, int len, unsigned char* mem,
+                                               BktShared& S, BktScratch<WARP>& X)
+{
+    constexpr bool kKeep = KPT <= 16;  // the thread's values stay in registers from the load to the quantizer
+    const int lane = threadIdx.x & 31;
+    const int t = WARP ? lane : (int)threadIdx.x, nt = WARP ? 32 : (int)blockDim.x;
+    const int tw = WARP ? 0 : (int)(threadIdx.x >> 5), ntw = nt >> 5;  // warp inside the team
+    const int s = A.s;
+    const bool orq = A.scheme == OGQ_ORQ, pbs = A.scheme == OGQ_BINGRAD_PB, threshold = A.scheme == OGQ_BINGRAD_B;
+    const int nl = orq ? s : 2;
+    float* sv = reinterpret_cast<float*>(mem);
+    uint32_t* cells = reinterpret_cast<uint32_t*>(mem);
+    double* pre = reinterpret_cast<double*>(mem + (size_t)nt * (KPT + (KPT >= 8 ? 4 : 0)) * sizeof(float));
+    const uint32_t tabaddr = (uint32_t)__cvta_generic_to_shared(S.tab);
+    const uint32_t tab4 = tabaddr * (1u + (1u << BITS) + (1u << (2 * BITS)) + (1u << (3 * BITS)));
+    {
+        const float* src = A.grad + (int64_t)j * A.d;
+        const int n = EXACT ? KPT * nt : len;
+        int stbits = 0;
+        // Element 4 u + c of thread t is value 4 (u nt + t) + c of the bucket: 128-bit loads, all issued
+        // before the first use, and the arrangement the quantizer works in.
+        auto index = [&](int e) -> int { return 4 * ((e >> 2) * nt + t) + (e & 3); };
+        auto have = [&](int e) -> bool { return EXACT || index(e) < n; };
+        auto load4 = [&](int u) -> float4 {
+            const int i = index(4 * u);
+            if (EXACT || i + 3 < n) return __ldg(reinterpret_cast<const float4*>(src + i));
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i < n) v.x = __ldg(src + i);
+            if (i + 1 < n) v.y = __ldg(src + i + 1);
+            if (i + 2 < n) v.z = __ldg(src + i + 2);
+            return v;
+        };
+        float raw[kKeep ? KPT : 1] = {};
+        if constexpr (kKeep) {
+#pragma unroll
+            for (int u = 0; u < KPT / 4; ++u) {
+                const float4 v = load4(u);
+                raw[4 * u] = v.x; raw[4 * u + 1] = v.y; raw[4 * u + 2] = v.z; raw[4 * u + 3] = v.w;
+            }
+        }
+        // the next bucket of this team: asked of L2 now
+        if (t == 0 && next_j < A.nb - 1) prefetch_l2(A.grad + (int64_t)next_j * A.d, (uint32_t)A.d * 4u);
+        auto value = [&](int e) -> float {
+            if constexpr (kKeep) return raw[e];
+            else return __ldg(src + (have(e) ? index(e) : 0));
+        };
+
+        // magnitudes: largest (also tells non-finite values), mean of the leading bits; variance if clipping
+        float tau = __int_as_float(0x7f800000);
+        uint32_t maxbits = 0u, meanbits = 0u;
+        {
+            const double v0 = A.clip_c > 0.f ? (double)__ldg(src) : 0.0;
+            double sums[2] = {0.0, 0.0};
 #pragma unroll
             for (int e = 0; e < KPT; ++e) {
-                if (e * (int)blockDim.x + (int)threadIdx.x < n) {
-                    const float raw = rawv[e];
-                    bad |= ((__float_as_uint(raw) & 0x7f800000u) == 0x7f800000u);
-                    sum += (double)copysignf(fminf(fabsf(raw), tau), raw);
+                if (have(e)) {
+                    const float v = value(e);
+                    const uint32_t m = __float_as_uint(v) & 0x7fffffffu;
+                    maxbits = max(maxbits, m);
+                    if (e % 4 == 0) meanbits += m >> 16;
+                    if (A.clip_c > 0.f) {
+                        const double dv = (double)v - v0;
+                        sums[0] += dv;
+                        sums[1] += dv * dv;
+                    }
                 }
             }
-            sum = bkt_block_sum(sum, sh_d);
-            if (__syncthreads_or(bad)) stbits |= OGQ_ST_NONFINITE;
-            float b0 = (float)(sum / (double)n);
+            team_max_sum<WARP>(maxbits, meanbits, X.u);
+            meanbits = (uint32_t)((float)meanbits / (float)((n + 3) >> 2));  // of every fourth value
+            if (A.clip_c > 0.f) {
+                team_sum<WARP>(sums, X.d);
+                double var = (sums[1] - sums[0] * sums[0] / (double)n) / (double)n;
+                if (!(var > 0.0)) var = 0.0;  // also a non-finite bucket: everything clips to 0
+                tau = (float)((double)A.clip_c * sqrt(var));
+            }
+        }
+        const bool bad = maxbits >= 0x7f800000u;
+        if (bad) stbits |= OGQ_ST_NONFINITE;
+        // clipped, and -0 as 0 (no clipping: tau = +Inf, which also turns a NaN into an infinity)
+        auto clip = [&](float x) -> float { return copysignf(fminf(fabsf(x), tau), x) + 0.0f; };
+        if constexpr (kKeep) {
+            if (A.clip_c > 0.f || bad) {
+#pragma unroll
+                for (int e = 0; e < KPT; ++e) raw[e] = clip(raw[e]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < KPT; ++e) raw[e] += 0.0f;
+            }
+        }
+        auto clipped = [&](int e) -> float {
+            if constexpr (kKeep) return raw[e];
+            else return clip(value(e));
+        };
+        float b0 = 0.f;
+
+        if (threshold) {
+            // ---- BinGrad-b: b_0 = mean, b_{-1}, b_1 = conditional means, optional Lloyd updates
+            double sum[1] = {0.0};
+#pragma unroll
+            for (int e = 0; e < KPT; ++e)
+                if (have(e)) sum[0] += (double)clipped(e);
+            team_sum<WARP>(sum, X.d);
+            b0 = (float)(sum[0] / (double)n);
             long long prev_lo = -1;
             float l_lo = 0.f, l_hi = 0.f;
             for (int it = 0;; ++it) {
-                double s_lo = 0.0, s_hi = 0.0, c_lo = 0.0;
+                double sp[2] = {0.0, 0.0};
+                uint32_t cnt = 0u, none = 0u;
 #pragma unroll
                 for (int e = 0; e < KPT; ++e) {
-                    if (e * (int)blockDim.x + (int)threadIdx.x < n) {
-                        const float raw = rawv[e];
-                        const float v = copysignf(fminf(fabsf(raw), tau), raw);
+                    if (have(e)) {
+                        const float v = clipped(e);
                         const bool below = v < b0;
-                        s_lo += below ? (double)v : 0.0;
-                        s_hi += below ? 0.0 : (double)v;
-                        c_lo += below ? 1.0 : 0.0;
+                        sp[0] += below ? (double)v : 0.0;
+                        sp[1] += below ? 0.0 : (double)v;
+                        cnt += below ? 1u : 0u;
                     }
                 }
-                s_lo = bkt_block_sum(s_lo, sh_d);
-                s_hi = bkt_block_sum(s_hi, sh_d);
-                c_lo = bkt_block_sum(c_lo, sh_d);
-                const long long n_lo = (long long)c_lo, n_hi = (long long)n - n_lo;
+                team_sum<WARP>(sp, X.d);
+                team_max_sum<WARP>(none, cnt, X.u);
+                const long long n_lo = (long long)cnt, n_hi = (long long)n - n_lo;
                 if (n_lo == 0 || n_hi == 0) {
-                    const double m = (n_lo == 0) ? s_hi / (double)n_hi : s_lo / (double)n_lo;
+                    const double m = (n_lo == 0) ? sp[1] / (double)n_hi : sp[0] / (double)n_lo;
                     l_lo = l_hi = (float)m;
                     stbits |= OGQ_ST_CONSTANT;
                     break;
                 }
-                const double m_lo = s_lo / (double)n_lo, m_hi = s_hi / (double)n_hi;
+                const double m_lo = sp[0] / (double)n_lo, m_hi = sp[1] / (double)n_hi;
                 l_lo = (float)m_lo;
                 l_hi = (float)m_hi;
                 if (n_lo == prev_lo) break;
@@ -359,264 +586,161 @@ k_bucket_encode(BktArgs A, const __grid_constant__ PhiloxKeys pk)
                 prev_lo = n_lo;
                 b0 = (float)((m_lo + m_hi) * 0.5);
             }
-            if (threadIdx.x == 0) {
+            if (t == 0) {
                 A.levels[2 * (int64_t)j] = l_lo;
                 A.levels[2 * (int64_t)j + 1] = l_hi;
                 A.thresh[j] = b0;
                 A.status[j] = stbits;
-                sh_b0 = b0;
             }
-            __syncthreads();
         } else {
-            // ---- sorted keys of the bucket (magnitudes for BinGrad-pb): KPT keys per thread, loaded
-            // coalesced (the arrangement before the sort does not matter), sorted in registers, then
-            // written to shared memory in order.  P = KPT * blockDim.x >= d; positions past n hold
-            // the largest key.
-            const int P = KPT * blockDim.x;
-            uint32_t r[KPT];
-            int bad = 0;
-#pragma unroll
-            for (int e = 0; e < KPT; ++e) {
-                const int i = e * blockDim.x + threadIdx.x;
-                uint32_t key = 0xffffffffu;
-                if (i < n) {
-                    const float raw = rawv[e];
-                    bad |= ((__float_as_uint(raw) & 0x7f800000u) == 0x7f800000u);
-                    uint32_t bits = __float_as_uint(copysignf(fminf(fabsf(raw), tau), raw));
-                    if (pbs) key = bits | 0x80000000u;
-                    else {
-                        if (bits == 0x80000000u) bits = 0u;
-                        key = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
-                    }
-                }
-                r[e] = key;
-            }
-            const bool nonfinite = __syncthreads_or(bad) != 0;
-            const int nl = pbs ? 2 : s;
-            if (nonfinite) {
-                stbits |= OGQ_ST_NONFINITE;
-                if (threadIdx.x < nl) sh_lv[threadIdx.x] = 0.f;
+            team_sync<WARP>();  // the previous bucket's levels and table have been read
+            if (bad) {
+                if (t < nl) S.lv[t].v = 0.f;
             } else {
-                bkt_sort_regs<KPT>(r, keys, P);
-                __syncthreads();
-                static_assert(KPT % 4 == 0, "a thread's keys are stored as 128-bit words");
-#pragma unroll
-                for (int e = 0; e < KPT; e += 4)
-                    *reinterpret_cast<uint4*>(keys + threadIdx.x * KPT + e) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
-                __syncthreads();
-                if (pre != nullptr) {
-                    // fp64 prefix sums of the sorted values, from the registers that hold them (thread t
-                    // owns positions t * KPT ...): local sums, one scan over the threads, running sums out
-                    const int p0 = threadIdx.x * KPT;
-                    double ls = 0.0;
-#pragma unroll
-                    for (int e = 0; e < KPT; ++e)
-                        if (p0 + e < n) ls += (double)key_to_float(r[e]);
-                    // exclusive scan of ls in thread order
-                    double inc = ls;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const double nbv = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc = nbv + inc;
-                    }
-                    double wbase = 0.0;
-                    if (nwarps > 1) {
-                        __syncthreads();
-                        if (lane == 31) sh_d[warp] = inc;
-                        __syncthreads();
-                        for (int w = 0; w < warp; ++w) wbase += sh_d[w];
-                    }
-                    double run = wbase + (inc - ls);
+                float r[KPT];
+                bkt_sort<KPT, WARP>(r, sv, cells, X.edge, X.u, n, meanbits, fminf(__uint_as_float(maxbits), tau), !pbs,
+                                    [&](int e) -> float {
+                                        const float v = clipped(e);
+                                        return pbs ? fabsf(v) : v;
+                                    },
+                                    have);
+                BktSorted<KPT, FULL> B;
+                B.sv = sv; B.pre = pre; B.n = n;
+                {
+                    double ls = 0.0, tot;
 #pragma unroll
                     for (int e = 0; e < KPT; ++e)
-                        if (p0 + e < n) { pre[p0 + e] = run; run += (double)key_to_float(r[e]); }
-                    if (n > p0 && n <= p0 + KPT) pre[n] = run;
-                    if (n == 0 && threadIdx.x == 0) pre[0] = 0.0;
-                    __syncthreads();
+                        if (t * KPT + e < n) ls += (double)r[e];
+                    const double base = team_excl_scan<WARP>(ls, X.d, tot);
+                    bkt_prefix<KPT, FULL>(r, pre, t, base);
+                    if (t == nt - 1 && n == KPT * nt) pre[FULL ? bkt_pre_at<KPT>(n) : nt] = tot;
                 }
+                team_sync<WARP>();
                 if (orq) {
-                    if (keys[0] == keys[n - 1]) stbits |= OGQ_ST_CONSTANT;
-                    if (threadIdx.x < s) sh_lvkey[threadIdx.x] = (threadIdx.x == s - 1) ? keys[n - 1] : keys[0];
-                    __syncthreads();
-                    // Algorithm 1: a level after its two brackets, the levels of one depth side by side
-                    for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
-                        if (pre != nullptr && nwarps == 1) {
-                            // one warp holds the bucket
-                            bkt_depth_warp<KPT>(r, keys, pre, sh_lvkey, s, stride, lane);
-                        } else if (pre != nullptr) {
-                            const int q = threadIdx.x;
-                            uint32_t res = 0u;
-                            const bool mine = q < s - 1 && q >= stride && ((q - stride) % (2 * stride)) == 0;
-                            if (mine) res = bkt_qstar_prefix(keys, pre, n, sh_lvkey[q - stride], sh_lvkey[q + stride]);
-                            __syncthreads();
-                            if (mine) sh_lvkey[q] = res;
-                            __syncthreads();
-                        } else {
-                            for (int q = stride; q < s - 1; q += 2 * stride) {
-                                const uint32_t res = bkt_qstar_block(keys, n, sh_lvkey[q - stride], sh_lvkey[q + stride], sh_d);
-                                __syncthreads();
-                                if (threadIdx.x == 0) sh_lvkey[q] = res;
-                                __syncthreads();
-                            }
+                    if (B.at(0) == B.at(n - 1)) stbits |= OGQ_ST_CONSTANT;
+                    if (tw == 0) {
+                        // Algorithm 1: a level after its two brackets, the levels of one depth side by side
+                        if (lane == 0) S.lv[0] = B.level_at(0);
+                        if (lane == 1) S.lv[s - 1] = B.level_at(n - 1);
+                        __syncwarp();
+                        for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
+                            const int q = stride + lane * 2 * stride;
+                            if (q < s - 1) S.lv[q] = B.qstar(S.lv[q - stride], S.lv[q + stride]);
+                            __syncwarp();
                         }
-                    }
-                    // refinement sweeps: every interior level again from its two current neighbours, ascending
-                    for (int it = 0; it < A.iters; ++it) {
-                        if (threadIdx.x == 0) sh_changed = 0;
-                        __syncthreads();
-                        if (pre != nullptr) {
-                            if (threadIdx.x == 0) {
+                        // refinement sweeps: every interior level again from its two current neighbours, ascending
+                        if (lane == 0) {
+                            for (int it = 0; it < A.iters; ++it) {
+                                bool changed = false;
                                 for (int q = 1; q < s - 1; ++q) {
-                                    const uint32_t res = bkt_qstar_prefix(keys, pre, n, sh_lvkey[q - 1], sh_lvkey[q + 1]);
-                                    if (res != sh_lvkey[q]) { sh_lvkey[q] = res; sh_changed = 1; }
+                                    const BktLevel l = B.qstar(S.lv[q - 1], S.lv[q + 1]);
+                                    if (l.v != S.lv[q].v) { S.lv[q] = l; changed = true; }
                                 }
-                            }
-                            __syncthreads();
-                        } else {
-                            for (int q = 1; q < s - 1; ++q) {
-                                const uint32_t res = bkt_qstar_block(keys, n, sh_lvkey[q - 1], sh_lvkey[q + 1], sh_d);
-                                __syncthreads();
-                                if (threadIdx.x == 0 && res != sh_lvkey[q]) { sh_lvkey[q] = res; sh_changed = 1; }
-                                __syncthreads();
+                                if (!changed) break;
                             }
                         }
-                        if (!sh_changed) break;
                     }
-                    if (threadIdx.x < s) sh_lv[threadIdx.x] = key_to_float(sh_lvkey[threadIdx.x]);
-                } else {
+                } else if (tw == 0) {
                     // BinGrad-pb: the last sorted magnitude x_c with g(x_c) = x_c n - sum_{|v| >= x_c} |v| <= 0;
-                    // the sign change lies in [x_c, next magnitude)
-                    auto suffix = [&](int from) -> double {  // sum of the magnitudes keys[from..n)
-                        if (pre != nullptr) return pre[n] - pre[from];
-                        double a = 0.0;
-                        for (int i = from + threadIdx.x; i < n; i += blockDim.x) a += (double)key_to_float(keys[i]);
-                        return bkt_block_sum(a, sh_d);
-                    };
-                    const double tot = suffix(0);
+                    // the sign change lies in [x_c, next magnitude).  g does not decrease along the sorted
+                    // magnitudes: 32 candidates are tried at a time.
+                    const double tot = B.before(n);
                     float b1 = 0.f;
                     if (!(tot > 0.0)) {
                         stbits |= OGQ_ST_CONSTANT;
                     } else {
-                        // g is non-decreasing along the sorted magnitudes: bisection on the index (all threads alike)
-                        int lo = -1, hi = n;  // g(x_lo) <= 0 < g(x_hi)
+                        int lo = 0, hi = n;  // the answer lies in [lo, hi) (position 0 when g is positive everywhere)
                         while (hi - lo > 1) {
-                            const int mid = (lo + hi) >> 1;
-                            const int first = bkt_lower(keys, n, keys[mid]);
-                            const double g = (double)key_to_float(keys[mid]) * (double)n - suffix(first);
-                            if (g <= 0.0) lo = mid; else hi = mid;
+                            const int step = (hi - lo + 31) >> 5;
+                            const int i = lo + lane * step;
+                            bool below = false;
+                            if (i < hi) {
+                                const float x = B.at(i);
+                                below = (double)x * (double)n - (tot - B.before(B.run_begin(i, x))) <= 0.0;
+                            }
+                            const unsigned m = __ballot_sync(0xffffffffu, below);
+                            const int k = m ? 31 - __clz(m) : 0;
+                            lo += k * step;
+                            hi = (lo + step < hi) ? lo + step : hi;
                         }
-                        const int c = lo < 0 ? 0 : lo;
-                        const double x = (double)key_to_float(keys[c]);
-                        const int up = bkt_upper(keys, n, keys[c]);
-                        const double stat_up = suffix(up) / (double)n;
-                        b1 = (float)(stat_up > x ? stat_up : x);
+                        const float x = B.at(lo);
+                        const double stat_up = (tot - B.before(B.run_end(lo, x))) / (double)n;
+                        b1 = (float)(stat_up > (double)x ? stat_up : (double)x);
                     }
-                    if (threadIdx.x == 0) { sh_lv[0] = -b1; sh_lv[1] = b1; }
+                    if (lane < 2) S.lv[lane].v = lane == 0 ? -b1 : b1;
                 }
             }
-            __syncthreads();
-            if (threadIdx.x < nl) {
-                const float cur = sh_lv[threadIdx.x];
-                const float prv = threadIdx.x > 0 ? sh_lv[threadIdx.x - 1] : cur;
-                const float nxt = (int)threadIdx.x + 1 < nl ? sh_lv[threadIdx.x + 1] : cur;
-                sh_w[threadIdx.x] = __fsub_rn(cur, prv);
-                sh_tab[threadIdx.x] = make_float2(cur, __fsub_rn(nxt, cur));
-                A.levels[(int64_t)j * nl + threadIdx.x] = cur;
+            team_sync<WARP>();
+            if (t < nl) {
+                const float cur = S.lv[t].v;
+                const float nxt = t + 1 < nl ? S.lv[t + 1].v : cur;
+                S.tab[t] = make_float2(cur, __fsub_rn(nxt, cur));
+                A.levels[(int64_t)j * nl + t] = cur;
             }
-            if (threadIdx.x == 0) A.status[j] = stbits;
-            __syncthreads();
+            if (t == 0) A.status[j] = stbits;
+            team_sync<WARP>();
         }
 
-        // ---- quantize + pack: the bucket is read again (it is in L2), 128 elements per warp and trip
+        // ---- quantize + pack: 128 consecutive elements per warp and trip
         uint32_t* out = A.packed + (int64_t)j * A.words_per_bucket;
-        const int64_t region = ((int64_t)n * BITS + 31) / 32;
-        const int64_t region4 = (region + 3) / 4 * 4;
-        const bool threshold = A.scheme == OGQ_BINGRAD_B;
-        const float b0 = sh_b0;
-        const int ngroups = (n + 127) >> 7, nfull = n >> 7;
-        const int nl = (orq ? s : 2);
-        constexpr bool kPow2 = (BITS == 1 || BITS == 2 || BITS == 4);
-        constexpr int L = kPow2 ? 8 / BITS : 1;
-        const uint32_t tabaddr = (uint32_t)__cvta_generic_to_shared(sh_tab);
-        const uint32_t tab4 = tabaddr * (1u + (1u << BITS) + (1u << (2 * BITS)) + (1u << (3 * BITS)));
-        float mid = 0.f;
-        PhiloxHoist hz = {};
-        if (!threshold) {
-            mid = sh_tab[(BITS >= 2) ? (1 << (BITS - 2)) : 0].x;
-            hz = philox_hoist(0u, (uint32_t)j, A.stream_id, pk);
-        }
-        uint32_t* wsm = sh_words[warp];
-        const int obit = (lane * 4 * BITS) & 31, oword = (lane * 4 * BITS) >> 5;
-        // (the next group's values are loaded before the current group is worked on)
-        const float4* src4 = reinterpret_cast<const float4*>(src) + lane;
-        float4 vnext = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (warp < nfull) vnext = __ldg(src4 + ((int64_t)warp << 5));
-        for (int g = warp; g < ngroups; g += nwarps) {
+        const int region4 = ((n * BITS + 31) / 32 + 3) / 4 * 4;
+        const int ngroups = (n + 127) >> 7;
+        const float mid = threshold ? 0.f : S.tab[(BITS >= 2) ? (1 << (BITS - 2)) : 0].x;
+        const PhiloxHoist hz = philox_hoist(0u, (uint32_t)j, A.stream_id, pk);
+        const bool writer = packs_word<BITS>(lane);
+        auto group = [&](int g, float4 v) {
+            if constexpr (!kKeep) { v.x = clip(v.x); v.y = clip(v.y); v.z = clip(v.z); v.w = clip(v.w); }
             uint32_t bits4;
-            float4 v = vnext;
-            if (g + nwarps < nfull) vnext = __ldg(src4 + ((int64_t)(g + nwarps) << 5));
-            if (g < nfull) {
-                v.x = copysignf(fminf(fabsf(v.x), tau), v.x);  // clipping (tau = +Inf: none)
-                v.y = copysignf(fminf(fabsf(v.y), tau), v.y);
-                v.z = copysignf(fminf(fabsf(v.z), tau), v.z);
-                v.w = copysignf(fminf(fabsf(v.w), tau), v.w);
-                if (threshold) {
-                    bits4 = ((v.x >= b0) ? 1u : 0u) | ((v.y >= b0) ? 2u : 0u) | ((v.z >= b0) ? 4u : 0u) |
-                            ((v.w >= b0) ? 8u : 0u);
-                } else {
-                    const uint4 r = philox4x32_10_tail(((uint32_t)g << 5) + (uint32_t)lane, hz, pk);
-                    const uint32_t a0 = entry_after_rounding<BITS>(v.x, r.x, tabaddr, mid),
-                                   a1 = entry_after_rounding<BITS>(v.y, r.y, tabaddr, mid),
-                                   a2 = entry_after_rounding<BITS>(v.z, r.z, tabaddr, mid),
-                                   a3 = entry_after_rounding<BITS>(v.w, r.w, tabaddr, mid);
-                    bits4 = (a0 + (a1 << BITS) + (a2 << (2 * BITS)) + (a3 << (3 * BITS)) - tab4) >> 3;
-                }
+            if (threshold) {
+                bits4 = ((v.x >= b0) ? 1u : 0u) | ((v.y >= b0) ? 2u : 0u) | ((v.z >= b0) ? 4u : 0u) | ((v.w >= b0) ? 8u : 0u);
             } else {
-                // the ragged end of the last bucket: element by element
-                const int i0 = (g << 7) + 4 * lane;
-                uint32_t c[4] = {0u, 0u, 0u, 0u};
-                uint4 r = make_uint4(0u, 0u, 0u, 0u);
-                if (!threshold) r = philox4x32_10((uint32_t)(i0 >> 2), 0u, (uint32_t)j, A.stream_id, pk);
-                const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
+                const uint4 rnd = philox4x32_10_tail(((uint32_t)g << 5) + (uint32_t)lane, hz, pk);
+                const uint32_t a0 = entry_after_rounding<BITS>(v.x, rnd.x, tabaddr, mid),
+                               a1 = entry_after_rounding<BITS>(v.y, rnd.y, tabaddr, mid),
+                               a2 = entry_after_rounding<BITS>(v.z, rnd.z, tabaddr, mid),
+                               a3 = entry_after_rounding<BITS>(v.w, rnd.w, tabaddr, mid);
+                bits4 = (a0 + (a1 << BITS) + (a2 << (2 * BITS)) + (a3 << (3 * BITS)) - tab4) >> 3;
+            }
+            const int left = n - ((g << 7) + 4 * lane);  // elements of this lane inside the bucket
+            if (!EXACT && left < 4) bits4 &= left > 0 ? (1u << (left * BITS)) - 1u : 0u;
+            const uint32_t word = assemble_words<BITS>(bits4, lane);
+            const int w = g * (4 * BITS) + packed_word<BITS>(lane);
+            if (writer && (EXACT || w < region4)) out[w] = word;
+        };
+        if constexpr (kKeep) {
+            // (rolled: the unrolled groups' instructions were too many for the instruction cache)
+            constexpr int kSide = KPT >= 8 ? 2 : 1;  // groups side by side
+#pragma unroll 1
+            for (int u = 0; u * ntw + tw < ngroups; u += kSide) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (i0 + e < n) {
-                        const float raw = __ldg(src + i0 + e);
-                        const float x = copysignf(fminf(fabsf(raw), tau), raw);
-                        if (threshold) {
-                            c[e] = (x >= b0) ? 1u : 0u;
-                        } else {
-                            int idx = 0;
-                            for (int step = (BITS >= 2) ? (1 << (BITS - 2)) : 0; step >= 1; step >>= 1)
-                                if (sh_lv[idx + step] <= x) idx += step;
-                            const float dd = __fsub_rn(x, sh_lv[idx]);
-                            const float lhs = __fmul_rn((float)(rw[e] >> 8), sh_w[idx + 1]);
-                            const float rhs = __fmul_rn(dd, 16777216.0f);
-                            c[e] = (uint32_t)idx + ((lhs < rhs) ? 1u : 0u);
-                        }
-                    }
-                }
-                bits4 = c[0] | (c[1] << BITS) | (c[2] << (2 * BITS)) | (c[3] << (3 * BITS));
+                for (int q = 0; q < kSide; ++q)
+                    if (EXACT || (u + q) * ntw + tw < ngroups)
+                        group((u + q) * ntw + tw, make_float4(raw[4 * q], raw[4 * q + 1], raw[4 * q + 2], raw[4 * q + 3]));
+#pragma unroll
+                for (int e = 0; e + 4 * kSide < KPT; ++e) raw[e] = raw[e + 4 * kSide];
             }
-            if constexpr (kPow2) {
-                const uint32_t word = assemble_words<BITS>(bits4, lane);
-                if ((lane & (L - 1)) == 0) {
-                    const int64_t widx = (int64_t)g * (4 * BITS) + lane / L;
-                    if (widx < region4) out[widx] = word;
-                }
-            } else {
-                atomicOr(wsm + oword, bits4 << obit);
-                if (obit + 4 * BITS > 32) atomicOr(wsm + oword + 1, bits4 >> (32 - obit));
-                __syncwarp();
-                if (lane < 4 * BITS) {
-                    const uint32_t word = atomicExch(wsm + lane, 0u);
-                    const int64_t widx = (int64_t)g * (4 * BITS) + lane;
-                    if (widx < region4) out[widx] = word;
-                }
-                __syncwarp();
-            }
+        } else {
+            for (int u = 0; u * ntw + tw < ngroups; ++u) group(u * ntw + tw, load4(u));
         }
-        (void)nl;
+    }
+}
+
+template <int BITS, int KPT, bool WARP, bool FULL, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_bucket_encode(BktArgs A, size_t team_bytes, const __grid_constant__ PhiloxKeys pk)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int kTeams = WARP ? kBktWarpsPerCta : 1;
+    __shared__ BktShared sh_team[kTeams];
+    __shared__ BktScratch<WARP> scratch;
+    const int team = WARP ? (int)(threadIdx.x >> 5) : 0;
+    const int P = KPT * (WARP ? 32 : (int)blockDim.x);
+    const int step = (int)gridDim.x * kTeams;
+    for (int j = (int)blockIdx.x * kTeams + team; j < A.nb; j += step) {
+        const int64_t left = A.total - (int64_t)j * A.d;
+        const int n = left < (int64_t)A.d ? (int)left : A.d;
+        unsigned char* mem = smem + (size_t)team * team_bytes;
+        if (n == P) bkt_encode_one<BITS, KPT, WARP, FULL, true>(A, pk, j, j + step, n, mem, sh_team[team], scratch);
+        else bkt_encode_one<BITS, KPT, WARP, FULL, false>(A, pk, j, j + step, n, mem, sh_team[team], scratch);
     }
 }
 
@@ -720,16 +844,6 @@ cudaError_t launch_bucket_decode_sum(const uint32_t* const* d_packed_k, const fl
     return cudaGetLastError();
 }
 
-static int bkt_pow2(int d);
-
-static size_t bkt_smem_bytes(int d)
-{
-    const size_t P = (size_t)bkt_pow2(d);
-    size_t b = P * sizeof(uint32_t);
-    if (d <= kBktPrefixMaxD) b += (P + 1) * sizeof(double);
-    return (b + 15) / 16 * 16;
-}
-
 static int bkt_pow2(int d)
 {
     int P = 128;
@@ -737,49 +851,65 @@ static int bkt_pow2(int d)
     return P;
 }
 
-// keys per thread of the register sort: 4 for the shortest buckets, 32 for the longest, else 16
-// (measured on 512- and 2048-element buckets: 16 keys per thread beat 8 and 4, although fewer
-// warps are resident: the stages that stay in registers are the cheapest)
-static int bkt_kpt(int d)
+// Shared memory of one team: the sorted values and their prefix sums, or the cells they are sorted with.
+template <int KPT, bool FULL>
+static size_t bkt_team_bytes(int threads)
 {
-    const int P = bkt_pow2(d);
-    return P <= 256 ? 4 : (P <= 16384 ? 16 : 32);
+    const size_t P = (size_t)KPT * threads;
+    const size_t sorted = (P + (KPT >= 8 ? P / KPT * 4 : 0)) * sizeof(float) +
+                          (FULL ? P + P / KPT + 2 : (size_t)threads + 1) * sizeof(double);
+    const size_t cells = (size_t)threads * (kBktCellsPerThread<KPT> + 4) * sizeof(uint32_t);
+    return ((sorted > cells ? sorted : cells) + 15) / 16 * 16;
 }
 
-template <int BITS, int KPT>
+template <int BITS, int KPT, bool WARP, bool FULL, int MAXT, int MINB>
 static cudaError_t bkt_launch(const BktArgs& A, const PhiloxKeys& pk, int sm_count, cudaStream_t stream)
 {
-    const size_t smem = bkt_smem_bytes(A.d);
-    const int threads = bkt_pow2(A.d) / KPT;
-    static std::atomic<size_t> attr_bytes[64];  // dynamic shared-memory limit set so far, per device
+    const int team_threads = WARP ? 32 : bkt_pow2(A.d) / KPT;
+    const int teams = WARP ? kBktWarpsPerCta : 1;
+    const size_t team_bytes = bkt_team_bytes<KPT, FULL>(team_threads);
+    const size_t smem = team_bytes * teams;
+    auto kernel = k_bucket_encode<BITS, KPT, WARP, FULL, MAXT, MINB>;
+    // The dynamic shared-memory limit and the resident CTAs per SM, looked up once per device and size.
+    struct Known { std::atomic<int> resident[6]; };
+    static Known known[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (smem > 48 * 1024 && (dev < 0 || dev >= 64 || attr_bytes[dev].load(std::memory_order_acquire) < smem)) {
-        e = cudaFuncSetAttribute(k_bucket_encode<BITS, KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(160 * 1024));
+    int slot = 0;
+    while ((32 << slot) < team_threads) ++slot;
+    int per_sm = (dev >= 0 && dev < 64) ? known[dev].resident[slot].load(std::memory_order_acquire) : 0;
+    if (per_sm == 0) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_bytes[dev].store(160 * 1024, std::memory_order_release);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, team_threads * teams, smem);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) per_sm = 1;
+        if (dev >= 0 && dev < 64) known[dev].resident[slot].store(per_sm, std::memory_order_release);
     }
-    int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bucket_encode<BITS, KPT>, threads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
     int64_t ctas = (int64_t)per_sm * sm_count;
-    if (ctas > A.nb) ctas = A.nb;
+    const int64_t need = ((int64_t)A.nb + teams - 1) / teams;
+    if (ctas > need) ctas = need;
     launch_begin("k_bucket_encode", stream);
-    k_bucket_encode<BITS, KPT><<<(int)ctas, threads, smem, stream>>>(A, pk);
+    kernel<<<(int)ctas, team_threads * teams, smem, stream>>>(A, team_bytes, pk);
     launch_end(stream);
     return cudaGetLastError();
 }
 
+// Values per thread: a bucket of up to 512 elements is one warp's (4, 8 or 16 per lane: its barriers are
+// warp barriers and the SM works on as many buckets as it has warps), longer ones a CTA's with 16 per
+// thread, the longest with 32.
 template <int BITS>
 static cudaError_t bkt_dispatch(const BktArgs& A, const PhiloxKeys& pk, int sm_count, cudaStream_t stream)
 {
-    switch (bkt_kpt(A.d)) {
-        case 4: return bkt_launch<BITS, 4>(A, pk, sm_count, stream);
-        case 16: return bkt_launch<BITS, 16>(A, pk, sm_count, stream);
-        default: return bkt_launch<BITS, 32>(A, pk, sm_count, stream);
-    }
+    const int P = bkt_pow2(A.d);
+    if (P == 128) return bkt_launch<BITS, 4, true, true, 128, 8>(A, pk, sm_count, stream);
+    if (P == 256) return bkt_launch<BITS, 8, true, true, 128, 8>(A, pk, sm_count, stream);
+    if (P <= kBktWarpD) return bkt_launch<BITS, 16, true, true, 128, 5>(A, pk, sm_count, stream);
+    if (P <= kBktPrefixMaxD) return bkt_launch<BITS, 16, false, true, 256, 3>(A, pk, sm_count, stream);
+    if (P == 8192) return bkt_launch<BITS, 16, false, false, 512, 2>(A, pk, sm_count, stream);
+    if (P == 16384) return bkt_launch<BITS, 16, false, false, 1024, 1>(A, pk, sm_count, stream);
+    return bkt_launch<BITS, 32, false, false, 1024, 1>(A, pk, sm_count, stream);
 }
 
 cudaError_t launch_bucket_encode(const float* d_grad, int64_t total, int d, int scheme, int s, int iters,

@@ -9,17 +9,52 @@ namespace ogq {
 constexpr int kMaxLevels = 32;
 constexpr int kMaxWorkers = 64;
 
-// OR-combine the 4*BITS-bit chunk of each lane into words, BITS = 1, 2 or 4: a word is made of
-// 8, 4, 2 neighbouring lanes and the first lane of each such set returns it (word index lane / L).
+// Combines the 4*BITS-bit chunk of each lane into the 4*BITS words of a 128-element group.  A word whose
+// width is a whole number of chunks (BITS = 1, 2, 4) is OR-ed together by a butterfly inside its 8, 4 or
+// 2 lanes.  3- and 5-bit chunks straddle words: eight lanes hold 3 or 5 words, and lane i of the eight
+// fetches the three or four chunks that touch word i by shuffle and shifts them into place (shl.b32 gives
+// 0 for shifts of 32 and more, which drops the chunks past the word).  Registers only: OR-ing the chunks
+// together with shared-memory atomics serialised on the words that neighbouring lanes share.
+// The lanes with packs_word() true then hold word packed_word() of the group.
+template <int BITS>
+__device__ __forceinline__ bool packs_word(int lane)
+{
+    constexpr bool kPow2 = (BITS & (BITS - 1)) == 0;
+    constexpr int L = kPow2 ? 8 / BITS : 1;
+    return kPow2 ? (lane & (L - 1)) == 0 : (lane & 7) < BITS;
+}
+
+template <int BITS>
+__device__ __forceinline__ int packed_word(int lane)
+{
+    constexpr bool kPow2 = (BITS & (BITS - 1)) == 0;
+    constexpr int L = kPow2 ? 8 / BITS : 1;
+    return kPow2 ? lane / L : (lane >> 3) * BITS + (lane & 7);
+}
+
 template <int BITS>
 __device__ __forceinline__ uint32_t assemble_words(uint32_t chunk, int lane)
 {
-    static_assert(BITS == 1 || BITS == 2 || BITS == 4, "other widths are combined in shared memory");
-    constexpr int L = 8 / BITS;
-    uint32_t x = chunk << (4 * BITS * (lane & (L - 1)));
+    if constexpr ((BITS & (BITS - 1)) == 0) {
+        constexpr int L = 8 / BITS;
+        uint32_t x = chunk << (4 * BITS * (lane & (L - 1)));
 #pragma unroll
-    for (int o = 1; o < L; o <<= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
+        for (int o = 1; o < L; o <<= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
+        return x;
+    } else {
+        constexpr int W = 4 * BITS;                 // bits per lane
+        const int bit = (lane & 7) * 32;            // first bit of this lane's word inside the eight chunks
+        const int a = (lane & 24) + bit / W, o = bit % W;
+        uint32_t x = __shfl_sync(0xffffffffu, chunk, a & 31) >> o;
+#pragma unroll
+        for (int u = 1; u <= (BITS == 3 ? 3 : 2); ++u) {
+            const uint32_t c = __shfl_sync(0xffffffffu, chunk, (a + u) & 31);
+            uint32_t y;
+            asm("shl.b32 %0, %1, %2;" : "=r"(y) : "r"(c), "r"(u * W - o));
+            x |= y;
+        }
+        return x;
+    }
 }
 
 // Segment search and rounding decision of one element on the fast path.  `tabaddr` is the shared
