@@ -13,6 +13,34 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kChunkAlign = 1024;   // flat chunk boundaries are multiples of this many elements
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch: a kernel of this library is put on the device while the kernel before it
+// in the stream is still running and waits, before its first access to global memory, until that one has
+// finished and its writes are visible.  The launch latency of every kernel of a chain so overlaps with the
+// kernel before it.  Every kernel launched with launch_pdl calls pdl_wait() in all its threads, so
+// completion passes from kernel to kernel, and only then allows its own successor to be launched: at most
+// two kernels of a chain are on the device.  What one kernel of a chain writes and a later one reads goes
+// through L2 (__ldcg), never through the read-only path, whose loads the compiler may move.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), int ctas, int threads, size_t smem, cudaStream_t stream, Args... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Flat partition of the bucket: CTA c owns elements [c*chunk, (c+1)*chunk).
 // ---------------------------------------------------------------------------
 struct FlatGrid {

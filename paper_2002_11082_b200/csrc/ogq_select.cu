@@ -27,8 +27,12 @@
 #include "ogq_common.cuh"
 #include "ogq_internal.h"
 #include "ogq_select_solver.cuh"
+#include "ogq_sort.cuh"
 #include "ogq_ws.h"
 
+#ifndef OGQ_CHUNK
+#define OGQ_CHUNK (total > ((int64_t)1 << 22) ? 131072 : 16384)
+#endif
 namespace ogq {
 
 constexpr int kSelThreads = 512;    // two CTAs are resident per SM: a CTA in a solver pass, a sort or a
@@ -37,14 +41,17 @@ constexpr int kSelResident = 2;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelW = 16;          // binades in the fine window of round 1
 constexpr int kSelM = 7;           // log2(cells per binade) in the window
-constexpr int kSmallN = 4096;      // tensors up to this size are sorted in shared memory
-constexpr int kMidN = 131072;      // tensors up to this size are solved start to finish by one CTA of their own
+constexpr int kSmallN = 8192;      // tensors up to this size are solved in shared memory
+constexpr int kSortN = 8192;       // candidates from which one CTA finishes a larger tensor
+constexpr int kAloneN = 131072;    // tensors up to this size are finished by one CTA after round 2
 constexpr int kStageCap = 320;     // per-warp staging entries for compaction
 constexpr int kParkMax = 256;      // values one warp can park between two checks in the tail of round 2 (32 lanes x 8)
 constexpr int kMaxSlices = 64;     // CTAs that share one tensor's copied keys in round 3
 constexpr int kSliceElems = 16384;
 constexpr int kMaxRounds = 32;
-constexpr int kSortScanMax = 65536;  // longest copied-key list one CTA filters for the sorting finish
+constexpr int kScanMax = 16384, kScanMaxAlone = 65536;  // longest list of copied keys one CTA looks through for the last few
+                                                        // thousand (the second where no other kernel would do it)
+constexpr int kRefineMax = 32;     // runs of candidate cells that make up the intervals of the next round
 
 constexpr int kRound1Mag = 256 - kSelW + (kSelW << kSelM);  // round-1 cells per sign
 constexpr int kRound1Cells = 2 * kRound1Mag;
@@ -53,13 +60,13 @@ static_assert(kRound1Cells <= kCells, "round-1 cells exceed the budget");
 struct TState {
     int done, round, m, hi_e;
     unsigned kmin_inv, kmax, nonfinite, arrive;
-    unsigned long long arrived;  // elements of the current pass whose counts have been flushed
     unsigned expected;
     int compact_only;  // the next pass only copies the keys inside the intervals: they fit one sort
     int overflow;      // the current pass dropped copies that did not fit the tensor's region
     int from_grad;     // the current pass (round >= 3) reads the gradient, not the previous pass's copies
     unsigned long long cursor[2];
     long long n;
+    long long cand;  // elements inside the intervals
     double stot;
     Interval iv[kMaxIv];
     ExactLv lv[kMaxLv];
@@ -115,8 +122,7 @@ static SelWs sel_carve(void* base, int T, int64_t total)
 // ---------------------------------------------------------------------------
 constexpr size_t kSmemHist = 3 * kCells * sizeof(uint32_t);
 constexpr size_t kSmemStage = kSelWarps * kStageCap * sizeof(uint32_t);
-constexpr size_t kSmemSolver = kSlots * (sizeof(uint32_t) + sizeof(double) + 1) + 32;
-constexpr size_t kSmemBytes = (kSmemHist + kSmemStage > kSmemSolver) ? kSmemHist + kSmemStage : kSmemSolver;
+constexpr size_t kSmemBytes = kSmemHist + kSmemStage;
 
 struct Table {  // interval lookup table of the tensor being streamed
     uint32_t klo[kMaxIv];
@@ -162,29 +168,29 @@ __device__ __forceinline__ void table_from_intervals_cta(Table& tb, const Interv
     }
 }
 
-// Round-1 intervals: coarse (one cell per binade) outside a window of kSelW binades that ends
-// at binade hi_e, fine inside.  Negative values only for signed keys.
-__device__ __forceinline__ int round1_intervals(int hi_e, bool magnitude_only, Interval* iv)
+// Round-1 interval j of the layout: coarse (one cell per binade) outside a window of kSelW binades that ends
+// at binade hi_e, fine inside; six of them, in key order, or the three of the non-negative values only.
+// (One of them may have no cells.)
+__device__ __forceinline__ Interval round1_interval(int hi_e, bool magnitude_only, int j)
 {
     const int lo_e = hi_e - kSelW;
-    int m = 0, cb = 0;
-    auto add = [&](uint32_t klo, int ncell, int sh) {
-        if (ncell <= 0) return;
-        Interval& x = iv[m++];
-        x.klo = klo; x.sh = sh; x.ncell = ncell;
-        x.khi = klo + (uint32_t)((((unsigned long long)ncell) << sh) - 1ull);
-        x.cellbase = cb; x.pad = 0; x.cbefore = 0; x.sbefore = 0.0;
-        cb += ncell;
-    };
-    if (!magnitude_only) {
-        add(0u, 256 - hi_e, 23);
-        add(0x80000000u - ((uint32_t)hi_e << 23), kSelW << kSelM, 23 - kSelM);
-        add(0x80000000u - ((uint32_t)lo_e << 23), lo_e, 23);
-    }
-    add(0x80000000u, lo_e, 23);
-    add(0x80000000u + ((uint32_t)lo_e << 23), kSelW << kSelM, 23 - kSelM);
-    add(0x80000000u + ((uint32_t)hi_e << 23), 256 - hi_e, 23);
-    return m;
+    if (magnitude_only) j += 3;
+    // cells of the coarse part below the window, of the window and of the part above it, mirrored for negative values
+    const int part = j < 3 ? 2 - j : j - 3;
+    const int ncell = part == 0 ? lo_e : part == 1 ? (kSelW << kSelM) : 256 - hi_e;
+    const int before = part == 0 ? 0 : part == 1 ? lo_e : lo_e + (kSelW << kSelM);  // cells nearer to zero
+    const int edge = part == 0 ? 0 : part == 1 ? lo_e : hi_e;                        // lowest binade
+    const int width = part == 1 ? kSelW : ncell;                                     // in binades
+    Interval x;
+    x.sh = part == 1 ? 23 - kSelM : 23;
+    x.ncell = ncell;
+    x.klo = j < 3 ? 0x80000000u - ((uint32_t)(edge + width) << 23) : 0x80000000u + ((uint32_t)edge << 23);
+    x.khi = x.klo + (uint32_t)((((unsigned long long)ncell) << x.sh) - 1ull);
+    x.cellbase = magnitude_only ? before : j < 3 ? kRound1Mag - before - ncell : kRound1Mag + before;
+    x.pad = 0;
+    x.cbefore = 0;
+    x.sbefore = 0.0;
+    return x;
 }
 
 // Round-1 cell of a value, computed directly (same layout as round1_intervals produces):
@@ -879,20 +885,6 @@ __device__ __forceinline__ void flush_hist(const uint32_t* smem_hist, int ncells
     }
 }
 
-// Sum of a double over the CTA in a fixed order; valid in thread 0.  scratch: kSelWarps doubles.
-__device__ __forceinline__ double sel_block_sum(double x, double* scratch)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = x;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < kSelWarps; ++i) r += scratch[i];
-    return r;
-}
-
 // ---------------------------------------------------------------------------
 // Block-wide exclusive scan of (count, sum) pairs in thread order (fixed order).
 // ---------------------------------------------------------------------------
@@ -927,6 +919,13 @@ __device__ __forceinline__ void block_excl_scan(unsigned long long& c, double& s
     s = (lane == 0) ? bs : bs + ps;
 }
 
+// The kernels from here to solver_round work on one tensor with one CTA and run their code once: what they
+// spend is the latency of barriers, of dependent loads and, most of all, of instructions that are not in the
+// instruction cache yet (about 300 cycles for every eight).  So loops stay rolled, values live in shared
+// memory instead of unrolled registers, a warp works on one level with searches spread over its lanes, and
+// fp64 division is one function.
+__device__ __noinline__ double fp64_div(double a, double b) { return a / b; }
+
 struct SolverShared {
     Interval iv[kMaxIv];
     Interval niv[kMaxIv];
@@ -935,573 +934,815 @@ struct SolverShared {
     unsigned long long sc[kSelWarps];
     double ss[kSelWarps];
     int pb_a, pb_b, pb_c;
-    int done, nm, internal;
+    int done, nm, internal, nopen;
     uint32_t offc[kMaxIv];    // per-interval shifts of the scanned prefix arrays
     double offs[kMaxIv];
-    int nr, ra[kMaxLv], rb[kMaxLv];  // open slot ranges of this pass
-    int pa[kMaxIv], pb[kMaxIv];      // pieces cut out of them
+    uint32_t marks[(kSlots + 31) / 32];  // candidate cells, one bit per slot
+    int pa[kRefineMax], pb[kRefineMax];  // runs of candidate cells
     long long cand;           // elements inside the new intervals
-    int n_keys, n_unique;     // sorting finish
-    int ivstart[kMaxIv], ivufirst[kMaxIv];
-    double ivpre[kMaxIv];
+    // sorting finish
+    uint32_t lo[kMaxIv], hi[kMaxIv];  // keys of the intervals (padded: no key lies in the surplus ones)
+    uint32_t base[kMaxIv];            // first cell of the interval
+    int sh[kMaxIv];                   // log2 of the keys per cell
+    int start[kMaxIv + 1];            // position of the interval's first value
+    double pre[kMaxIv];               // sum of the values before it
+    int n_keys;
+    uint32_t below[kSelWarps];
 };
 
-__device__ __forceinline__ int find_new_interval(const SolverShared& S, uint32_t key)
+// First of the ascending a[0 .. n) that exceeds pos (n if none does), by the 32 lanes of a warp: 32 probes a
+// step, three steps for 16384 entries (a binary search is fourteen dependent shared-memory reads).
+__device__ __forceinline__ int warp_upper_bound(const uint32_t* a, int n, uint32_t pos)
 {
-    int lo = 0, hi = S.nm;  // last interval with klo <= key
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (S.niv[mid].klo <= key) lo = mid; else hi = mid;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = n;  // the answer lies in [lo, hi]
+#pragma unroll 1
+    while (lo < hi) {
+        const int step = (hi - lo + 31) >> 5;
+        const int i = lo + lane * step;
+        const int k = __popc(__ballot_sync(0xffffffffu, i < hi && a[i] <= pos));  // a prefix of the lanes
+        const int nhi = lo + k * step;
+        if (k > 0) lo += (k - 1) * step + 1;
+        if (nhi < hi) hi = nhi;
     }
-    return (key >= S.niv[lo].klo && key <= S.niv[lo].khi) ? lo : -1;
+    return lo;
 }
 
 // ---------------------------------------------------------------------------
-// Ascending bitonic sort of P keys in shared memory (P a power of two, at most 8 * kSelThreads),
-// called by all threads of the CTA; the keys are ordered on return (a barrier has been passed).
-// Compare-exchange distances of 256 and more are done by the whole CTA with a barrier per stage;
-// distances 8..128 stay inside an aligned block of 256 keys, which one warp owns and orders with
-// warp barriers only; distances 4, 2, 1 stay inside 8 consecutive keys, which one lane holds in
-// registers.  For 4096 keys that is 10 CTA barriers instead of 78.
+// Order statistics of up to kSortN values in shared memory.  The values are grouped by cells, a monotone
+// function of the value with about one value to a cell, in ascending order of the cells and in any order
+// inside one; a rank is found by a search over the cells and a selection inside its cell, both by a warp.
+// (Nothing is sorted: a level needs one rank, and the sums before it need only know which values are
+// smaller.)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void cmpx(uint32_t& a, uint32_t& b, bool up)
+constexpr int kChunkN = kSortN / kSelThreads;  // values per prefix sum
+
+struct CellIndex {
+    float* sv;          // the values
+    uint32_t* end;      // [nc] position after the last value of every cell
+    uint16_t* cell;     // [n] cell of every value, while they are being placed
+    double* pre;        // [kSelThreads + 1] sum of the values before every kChunkN-th position
+    int n, nc;
+};
+
+// Shared memory: the cells, the values, their cells' numbers, the prefix sums, the list of the gathered keys.
+constexpr int kFinishCells = 16384, kSmallCells = 8192;
+template <int NC>
+constexpr size_t kIndexBytes = (size_t)NC * 4 + (size_t)kSortN * 6 + (kSelThreads + 1) * 8;
+
+__device__ __forceinline__ CellIndex index_at(unsigned char* smem, int n, int nc)
 {
-    const uint32_t lo = a < b ? a : b, hi = a < b ? b : a;
-    a = up ? lo : hi;
-    b = up ? hi : lo;
+    CellIndex X;
+    X.end = reinterpret_cast<uint32_t*>(smem);
+    X.sv = reinterpret_cast<float*>(smem + (size_t)nc * 4);
+    X.cell = reinterpret_cast<uint16_t*>(smem + (size_t)nc * 4 + (size_t)kSortN * 4);
+    X.pre = reinterpret_cast<double*>(smem + (size_t)nc * 4 + (size_t)kSortN * 6);
+    X.n = n;
+    X.nc = nc;
+    return X;
 }
 
-__device__ void block_bitonic_sort(uint32_t* keys, int P)
+// fetch(i): value i of n, cell_of(i): its cell.  Called by every thread of the CTA; nc is a multiple of
+// 128 kSelWarps.
+template <class Fetch, class CellOf>
+__device__ __forceinline__ void index_build(const CellIndex& X, SolverShared& S, Fetch fetch, CellOf cell_of)
 {
-    if (P < 256) {  // few stages: the plain network
-        for (int k = 2; k <= P; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < P; i += kSelThreads) {
-                    const int ixj = i ^ j;
-                    if (ixj > i) {
-                        const uint32_t a = keys[i], b = keys[ixj];
-                        const bool up = (i & k) == 0;
-                        if ((a > b) == up) { keys[i] = b; keys[ixj] = a; }
-                    }
-                }
-                __syncthreads();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint4* rows = reinterpret_cast<uint4*>(X.end);
+#pragma unroll 1
+    for (int i = tid; i < X.nc / 4; i += kSelThreads) rows[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < X.n; i += kSelThreads) {
+        const uint32_t c = cell_of(i);
+        X.cell[i] = (uint16_t)c;
+        atomicAdd(X.end + c, 1u);
+    }
+    __syncthreads();
+    // exclusive sums over the cells, in place: a warp takes rows of 128 cells
+    const int nrows = X.nc / 128 / kSelWarps;
+    uint4* mine = rows + warp * nrows * 32 + lane;
+    uint32_t sum = 0u;
+#pragma unroll 1
+    for (int q = 0; q < nrows; ++q) {
+        const uint4 w = mine[q * 32];
+        sum += (w.x + w.y) + (w.z + w.w);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) S.below[warp] = sum;
+    __syncthreads();
+    uint32_t run = __reduce_add_sync(0xffffffffu, lane < warp ? S.below[lane & (kSelWarps - 1)] : 0u);
+#pragma unroll 1
+    for (int q = 0; q < nrows; ++q) {
+        uint4 w = mine[q * 32];
+        const uint32_t own = (w.x + w.y) + (w.z + w.w);
+        uint32_t inc = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t nb = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += nb;
+        }
+        uint4 x;
+        x.x = run + inc - own; x.y = x.x + w.x; x.z = x.y + w.y; x.w = x.z + w.z;
+        run += __shfl_sync(0xffffffffu, inc, 31);
+        mine[q * 32] = x;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < X.n; i += kSelThreads) X.sv[atomicAdd(X.end + X.cell[i], 1u)] = fetch(i);
+    __syncthreads();
+    // fp64 sums of the kChunkN values of every thread, scanned
+    double ls = 0.0;
+#pragma unroll 1
+    for (int i = tid * kChunkN; i < tid * kChunkN + kChunkN && i < X.n; ++i) ls += (double)X.sv[i];
+    unsigned long long none = 0, tc;
+    double tot;
+    block_excl_scan(none, ls, S.sc, S.ss, tc, tot);
+    X.pre[tid] = ls;
+    if (tid == 0) X.pre[kSelThreads] = tot;
+    __syncthreads();
+}
+
+struct Ranked {
+    float v;
+    int i_lt, i_le;    // #{values < v}, #{values <= v}
+    double s_lt, s_le; // their sums
+};
+
+// Sum of the values before position a (lane's share of it; add up over the warp).
+__device__ __forceinline__ double index_before_lane(const CellIndex& X, int a)
+{
+    const int lane = threadIdx.x & 31, q = a / kChunkN;
+    double x = lane == 0 ? X.pre[q] : 0.0;
+    if (q * kChunkN + lane < a) x += (double)X.sv[q * kChunkN + lane];
+    return x;
+}
+static_assert(kChunkN <= 32, "a lane for every value of a chunk");
+
+// The value of ascending rank p, by the 32 lanes of a warp.
+__device__ __forceinline__ Ranked index_select(const CellIndex& X, int p)
+{
+    const int lane = threadIdx.x & 31;
+    const int c = warp_upper_bound(X.end, X.nc, (uint32_t)p);
+    const int a = c > 0 ? (int)X.end[c - 1] : 0, b = (int)X.end[c], k = p - a;
+    Ranked r;
+    int lt = 0, eq = 0;
+    double s = index_before_lane(X, a);
+    if (b - a <= 32) {
+        const float v = a + lane < b ? X.sv[a + lane] : __int_as_float(0x7f800000);
+#pragma unroll 1
+        for (int j = 0; j < b - a; ++j) {
+            const float w = __shfl_sync(0xffffffffu, v, j);
+            lt += w < v ? 1 : 0;
+            eq += w == v ? 1 : 0;
+        }
+        const int src = __ffs(__ballot_sync(0xffffffffu, a + lane < b && lt <= k && k < lt + eq)) - 1;
+        r.v = __shfl_sync(0xffffffffu, v, src);
+        lt = __shfl_sync(0xffffffffu, lt, src);
+        eq = __shfl_sync(0xffffffffu, eq, src);
+        if (v < r.v) s += (double)v;
+    } else {
+        // a crowded cell (mostly one value many times over): its keys are bisected bit by bit
+        uint32_t key = 0u;
+#pragma unroll 1
+        for (int bit = 31; bit >= -1; --bit) {
+            const uint32_t cand = bit >= 0 ? key | (1u << bit) : key;
+            int n_lt = 0, n_eq = 0;
+#pragma unroll 1
+            for (int i = a + lane; i < b; i += 32) {
+                const uint32_t w = float_to_key(X.sv[i]);
+                n_lt += w < cand ? 1 : 0;
+                n_eq += w == cand ? 1 : 0;
+            }
+            n_lt = __reduce_add_sync(0xffffffffu, n_lt);
+            if (bit >= 0) {
+                if (n_lt <= k) key = cand;
+            } else {
+                lt = n_lt;
+                eq = __reduce_add_sync(0xffffffffu, n_eq);
             }
         }
-        return;
+        r.v = key_to_float(key);
+#pragma unroll 1
+        for (int i = a + lane; i < b; i += 32)
+            if (X.sv[i] < r.v) s += (double)X.sv[i];
     }
+    r.i_lt = a + lt;
+    r.i_le = a + lt + eq;
+    r.s_lt = warp_sum(s);
+    r.s_le = r.s_lt + (double)r.v * (double)eq;
+    return r;
+}
+
+// Levels from the indexed values: those of the m intervals iv (S.start, S.pre: where each begins), whose
+// cbefore and sbefore tie them to the whole tensor of n elements with sum stot.  ORQ: the open levels of
+// S.lv, one warp per level, one depth of Algorithm 1 at a time.  BinGrad-pb: the sign change of g.
+// Called by every thread of the CTA.
+__device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared& S, const Interval* iv, int m, bool pb, int s,
+                                               long long n, double stot, int t, float* __restrict__ levels,
+                                               int32_t* __restrict__ status)
+{
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 2; k <= P; k <<= 1) {
-        int j = k >> 1;
-        for (; j >= 256; j >>= 1) {  // CTA-wide stages
-            for (int q = threadIdx.x; q < (P >> 1); q += kSelThreads) {
-                const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
-                uint32_t a = keys[i], b = keys[i | j];
-                cmpx(a, b, (i & k) == 0);
-                keys[i] = a; keys[i | j] = b;
+    if (!pb) {
+        static_assert(kSelWarps >= kMaxLv - 1, "one warp per interior level");
+#pragma unroll 1
+        for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
+            const int q = warp;
+            if (q < s - 1 && q >= stride && ((q - stride) & (2 * stride - 1)) == 0 && !S.lv[q].exact) {
+                const LvInfo &L = S.lv[q - stride], &R = S.lv[q + stride];
+                LvInfo& o = S.lv[q];
+                if (!(R.val > L.val)) {
+                    if (lane == 0) o = L;
+                } else {
+                    const long long nseg = R.c_le - L.c_lt;
+                    const double A = (R.s_le - L.s_lt) - L.val * (double)nseg;
+                    long long k = (long long)floor(fp64_div(A, R.val - L.val));
+                    if (k < 0) k = 0;
+                    if (k > nseg - 1) k = nseg - 1;
+                    const long long p = R.c_le - 1 - k;
+                    // the interval that holds rank p: the last one that begins at or before it
+                    const int j = __popc(__ballot_sync(0xffffffffu, lane < m && iv[lane].cbefore <= p)) +
+                                  __popc(__ballot_sync(0xffffffffu, lane + 32 < m && iv[lane + 32].cbefore <= p)) - 1;
+                    const long long i = j >= 0 ? S.start[j] + (p - iv[j].cbefore) : -1;
+                    if (i < 0 || i >= S.start[j + 1]) {
+                        if (lane == 0) { o = L; S.internal = 1; }
+                    } else {
+                        const Ranked r = index_select(X, (int)i);
+                        if (lane == 0) {
+                            o.exact = 1;
+                            o.val = (double)r.v;
+                            o.key = float_to_key(r.v);
+                            o.c_lt = iv[j].cbefore + (r.i_lt - S.start[j]);
+                            o.c_le = iv[j].cbefore + (r.i_le - S.start[j]);
+                            o.s_lt = iv[j].sbefore + (r.s_lt - S.pre[j]);
+                            o.s_le = iv[j].sbefore + (r.s_le - S.pre[j]);
+                        }
+                    }
+                }
             }
             __syncthreads();
         }
-        for (int wb = warp * 256; wb < P; wb += kSelWarps * 256) {  // the 256-key blocks of this warp
-            uint32_t* blk = keys + wb;
-            int jj = j;
-            for (; jj >= 8; jj >>= 1) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int q = lane + 32 * u;
-                    const int i = ((q & ~(jj - 1)) << 1) | (q & (jj - 1));
-                    uint32_t a = blk[i], b = blk[i | jj];
-                    cmpx(a, b, ((wb + i) & k) == 0);
-                    blk[i] = a; blk[i | jj] = b;
-                }
-                __syncwarp();
+        const bool fail = S.internal != 0;
+        if ((int)threadIdx.x < s) levels[(int64_t)t * s + threadIdx.x] = fail ? 0.f : (float)S.lv[threadIdx.x].val;
+        if (threadIdx.x == 0 && fail) status[t] |= OGQ_ST_INTERNAL;
+        return;
+    }
+    // BinGrad-pb: the values with g(x) = x n - sum_{|v| >= x} |v| <= 0 come first; a warp per candidate rank
+    int lo = -1, hi = X.n;  // g <= 0 at lo (or lo = -1), g > 0 at hi (or hi = n)
+    double b1 = fp64_div(stot - iv[0].sbefore, (double)n);  // the zero when it lies below every value of the bracket
+#pragma unroll 1
+    while (true) {
+        const bool last = hi - lo <= 1;
+        const int step = (hi - lo + kSelWarps - 1) / kSelWarps;
+        const int i = last ? lo : lo + 1 + warp * step;
+        if (last && lo < 0) break;
+        bool below = false;
+        if (i < hi && (!last || warp == 0)) {
+            const Ranked r = index_select(X, i);
+            const int j = __popc(__ballot_sync(0xffffffffu, lane < m && S.start[lane] <= i)) +
+                          __popc(__ballot_sync(0xffffffffu, lane + 32 < m && S.start[lane + 32] <= i)) - 1;
+            const double x = (double)r.v, before = iv[j].sbefore + (r.s_lt - S.pre[j]);
+            below = x * (double)n - (stot - before) <= 0.0;
+            if (last) {
+                const double up = fp64_div(stot - (iv[j].sbefore + (r.s_le - S.pre[j])), (double)n);
+                b1 = up > x ? up : x;
             }
-            // distances 4, 2, 1 (those not above k / 2) on this lane's 8 consecutive keys
-            uint4* v4 = reinterpret_cast<uint4*>(blk + 8 * lane);
-            uint4 lo4 = v4[0], hi4 = v4[1];
-            uint32_t r[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-            const int i0 = wb + 8 * lane;
-#pragma unroll
-            for (int d = 4; d >= 1; d >>= 1) {
-                if (d <= jj) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        if ((e & d) == 0) cmpx(r[e], r[e | d], ((i0 + e) & k) == 0);
-                }
-            }
-            v4[0] = make_uint4(r[0], r[1], r[2], r[3]);
-            v4[1] = make_uint4(r[4], r[5], r[6], r[7]);
-            __syncwarp();
         }
-        // the next k starts with a CTA-wide stage only when k >= 256
-        if ((k << 1) >= 512 || k == P) __syncthreads();
+        if (last) break;
+        if (lane == 0) S.below[warp] = below ? 1u : 0u;
+        __syncthreads();
+        const int k = __popc(__ballot_sync(0xffffffffu, lane < kSelWarps && S.below[lane & (kSelWarps - 1)]));
+        __syncthreads();
+        const int nhi = lo + 1 + k * step;
+        if (k > 0) lo += 1 + (k - 1) * step;
+        if (nhi < hi) hi = nhi;
+    }
+    if (threadIdx.x == 0) {
+        if (S.internal) { status[t] |= OGQ_ST_INTERNAL; b1 = 0.0; }
+        levels[2 * t] = -(float)b1;
+        levels[2 * t + 1] = (float)b1;
     }
 }
 
-// Sorting finish (ORQ): when the elements left inside the candidate intervals fit in shared
-// memory, they are sorted, run-length encoded into single-key cells with exact prefix counts
-// and sums, and one more solver pass resolves every open level at once.
-__device__ void sort_finish(TState* st, int t, int s, const uint32_t* buf, long long src_cnt,
-                            float* __restrict__ levels, int32_t* __restrict__ status, unsigned char* smem,
-                            SolverShared& S)
+// Gathers the keys of src[0 .. src_cnt) that lie inside the intervals S.niv (all of them when `filtered`),
+// indexes them and finishes the tensor from there: called when they fit kSortN.  4096 keys take about 5 us;
+// a bitonic sort in shared memory with binary searches per level took 20.
+__device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s, const uint32_t* src, int src_cnt, bool filtered,
+                                              float* __restrict__ levels, int32_t* __restrict__ status, unsigned char* smem,
+                                              SolverShared& S)
 {
-    constexpr int kPer = kSmallN / kSelThreads;
-    uint32_t* skeys = reinterpret_cast<uint32_t*>(smem);
-    uint32_t* xkeys = skeys + kSmallN;
-    uint32_t* xcpre = xkeys + kSmallN;
-    double* xspre = reinterpret_cast<double*>(smem + ((3 * kSmallN + kMaxIv + 2) * sizeof(uint32_t) + 15) / 16 * 16);
-    __syncthreads();
-    if (threadIdx.x == 0) S.n_keys = 0;
-    if (threadIdx.x < kMaxIv) { S.ivstart[threadIdx.x] = 0; S.ivufirst[threadIdx.x] = -1; S.ivpre[threadIdx.x] = 0.0; }
-    __syncthreads();
-    // Filter of the copied keys: the lower and upper keys of the new intervals in two compact arrays
-    // (padded to 64 entries), a six-step search without branches, eight keys per thread in flight, and
-    // one shared counter update per warp and key column instead of one per accepted key.
-    __shared__ uint32_t f_lo[kMaxIv], f_hi[kMaxIv];
-    static_assert(kMaxIv == 64, "the search below takes six halving steps");
-    if (threadIdx.x < kMaxIv) {
-        const bool real = (int)threadIdx.x < S.nm;
-        f_lo[threadIdx.x] = real ? S.niv[threadIdx.x].klo : 0xffffffffu;  // no key has this value (NaN pattern)
-        f_hi[threadIdx.x] = real ? S.niv[threadIdx.x].khi : 0u;
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint32_t* list = reinterpret_cast<uint32_t*>(smem + kIndexBytes<kFinishCells> + 8);
+    __syncthreads();  // S.nm and S.niv are complete
+    const int m = S.nm;
+    if (tid < kMaxIv) {
+        const bool real = tid < m;
+        const uint32_t lo = real ? S.niv[tid].klo : 0xffffffffu, hi = real ? S.niv[tid].khi : 0u;  // (no key has the value of lo: NaN)
+        S.lo[tid] = lo;
+        S.hi[tid] = hi;
+        // equal shares of the cells: an interval is a narrow slice of a binade, its values are spread evenly
+        const uint32_t share = (uint32_t)(kFinishCells / m);
+        S.sh[tid] = real ? max(0, 32 - __clz((hi - lo) / share)) : 0;
+        S.base[tid] = tid * share;
     }
+    if (tid == 0) { S.n_keys = 0; S.internal = 0; }
+    int top = 2;
+    while (top < m) top <<= 1;
     __syncthreads();
-    {
-        const int lane = threadIdx.x & 31;
-        constexpr int kCols = 8;
-        // the keys come from L2 (another SM wrote them): the loads of the next trip are issued before
-        // this trip's keys are searched, so that one round trip is hidden behind the other's work
-        auto fetch = [&](uint32_t* k, long long at) {
+    auto interval = [&](uint32_t key) -> int {
+        int j = 0;
+#pragma unroll 1
+        for (int step = top >> 1; step >= 1; step >>= 1)
+            if (S.lo[j + step] <= key) j += step;
+        return j;
+    };
+    int c = src_cnt;
+    if (filtered) {
+#pragma unroll 4
+        for (int i = tid; i < c; i += kSelThreads) list[i] = __ldcg(src + i);
+    } else {
+        constexpr int kCols = 4;  // loads in flight per thread
+#pragma unroll 1
+        for (int i0 = tid & ~31; i0 < src_cnt; i0 += kCols * kSelThreads) {
+            uint32_t k[kCols];
 #pragma unroll
             for (int u = 0; u < kCols; ++u) {
-                const long long i = at + u * 32 + lane;
-                k[u] = (i < src_cnt) ? __ldcg(buf + i) : 0u;
+                const int i = i0 + u * kSelThreads + lane;
+                k[u] = i < src_cnt ? __ldcg(src + i) : 0u;
             }
-        };
-        int top = 2;
-        while (top < S.nm) top <<= 1;
-        uint32_t nxt[kCols];
-        long long i0 = (long long)(threadIdx.x & ~31) * kCols;
-        if (i0 < src_cnt) fetch(nxt, i0);
-        for (; i0 < src_cnt; i0 += (long long)kCols * kSelThreads) {
-            uint32_t key[kCols];
-            bool in[kCols];
+            int j[kCols];
 #pragma unroll
-            for (int u = 0; u < kCols; ++u) key[u] = nxt[u];
-            if (i0 + (long long)kCols * kSelThreads < src_cnt) fetch(nxt, i0 + (long long)kCols * kSelThreads);
-            int idx[kCols];
-#pragma unroll
-            for (int u = 0; u < kCols; ++u) idx[u] = 0;
-            // halving steps over the first `top` entries only (top = the power of two that covers the
-            // intervals): the table reads of 16 warps are what this loop is bound by
+            for (int u = 0; u < kCols; ++u) j[u] = 0;
+#pragma unroll 1
             for (int step = top >> 1; step >= 1; step >>= 1) {
 #pragma unroll
                 for (int u = 0; u < kCols; ++u)
-                    if (f_lo[idx[u] + step] <= key[u]) idx[u] += step;
+                    if (S.lo[j[u] + step] <= k[u]) j[u] += step;
             }
-            unsigned m[kCols];
-            int total = 0;
 #pragma unroll
             for (int u = 0; u < kCols; ++u) {
-                in[u] = (i0 + u * 32 + lane < src_cnt) && key[u] >= f_lo[idx[u]] && key[u] <= f_hi[idx[u]];
-                m[u] = __ballot_sync(0xffffffffu, in[u]);
-                total += __popc(m[u]);
-            }
-            if (total) {  // one counter update per warp and trip
-                int pos = 0;
-                if (lane == 0) pos = atomicAdd(&S.n_keys, total);
-                pos = __shfl_sync(0xffffffffu, pos, 0);
-#pragma unroll
-                for (int u = 0; u < kCols; ++u) {
-                    const int at = pos + __popc(m[u] & ((1u << lane) - 1u));
-                    if (in[u] && at < kSmallN) skeys[at] = key[u];
-                    pos += __popc(m[u]);
+                const bool in = i0 + u * kSelThreads + lane < src_cnt && k[u] >= S.lo[j[u]] && k[u] <= S.hi[j[u]];
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                if (b) {
+                    int pos = 0;
+                    if (lane == 0) pos = atomicAdd(&S.n_keys, __popc(b));
+                    pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(b & ((1u << lane) - 1u));
+                    if (in && pos < kSortN) list[pos] = k[u];
                 }
             }
         }
-    }
-    __syncthreads();
-    const int c = S.n_keys < kSmallN ? S.n_keys : kSmallN;
-    int P = 1;
-    while (P < c) P <<= 1;
-    for (int i = c + threadIdx.x; i < kSmallN; i += kSelThreads) skeys[i] = 0xffffffffu;
-    __syncthreads();
-    block_bitonic_sort(skeys, P);
-    // pass 1: run starts and value sums of this thread's kPer consecutive sorted elements
-    const int base = threadIdx.x * kPer;
-    uint32_t k[kPer];
-    unsigned long long lu = 0;
-    double ls = 0.0;
-    uint32_t prev = (base > 0 && base <= c) ? skeys[base - 1] : 0u;
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) {
-        const int i = base + e;
-        k[e] = (i < c) ? skeys[i] : 0xffffffffu;
-        if (i < c) {
-            const bool flag = (i == 0) || (k[e] != (e == 0 ? prev : k[e - 1]));
-            lu += flag ? 1 : 0;
-            ls += (double)sel_key_to_float(k[e]);
-        }
-    }
-    unsigned long long ubase = lu, tu;
-    double sbase = ls, tsum;
-    block_excl_scan(ubase, sbase, S.sc, S.ss, tu, tsum);
-    if (threadIdx.x == 0) S.n_unique = (int)tu;
-    // interval of each of this thread's keys, of the key before them and of the key after them
-    // (searched once; the passes below reuse them)
-    int jv[kPer];
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) jv[e] = (base + e < c) ? find_new_interval(S, k[e]) : -1;
-    const int jprev = (base > 0 && base <= c) ? find_new_interval(S, prev) : -2;
-    const uint32_t knext = (base + kPer < c) ? skeys[base + kPer] : 0u;
-    const int jnext = (base + kPer < c) ? find_new_interval(S, knext) : -3;
-    // pass 2: first element of every interval
-    {
-        int nf = 0;
-        double run = sbase;
-#pragma unroll
-        for (int e = 0; e < kPer; ++e) {
-            const int i = base + e;
-            if (i < c) {
-                const uint32_t pk = (e == 0) ? prev : k[e - 1];
-                const bool flag = (i == 0) || (k[e] != pk);
-                if (flag) {
-                    const int j = jv[e];
-                    const int jp = (i == 0) ? -2 : ((e == 0) ? jprev : jv[e - 1]);
-                    if (j >= 0 && j != jp) {
-                        S.ivstart[j] = i;
-                        S.ivpre[j] = run;
-                        S.ivufirst[j] = (int)ubase + nf;
-                    }
-                    ++nf;
-                }
-                run += (double)sel_key_to_float(k[e]);
-            }
-        }
-    }
-    __syncthreads();
-    // pass 3: explicit cells (slot = unique index + interval index) and the end slot of every interval
-    {
-        int nf = 0;
-        double run = sbase;
-#pragma unroll
-        for (int e = 0; e < kPer; ++e) {
-            const int i = base + e;
-            if (i < c) {
-                const uint32_t pk = (e == 0) ? prev : k[e - 1];
-                const bool flag = (i == 0) || (k[e] != pk);
-                const int j = jv[e];
-                const double val = (double)sel_key_to_float(k[e]);
-                if (flag) {
-                    const int u = (int)ubase + nf;
-                    xkeys[u] = k[e];
-                    if (j >= 0) {
-                        xcpre[u + j] = (uint32_t)(S.niv[j].cbefore + (long long)(i - S.ivstart[j]));
-                        xspre[u + j] = S.niv[j].sbefore + (run - S.ivpre[j]);
-                    }
-                    ++nf;
-                }
-                const int jn = (i + 1 < c) ? ((e + 1 < kPer) ? jv[e + 1] : jnext) : -4;
-                const bool last_of_iv = (i + 1 >= c) || (jn != j);
-                if (last_of_iv && j >= 0) {
-                    const int u = (int)ubase + nf - 1;
-                    xcpre[u + 1 + j] = (uint32_t)(S.niv[j].cbefore + (long long)(i + 1 - S.ivstart[j]));
-                    xspre[u + 1 + j] = S.niv[j].sbefore + ((run + val) - S.ivpre[j]);
-                    S.niv[j].ncell = u - S.ivufirst[j] + 1;
-                }
-                run += val;
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int next = S.n_unique;
-        for (int j = S.nm - 1; j >= 0; --j) {
-            if (S.ivufirst[j] < 0) {  // no element left in this interval: only its end slot
-                S.niv[j].ncell = 0;
-                xcpre[next + j] = (uint32_t)S.niv[j].cbefore;
-                xspre[next + j] = S.niv[j].sbefore;
-            } else {
-                next = S.ivufirst[j];
-            }
-        }
-        int cb = 0;
-        for (int j = 0; j < S.nm; ++j) { S.niv[j].sh = 0; S.niv[j].cellbase = cb; cb += S.niv[j].ncell; }
-        S.view.slot_iv = nullptr; S.view.xkeys = xkeys; S.view.cpre = xcpre; S.view.spre = xspre;
-        S.view.iv = S.niv; S.view.m = S.nm;
-        sel_init_slots(S.view);
-        S.internal = (S.n_keys > kSmallN) ? 1 : 0;
-    }
-    // one thread per level, one depth at a time (every cell is a single key now, so each solve is exact)
-    for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
         __syncthreads();
-        const int q = threadIdx.x >> 5;  // one warp per level, as in solver_round
-        if ((threadIdx.x & 31) == 0 && !S.internal && q < s - 1 && q >= stride && ((q - stride) % (2 * stride)) == 0 &&
-            !S.lv[q].exact) {
-            if (!sel_orq_solve(S.view, S.lv[q - stride], S.lv[q + stride], S.lv[q])) S.internal = 1;
+        c = S.n_keys;
+        if (c > kSortN) { c = kSortN; if (tid == 0) S.internal = 1; }
+    }
+    const CellIndex X = index_at(smem, c, kFinishCells);
+    // (index_build begins with a barrier)
+    index_build(X, S, [&](int i) { return sel_key_to_float(list[i]); },
+                [&](int i) -> uint32_t {
+                    const uint32_t key = list[i];
+                    const int j = interval(key);
+                    return S.base[j] + ((key - S.lo[j]) >> S.sh[j]);
+                });
+    for (int j = tid >> 5; j <= m; j += kSelWarps) {
+        // where interval j begins: after the last value of the cell before its first
+        const int a = j == m ? c : (j > 0 ? (int)X.end[S.base[j] - 1] : 0);
+        const double x = warp_sum(index_before_lane(X, a));
+        if (lane == 0) {
+            S.start[j] = a;
+            if (j < m) S.pre[j] = x;
         }
     }
     __syncthreads();
+    levels_from_index(X, S, S.niv, m, pb, s, S.view.n, S.view.stot, t, levels, status);
+    if (tid == 0) st->done = 1;
+    __threadfence();
+    __syncthreads();
+}
+
+// Small tensors: all values indexed, the definitions applied directly.
+__device__ void small_tensor(const float* __restrict__ src, int n, int t, bool pb, int s, float* __restrict__ levels,
+                             int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, float tau)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto value = [&](int i) -> float {
+        const float x = __ldg(src + i);
+        const float v = copysignf(fminf(fabsf(x), tau), x) + 0.0f;  // clipped, -0 counts as 0
+        return pb ? fabsf(v) : v;
+    };
+    uint32_t kmin = 0xffffffffu, kmax = 0u, sum = 0u;
+#pragma unroll 4
+    for (int i = tid; i < n; i += kSelThreads) {
+        const float v = value(i);
+        const uint32_t k = float_to_key(v);
+        kmin = min(kmin, k);
+        kmax = max(kmax, k);
+        sum += (__float_as_uint(v) & 0x7fffffffu) >> 16;
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) { S.lo[warp] = kmin; S.hi[warp] = kmax; S.base[warp] = sum; }
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, S.lo[lane & (kSelWarps - 1)]);
+    kmax = __reduce_max_sync(0xffffffffu, S.hi[lane & (kSelWarps - 1)]);
+    sum = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? S.base[lane & (kSelWarps - 1)] : 0u);
+    const float vmin = key_to_float(kmin), vmax = key_to_float(kmax);
+    const int nl = pb ? 2 : s;
+    // (keys order Inf and NaN beyond the finite values at either end)
+    const bool bad = kmax >= 0xff800000u || kmin <= 0x007fffffu;
+    if (bad || kmin == kmax) {
+        // non-finite, or all values equal: level = value (BinGrad-pb: b_1 = the magnitude, b_0 = b_1 = 0 for zeros)
+        if (tid < nl) levels[(int64_t)t * nl + tid] = bad ? 0.f : pb ? (tid == 0 ? -vmax : vmax) : vmax;
+        if (tid == 0) status[t] = bad ? OGQ_ST_NONFINITE : (!pb || vmax == 0.f) ? OGQ_ST_CONSTANT : 0;
+        return;
+    }
+    const MagnitudeCells cell((uint32_t)((float)sum / (float)n), fmaxf(fabsf(vmin), fabsf(vmax)), !pb, kSmallCells);
+    const CellIndex X = index_at(smem, n, kSmallCells);
+    index_build(X, S, value, [&](int i) { return cell(value(i)); });
+    if (tid == 0) {
+        S.internal = 0;
+        S.start[0] = 0; S.start[1] = n; S.pre[0] = 0.0;
+        S.niv[0].cbefore = 0; S.niv[0].sbefore = 0.0;
+    }
+    if (tid < s) {
+        LvInfo& l = S.lv[tid];
+        l.exact = tid == 0 || tid == s - 1;
+        l.val = (double)(tid == 0 ? vmin : vmax);
+        l.key = tid == 0 ? kmin : kmax;
+        l.c_lt = 0; l.s_lt = 0.0;
+        l.c_le = n; l.s_le = X.pre[kSelThreads];
+    }
+    if (tid == 0) status[t] = 0;
+    __syncthreads();
+    levels_from_index(X, S, S.niv, 1, pb, s, n, X.pre[kSelThreads], t, levels, status);
+}
+
+// Finishes a tensor whose last pass only copied the keys inside its intervals (TState::compact_only): the
+// solver state the previous pass left in global memory is loaded back.  Called by every thread of the CTA.
+__device__ void finish_sorted(TState* st, int t, bool pb, int s, const uint32_t* copied, float* __restrict__ levels,
+                              int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, int cursor_idx)
+{
+    __syncthreads();
+    const int m = __ldcg(&st->m);
+    if ((int)threadIdx.x < m) S.niv[threadIdx.x] = st->iv[threadIdx.x];
+    if (!pb && (int)threadIdx.x >= 64 && (int)threadIdx.x - 64 < s) {
+        const ExactLv& e = st->lv[threadIdx.x - 64];
+        LvInfo& l = S.lv[threadIdx.x - 64];
+        l.exact = e.exact; l.key = e.key; l.val = (double)sel_key_to_float(e.key);
+        l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
+    }
     if (threadIdx.x == 0) {
-        bool ok = !S.internal;
-        for (int q = 0; q < s; ++q) ok = ok && S.lv[q].exact;
-        if (ok) {
-            for (int q = 0; q < s; ++q) levels[(int64_t)t * s + q] = sel_key_to_float(S.lv[q].key);
-        } else {
-            status[t] |= OGQ_ST_INTERNAL;
-            for (int q = 0; q < s; ++q) levels[(int64_t)t * s + q] = 0.f;
-        }
-        st->done = 1;
-        __threadfence();
+        S.nm = m;
+        S.view.n = st->n;
+        S.view.stot = st->stot;
+    }
+    const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[cursor_idx]);
+    finish_from_keys(st, t, pb, s, copied, (int)src_cnt, src_cnt == cand, levels, status, smem, S);
+}
+
+// Shared memory of a solver pass: the prefix arrays over the slots, and the raw cells as they come from L2.
+constexpr size_t kOffSpre = (kSlots * sizeof(uint32_t) + 15) / 16 * 16;
+constexpr size_t kOffSlotIv = kOffSpre + kSlots * sizeof(double);
+constexpr size_t kOffRawSum = (kOffSlotIv + kSlots + 15) / 16 * 16;
+constexpr size_t kOffRawCnt = kOffRawSum + kCells * sizeof(unsigned long long);
+constexpr size_t kPrefixBytes = kOffRawCnt + kCells * sizeof(uint32_t);
+constexpr size_t kFinishBytes = kIndexBytes<kFinishCells> + 8 + kSortN * sizeof(uint32_t);
+constexpr size_t kSolveBytes = kPrefixBytes > kFinishBytes ? kPrefixBytes : kFinishBytes;
+constexpr size_t kRound3Bytes = kSolveBytes > kSmemBytes ? kSolveBytes : kSmemBytes;  // of a CTA that also streams
+static_assert(kIndexBytes<kSmallCells> <= kSmemBytes, "small tensors are solved in a streaming CTA");
+
+// Prefix arrays over all slots of the intervals S.iv (S.view.m of them): counts and sums of the elements
+// before every slot.  A thread takes consecutive slots; a slot's cell is its index minus the number of
+// intervals before it (every interval has one end slot).
+__device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* gcnt, const unsigned long long* glsum, bool first,
+                                              unsigned char* smem)
+{
+    uint32_t* cpre = reinterpret_cast<uint32_t*>(smem);
+    double* spre = reinterpret_cast<double*>(smem + kOffSpre);
+    uint8_t* slot_iv = smem + kOffSlotIv;
+    unsigned long long* raw_sum = reinterpret_cast<unsigned long long*>(smem + kOffRawSum);
+    uint32_t* raw_cnt = reinterpret_cast<uint32_t*>(smem + kOffRawCnt);
+    const int tid = threadIdx.x, m = S.view.m;
+    const int ncells = S.iv[m - 1].cellbase + S.iv[m - 1].ncell, nslots = ncells + m;
+    {
+        constexpr int kC = (kCells / 4 + kSelThreads - 1) / kSelThreads, kL = (kCells / 2 + kSelThreads - 1) / kSelThreads;
+        uint4 c[kC];
+        ulonglong2 l[kL];
+#pragma unroll
+        for (int u = 0; u < kC; ++u)
+            if ((tid + u * kSelThreads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSelThreads);
+#pragma unroll
+        for (int u = 0; u < kL; ++u)
+            if ((tid + u * kSelThreads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSelThreads);
+        if (tid < m) S.view.slotbase[tid] = S.iv[tid].cellbase + tid;
+        if (tid == 0) { S.view.slotbase[m] = nslots; S.view.nslots = nslots; }
+#pragma unroll
+        for (int u = 0; u < kC; ++u)
+            if ((tid + u * kSelThreads) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * kSelThreads] = c[u];
+#pragma unroll
+        for (int u = 0; u < kL; ++u)
+            if ((tid + u * kSelThreads) * 2 < ncells) reinterpret_cast<ulonglong2*>(raw_sum)[tid + u * kSelThreads] = l[u];
+    }
+    __syncthreads();
+    const int per = (nslots + kSelThreads - 1) / kSelThreads;
+    const int s0 = tid * per < nslots ? tid * per : nslots, s1 = s0 + per < nslots ? s0 + per : nslots;
+    int j = 0;
+    {
+        int hi = m;
+#pragma unroll 1
+        while (hi - j > 1) { const int mid = (j + hi) >> 1; if (S.view.slotbase[mid] <= s0) j = mid; else hi = mid; }
+    }
+    unsigned long long lc = 0;
+    double ls = 0.0;
+#pragma unroll 1
+    for (int slot = s0; slot < s1; ++slot) {
+        while (slot >= S.view.slotbase[j + 1]) ++j;
+        slot_iv[slot] = (uint8_t)j;
+        const uint32_t n = slot + 1 < S.view.slotbase[j + 1] ? raw_cnt[slot - j] : 0u;
+        double x = 0.0;
+        if (n) x = sel_cell_sum(S.iv[j].klo + ((uint32_t)(slot - S.view.slotbase[j]) << S.iv[j].sh), S.iv[j].sh, n, raw_sum[slot - j]);
+        cpre[slot] = n;
+        spre[slot] = x;
+        lc += n;
+        ls += x;
+    }
+    unsigned long long tc;
+    double ts;
+    block_excl_scan(lc, ls, S.sc, S.ss, tc, ts);
+#pragma unroll 1
+    for (int slot = s0; slot < s1; ++slot) {
+        const uint32_t n = cpre[slot];
+        const double x = spre[slot];
+        cpre[slot] = (uint32_t)lc;
+        spre[slot] = ls;
+        lc += n;
+        ls += x;
+    }
+    __syncthreads();
+    if (first) return;
+    // rounds >= 2: shift every interval so that it starts from the exact (count, sum) before it
+    if (tid < m) {
+        const int sb = S.view.slotbase[tid];
+        S.offc[tid] = (uint32_t)((unsigned long long)S.iv[tid].cbefore - cpre[sb]);
+        S.offs[tid] = S.iv[tid].sbefore - spre[sb];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int slot = s0; slot < s1; ++slot) {
+        cpre[slot] += S.offc[slot_iv[slot]];
+        spre[slot] += S.offs[slot_iv[slot]];
     }
     __syncthreads();
 }
 
-// Warp-parallel version of the common case of sel_refine: the open ranges are sorted and do not
-// touch, every range yields at most four pieces, there are at most 32 pieces and none is wider
-// than an equal share of the cell budget.  Lane i first cuts range i into pieces, then lane k
-// builds interval k.  Returns false (nothing written) when the case is not the common one; the
-// caller then runs the general single-thread routine.  Called by the 32 lanes of warp 0.
-__device__ bool refine_parallel(SolverShared& S, bool trim_empty)
+// Q*(L, R) on the current cells, by the 32 lanes of a warp: exact when both brackets are exact and the target
+// rank sits in a single-key cell, otherwise a conservative range of cells [sa, sb].  The lower half of the
+// lanes works out the range's first rank and its cell, the upper half the last; both are the same when the
+// brackets are exact.  Returns false on an internal inconsistency.
+//   With M the elements strictly between L's cells and R's cells (count cntM, sum sumM), T = [t_L + (sumM -
+// L cntM) + t_R] / (R - L), t_L and t_R the contributions of the elements of L's and R's own cells.
+// (sumM - L cntM) / (R - L) decreases in L and in R, so its extremes are taken at matching corners, which
+// stays tight even when a bracket is only known to lie somewhere in a sparse stretch of cells.
+__device__ __noinline__ bool warp_orq_solve(const SolverView& v, const LvInfo& L, const LvInfo& R, LvInfo& out)
+{
+    const int lane = threadIdx.x & 31;
+    const bool upper = lane >= 16;
+    if (L.exact && R.exact && !(R.val > L.val)) {
+        if (lane == 0) out = L;
+        return true;
+    }
+    const bool exact = L.exact && R.exact;
+    // (an exact level's range is its value: vlo = vhi = val, and c_lt .. c_le, s_lt .. s_le its elements; one
+    // that is only known as a range has the counts and sums of the whole range there)
+    const long long floor_pos = L.c_lt, ceil_pos = R.c_le - 1;
+    long long pos;
+    if (exact) {
+        const long long nseg = R.c_le - L.c_lt;
+        const double A = (R.s_le - L.s_lt) - L.val * (double)nseg;
+        long long k = (long long)floor(fp64_div(A, R.val - L.val));
+        if (k < 0) k = 0;
+        if (k > nseg - 1) k = nseg - 1;
+        pos = R.c_le - 1 - k;
+    } else {
+        const long long Cs = L.exact ? L.c_lt : L.c_le, Ce = R.exact ? R.c_le : R.c_lt;
+        const double Ss = L.exact ? L.s_lt : L.s_le, Se = R.exact ? R.s_le : R.s_lt;
+        const double cntL = L.exact ? 0.0 : (double)(L.c_le - L.c_lt), cntR = R.exact ? 0.0 : (double)(R.c_le - R.c_lt);
+        const double cntM = (double)(Ce - Cs), sumM = Se - Ss;
+        pos = upper ? ceil_pos : floor_pos;
+        if (cntM >= 0.0 && R.vlo > L.vhi) {
+            double num = fmax(sumM - (upper ? L.vhi : L.vlo) * cntM, 0.0);
+            num = upper ? cntR * (R.vhi - R.vlo) - num : -(cntL * (L.vhi - L.vlo) + num);
+            const double den = upper ? R.vhi - L.vhi : R.vlo - L.vlo;
+            const double delta = 2.0 + 1e-9 * (double)v.n;
+            const double p = ceil((double)Ce + fp64_div(num, den) + (upper ? delta : -delta)) - 1.0;
+            if (upper ? p < (double)pos : p > (double)pos) pos = (long long)p;
+        }
+        if (pos < floor_pos) pos = floor_pos;
+        if (pos > ceil_pos) pos = ceil_pos;
+        const long long other = __shfl_xor_sync(0xffffffffu, pos, 16);
+        if (!upper && pos > other) pos = other;
+        if (pos < 0) pos = 0;
+        if (pos > v.n - 1) pos = v.n - 1;
+    }
+    // the cells of the two ranks: each half of the warp searches for the first slot whose prefix exceeds its own
+    int lo = 0, hi = v.nslots;
+#pragma unroll 1
+    while (__any_sync(0xffffffffu, lo < hi)) {
+        const int step = (hi - lo + 15) >> 4;
+        const int i = lo + (lane & 15) * step;
+        const unsigned b = __ballot_sync(0xffffffffu, i < hi && (long long)v.cpre[i] <= pos);
+        const int k = __popc(upper ? b >> 16 : b & 0xffffu);
+        const int nhi = lo + k * step;
+        if (k > 0) lo += (k - 1) * step + 1;
+        if (nhi < hi) hi = nhi;
+    }
+    // lo - 1 is the cell's slot; the end slot of an interval there means that the rank lies between two
+    // intervals: the first cell after the gap for the lower rank, the last one before it for the upper
+    int slot = lo - 1;
+    const bool gap = slot < 0 || sel_is_end_slot(v, slot);
+    if (gap) slot = (upper && !exact) ? slot - 1 : slot + 1;
+    bool ok = slot >= 0 && slot < v.nslots && !(exact && gap);
+    const int sa = __shfl_sync(0xffffffffu, slot, 0), sb = __shfl_sync(0xffffffffu, slot, 16);
+    ok = __all_sync(0xffffffffu, ok) && sa <= sb;
+    if (!ok) return false;
+    // value bounds: the low end of the first cell, the high end of the last
+    const int sh = sel_slot_shift(v, slot);
+    const double val = (double)sel_key_to_float(sel_slot_kbase(v, slot) + (upper && sh > 0 ? (1u << sh) - 1u : 0u));
+    const double vhi = __shfl_sync(0xffffffffu, val, 16);
+    if (lane == 0) {
+        out.exact = exact && sh == 0;
+        out.key = sel_slot_kbase(v, sa);
+        out.val = val;
+        out.vlo = val;
+        out.vhi = vhi;
+        out.c_lt = v.cpre[sa];
+        out.s_lt = v.spre[sa];
+        out.c_le = v.cpre[sb + 1];
+        out.s_le = v.spre[sb + 1];
+        out.sa = sa;
+        out.sb = sb;
+    }
+    return true;
+}
+
+// Turns the candidate cells (S.marks) into the intervals of the next round (S.niv, S.nm, S.cand): a run of
+// neighbouring candidate cells is an interval, and the cell budget is shared out equally among the runs,
+// each taking as many halvings of its cells as its share allows (a run that is longer than its share keeps
+// its cells and the others share the rest).  Returns false when there are more than kRefineMax runs or the
+// shares do not work out.  Called by the 32 lanes of warp 0.
+__device__ __forceinline__ bool refine_marked(SolverShared& S)
 {
     const SolverView& v = S.view;
     const int lane = threadIdx.x & 31;
-    const int nr = S.nr;
-    int p_a[4], p_b[4], np = 0;
-    bool fail = nr > 32;
-    if (lane < nr && !fail) {
-        const int a = S.ra[lane], b = S.rb[lane];
-        if (lane > 0 && a <= S.rb[lane - 1] + 1) fail = true;
-        int first = a, last = b;
-        long long cnt = 1;
-        if (trim_empty) {
-            cnt = (long long)v.cpre[b + 1] - (long long)v.cpre[a];
-            if (cnt > 0) {
-                bool gap;
-                first = sel_locate(v, (long long)v.cpre[a], true, &gap);
-                last = sel_locate(v, (long long)v.cpre[b + 1] - 1, false, &gap);
-                if (first < a || last > b || first > last) fail = true;
-            }
-        }
-        if (cnt > 0 && !fail) {
-            const int width = last - first + 1;
-            if (trim_empty && width <= 12) {
-                int run_a = -1, lastp = -1;
-                for (int c = first; c <= last + 1; ++c) {
-                    const bool boundary = (c > last) || sel_is_end_slot(v, c);
-                    const bool populated = !boundary && v.cpre[c + 1] != v.cpre[c];
-                    if (run_a >= 0 && (boundary || (!populated && c - lastp > 1))) {
-                        if (np >= 4) { fail = true; break; }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) if (u == np) { p_a[u] = run_a; p_b[u] = lastp; }
-                        ++np;
-                        run_a = -1;
-                    }
-                    if (populated) { if (run_a < 0) run_a = c; lastp = c; }
-                }
+    constexpr int kWords = (kSlots + 31) / 32, kWpl = (kWords + 31) / 32;
+    const int w0 = lane * kWpl, w1 = w0 + kWpl < kWords ? w0 + kWpl : kWords;
+    // first and last cells of runs in this lane's words: counted, then written out
+    int is = 0, ie = 0, m = 0;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        int ns = 0, ne = 0;
+#pragma unroll 1
+        for (int w = w0; w < w1; ++w) {
+            const uint32_t x = S.marks[w];
+            if (x == 0u) continue;
+            uint32_t a = x & ~((x << 1) | (w > 0 ? S.marks[w - 1] >> 31 : 0u));
+            uint32_t b = x & ~((x >> 1) | (w + 1 < kWords ? S.marks[w + 1] << 31 : 0u));
+            if (pass == 0) {
+                ns += __popc(a);
+                ne += __popc(b);
             } else {
-                // wide: the trimmed hull, cut where it crosses into another interval (if it is too wide
-                // for its share of the cells the general routine takes over below)
-                const int j0 = sel_interval_of_slot(v, first), j1 = sel_interval_of_slot(v, last);
-                for (int j = j0; j <= j1; ++j) {
-                    const int lo = v.slotbase[j], hi = v.slotbase[j] + v.iv[j].ncell - 1;
-                    const int x = first > lo ? first : lo, y = last < hi ? last : hi;
-                    if (x > y) continue;
-                    if (np >= 4) { fail = true; break; }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) if (u == np) { p_a[u] = x; p_b[u] = y; }
-                    ++np;
-                }
+                for (; a; a &= a - 1) S.pa[is++] = w * 32 + __ffs(a) - 1;
+                for (; b; b &= b - 1) S.pb[ie++] = w * 32 + __ffs(b) - 1;
             }
         }
-    }
-    if (__any_sync(0xffffffffu, fail)) return false;
-    // piece offsets
-    int incl = np;
+        if (pass == 0) {
+            is = ns;
+            ie = ne;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int nb = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += nb;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int a = __shfl_up_sync(0xffffffffu, is, o), b = __shfl_up_sync(0xffffffffu, ie, o);
+                if (lane >= o) { is += a; ie += b; }
+            }
+            m = __shfl_sync(0xffffffffu, is, 31);
+            if (m == 0 || m > kRefineMax) return false;
+            is -= ns;
+            ie -= ne;
+        }
     }
-    const int m = __shfl_sync(0xffffffffu, incl, 31);
-    if (m == 0 || m > 32) return false;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (u < np) { S.pa[incl - np + u] = p_a[u]; S.pb[incl - np + u] = p_b[u]; }
     __syncwarp();
-    // one lane per piece: equal share of the cell budget
-    const int share = kCells / m;
-    int cells = 0, sh = 0, r = 0, j = 0, pa = 0, pb = 0;
-    long long elems = 0;
-    if (lane < m) {
-        pa = S.pa[lane]; pb = S.pb[lane];
-        cells = pb - pa + 1;
-        j = sel_interval_of_slot(v, pa);
-        sh = v.iv[j].sh;
-        r = (cells <= share) ? sel_floor_log2(share / cells) : -1;
-        if (r > sh) r = sh;
-        elems = (long long)v.cpre[pb + 1] - (long long)v.cpre[pa];
-    }
-    if (__any_sync(0xffffffffu, lane < m && r < 0)) return false;  // a piece wider than its share
-    const int ncell = (lane < m) ? (cells << r) : 0;
-    int cinc = ncell;
-    long long einc = elems;
+    static_assert(kRefineMax == 32, "a lane per run");
+    const bool have = lane < m;
+    const int pa = have ? S.pa[lane] : 0, pb = have ? S.pb[lane] : 0;
+    const int len = have ? pb - pa + 1 : 0, j = have ? v.slot_iv[pa] : 0;
+    int sh = have ? v.iv[j].sh : 0;
+    const bool large = len > kCells / m;
+    const int big = __reduce_add_sync(0xffffffffu, large ? len : 0), nbig = __popc(__ballot_sync(0xffffffffu, large));
+    const int share = nbig < m ? (kCells - big) / (m - nbig) : 0;
+    const int r = have && len <= share ? min(31 - __clz(share / len), sh) : 0;
+    const int ncell = len << r;
+    sh -= r;
+    const bool progress = __any_sync(0xffffffffu, r > 0), open_shift = __any_sync(0xffffffffu, sh > 0);
+    int at = ncell;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int nb = __shfl_up_sync(0xffffffffu, cinc, o);
-        const long long eb = __shfl_up_sync(0xffffffffu, einc, o);
-        if (lane >= o) { cinc += nb; einc += eb; }
+        const int a = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += a;
     }
-    const bool progress = __any_sync(0xffffffffu, lane < m && r > 0);
-    const bool open_shift = __any_sync(0xffffffffu, lane < m && sh - r > 0);
-    if (open_shift && !progress) return false;
-    if (lane < m) {
+    if (__shfl_sync(0xffffffffu, at, 31) > kCells || (open_shift && !progress)) return false;
+    if (have) {
         const Interval& o = v.iv[j];
         Interval& ni = S.niv[lane];
-        ni.sh = sh - r;
+        ni.sh = sh;
         ni.ncell = ncell;
         ni.klo = o.klo + ((uint32_t)(pa - v.slotbase[j]) << o.sh);
-        ni.khi = ni.klo + (uint32_t)((((unsigned long long)ncell) << ni.sh) - 1ull);
-        ni.cellbase = cinc - ncell;
+        ni.khi = ni.klo + (uint32_t)((((unsigned long long)ncell) << sh) - 1ull);
+        ni.cellbase = at - ncell;
         ni.pad = 0;
         ni.cbefore = v.cpre[pa];
         ni.sbefore = v.spre[pa];
+        atomicAdd((unsigned long long*)&S.cand, (unsigned long long)(v.cpre[pb + 1] - v.cpre[pa]));
     }
-    if (lane == 31) { S.cand = einc; S.nm = m; }
+    if (lane == 0) S.nm = m;
     __syncwarp();
     return true;
 }
 
-// Runs one solver pass for tensor t after all of its pieces of the current round arrived.
-// Called by every thread of the CTA; returns true when the tensor is finished.
+// Runs one solver pass for tensor t after a pass over it is complete: prefix arrays, then the levels or a
+// conservative range of cells for each, then the intervals of the next pass, or the finish when the copied
+// keys inside the new intervals are few enough.  Called by every thread of the CTA; returns true when the
+// tensor is finished.  S.iv, S.view.m / n / stot and S.lv describe the pass that just ended.
+//   round_buf: the keys copied by the pass (null: none were), cap: words of the tensor's key region.
 __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long long* glsum, int scheme,
                              int s, float* __restrict__ levels, int32_t* __restrict__ status,
                              unsigned* nitems, int2* items, const uint32_t* round_buf, bool enqueue,
-                             unsigned char* smem, SolverShared& S, int64_t cap)
+                             unsigned char* smem, SolverShared& S, int64_t cap, int round)
 {
-    constexpr size_t kOffSpre = (kSlots * sizeof(uint32_t) + 15) / 16 * 16;
     uint32_t* cpre = reinterpret_cast<uint32_t*>(smem);
     double* spre = reinterpret_cast<double*>(smem + kOffSpre);
-    uint8_t* slot_iv = smem + kOffSpre + kSlots * sizeof(double);
     const bool pb = scheme == OGQ_BINGRAD_PB;
-    const int round = st->round;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
 
-    __syncthreads();
-    if ((int)threadIdx.x < st->m) S.iv[threadIdx.x] = st->iv[threadIdx.x];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        S.view.m = st->m;
+    if (tid == 0) {
         S.view.iv = S.iv;
-        S.view.slot_iv = slot_iv;
-        S.view.xkeys = nullptr;
+        S.view.slot_iv = smem + kOffSlotIv;
         S.view.cpre = cpre;
         S.view.spre = spre;
-        S.view.n = st->n;
-        sel_init_slots(S.view);
-        S.done = 0; S.nm = 0; S.internal = 0;
+        S.done = 0; S.nm = -100; S.internal = 0; S.cand = 0; S.nopen = 0;
         S.pb_a = -1; S.pb_b = -1; S.pb_c = -1;
     }
+    for (int i = tid; i < (kSlots + 31) / 32; i += kSelThreads) S.marks[i] = 0u;
     __syncthreads();
-
-    // ---- prefix arrays over all slots: raw cell values, one block scan, per-interval shifts
-    const int nslots = S.view.nslots, m = S.view.m;
-    const int per = (nslots + kSelThreads - 1) / kSelThreads;
-    const int s0 = (int)threadIdx.x * per < nslots ? (int)threadIdx.x * per : nslots;
-    const int s1 = s0 + per < nslots ? s0 + per : nslots;
-    {
-        // interval index of every slot (blocked over threads, no global traffic)
-        int j = 0;
-        if (s0 < nslots) {
-            int lo = 0, hi = m;
-            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (S.view.slotbase[mid] <= s0) lo = mid; else hi = mid; }
-            j = lo;
-        }
-        for (int slot = s0; slot < s1; ++slot) {
-            while (slot >= S.view.slotbase[j + 1]) ++j;
-            slot_iv[slot] = (uint8_t)j;
+    solver_prefix(S, gcnt, glsum, round == 1, smem);
+    const int nslots = S.view.nslots;
+    if (round == 1) {
+        if (tid == 0) {
+            const double stot = spre[nslots - 1];
+            S.view.stot = stot;
+            st->stot = stot;
+            LvInfo& l = S.lv[pb ? 1 : s - 1];
+            l.c_le = S.view.n;
+            l.s_le = stot;
+            if ((long long)cpre[nslots - 1] != S.view.n) S.internal = 1;
         }
         __syncthreads();
-        // raw (count, sum) of every cell: strided so that the global loads are coalesced and independent
-        // (all of a thread's loads are issued before the first is used: they come from L2)
-        constexpr int kPerThread = (kSlots + kSelThreads - 1) / kSelThreads;
-        uint32_t rc[kPerThread];
-        unsigned long long rl[kPerThread];
-#pragma unroll
-        for (int u = 0; u < kPerThread; ++u) {
-            const int slot = threadIdx.x + u * kSelThreads;
-            rc[u] = 0u;
-            rl[u] = 0ull;
-            if (slot < nslots) {
-                const int jj = slot_iv[slot];
-                const int c = slot - S.view.slotbase[jj];
-                if (c < S.iv[jj].ncell) {
-                    rc[u] = __ldcg(gcnt + S.iv[jj].cellbase + c);
-                    rl[u] = __ldcg(glsum + S.iv[jj].cellbase + c);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kPerThread; ++u) {
-            const int slot = threadIdx.x + u * kSelThreads;
-            if (slot < nslots) {
-                double sm = 0.0;
-                if (rc[u]) {
-                    const int jj = slot_iv[slot];
-                    const int c = slot - S.view.slotbase[jj];
-                    sm = sel_cell_sum(S.iv[jj].klo + ((uint32_t)c << S.iv[jj].sh), S.iv[jj].sh, rc[u], rl[u]);
-                }
-                cpre[slot] = rc[u];
-                spre[slot] = sm;
-            }
-        }
-        __syncthreads();
-        // exclusive prefix: per-thread blocks, one block scan, in place
-        unsigned long long lc = 0;
-        double ls = 0.0;
-        for (int slot = s0; slot < s1; ++slot) { lc += cpre[slot]; ls += spre[slot]; }
-        unsigned long long tc;
-        double ts;
-        block_excl_scan(lc, ls, S.sc, S.ss, tc, ts);
-        for (int slot = s0; slot < s1; ++slot) {
-            const unsigned long long cn = cpre[slot];
-            const double sm = spre[slot];
-            cpre[slot] = (uint32_t)lc;
-            spre[slot] = ls;
-            lc += cn;
-            ls += sm;
-        }
     }
-    __syncthreads();
-    if ((int)threadIdx.x < m) {
-        // rounds >= 2: shift every interval so that it starts from the exact (count, sum) before it
-        const int sb = S.view.slotbase[threadIdx.x];
-        S.offc[threadIdx.x] = (round == 1) ? 0u : (uint32_t)((unsigned long long)S.iv[threadIdx.x].cbefore - cpre[sb]);
-        S.offs[threadIdx.x] = (round == 1) ? 0.0 : S.iv[threadIdx.x].sbefore - spre[sb];
-    }
-    __syncthreads();
-    if (round != 1)
-        for (int slot = s0; slot < s1; ++slot) {
-            const int j = slot_iv[slot];
-            cpre[slot] += S.offc[j];
-            spre[slot] += S.offs[j];
-        }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (round == 1) {
-            st->stot = spre[nslots - 1];
-            if ((long long)cpre[nslots - 1] != st->n) S.internal = 1;
-        }
-        S.view.stot = st->stot;
-    }
-    __syncthreads();
+    const double stot = S.view.stot;
+    int range_a = -1, range_b = -1;  // this warp's open range
 
-    if (pb && !S.internal && S.view.stot > 0.0) {
+    if (!pb) {
+        // one warp per level, one depth of Algorithm 1 at a time
+        static_assert(kSelWarps >= kMaxLv - 1, "one warp per interior level");
+#pragma unroll 1
+        for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
+            const int q = warp;
+            if (q < s - 1 && q >= stride && ((q - stride) & (2 * stride - 1)) == 0 && !S.lv[q].exact) {
+                const bool ok = warp_orq_solve(S.view, S.lv[q - stride], S.lv[q + stride], S.lv[q]);
+                __syncwarp();
+                if (!ok) {
+                    if (lane == 0) S.internal = 1;
+                } else if (!S.lv[q].exact) {
+                    range_a = S.lv[q].sa;
+                    range_b = S.lv[q].sb;
+                    if (lane == 0) S.nopen = 1;
+                }
+            }
+            __syncthreads();
+        }
+        if (tid < s) {
+            ExactLv& e = st->lv[tid];
+            const LvInfo& l = S.lv[tid];
+            e.exact = l.exact; e.key = l.key; e.c_lt = l.c_lt; e.c_le = l.c_le; e.s_lt = l.s_lt; e.s_le = l.s_le;
+        }
+    } else if (!S.internal && stot > 0.0) {
         // bracket of the sign change of g, evaluated at the lower edge of every cell
         int a = -1, b = -1, cs = -1;
-        for (int sl = threadIdx.x; sl < nslots; sl += kSelThreads) {
+#pragma unroll 1
+        for (int sl = tid; sl < nslots; sl += kSelThreads) {
             if (sel_is_end_slot(S.view, sl)) continue;
             double x;
             const double g = sel_pb_g(S.view, sl, &x);
             if (!(x < INFINITY)) continue;
-            const double eps = 1e-11 * (x * (double)S.view.n + S.view.stot);
+            const double eps = 1e-11 * (x * (double)S.view.n + stot);
             if (g < -eps) a = sl;
             if (g <= eps) b = sl;
             if (g <= 0.0) cs = sl;
@@ -1509,151 +1750,113 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
         if (a >= 0) atomicMax(&S.pb_a, a);
         if (b >= 0) atomicMax(&S.pb_b, b);
         if (cs >= 0) atomicMax(&S.pb_c, cs);
-    }
-    if (!pb && !S.internal) {
-        // one thread per level, one depth of Algorithm 1 at a time
-        if ((int)threadIdx.x < s) {
-            LvInfo& l = S.lv[threadIdx.x];
-            if (round == 1) {
-                l.exact = 0;
-                if (threadIdx.x == 0) {
-                    l.exact = 1; l.key = ~__ldcg(&st->kmin_inv); l.val = (double)sel_key_to_float(l.key);
-                    l.c_lt = 0; l.s_lt = 0.0; l.c_le = 0; l.s_le = 0.0;
-                } else if ((int)threadIdx.x == s - 1) {
-                    l.exact = 1; l.key = __ldcg(&st->kmax); l.val = (double)sel_key_to_float(l.key);
-                    l.c_lt = 0; l.s_lt = 0.0; l.c_le = S.view.n; l.s_le = S.view.stot;
-                }
-            } else {
-                const ExactLv& e = st->lv[threadIdx.x];
-                l.exact = e.exact; l.key = e.key; l.val = (double)sel_key_to_float(e.key);
-                l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
+        __syncthreads();
+        a = S.pb_a < 0 ? 0 : S.pb_a;
+        b = S.pb_b < a ? a : S.pb_b;
+        cs = S.pb_c < a ? a : S.pb_c;
+        if (cs > b) cs = b;
+        bool coarse = false;  // some cell of the bracket holds more than one key
+        for (int sl = a + tid; sl <= b; sl += kSelThreads)
+            coarse |= !sel_is_end_slot(S.view, sl) && sel_slot_shift(S.view, sl) != 0;
+        coarse = __syncthreads_or(coarse);
+        if (cpre[b + 1] == cpre[a]) {
+            // no element in the bracket: g is zero between two magnitudes
+            if (tid == 0) {
+                const float b1 = (float)((stot - spre[a]) / (double)S.view.n);
+                levels[2 * t] = -b1; levels[2 * t + 1] = b1;
             }
-        }
-        // (one warp per level: the solves of one depth are long chains of dependent shared-memory
-        // reads and fp64 divisions, and lanes of one warp that take different branches would run
-        // one after the other)
-        static_assert(kSelWarps >= kMaxLv - 1, "one warp per interior level");
-        for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
-            __syncthreads();
-            const int q = threadIdx.x >> 5;
-            if ((threadIdx.x & 31) == 0 && q < s - 1 && q >= stride && ((q - stride) % (2 * stride)) == 0 &&
-                !S.lv[q].exact) {
-                if (!sel_orq_solve(S.view, S.lv[q - stride], S.lv[q + stride], S.lv[q])) S.internal = 1;
-            }
-        }
-    }
-    __syncthreads();
-
-    if (threadIdx.x == 0) {
-        int open = 0;
-        int stbits = 0;
-        if (S.internal) {
-            stbits = OGQ_ST_INTERNAL;
-            S.done = 1;
-        } else if (pb) {
-            if (!(S.view.stot > 0.0)) {
-                levels[2 * t] = 0.f; levels[2 * t + 1] = 0.f;
-                stbits = OGQ_ST_CONSTANT;
-                S.done = 1;
-            } else {
-                int a = S.pb_a < 0 ? 0 : S.pb_a;
-                int b = S.pb_b < a ? a : S.pb_b;
-                int cs = S.pb_c < a ? a : S.pb_c;
-                if (cs > b) cs = b;
-                bool fine = true;
-                for (int sl = a; sl <= b; ++sl)
-                    if (!sel_is_end_slot(S.view, sl) && sel_slot_shift(S.view, sl) != 0) fine = false;
-                if (fine && !sel_is_end_slot(S.view, cs)) {
-                    const float b1 = (float)sel_pb_final(S.view, cs);
-                    levels[2 * t] = -b1; levels[2 * t + 1] = b1;
-                    S.done = 1;
-                } else {
-                    S.ra[0] = a; S.rb[0] = b; open = 1;
-                }
+        } else if (!coarse && !sel_is_end_slot(S.view, cs)) {
+            if (tid == 0) {
+                const float b1 = (float)sel_pb_final(S.view, cs);
+                levels[2 * t] = -b1; levels[2 * t + 1] = b1;
             }
         } else {
-            for (int q = 1; q < s - 1; ++q)
-                if (!S.lv[q].exact) { S.ra[open] = S.lv[q].sa; S.rb[open] = S.lv[q].sb; ++open; }
-            if (open == 0) S.done = 1;
+            if (warp == 0) { range_a = a; range_b = b; }
+            if (tid == 0) S.nopen = 1;
         }
-        S.nr = open;
-        S.nm = -100;
-        S.cand = 0;
-        if (!S.done && round + 1 > kMaxRounds) { stbits = OGQ_ST_ITER_CAP; S.done = 1; }
-        if (stbits) {
-            // unresolved: leave zeros rather than garbage
-            if (pb) { levels[2 * t] = 0.f; levels[2 * t + 1] = 0.f; }
-            else for (int q = 0; q < s; ++q) levels[(int64_t)t * s + q] = 0.f;
-            status[t] |= stbits;
+        __syncthreads();
+    }
+    const bool fail = S.internal != 0, zero = pb && !fail && !(stot > 0.0);
+    const bool capped = round + 1 > kMaxRounds && S.nopen;
+    if (fail || zero || !S.nopen || capped) {
+        const int nl = pb ? 2 : s;
+        if (fail || zero || capped) {
+            // unresolved: zeros rather than garbage
+            if (tid < nl) levels[(int64_t)t * nl + tid] = 0.f;
+            if (tid == 0) status[t] |= fail ? OGQ_ST_INTERNAL : zero ? OGQ_ST_CONSTANT : OGQ_ST_ITER_CAP;
+        } else if (!pb && tid < s) {
+            levels[(int64_t)t * s + tid] = sel_key_to_float(S.lv[tid].key);
+        }
+        if (tid == 0) st->done = 1;
+        __threadfence();
+        __syncthreads();
+        return true;
+    }
+    // candidate cells: the populated cells of the open ranges
+    if (range_a >= 0) {
+#pragma unroll 1
+        for (int c0 = range_a & ~31; c0 <= range_b; c0 += 32) {
+            const int c = c0 + lane;
+            const bool in = c >= range_a && c <= range_b && !sel_is_end_slot(S.view, c) && cpre[c + 1] != cpre[c];
+            const uint32_t w = __ballot_sync(0xffffffffu, in);
+            if (lane == 0 && w) atomicOr(&S.marks[c0 >> 5], w);
         }
     }
     __syncthreads();
-    if (!pb && !S.internal && (int)threadIdx.x < s) {
-        if (S.done) {
-            if (S.nr == 0 && !(status[t] & (OGQ_ST_ITER_CAP | OGQ_ST_INTERNAL)))
-                levels[(int64_t)t * s + threadIdx.x] = sel_key_to_float(S.lv[threadIdx.x].key);
-        } else {
-            ExactLv& e = st->lv[threadIdx.x];
-            const LvInfo& l = S.lv[threadIdx.x];
-            e.exact = l.exact; e.key = l.key; e.c_lt = l.c_lt; e.c_le = l.c_le; e.s_lt = l.s_lt; e.s_le = l.s_le;
-        }
-    }
-    if (!S.done) {
-        // intervals of the next round: warp-parallel common case, single-thread general case
-        bool ok = true;
-        if (threadIdx.x < 32) ok = refine_parallel(S, !pb);
-        if (threadIdx.x == 0 && !ok) {
-            const int nm = sel_refine(S.view, S.nr, S.ra, S.rb, !pb, S.niv, &S.cand);
-            if (nm < 0) {
-                if (pb) { levels[2 * t] = 0.f; levels[2 * t + 1] = 0.f; }
-                else for (int q = 0; q < s; ++q) levels[(int64_t)t * s + q] = 0.f;
-                status[t] |= OGQ_ST_INTERNAL;
-                S.done = 1;
-            } else {
-                S.nm = nm;
-            }
+    if (warp == 0) {
+        const bool ok = refine_marked(S);
+        if (lane == 0 && !ok) {
+            // too many scattered cells: the general single-thread routine, which may keep empty stretches
+            int nr = 0, ra[kMaxLv], rb[kMaxLv];
+            if (pb) { ra[0] = range_a; rb[0] = range_b; nr = 1; }
+            else
+                for (int q = 1; q < s - 1; ++q)
+                    if (!S.lv[q].exact) { ra[nr] = S.lv[q].sa; rb[nr] = S.lv[q].sb; ++nr; }
+            S.nm = sel_refine(S.view, nr, ra, rb, !pb, S.niv, &S.cand);
         }
     }
     __syncthreads();
-
-    if (S.done) {
-        if (threadIdx.x == 0) { st->done = 1; __threadfence(); }
+    if (S.nm < 0) {
+        const int nl = pb ? 2 : s;
+        if (tid < nl) levels[(int64_t)t * nl + tid] = 0.f;
+        if (tid == 0) { status[t] |= OGQ_ST_INTERNAL; st->done = 1; }
+        __threadfence();
+        __syncthreads();
         return true;
     }
     // (the copies of the pass that just ended are complete unless it overflowed its region)
     const bool incomplete = round >= 2 && __ldcg(&st->overflow) != 0;
-    if (!pb && round >= 2 && S.cand <= kSmallN && round_buf != nullptr && !incomplete) {
+    const bool few = S.cand <= kSortN;
+    if (round >= 2 && few && round_buf != nullptr && !incomplete) {
         const long long src_cnt = (long long)__ldcg(&st->cursor[round & 1]);
-        if (src_cnt <= kSortScanMax) {
-            sort_finish(st, t, s, round_buf, src_cnt, levels, status, smem, S);
+        if (src_cnt <= (enqueue ? kScanMax : kScanMaxAlone)) {
+            finish_from_keys(st, t, pb, s, round_buf, (int)src_cnt, src_cnt == S.cand, levels, status, smem, S);
             return true;
         }
     }
-    // prepare the next round: clear the cells it will use, publish the new intervals.  When the
-    // elements inside the new intervals already fit one sort (ORQ), the next pass only copies them
-    // and its last CTA sorts and finishes the tensor (finish_sorted): no cells, no further solver pass.
-    const bool compact_only = !pb && S.cand <= kSmallN && S.cand <= cap;
+    // prepare the next round: clear the cells it will use, publish the new intervals.  When the elements
+    // inside the new intervals are few enough, the next pass only copies them and finish_sorted finishes
+    // the tensor: no cells, no further solver pass.
+    const bool compact_only = few && S.cand <= cap;
     const int ncells_next = S.niv[S.nm - 1].cellbase + S.niv[S.nm - 1].ncell;
-    if (!compact_only)
-        for (int i = threadIdx.x; i < ncells_next; i += kSelThreads) {
-            gcnt[i] = 0u;
-            glsum[i] = 0ull;
-        }
-    if ((int)threadIdx.x < S.nm) st->iv[threadIdx.x] = S.niv[threadIdx.x];
-    if (threadIdx.x == 0) {
+    if (!compact_only) {
+        for (int i = tid; i < ncells_next; i += kSelThreads) { gcnt[i] = 0u; glsum[i] = 0ull; }
+    }
+    if (tid < S.nm) st->iv[tid] = S.niv[tid];
+    if (tid == 0) {
         st->m = S.nm;
+        st->cand = S.cand;
         st->compact_only = compact_only ? 1 : 0;
         st->from_grad = incomplete ? 1 : 0;  // the next pass cannot read copies that were cut short
         st->overflow = 0;
         st->round = round + 1;
         st->arrive = 0;
-        st->arrived = 0ull;
         const int next = round + 1;
         st->cursor[next & 1] = 0ull;  // buffer the next round writes
         if (next == 3 && enqueue) {
             // work items of the round-3 kernel: slices of the copied keys, or of the tensor itself when
             // the copies were cut short
-            const unsigned long long cntk = incomplete ? (unsigned long long)(st->n / 16) : __ldcg(&st->cursor[0]);
+            const unsigned long long cntk = incomplete ? (unsigned long long)(S.view.n / 16) : __ldcg(&st->cursor[0]);
             unsigned ns = (unsigned)((cntk + kSliceElems - 1) / kSliceElems);
             if (ns < 1) ns = 1;
             if (ns > kMaxSlices) ns = kMaxSlices;
@@ -1667,166 +1870,25 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
     return false;
 }
 
-// Finishes a tensor whose last pass only copied the keys inside its intervals (TState::compact_only):
-// the solver state the previous pass left in global memory is loaded back, then the copied keys are
-// sorted and every open level is solved on single-key cells.  Called by every thread of the CTA that
-// arrived last for the tensor.
-__device__ void finish_sorted(TState* st, int t, int s, const uint32_t* copied, float* __restrict__ levels,
-                              int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, int cursor_idx)
+// Loads what solver_round needs of a tensor in round >= 2 back from its state.
+__device__ __forceinline__ int solver_load(const TState* st, SolverShared& S, bool pb, int s)
 {
+    const int tid = threadIdx.x, m = __ldcg(&st->m);
     __syncthreads();
-    const int m = __ldcg(&st->m);
-    if ((int)threadIdx.x < m) S.niv[threadIdx.x] = st->iv[threadIdx.x];
-    if ((int)threadIdx.x < s) {
-        const ExactLv& e = st->lv[threadIdx.x];
-        LvInfo& l = S.lv[threadIdx.x];
-        l.exact = e.exact; l.key = e.key; l.val = (double)sel_key_to_float(e.key);
+    if (tid < m) S.iv[tid] = st->iv[tid];
+    if (!pb && tid >= 64 && tid - 64 < s) {
+        const ExactLv& e = st->lv[tid - 64];
+        LvInfo& l = S.lv[tid - 64];
+        l.exact = e.exact; l.key = e.key;
+        l.val = l.vlo = l.vhi = (double)sel_key_to_float(e.key);
         l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
-        l.sa = l.sb = 0; l.vlo = l.vhi = l.val;
     }
-    if (threadIdx.x == 0) {
-        S.nm = m;
+    if (tid == 0) {
+        S.view.m = m;
         S.view.n = st->n;
         S.view.stot = st->stot;
-        S.internal = 0;
     }
-    __syncthreads();
-    const long long src_cnt = (long long)__ldcg(&st->cursor[cursor_idx]);
-    sort_finish(st, t, s, copied, src_cnt, levels, status, smem, S);
-}
-
-// ---------------------------------------------------------------------------
-// Small tensors: sort the keys in shared memory and apply the definitions directly.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int lower_bound_u32(const uint32_t* a, int n, uint32_t k)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) { const int mid = (lo + hi) >> 1; if (a[mid] < k) lo = mid + 1; else hi = mid; }
-    return lo;
-}
-
-__device__ __forceinline__ int upper_bound_u32(const uint32_t* a, int n, uint32_t k)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) { const int mid = (lo + hi) >> 1; if (a[mid] <= k) lo = mid + 1; else hi = mid; }
-    return lo;
-}
-
-__device__ void small_tensor(const float* __restrict__ grad, int64_t tb, int n, int t, int scheme, int s,
-                             float* __restrict__ levels, int32_t* __restrict__ status, TState* st,
-                             unsigned char* smem, float tau)
-{
-    __shared__ double sh_d[kSelWarps];
-    __shared__ uint32_t sh_lvkey[kMaxLv];
-    __shared__ int sh_flag;
-    __shared__ double sh_bcast;
-    uint32_t* keys = reinterpret_cast<uint32_t*>(smem);
-    const bool pb = scheme == OGQ_BINGRAD_PB;
-    int P = 1;
-    while (P < n) P <<= 1;
-    if (threadIdx.x == 0) sh_flag = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < P; i += kSelThreads) {
-        uint32_t key = 0xffffffffu;
-        if (i < n) {
-            const float raw = __ldg(grad + tb + i);
-            uint32_t bits = __float_as_uint(copysignf(fminf(fabsf(raw), tau), raw));
-            if ((bits & 0x7f800000u) == 0x7f800000u) sh_flag = 1;
-            if (pb) key = bits | 0x80000000u;
-            else {
-                if (bits == 0x80000000u) bits = 0u;
-                key = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
-            }
-        }
-        keys[i] = key;
-    }
-    __syncthreads();
-    block_bitonic_sort(keys, P);  // ascending
-    int stbits = 0;
-    if (sh_flag) {
-        if (threadIdx.x == 0) {
-            const int nl = pb ? 2 : s;
-            for (int q = 0; q < nl; ++q) levels[(int64_t)t * nl + q] = 0.f;
-            status[t] = OGQ_ST_NONFINITE;
-            st->done = 1;
-        }
-        return;
-    }
-    if (!pb) {
-        if (keys[0] == keys[n - 1]) stbits |= OGQ_ST_CONSTANT;
-        if (threadIdx.x == 0) {
-            for (int q = 0; q < s; ++q) sh_lvkey[q] = keys[0];
-            sh_lvkey[s - 1] = keys[n - 1];
-        }
-        __syncthreads();
-        for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
-            for (int q = stride; q < s - 1; q += 2 * stride) {
-                const uint32_t kl = sh_lvkey[q - stride], kr = sh_lvkey[q + stride];
-                uint32_t res = kl;
-                if (kr > kl) {
-                    const int i0 = lower_bound_u32(keys, n, kl), i1 = upper_bound_u32(keys, n, kr);
-                    const double Lv = (double)sel_key_to_float(kl), Rv = (double)sel_key_to_float(kr);
-                    double a = 0.0;
-                    for (int i = i0 + threadIdx.x; i < i1; i += kSelThreads) a += (double)sel_key_to_float(keys[i]) - Lv;
-                    a = sel_block_sum(a, sh_d);
-                    if (threadIdx.x == 0) sh_bcast = a;
-                    __syncthreads();
-                    a = sh_bcast;
-                    const double T = a / (Rv - Lv);
-                    long long k = (long long)floor(T);
-                    const long long m = i1 - i0;
-                    if (k < 0) k = 0;
-                    if (k > m - 1) k = m - 1;
-                    res = keys[i1 - 1 - (int)k];
-                }
-                __syncthreads();
-                if (threadIdx.x == 0) sh_lvkey[q] = res;
-                __syncthreads();
-            }
-        }
-        if (threadIdx.x < s) levels[(int64_t)t * s + threadIdx.x] = sel_key_to_float(sh_lvkey[threadIdx.x]);
-        if (threadIdx.x == 0) { status[t] = stbits; st->done = 1; }
-        return;
-    }
-    // BinGrad-pb: prefix sums of the sorted magnitudes, then the sign change of g
-    double* pre = reinterpret_cast<double*>(smem + kSmallN * sizeof(uint32_t));  // [n + 1]
-    __shared__ unsigned long long sc_[kSelWarps];
-    __shared__ double ss_[kSelWarps];
-    __shared__ int sh_c;
-    const int per = (n + kSelThreads - 1) / kSelThreads;
-    const int c0 = threadIdx.x * per < n ? threadIdx.x * per : n;
-    const int c1 = c0 + per < n ? c0 + per : n;
-    unsigned long long dummy = 0, dt;
-    double ls = 0.0, tot;
-    for (int i = c0; i < c1; ++i) ls += (double)sel_key_to_float(keys[i]);
-    block_excl_scan(dummy, ls, sc_, ss_, dt, tot);
-    double run = ls;
-    for (int i = c0; i < c1; ++i) { pre[i] = run; run += (double)sel_key_to_float(keys[i]); }
-    if (threadIdx.x == 0) { pre[n] = tot; sh_c = -1; }
-    __syncthreads();
-    int best = -1;
-    for (int i = threadIdx.x; i < n; i += kSelThreads) {
-        const double x = (double)sel_key_to_float(keys[i]);
-        const int first = lower_bound_u32(keys, n, keys[i]);
-        const double g = x * (double)n - (tot - pre[first]);
-        if (g <= 0.0) best = i;
-    }
-    if (best >= 0) atomicMax(&sh_c, best);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float b1 = 0.f;
-        if (!(tot > 0.0)) stbits |= OGQ_ST_CONSTANT;
-        else {
-            const int c = sh_c < 0 ? 0 : sh_c;
-            const double x = (double)sel_key_to_float(keys[c]);
-            const int up = upper_bound_u32(keys, n, keys[c]);
-            const double stat_up = (tot - pre[up]) / (double)n;
-            b1 = (float)(stat_up > x ? stat_up : x);
-        }
-        levels[2 * t] = -b1; levels[2 * t + 1] = b1;
-        status[t] = stbits;
-        st->done = 1;
-    }
+    return __ldcg(&st->round);
 }
 
 // ---------------------------------------------------------------------------
@@ -1857,7 +1919,7 @@ __device__ __forceinline__ void grad_pass(const SelArgs& A, int t, int64_t tbeg,
     const bool mag = A.scheme == OGQ_BINGRAD_PB;
     if (A.tau)
         stream_round2<true>(A.grad, pb_, pe_, mag, tb, hist, hist + kCells, hist + 2 * kCells, stage, dst, cap,
-                            &st->cursor[k], &st->overflow, copy_only, __ldg(A.tau + t));
+                            &st->cursor[k], &st->overflow, copy_only, __ldcg(A.tau + t));
     else
         stream_round2<false>(A.grad, pb_, pe_, mag, tb, hist, hist + kCells, hist + 2 * kCells, stage, dst, cap,
                              &st->cursor[k], &st->overflow, copy_only, 0.f);
@@ -1873,7 +1935,7 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
     const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
     for (int guard = 0; guard < kMaxRounds; ++guard) {
-        const int round = st->round;
+        const int round = __ldcg(&st->round);
         const uint32_t* src = A.ws.buf[(round - 1) & 1];  // 16-byte aligned base; indices are absolute
         const int64_t cnt = (int64_t)__ldcg(&st->cursor[(round - 1) & 1]);
         const bool copy_only = st->compact_only != 0;
@@ -1901,14 +1963,15 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
         if (copy_only) {
             __threadfence();
             __syncthreads();
-            finish_sorted(st, t, A.s, A.ws.buf[round & 1] + sel_region(tbeg), A.levels, A.status, smem, S, round & 1);
+            finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[round & 1] + sel_region(tbeg), A.levels, A.status, smem, S, round & 1);
             return;
         }
         flush_hist(hist, tb.ncells, gcnt, glsum);
         __threadfence();
+        solver_load(st, S, A.scheme == OGQ_BINGRAD_PB, A.s);
         __syncthreads();
         if (solver_round(st, t, gcnt, glsum, A.scheme, A.s, A.levels, A.status, A.ws.nitems, A.ws.items,
-                         A.ws.buf[round & 1] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg)))
+                         A.ws.buf[round & 1] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg), round))
             return;
     }
     if (threadIdx.x == 0) {
@@ -1917,327 +1980,228 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
     }
 }
 
+// Clears what the passes over tensor t add to and fixes the tensor's window: one CTA per tensor.
+__global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
+{
+    __shared__ int sh_i[kSelWarps];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = blockIdx.x;
+    const int64_t tbeg = __ldg(A.off + t), n = __ldg(A.off + t + 1) - tbeg;
+    if (t == 0 && threadIdx.x == 0) *A.ws.nitems = 0u;
+    if (n <= kSmallN) return;
+    // Anchor of the fine window: largest binade among strided samples, plus two.
+    int e = (int)((__float_as_uint(__ldg(A.grad + tbeg + (int64_t)threadIdx.x * n / kSelThreads)) >> 23) & 255u);
+    if (e == 255) e = 0;
+    const int ncells = A.scheme == OGQ_BINGRAD_PB ? kRound1Mag : kRound1Cells;
+    uint4* cnt = reinterpret_cast<uint4*>(A.ws.gcnt + (size_t)t * kCells);
+    uint4* sum = reinterpret_cast<uint4*>(A.ws.glsum + (size_t)t * kCells);
+    for (int i = threadIdx.x; i < ncells / 4; i += kSelThreads) cnt[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < ncells / 2; i += kSelThreads) sum[i] = make_uint4(0u, 0u, 0u, 0u);
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) sh_i[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int hi_e = 0;
+        for (int w = 0; w < kSelWarps; ++w) hi_e = max(hi_e, sh_i[w]);
+        hi_e += 2;
+        if (hi_e < kSelW) hi_e = kSelW;
+        if (hi_e > 255) hi_e = 255;  // binade 255 (Inf / NaN) always stays outside the fine window
+        TState* st = A.ws.st + t;
+        st->hi_e = hi_e;
+        st->done = 0;
+        st->kmin_inv = 0u;
+        st->kmax = 0u;
+        st->nonfinite = 0u;
+        st->arrive = 0u;
+        st->overflow = 0;
+        st->from_grad = 0;
+        st->compact_only = 0;
+        st->cursor[0] = 0ull;
+        st->cursor[1] = 0ull;
+    }
+}
+
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SolverShared S;
-    __shared__ Interval r1iv[kMaxIv];
-    __shared__ int sh_i[kSelWarps];
-    __shared__ int sh_last;
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
     const int nl = pb ? 2 : A.s;
-
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
-
-    // Anchor of the fine window of tensor [tbeg, tbeg + n): largest binade among strided samples, plus
-    // two (every CTA of the tensor samples the same elements and so arrives at the same window).
-    auto window_anchor = [&](int64_t tbeg, int64_t n) -> int {
-        int hi_e;
-        {
-            const int64_t idx = tbeg + (int64_t)threadIdx.x * n / kSelThreads;
-            int e = (int)((__float_as_uint(__ldg(A.grad + idx)) >> 23) & 255u);
-            if (e == 255) e = 0;
-            e = __reduce_max_sync(0xffffffffu, e);
-            __syncthreads();  // earlier readers of sh_i are done
-            if ((threadIdx.x & 31) == 0) sh_i[threadIdx.x >> 5] = e;
-            __syncthreads();
-            hi_e = __reduce_max_sync(0xffffffffu, ((threadIdx.x & 31) < kSelWarps) ? sh_i[threadIdx.x & 31] : 0) + 2;
-            if (hi_e < kSelW) hi_e = kSelW;
-            if (hi_e > 255) hi_e = 255;  // binade 255 (Inf / NaN) always stays outside the fine window
-        }
-        return hi_e;
-    };
-
-    // Round 1 of a tensor on this CTA, in three steps: r1_begin clears the CTA's cells, r1_add streams
-    // a piece of the tensor into them (any number of pieces), r1_flush adds the cells to the tensor's
-    // global ones, reports `elems` streamed elements and returns true when that completes the tensor;
-    // the CTA for which it does runs r1_solve.
-    float r1_vmin = 0.f, r1_vmax = 0.f, r1_tau = 0.f;
-    uint32_t r1_nf = 0u;
-    int r1_lo_e = 0;
-    uint32_t* packed_cells = reinterpret_cast<uint32_t*>(smem + kSmemHist);
-    const int r1_ncells = pb ? kRound1Mag : kRound1Cells;
-    auto r1_begin = [&](int t, int64_t tbeg, int64_t tend) {
-        r1_lo_e = window_anchor(tbeg, tend - tbeg) - kSelW;
-        r1_tau = A.tau ? __ldg(A.tau + t) : 0.f;
-        r1_vmin = __int_as_float(0x7f800000);
-        r1_vmax = __int_as_float(0xff800000);
-        r1_nf = 0u;
-        __syncthreads();
-        zero_hist(hist, r1_ncells);
-        for (int i = threadIdx.x; i < kPackedCells; i += kSelThreads) packed_cells[i] = 0u;
-        __syncthreads();
-    };
-    auto r1_add = [&](int64_t pb_, int64_t pe_) {
-        const bool clip = A.tau != nullptr;
-        if (pb) {
-            if (clip) stream_round1<true, true>(A.grad, pb_, pe_, r1_lo_e, hist, packed_cells, r1_vmin, r1_vmax, r1_nf, r1_tau);
-            else stream_round1<true, false>(A.grad, pb_, pe_, r1_lo_e, hist, packed_cells, r1_vmin, r1_vmax, r1_nf, r1_tau);
-        } else {
-            if (clip) stream_round1<false, true>(A.grad, pb_, pe_, r1_lo_e, hist, packed_cells, r1_vmin, r1_vmax, r1_nf, r1_tau);
-            else stream_round1<false, false>(A.grad, pb_, pe_, r1_lo_e, hist, packed_cells, r1_vmin, r1_vmax, r1_nf, r1_tau);
-        }
-    };
-    auto r1_flush = [&](int t, int64_t n, int64_t elems) -> bool {
-        TState* st = A.ws.st + t;
-        __syncthreads();
-        flush_hist(hist, r1_ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
-        // min / max / non-finite: one atomic per warp
-        {
-            const uint32_t kmin = __reduce_min_sync(0xffffffffu, float_to_key(r1_vmin));  // +Inf / -Inf when the
-            const uint32_t kmax = __reduce_max_sync(0xffffffffu, float_to_key(r1_vmax));  // thread saw nothing
-            const bool anynf = __any_sync(0xffffffffu, r1_nf != 0u);
-            if ((threadIdx.x & 31) == 0) {
-                atomicMax(&st->kmin_inv, ~kmin);
-                atomicMax(&st->kmax, kmax);
-                if (anynf) atomicOr(&st->nonfinite, 1u);
-            }
-        }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const unsigned long long prev = atomicAdd(&st->arrived, (unsigned long long)elems);
-            sh_last = (prev + (unsigned long long)elems == (unsigned long long)n);
-        }
-        __syncthreads();
-        if (!sh_last) return false;
-        __threadfence();
-        return true;
-    };
-
-    // Last CTA of tensor t: sets up the state and runs the first solver pass.  Returns true when the
-    // tensor is finished.
-    auto r1_solve = [&](int t, int64_t tbeg, int64_t tend, bool alone) -> bool {
-        const int64_t n = tend - tbeg;
-        TState* st = A.ws.st + t;
-        const int hi_e = window_anchor(tbeg, n);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            st->n = n;
-            st->round = 1;
-            st->hi_e = hi_e;
-            const int m = round1_intervals(hi_e, pb, r1iv);
-            st->m = m;
-            for (int j = 0; j < m; ++j) st->iv[j] = r1iv[j];
-            int stb = 0;
-            const uint32_t kmn = ~__ldcg(&st->kmin_inv), kmx = __ldcg(&st->kmax);
-            if (__ldcg(&st->nonfinite)) stb |= OGQ_ST_NONFINITE;
-            else if (!pb && kmn == kmx) stb |= OGQ_ST_CONSTANT;
-            A.status[t] = stb;
-            sh_last = stb;
-            if (stb & OGQ_ST_NONFINITE) {
-                for (int q = 0; q < nl; ++q) A.levels[(int64_t)t * nl + q] = 0.f;
-                st->done = 1;
-            } else if (stb & OGQ_ST_CONSTANT) {
-                const float v = sel_key_to_float(kmn);
-                for (int q = 0; q < nl; ++q) A.levels[(int64_t)t * nl + q] = v;
-                st->done = 1;
-            }
-        }
-        __syncthreads();
-        if (sh_last & (OGQ_ST_NONFINITE | OGQ_ST_CONSTANT)) return true;
-        bool done;
-        done = solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells,
-                                           A.scheme, A.s, A.levels, A.status, A.ws.nitems, A.ws.items, nullptr,
-                                           !alone, smem, S, sel_region(tend) - sel_region(tbeg));
-        return done;
-    };
+    pdl_wait();
+    pdl_launch_dependents();
 
     if ((int)blockIdx.x < A.T) {
-        // the first T CTAs, one per tensor, settle the empty, small and mid-size tensors; they come
-        // first in the grid because the mid-size ones run longest
-        [&]() {
+        // the first T CTAs, one per tensor, settle the empty and small tensors
         const int t = blockIdx.x;
         const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
         const int64_t n = tend - tbeg;
         if (n <= 0) {
             if (threadIdx.x < nl) A.levels[(int64_t)t * nl + threadIdx.x] = 0.f;
-            if (threadIdx.x == 0) { A.status[t] = OGQ_ST_EMPTY; A.ws.st[t].done = 1; }
+            if (threadIdx.x == 0) A.status[t] = OGQ_ST_EMPTY;
         } else if (n <= kSmallN) {
-            small_tensor(A.grad, tbeg, (int)n, t, A.scheme, A.s, A.levels, A.status, A.ws.st + t, smem,
-                         A.tau ? __ldg(A.tau + t) : __int_as_float(0x7f800000));
-        } else if (n <= kMidN) {
-            // round 1 and its solver pass on this CTA; the tensor's CTA of the round-2 kernel goes on from there
-            r1_begin(t, tbeg, tend);
-            r1_add(tbeg, tend);
-            r1_flush(t, n, n);
-            r1_solve(t, tbeg, tend, true);
+            small_tensor(A.grad + tbeg, (int)n, t, pb, A.s, A.levels, A.status, smem, S,
+                         A.tau ? __ldcg(A.tau + t) : __int_as_float(0x7f800000));
         }
-        }();
         return;
     }
 
-    // Flat CTAs: one chunk of the bucket each.  The solver passes of the tensors this CTA completed wait
-    // until its chunk has been streamed, so that a solver pass never holds up another tensor's arrival.
-    // (Handing smaller chunks out from a counter was tried and lost: the CTAs of a launch already finish
-    // within a few percent of one another, what ends late are the solver passes, and every extra chunk
-    // boundary costs a set-up and, in round 2, a drain of the compaction stages.)
-    constexpr int kDefer = 8;
-    int dt[kDefer];
-    int nd = 0;
-    int cur_t = -1;
-    int64_t cur_n = 0, cur_elems = 0;
-    auto done_with_current = [&]() {
-        if (cur_t < 0) return;
-        if (r1_flush(cur_t, cur_n, cur_elems)) {
-            if (nd < kDefer) {
-#pragma unroll
-                for (int u = 0; u < kDefer; ++u)
-                    if (u == nd) dt[u] = cur_t;
-                ++nd;
-            } else {
-                r1_solve(cur_t, __ldg(A.off + cur_t), __ldg(A.off + cur_t + 1), false);
-            }
+    // Flat CTAs: one chunk of the bucket each.  A piece of a tensor is streamed into the CTA's cells, which
+    // are then added to the tensor's global ones.
+    float vmin = 0.f, vmax = 0.f, tau = 0.f;
+    uint32_t nf = 0u;
+    int lo_e = 0;
+    uint32_t* packed_cells = reinterpret_cast<uint32_t*>(smem + kSmemHist);
+    const int ncells = pb ? kRound1Mag : kRound1Cells;
+    const int64_t lo = (int64_t)(blockIdx.x - A.T) * A.chunk;
+    const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
+    for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
+        if (tend - tbeg <= kSmallN) return;
+        TState* st = A.ws.st + t;
+        lo_e = __ldcg(&st->hi_e) - kSelW;
+        tau = A.tau ? __ldcg(A.tau + t) : 0.f;
+        vmin = __int_as_float(0x7f800000);
+        vmax = __int_as_float(0xff800000);
+        nf = 0u;
+        __syncthreads();
+        zero_hist(hist, ncells);
+        for (int i = threadIdx.x; i < kPackedCells; i += kSelThreads) packed_cells[i] = 0u;
+        __syncthreads();
+        const bool clip = A.tau != nullptr;
+        if (pb) {
+            if (clip) stream_round1<true, true>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
+            else stream_round1<true, false>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
+        } else {
+            if (clip) stream_round1<false, true>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
+            else stream_round1<false, false>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
         }
-        cur_t = -1;
-    };
-    {
-        const int64_t lo = (int64_t)(blockIdx.x - A.T) * A.chunk;
-        const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
-        for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
-            if (tend - tbeg <= kMidN) return;
-            if (t != cur_t) {
-                done_with_current();
-                r1_begin(t, tbeg, tend);
-                cur_t = t;
-                cur_n = tend - tbeg;
-                cur_elems = 0;
-            }
-            r1_add(pb_, pe_);
-            cur_elems += pe_ - pb_;
-        });
+        __syncthreads();
+        flush_hist(hist, ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
+        // min / max / non-finite: one atomic per warp
+        const uint32_t kmin = __reduce_min_sync(0xffffffffu, float_to_key(vmin));  // +Inf / -Inf when the
+        const uint32_t kmax = __reduce_max_sync(0xffffffffu, float_to_key(vmax));  // thread saw nothing
+        const bool anynf = __any_sync(0xffffffffu, nf != 0u);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&st->kmin_inv, ~kmin);
+            atomicMax(&st->kmax, kmax);
+            if (anynf) atomicOr(&st->nonfinite, 1u);
+        }
+    });
+}
+
+// The first solver pass of every streamed tensor: one CTA per tensor.
+__global__ void __launch_bounds__(kSelThreads) k_sel_solve1(SelArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ SolverShared S;
+    const bool pb = A.scheme == OGQ_BINGRAD_PB;
+    const int nl = pb ? 2 : A.s;
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = blockIdx.x;
+    const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
+    const int64_t n = tend - tbeg;
+    if (n <= kSmallN) return;
+    TState* st = A.ws.st + t;
+    const int tid = threadIdx.x;
+    const uint32_t kmn = ~__ldcg(&st->kmin_inv), kmx = __ldcg(&st->kmax);
+    const int hi_e = __ldcg(&st->hi_e);
+    const bool bad = __ldcg(&st->nonfinite) != 0u, constant = !bad && !pb && kmn == kmx;
+    if (bad || constant) {
+        if (tid < nl) A.levels[(int64_t)t * nl + tid] = bad ? 0.f : sel_key_to_float(kmn);
+        if (tid == 0) {
+            A.status[t] = bad ? OGQ_ST_NONFINITE : OGQ_ST_CONSTANT;
+            st->done = 1;
+        }
+        return;
     }
-    done_with_current();
-#pragma unroll
-    for (int u = 0; u < kDefer; ++u)
-        if (u < nd) r1_solve(dt[u], __ldg(A.off + dt[u]), __ldg(A.off + dt[u] + 1), false);
+    if (tid < (pb ? 3 : 6)) S.iv[tid] = round1_interval(hi_e, pb, tid);
+    if (tid >= 64 && tid - 64 < A.s) {
+        const int q = tid - 64;
+        LvInfo& l = S.lv[q];
+        l.exact = (q == 0 || q == A.s - 1) ? 1 : 0;
+        l.key = q == 0 ? kmn : kmx;
+        l.val = l.vlo = l.vhi = (double)sel_key_to_float(l.key);
+        l.c_lt = 0; l.s_lt = 0.0; l.c_le = 0; l.s_le = 0.0;
+    }
+    if (tid == 0) {
+        st->n = n;
+        A.status[t] = 0;
+        S.view.m = pb ? 3 : 6;
+        S.view.n = n;
+        S.view.stot = 0.0;
+    }
+    solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s, A.levels, A.status,
+                 A.ws.nitems, A.ws.items, nullptr, false, smem, S, sel_region(tend) - sel_region(tbeg), 1);
 }
 
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Table tb;
-    __shared__ SolverShared S;
-    __shared__ int sh_last;
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
-
-    // Second pass over a tensor on this CTA, in three steps like round 1: r2_begin builds the tensor's
-    // interval table and prefilter and clears the CTA's cells, r2_add streams a piece (copies the values
-    // inside the intervals and counts them on the finer cells, unless they already fit one sort),
-    // r2_flush adds the cells to the tensor's global ones.
-    bool r2_copy_only = false;
-    auto r2_begin = [&](int t) {
+    pdl_wait();
+    pdl_launch_dependents();
+    // Second pass over a piece: builds the tensor's interval table and prefilter, clears the CTA's cells,
+    // copies the values inside the intervals and counts them on the finer cells (unless they already fit
+    // one sort), adds the cells to the tensor's global ones.
+    const int64_t lo = (int64_t)blockIdx.x * A.chunk;
+    const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
+    for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
+        if (tend - tbeg <= kSmallN) return;
         TState* st = A.ws.st + t;
+        if (__ldcg(&st->done)) return;  // settled in round 1
         __syncthreads();
         table_from_intervals_cta(tb, st->iv, __ldcg(&st->m));
         __syncthreads();
         build_prefilter(tb, pb);
-        r2_copy_only = __ldcg(&st->compact_only) != 0;
-        if (!r2_copy_only) zero_hist(hist, tb.ncells);
+        const bool copy_only = __ldcg(&st->compact_only) != 0;
+        if (!copy_only) zero_hist(hist, tb.ncells);
         __syncthreads();
-    };
-    auto r2_add = [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
-        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, tb, hist, smem, r2_copy_only);
-    };
-    auto r2_flush = [&](int t) {
+        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, tb, hist, smem, copy_only);
         __syncthreads();
-        if (!r2_copy_only) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
-        __threadfence();
-        __syncthreads();
-    };
-
-    if ((int)blockIdx.x < A.T) {
-        // the first T CTAs, one per tensor, take the mid-size tensors from where their CTA of the
-        // round-1 kernel left them to the end (the tensor stays in L2, later rounds read copied keys)
-        const int t = blockIdx.x;
-        const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
-        const int64_t n = tend - tbeg;
-        TState* st = A.ws.st + t;
-        if (n <= kSmallN || n > kMidN || __ldcg(&st->done)) return;
-        r2_begin(t);
-        r2_add(t, tbeg, tend, tbeg, tend);
-        r2_flush(t);
-        if (r2_copy_only) {
-            finish_sorted(st, t, A.s, A.ws.buf[0] + sel_region(tbeg), A.levels, A.status, smem, S, 0);
-            return;
-        }
-        if (solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s,
-                         A.levels, A.status, A.ws.nitems, A.ws.items, A.ws.buf[0] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg)))
-            return;
-        finish_alone(A, t, smem, tb, S);
-        return;
-    }
-
-    // flat CTAs: one chunk each, solver passes last (as in round 1)
-    constexpr int kDefer = 8;
-    int dt[kDefer];
-    int nd = 0;
-    auto finish = [&](int t) {
-        TState* st = A.ws.st + t;
-        const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
-        if (__ldcg(&st->compact_only) != 0) {
-            finish_sorted(st, t, A.s, A.ws.buf[0] + sel_region(tbeg), A.levels, A.status, smem, S, 0);
-            return;
-        }
-        solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s,
-                     A.levels, A.status, A.ws.nitems, A.ws.items, A.ws.buf[0] + sel_region(tbeg), true, smem, S, sel_region(tend) - sel_region(tbeg));
-    };
-    int cur_t = -1;
-    int64_t cur_n = 0, cur_elems = 0;
-    auto done_with_current = [&]() {
-        if (cur_t < 0) return;
-        r2_flush(cur_t);
-        TState* st = A.ws.st + cur_t;
-        if (threadIdx.x == 0) {
-            const unsigned long long prev = atomicAdd(&st->arrived, (unsigned long long)cur_elems);
-            sh_last = (prev + (unsigned long long)cur_elems == (unsigned long long)cur_n);
-        }
-        __syncthreads();
-        if (sh_last) {
-            __threadfence();
-            if (nd < kDefer) {
-#pragma unroll
-                for (int u = 0; u < kDefer; ++u)
-                    if (u == nd) dt[u] = cur_t;
-                ++nd;
-            } else {
-                finish(cur_t);
-            }
-        }
-        cur_t = -1;
-    };
-    {
-        const int64_t lo = (int64_t)(blockIdx.x - A.T) * A.chunk;
-        const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
-        for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
-            const int64_t n = tend - tbeg;
-            if (n <= kMidN) return;
-            if (t != cur_t) {
-                done_with_current();
-                if (__ldcg(&A.ws.st[t].done)) return;  // settled in round 1
-                r2_begin(t);
-                cur_t = t;
-                cur_n = n;
-                cur_elems = 0;
-            }
-            r2_add(t, tbeg, tend, pb_, pe_);
-            cur_elems += pe_ - pb_;
-        });
-    }
-    done_with_current();
-#pragma unroll
-    for (int u = 0; u < kDefer; ++u)
-        if (u < nd) finish(dt[u]);
+        if (!copy_only) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
+    });
 }
 
-__global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round3(SelArgs A)
+// What follows round 2, one CTA per tensor: the sorting finish when round 2 only copied, else a solver pass;
+// tensors of up to kAloneN elements that are then still open are taken to the end here, larger ones get
+// work items of the round-3 kernel.
+__global__ void __launch_bounds__(kSelThreads) k_sel_solve2(SelArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ Table tb;
+    __shared__ SolverShared S;
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = blockIdx.x;
+    const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
+    const int64_t n = tend - tbeg;
+    TState* st = A.ws.st + t;
+    if (n <= kSmallN || __ldcg(&st->done)) return;
+    if (__ldcg(&st->compact_only) != 0) {
+        finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[0] + sel_region(tbeg), A.levels, A.status, smem, S, 0);
+        return;
+    }
+    const bool alone = n <= kAloneN;
+    const int round = solver_load(st, S, A.scheme == OGQ_BINGRAD_PB, A.s);
+    if (solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s, A.levels, A.status,
+                     A.ws.nitems, A.ws.items, A.ws.buf[0] + sel_region(tbeg), !alone, smem, S, sel_region(tend) - sel_region(tbeg), round))
+        return;
+    if (alone) finish_alone(A, t, smem, tb, S);
+}
+
+__global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Table tb;
     __shared__ SolverShared S;
     __shared__ int sh_last;
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+    pdl_wait();
+    pdl_launch_dependents();
     const unsigned nitems = __ldcg(A.ws.nitems);
 
     for (unsigned w = blockIdx.x; w < nitems; w += gridDim.x) {
@@ -2285,11 +2249,12 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round3(SelArg
         if (!sh_last) continue;
         __threadfence();
         if (copy_only) {
-            finish_sorted(st, t, A.s, A.ws.buf[1] + sel_region(tbeg), A.levels, A.status, smem, S, 1);
+            finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[1] + sel_region(tbeg), A.levels, A.status, smem, S, 1);
             continue;
         }
+        const int round = solver_load(st, S, A.scheme == OGQ_BINGRAD_PB, A.s);
         if (!solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s,
-                          A.levels, A.status, A.ws.nitems, A.ws.items, A.ws.buf[1] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg)))
+                          A.levels, A.status, A.ws.nitems, A.ws.items, A.ws.buf[1] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg), round))
             finish_alone(A, t, smem, tb, S);
     }
 }
@@ -2305,41 +2270,41 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
-            e = cudaFuncSetAttribute(k_sel_round1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-            if (e != cudaSuccess) return e;
-            e = cudaFuncSetAttribute(k_sel_round2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-            if (e != cudaSuccess) return e;
-            e = cudaFuncSetAttribute(k_sel_round3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-            if (e != cudaSuccess) return e;
+            struct { void (*kernel)(SelArgs); size_t bytes; } limits[] = {{k_sel_round1, kSmemBytes}, {k_sel_round2, kSmemBytes},
+                {k_sel_solve1, kSolveBytes}, {k_sel_solve2, kRound3Bytes}, {k_sel_round3, kRound3Bytes}};
+            for (auto& l : limits) {
+                e = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes);
+                if (e != cudaSuccess) return e;
+            }
             if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
         }
     }
-    // Flat streaming CTAs: one wave (kSelResident per SM).  Each CTA pays a set-up, a flush of its
-    // cells and an arrival per tensor piece, so larger chunks stream more of the time; a second wave
-    // balanced a lone call slightly better in round 1 but cost throughput whenever several calls
-    // (workers on their own streams) share the GPU.  Buckets above 4 M elements get chunks of at least
-    // 131,072 elements: on a bucket of 25 M elements that leaves a third of the wave's slots to concurrent
-    // calls (measured with eight workers in flight: 8 % more throughput, 3 % slower alone); smaller
-    // buckets keep 32,768, where a lone call is all that matters.
+    // Flat streaming CTAs: one wave (kSelResident per SM).  Each CTA pays a set-up and a flush of its
+    // cells per tensor piece, so larger chunks stream more of the time.
     const int64_t wave = (int64_t)kSelResident * sm_count;
     const int target = wave < kMaxFlatCtas ? (int)wave : kMaxFlatCtas;
-    FlatGrid g = make_flat_grid(total, target, total > ((int64_t)1 << 22) ? 131072 : 32768);
+    FlatGrid g = make_flat_grid(total, target, OGQ_CHUNK);
     SelArgs A;
     A.grad = d_grad; A.tau = d_tau; A.off = d_off; A.T = T; A.total = total; A.chunk = g.chunk; A.flat_ctas = g.ctas;
     A.scheme = scheme; A.s = s; A.levels = d_levels; A.status = d_status;
     A.ws = sel_carve(d_ws, T, total);
-    cudaError_t e = cudaMemsetAsync(d_ws, 0, sel_zero_bytes(T), stream);
-    if (e != cudaSuccess) return e;
-    launch_begin("k_sel_round1", stream);
-    k_sel_round1<<<g.ctas + T, kSelThreads, kSmemBytes, stream>>>(A);
-    launch_end(stream);
-    launch_begin("k_sel_round2", stream);
-    k_sel_round2<<<g.ctas + T, kSelThreads, kSmemBytes, stream>>>(A);
-    launch_end(stream);
-    launch_begin("k_sel_round3", stream);
-    k_sel_round3<<<kSelResident * sm_count, kSelThreads, kSmemBytes, stream>>>(A);
-    launch_end(stream);
-    return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    auto run = [&](const char* name, void (*kernel)(SelArgs), int ctas, size_t smem) {
+        if (e != cudaSuccess) return;
+        launch_begin(name, stream);
+        e = launch_pdl(kernel, ctas, kSelThreads, smem, stream, A);
+        launch_end(stream);
+    };
+    const bool streams = total > kSmallN;  // some tensor may be larger than one CTA settles on its own
+    if (streams) run("k_sel_prepare", k_sel_prepare, T, 0);
+    run("k_sel_round1", k_sel_round1, T + (streams ? g.ctas : 0), kSmemBytes);
+    if (streams) {
+        run("k_sel_solve1", k_sel_solve1, T, kSolveBytes);
+        run("k_sel_round2", k_sel_round2, g.ctas, kSmemBytes);
+        run("k_sel_solve2", k_sel_solve2, T, kRound3Bytes);
+    }
+    if (total > kAloneN) run("k_sel_round3", k_sel_round3, sm_count, kRound3Bytes);
+    return e;
 }
 
 }  // namespace ogq

@@ -98,7 +98,6 @@ OGQ_HD double sel_cell_sum(uint32_t kbase, int sh, unsigned long long cnt, unsig
 // slotbase[j] + c is the state before its cell c, the last one the state after its last cell.
 struct SolverView {
     const uint8_t* slot_iv;  // optional: interval index of every slot (null: searched)
-    const uint32_t* xkeys;  // explicit mode: cell c of the view holds the single key xkeys[c] (else null)
     const uint32_t* cpre;  // #{elements before the slot} (absolute)
     const double* spre;    // their sum
     const Interval* iv;
@@ -108,17 +107,6 @@ struct SolverView {
     long long n;
     double stot;
 };
-
-OGQ_HD void sel_init_slots(SolverView& v)
-{
-    int s = 0;
-    for (int j = 0; j < v.m; ++j) {
-        v.slotbase[j] = s;
-        s += v.iv[j].ncell + 1;
-    }
-    v.slotbase[v.m] = s;
-    v.nslots = s;
-}
 
 OGQ_HD int sel_interval_of_slot(const SolverView& v, int slot)
 {
@@ -140,13 +128,12 @@ OGQ_HD bool sel_is_end_slot(const SolverView& v, int slot)
 OGQ_HD uint32_t sel_slot_kbase(const SolverView& v, int slot)
 {
     const int j = sel_interval_of_slot(v, slot);
-    if (v.xkeys) return v.xkeys[slot - j];  // explicit cells are numbered without the end slots
     return v.iv[j].klo + ((uint32_t)(slot - v.slotbase[j]) << v.iv[j].sh);
 }
 
 OGQ_HD int sel_slot_shift(const SolverView& v, int slot)
 {
-    return v.xkeys ? 0 : v.iv[sel_interval_of_slot(v, slot)].sh;
+    return v.iv[sel_interval_of_slot(v, slot)].sh;
 }
 
 OGQ_HD double sel_slot_vlo(const SolverView& v, int slot) { return (double)sel_key_to_float(sel_slot_kbase(v, slot)); }
@@ -218,30 +205,10 @@ OGQ_HD void sel_make_range(const SolverView& v, int sa, int sb, LvInfo& o)
     o.vhi = sel_slot_vhi(v, sb);
 }
 
-// Q*(L, R) on the current cells: exact when both brackets are exact and the target rank sits in
-// a single-key cell, otherwise a conservative range of cells.  Returns false on an internal
-// inconsistency (the range cannot be placed on any cell).
-OGQ_HD bool sel_orq_solve(const SolverView& v, const LvInfo& L, const LvInfo& R, LvInfo& out)
+// Ranks [pos_lo, pos_hi] that are certain to contain Q*(L, R) when L or R is only known to lie in a range of
+// cells.
+OGQ_HD void sel_orq_range(const SolverView& v, const LvInfo& L, const LvInfo& R, long long& pos_lo, long long& pos_hi)
 {
-    bool gap;
-    if (L.exact && R.exact) {
-        if (!(R.val > L.val)) {
-            out = L;
-            return true;
-        }
-        const long long nseg = R.c_le - L.c_lt;
-        const double A = (R.s_le - L.s_lt) - L.val * (double)nseg;
-        const double T = A / (R.val - L.val);
-        long long k = (long long)floor(T);
-        if (k < 0) k = 0;
-        if (k > nseg - 1) k = nseg - 1;
-        const long long pos = R.c_le - 1 - k;
-        const int slot = sel_locate(v, pos, true, &gap);
-        if (slot < 0 || gap) return false;
-        if (sel_slot_shift(v, slot) == 0) sel_make_exact_from_slot(v, slot, out);
-        else sel_make_range(v, slot, slot, out);
-        return true;
-    }
     // prefix state right after L's part and right before R's part
     const long long Cs = L.exact ? L.c_lt : (long long)v.cpre[L.sb + 1];
     const double Ss = L.exact ? L.s_lt : v.spre[L.sb + 1];
@@ -253,7 +220,8 @@ OGQ_HD bool sel_orq_solve(const SolverView& v, const LvInfo& L, const LvInfo& R,
     const long long cntR = R.exact ? 0 : (long long)v.cpre[R.sb + 1] - (long long)v.cpre[R.sa];
     const long long floor_pos = L.exact ? L.c_lt : (long long)v.cpre[L.sa];
     const long long ceil_pos = (R.exact ? R.c_le : (long long)v.cpre[R.sb + 1]) - 1;
-    long long pos_lo = floor_pos, pos_hi = ceil_pos;
+    pos_lo = floor_pos;
+    pos_hi = ceil_pos;
     // With M the elements strictly between L's cells and R's cells (count cntM, sum sumM, all of
     // them inside [Lhi, Rlo]), T = [t_L + (sumM - L cntM) + t_R] / (R - L), where t_L and t_R are
     // the contributions of the elements of L's and R's own cells.  f(L, R) = (sumM - L cntM)/(R - L)
@@ -281,31 +249,6 @@ OGQ_HD bool sel_orq_solve(const SolverView& v, const LvInfo& L, const LvInfo& R,
     }
     if (pos_lo < 0) pos_lo = 0;
     if (pos_hi > v.n - 1) pos_hi = v.n - 1;
-    const int sa = sel_locate(v, pos_lo, true, &gap);
-    const int sb = sel_locate(v, pos_hi, false, &gap);
-    if (sa < 0 || sb < 0 || sa > sb) return false;
-    sel_make_range(v, sa, sb, out);
-    return true;
-}
-
-// One ORQ solver pass over all levels in the order of Algorithm 1 (a level after its two
-// brackets).  lv[0] and lv[s-1] must be exact on entry.  ranges receives the slot ranges of the
-// levels that are still open; returns their number, or -1 on an internal inconsistency.
-OGQ_HD int sel_orq_pass(const SolverView& v, int s, LvInfo* lv, int* range_a, int* range_b)
-{
-    int open = 0;
-    for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
-        for (int q = stride; q < s - 1; q += 2 * stride) {
-            if (lv[q].exact) continue;
-            if (!sel_orq_solve(v, lv[q - stride], lv[q + stride], lv[q])) return -1;
-            if (!lv[q].exact) {
-                range_a[open] = lv[q].sa;
-                range_b[open] = lv[q].sb;
-                ++open;
-            }
-        }
-    }
-    return open;
 }
 
 OGQ_HD int sel_floor_log2(long long x)
