@@ -35,12 +35,14 @@ struct BktArgs {
     int32_t* status;
     uint32_t* packed;
     int64_t words_per_bucket;
+    QuantSteps steps;
 };
 
 // Shared memory of one team besides the sort's: level records and the quantizer's table.
 struct BktShared {
     SortedLevel lv[kSortedLevels];
-    float2 tab[kMaxLevels];  // {level k, width of the segment above it}
+    float2 tab[kMaxLevels];  // see quant_table_entry
+    int plain;               // the table does not scale
 };
 
 // The whole path on bucket j.  EXACT: the bucket fills the team, KPT values for every thread (every full
@@ -60,7 +62,6 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
     uint32_t* cells = reinterpret_cast<uint32_t*>(mem);
     double* pre = reinterpret_cast<double*>(mem + (size_t)nt * (KPT + (KPT >= 8 ? 4 : 0)) * sizeof(float));
     const uint32_t tabaddr = (uint32_t)__cvta_generic_to_shared(S.tab);
-    const uint32_t tab4 = tabaddr * (1u + (1u << BITS) + (1u << (2 * BITS)) + (1u << (3 * BITS)));
     {
         const float* src = A.grad + (int64_t)j * A.d;
         const int n = EXACT ? KPT * nt : len;
@@ -192,6 +193,7 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
             }
         } else {
             team_sync<WARP>();  // the previous bucket's levels and table have been read
+            if (t == 0) S.plain = 0;
             if (bad) {
                 if (t < nl) S.lv[t].v = 0.f;
             } else {
@@ -229,7 +231,8 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
             if (t < nl) {
                 const float cur = S.lv[t].v;
                 const float nxt = t + 1 < nl ? S.lv[t + 1].v : cur;
-                S.tab[t] = make_float2(cur, __fsub_rn(nxt, cur));
+                S.tab[t] = quant_table_entry(cur, nxt);
+                if (!quant_table_scales(cur, nxt)) S.plain = 1;
                 A.levels[(int64_t)j * nl + t] = cur;
             }
             if (t == 0) A.status[j] = stbits;
@@ -242,7 +245,6 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
         const int ngroups = (n + 127) >> 7;
         const float mid = threshold ? 0.f : S.tab[(BITS >= 2) ? (1 << (BITS - 2)) : 0].x;
         const PhiloxHoist hz = philox_hoist(0u, (uint32_t)j, A.stream_id, pk);
-        const bool writer = packs_word<BITS>(lane);
         auto group = [&](int g, float4 v) {
             if constexpr (!kKeep) { v.x = clip(v.x); v.y = clip(v.y); v.z = clip(v.z); v.w = clip(v.w); }
             uint32_t bits4;
@@ -250,17 +252,24 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
                 bits4 = ((v.x >= b0) ? 1u : 0u) | ((v.y >= b0) ? 2u : 0u) | ((v.z >= b0) ? 4u : 0u) | ((v.w >= b0) ? 8u : 0u);
             } else {
                 const uint4 rnd = philox4x32_10_tail(((uint32_t)g << 5) + (uint32_t)lane, hz, pk);
-                const uint32_t a0 = entry_after_rounding<BITS>(v.x, rnd.x, tabaddr, mid),
-                               a1 = entry_after_rounding<BITS>(v.y, rnd.y, tabaddr, mid),
-                               a2 = entry_after_rounding<BITS>(v.z, rnd.z, tabaddr, mid),
-                               a3 = entry_after_rounding<BITS>(v.w, rnd.w, tabaddr, mid);
-                bits4 = (a0 + (a1 << BITS) + (a2 << (2 * BITS)) + (a3 << (3 * BITS)) - tab4) >> 3;
+                if (S.plain) {
+                    auto level = [&](int k) { return S.lv[k].v; };
+                    bits4 = code_as_written<BITS>(v.x, rnd.x, level) | code_as_written<BITS>(v.y, rnd.y, level) << BITS |
+                            code_as_written<BITS>(v.z, rnd.z, level) << (2 * BITS) | code_as_written<BITS>(v.w, rnd.w, level) << (3 * BITS);
+                } else bits4 = codes_of_entries<BITS>(entry_after_rounding<BITS>(v.x, rnd.x, tabaddr, mid, A.steps),
+                                               entry_after_rounding<BITS>(v.y, rnd.y, tabaddr, mid, A.steps),
+                                               entry_after_rounding<BITS>(v.z, rnd.z, tabaddr, mid, A.steps),
+                                               entry_after_rounding<BITS>(v.w, rnd.w, tabaddr, mid, A.steps), tabaddr);
             }
             const int left = n - ((g << 7) + 4 * lane);  // elements of this lane inside the bucket
             if (!EXACT && left < 4) bits4 &= left > 0 ? (1u << (left * BITS)) - 1u : 0u;
-            const uint32_t word = assemble_words<BITS>(bits4, lane);
-            const int w = g * (4 * BITS) + packed_word<BITS>(lane);
-            if (writer && (EXACT || w < region4)) out[w] = word;
+            if constexpr (EXACT) {
+                store_chunks<BITS>(out + g * (4 * BITS), bits4, lane);
+            } else {
+                const uint32_t word = assemble_words<BITS>(bits4, lane);
+                const int w = g * (4 * BITS) + packed_word<BITS>(lane);
+                if (packs_word<BITS>(lane) && w < region4) out[w] = word;
+            }
         };
         if constexpr (kKeep) {
             // (rolled: the unrolled groups' instructions were too many for the instruction cache)
@@ -477,6 +486,7 @@ cudaError_t launch_bucket_encode(const float* d_grad, int64_t total, int d, int 
     A.levels = d_levels; A.thresh = d_thresh; A.status = d_status; A.packed = d_packed;
     const int bits = ogq_bits_for_levels(s);
     A.words_per_bucket = (int64_t)d * bits / 32;
+    A.steps = quant_steps();
     const PhiloxKeys pk = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     switch (bits) {
         case 1: return bkt_dispatch<1>(A, pk, sm_count, stream);

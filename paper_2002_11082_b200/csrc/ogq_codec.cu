@@ -17,121 +17,97 @@ namespace ogq {
 
 // CLIP: every value is first clamped to [-tau_arr[t], tau_arr[t]] (gradient clipping).
 template <int BITS, bool THRESHOLD, bool CLIP>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, int64_t total,
-                int64_t chunk, int s, const float* __restrict__ levels, const float* __restrict__ thresh,
-                const float* __restrict__ tau_arr,
+                int64_t chunk, int s, const float* levels, const float* thresh, const float* tau_arr,
                 const __grid_constant__ PhiloxKeys keys, uint32_t stream_id,
-                const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed)
+                const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed, const __grid_constant__ QuantSteps steps)
 {
     __shared__ float sh_lv[kMaxLevels];
-    __shared__ float sh_w[kMaxLevels];
-    __shared__ float2 sh_tab[kMaxLevels];  // {level k, width of the segment above it}
-    // 3- and 5-bit codes: the 4*BITS words of a warp's group are OR-ed together here (kept zero between uses)
-    __shared__ uint32_t sh_words[kWarps][(BITS == 3 || BITS == 5) ? 4 * BITS : 1];
-    if ((BITS == 3 || BITS == 5) && (threadIdx.x & 31) < 4 * BITS) sh_words[threadIdx.x >> 5][threadIdx.x & 31] = 0u;
-    __syncthreads();
+    __shared__ float2 sh_tab[kMaxLevels];
+    pdl_wait();
+    pdl_launch_dependents();
 
     const int64_t lo = (int64_t)blockIdx.x * chunk;
     const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kWords = 4 * BITS;  // words of a group
 
     for_each_piece(off, T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + 127) >> 7, g_end = (pe - tb + 127) >> 7;
         if (g_beg >= g_end) return;
         float b0 = 0.f;
-        const float tau = CLIP ? __ldg(tau_arr + t) : 0.f;
+        const float tau = CLIP ? __ldcg(tau_arr + t) : 0.f;
         auto clip = [&](float x) -> float { return CLIP ? copysignf(fminf(fabsf(x), tau), x) : x; };
+        bool scales = true;
         if (THRESHOLD) {
-            b0 = __ldg(thresh + t);
+            b0 = __ldcg(thresh + t);
         } else {
             __syncthreads();
+            bool ok = true;
             if (threadIdx.x < s) {
-                const float cur = __ldg(levels + (int64_t)t * s + threadIdx.x);
-                const float prv = threadIdx.x > 0 ? __ldg(levels + (int64_t)t * s + threadIdx.x - 1) : cur;
+                const float cur = __ldcg(levels + (int64_t)t * s + threadIdx.x);
+                const float nxt = (int)threadIdx.x + 1 < s ? __ldcg(levels + (int64_t)t * s + threadIdx.x + 1) : cur;
                 sh_lv[threadIdx.x] = cur;
-                sh_w[threadIdx.x] = __fsub_rn(cur, prv);  // width of the segment below level k
-                const float nxt = (int)threadIdx.x + 1 < s ? __ldg(levels + (int64_t)t * s + threadIdx.x + 1) : cur;
-                sh_tab[threadIdx.x] = make_float2(cur, __fsub_rn(nxt, cur));
+                sh_tab[threadIdx.x] = quant_table_entry(cur, nxt);
+                ok = quant_table_scales(cur, nxt);
             }
-            __syncthreads();
+            scales = __syncthreads_and(ok);
         }
         const int64_t region = __ldg(packed_off + t + 1) - __ldg(packed_off + t);
         uint32_t* out = packed + __ldg(packed_off + t);
         const bool aligned = (tb & 3) == 0;
         const float* base = grad + tb;
 
-        // Fast path: groups that lie wholly inside the tensor, 128-bit loads, four groups in flight
-        // per warp, no bounds checks.  The generic loop below takes what is left (the last, partial
-        // group; everything when the tensor does not start on a 16-byte boundary, or when its Philox
-        // counters do not fit 32 bits).
+        // Fast path: groups that lie wholly inside the tensor, 128-bit loads, kU groups in flight per warp, no
+        // bounds checks.  The generic loop below takes what is left (the last, partial group; everything
+        // when the tensor does not start on a 16-byte boundary, when its Philox counters do not fit 32 bits
+        // or its levels are outside the range of quant_table_scales).
         int64_t g_rest = g_beg;
-        if (aligned && n <= ((int64_t)1 << 34)) {
+        if (aligned && scales && n <= ((int64_t)1 << 34)) {
             const int64_t g_full = (n >> 7) < g_end ? (n >> 7) : g_end;
             if (g_full > g_beg) {
                 g_rest = g_full;
-                constexpr bool kPow2 = (BITS == 1 || BITS == 2 || BITS == 4);
-                constexpr int L = kPow2 ? 8 / BITS : 1;  // lanes per word when a word is a whole number of lanes
                 const int ng = (int)(g_full - g_beg);
                 const float4* src = reinterpret_cast<const float4*>(base + (g_beg << 7)) + lane;
-                // which word of the group this lane stores: the first lane of each set of L lanes (see
-                // assemble_words), or, for 3 and 5 bits, lane w stores word w after the shared-memory OR
-                const bool writer = kPow2 ? (lane & (L - 1)) == 0 : lane < 4 * BITS;
-                uint32_t* dstw = out + g_beg * (4 * BITS) + (kPow2 ? lane / L : lane);
-                uint32_t* wsm = sh_words[warp];
-                const int obit = (lane * 4 * BITS) & 31, oword = (lane * 4 * BITS) >> 5;  // kPow2 == false only
+                uint32_t* dst = out + g_beg * kWords;
                 const uint32_t c0_first = (uint32_t)(g_beg << 5) + (uint32_t)lane;  // counters fit 32 bits here
                 const uint32_t tabaddr = (uint32_t)__cvta_generic_to_shared(sh_tab);
-                // the sum of the four entry addresses of a lane carries this multiple of the table's base
-                const uint32_t tab4 = tabaddr * (1u + (1u << BITS) + (1u << (2 * BITS)) + (1u << (3 * BITS)));
                 float mid = 0.f;
                 PhiloxHoist hz = {};
                 if constexpr (!THRESHOLD) {
                     mid = sh_tab[(BITS >= 2) ? (1 << (BITS - 2)) : 0].x;
                     hz = philox_hoist(0u, (uint32_t)t, stream_id, keys);
                 }
-                auto code4 = [&](float4 v, int gl) -> uint32_t {
+                auto code4 = [&](float4 v, int gl) {
                     if constexpr (CLIP) { v.x = clip(v.x); v.y = clip(v.y); v.z = clip(v.z); v.w = clip(v.w); }
+                    uint32_t chunk4;
                     if constexpr (THRESHOLD) {
-                        const uint32_t b4 = ((v.x >= b0) ? 1u : 0u) | ((v.y >= b0) ? 2u : 0u) |
-                                            ((v.z >= b0) ? 4u : 0u) | ((v.w >= b0) ? 8u : 0u);
-                        return assemble_words<BITS>(b4, lane);
+                        chunk4 = ((v.x >= b0) ? 1u : 0u) | ((v.y >= b0) ? 2u : 0u) | ((v.z >= b0) ? 4u : 0u) | ((v.w >= b0) ? 8u : 0u);
                     } else {
                         const uint4 r = philox4x32_10_tail(c0_first + ((uint32_t)gl << 5), hz, keys);
-                        const uint32_t a0 = entry_after_rounding<BITS>(v.x, r.x, tabaddr, mid),
-                                       a1 = entry_after_rounding<BITS>(v.y, r.y, tabaddr, mid),
-                                       a2 = entry_after_rounding<BITS>(v.z, r.z, tabaddr, mid),
-                                       a3 = entry_after_rounding<BITS>(v.w, r.w, tabaddr, mid);
-                        // entries are 8 bytes apart: (address - base) / 8 is the code
-                        const uint32_t bits4 =
-                            (a0 + (a1 << BITS) + (a2 << (2 * BITS)) + (a3 << (3 * BITS)) - tab4) >> 3;
-                        if constexpr (kPow2) {
-                            return assemble_words<BITS>(bits4, lane);
-                        } else {
-                            // a lane's 4*BITS bits touch at most two words of the group
-                            atomicOr(wsm + oword, bits4 << obit);
-                            if (obit + 4 * BITS > 32) atomicOr(wsm + oword + 1, bits4 >> (32 - obit));
-                            __syncwarp();
-                            const uint32_t word = writer ? atomicExch(wsm + lane, 0u) : 0u;
-                            __syncwarp();
-                            return word;
-                        }
+                        chunk4 = codes_of_entries<BITS>(entry_after_rounding<BITS>(v.x, r.x, tabaddr, mid, steps),
+                                                        entry_after_rounding<BITS>(v.y, r.y, tabaddr, mid, steps),
+                                                        entry_after_rounding<BITS>(v.z, r.z, tabaddr, mid, steps),
+                                                        entry_after_rounding<BITS>(v.w, r.w, tabaddr, mid, steps), tabaddr);
                     }
+                    store_chunks<BITS>(dst + (size_t)gl * kWords, chunk4, lane);
                 };
-                constexpr int U = 4;  // groups per warp and trip: all loads are issued before the first use
-                for (int gl = warp; gl < ng; gl += U * kWarps) {
-                    float4 v[U];
+                constexpr int kU = 4;  // groups per warp and trip: all loads are issued before the first use
+                int gl = warp;
+                for (; gl + (kU - 1) * kWarps < ng; gl += kU * kWarps) {
+                    // L2 is asked for the block (kU kWarps groups, 512 bytes each) two trips ahead: the random-rounding
+                    // variants compute long enough between their loads for it to pay
+                    if (!THRESHOLD && threadIdx.x == 0 && gl + 3 * kU * kWarps <= ng)
+                        prefetch_l2(src + (size_t)(gl + 2 * kU * kWarps) * 32, kU * kWarps * 512u);
+                    float4 v[kU];
 #pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (gl + u * kWarps < ng) v[u] = __ldg(src + (size_t)(gl + u * kWarps) * 32);
+                    for (int u = 0; u < kU; ++u) v[u] = __ldg(src + (size_t)(gl + u * kWarps) * 32);
 #pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (gl + u * kWarps < ng) {
-                            const uint32_t w = code4(v[u], gl + u * kWarps);
-                            if (writer) dstw[(size_t)(gl + u * kWarps) * (4 * BITS)] = w;
-                        }
+                    for (int u = 0; u < kU; ++u) code4(v[u], gl + u * kWarps);
                 }
+                for (; gl < ng; gl += kWarps) code4(__ldg(src + (size_t)gl * 32), gl);
             }
         }
 
@@ -158,45 +134,16 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
                 const uint4 r = philox4x32_10((uint32_t)q, (uint32_t)(q >> 32), (uint32_t)t, stream_id, keys);
                 const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    // s = 2^(BITS-1) + 1 levels (s = 2 for BITS = 1): BITS - 1 halving steps
-                    int idx = 0;
-#pragma unroll
-                    for (int step = (BITS >= 2) ? (1 << (BITS - 2)) : 0; step >= 1; step >>= 1)
-                        if (sh_lv[idx + step] <= x[j]) idx += step;
-                    const float d = __fsub_rn(x[j], sh_lv[idx]);
-                    const float lhs = __fmul_rn((float)(rw[j] >> 8), sh_w[idx + 1]);
-                    const float rhs = __fmul_rn(d, 16777216.0f);
-                    c[j] = (uint32_t)idx + ((lhs < rhs) ? 1u : 0u);
-                }
+                for (int j = 0; j < 4; ++j) c[j] = code_as_written<BITS>(x[j], rw[j], [&](int k) { return sh_lv[k]; });
             }
             if (i0 + 3 >= n) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (i0 + j >= n) c[j] = 0u;  // zero padding beyond the tensor
             }
-            const uint32_t bits4 = c[0] | (c[1] << BITS) | (c[2] << (2 * BITS)) | (c[3] << (3 * BITS));
-            if constexpr (BITS == 1 || BITS == 2 || BITS == 4) {
-                const uint32_t word = assemble_words<BITS>(bits4, lane);
-                constexpr int L = 8 / (BITS == 3 || BITS == 5 ? 1 : BITS);
-                if ((lane & (L - 1)) == 0) {
-                    const int64_t widx = g * (4 * BITS) + lane / L;
-                    if (widx < region) out[widx] = word;
-                }
-            } else {
-                // 3 and 5 bits: OR the lanes' bits into the group's 4*BITS words in shared memory
-                uint32_t* wsm = sh_words[warp];
-                const int obit = (lane * 4 * BITS) & 31, oword = (lane * 4 * BITS) >> 5;
-                atomicOr(wsm + oword, bits4 << obit);
-                if (obit + 4 * BITS > 32) atomicOr(wsm + oword + 1, bits4 >> (32 - obit));
-                __syncwarp();
-                if (lane < 4 * BITS) {
-                    const uint32_t word = atomicExch(wsm + lane, 0u);
-                    const int64_t widx = g * (4 * BITS) + lane;
-                    if (widx < region) out[widx] = word;
-                }
-                __syncwarp();
-            }
+            const uint32_t word = assemble_words<BITS>(c[0] | (c[1] << BITS) | (c[2] << (2 * BITS)) | (c[3] << (3 * BITS)), lane);
+            const int64_t widx = g * kWords + packed_word<BITS>(lane);
+            if (packs_word<BITS>(lane) && widx < region) out[widx] = word;
         }
     });
 }
@@ -356,10 +303,10 @@ cudaError_t launch_quantize_pack(const float* d_grad, const int64_t* d_off, int 
     FlatGrid g = make_flat_grid(total, flat_target(sm_count), 8192);
     const PhiloxKeys keys = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     const int bits = ogq_bits_for_levels(s);
+    cudaError_t e = cudaErrorInvalidValue;
 #define OGQ_LAUNCH_QC(B, TH, CL)                                                                        \
-    k_quantize_pack<B, TH, CL><<<g.ctas, kThreads, 0, stream>>>(d_grad, d_off, T, total, g.chunk, s,    \
-                                                                d_levels, d_thresh, d_tau, keys,        \
-                                                                stream_id, d_packed_off, d_packed)
+    e = launch_pdl(k_quantize_pack<B, TH, CL>, g.ctas, kThreads, 0, stream, d_grad, d_off, T, total, g.chunk, s, \
+                   d_levels, d_thresh, d_tau, keys, stream_id, d_packed_off, d_packed, quant_steps())
 #define OGQ_LAUNCH_Q(B, TH)                    \
     do {                                       \
         if (d_tau) OGQ_LAUNCH_QC(B, TH, true); \
@@ -381,7 +328,7 @@ cudaError_t launch_quantize_pack(const float* d_grad, const int64_t* d_off, int 
 #undef OGQ_LAUNCH_Q
 #undef OGQ_LAUNCH_QC
     launch_end(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* const* d_levels_k, int K,

@@ -44,11 +44,10 @@ template <int S>
 __global__ void __launch_bounds__(kThreads)
 k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, int64_t total,
                       int64_t chunk, const float* __restrict__ levels, const __grid_constant__ PhiloxKeys keys,
-                      uint32_t stream_id, const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed)
+                      uint32_t stream_id, const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed, const __grid_constant__ QuantSteps steps)
 {
     constexpr int M = Dense<S>::M, U = Dense<S>::U, BITS = Dense<S>::BITS, W = U / M, Q = U / 4;
     __shared__ float sh_lv[kMaxLevels];
-    __shared__ float sh_w[kMaxLevels];
     __shared__ float2 sh_tab[kMaxLevels];
 
     const int64_t lo = (int64_t)blockIdx.x * chunk;
@@ -60,22 +59,22 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
         const int64_t g_beg = (pb - tb + U - 1) / U, g_end = (pe - tb + U - 1) / U;
         if (g_beg >= g_end) return;
         __syncthreads();
+        bool ok = true;
         if (threadIdx.x < S) {
             const float cur = __ldg(levels + (int64_t)t * S + threadIdx.x);
-            const float prv = threadIdx.x > 0 ? __ldg(levels + (int64_t)t * S + threadIdx.x - 1) : cur;
             const float nxt = (int)threadIdx.x + 1 < S ? __ldg(levels + (int64_t)t * S + threadIdx.x + 1) : cur;
             sh_lv[threadIdx.x] = cur;
-            sh_w[threadIdx.x] = __fsub_rn(cur, prv);
-            sh_tab[threadIdx.x] = make_float2(cur, __fsub_rn(nxt, cur));
+            sh_tab[threadIdx.x] = quant_table_entry(cur, nxt);
+            ok = quant_table_scales(cur, nxt);
         }
-        __syncthreads();
+        const bool scales = __syncthreads_and(ok);
         const int64_t region = __ldg(packed_off + t + 1) - __ldg(packed_off + t);
         uint32_t* out = packed + __ldg(packed_off + t);
         const float* base = grad + tb;
         const bool aligned = (tb & 3) == 0;
 
         int64_t g_rest = g_beg;
-        if (aligned && n <= ((int64_t)1 << 34)) {
+        if (aligned && scales && n <= ((int64_t)1 << 34)) {
             const int64_t g_full = (n / U) < g_end ? (n / U) : g_end;
             if (g_full > g_beg) {
                 g_rest = g_full;
@@ -99,7 +98,7 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             const int e = 4 * q + j;  // position in the group (compile time after unrolling)
-                            const uint32_t code = (entry_after_rounding<BITS>(x[j], rw[j], tabaddr, mid) - tabaddr) >> 3;
+                            const uint32_t code = (entry_after_rounding<BITS>(x[j], rw[j], tabaddr, mid, steps) - tabaddr) >> 3;
                             word[e / M] += code * dense_pow(S, e % M);
                         }
                     }
@@ -125,13 +124,7 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
                     const uint64_t blk = (uint64_t)i >> 2;
                     const uint4 r = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)t, stream_id, keys);
                     const uint32_t rnd = (i & 3) == 0 ? r.x : ((i & 3) == 1 ? r.y : ((i & 3) == 2 ? r.z : r.w));
-                    int idx = 0;
-                    for (int step = 1 << (BITS - 2); step >= 1; step >>= 1)
-                        if (sh_lv[idx + step] <= x) idx += step;
-                    const float dd = __fsub_rn(x, sh_lv[idx]);
-                    const float lhs = __fmul_rn((float)(rnd >> 8), sh_w[idx + 1]);
-                    const float rhs = __fmul_rn(dd, 16777216.0f);
-                    word += ((uint32_t)idx + ((lhs < rhs) ? 1u : 0u)) * p;
+                    word += code_as_written<BITS>(x, rnd, [&](int k) { return sh_lv[k]; }) * p;
                 }
                 p *= (uint32_t)S;
             }
@@ -240,7 +233,7 @@ cudaError_t launch_quantize_pack_dense(const float* d_grad, const int64_t* d_off
     launch_begin("k_quantize_pack_dense", stream);
 #define OGQ_LAUNCH_D(SS)                                                                                     \
     k_quantize_pack_dense<SS><<<g.ctas, kThreads, 0, stream>>>(d_grad, d_off, T, total, g.chunk, d_levels,  \
-                                                               keys, stream_id, d_packed_off, d_packed)
+                                                               keys, stream_id, d_packed_off, d_packed, quant_steps())
     switch (s) {
         case 3: OGQ_LAUNCH_D(3); break;
         case 5: OGQ_LAUNCH_D(5); break;

@@ -30,9 +30,6 @@
 #include "ogq_sort.cuh"
 #include "ogq_ws.h"
 
-#ifndef OGQ_CHUNK
-#define OGQ_CHUNK (total > ((int64_t)1 << 22) ? 131072 : 16384)
-#endif
 namespace ogq {
 
 constexpr int kSelThreads = 512;    // two CTAs are resident per SM: a CTA in a solver pass, a sort or a
@@ -2283,7 +2280,7 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
     // cells per tensor piece, so larger chunks stream more of the time.
     const int64_t wave = (int64_t)kSelResident * sm_count;
     const int target = wave < kMaxFlatCtas ? (int)wave : kMaxFlatCtas;
-    FlatGrid g = make_flat_grid(total, target, OGQ_CHUNK);
+    FlatGrid g = make_flat_grid(total, target, 16384);
     SelArgs A;
     A.grad = d_grad; A.tau = d_tau; A.off = d_off; A.T = T; A.total = total; A.chunk = g.chunk; A.flat_ctas = g.ctas;
     A.scheme = scheme; A.s = s; A.levels = d_levels; A.status = d_status;
