@@ -1,4 +1,8 @@
-"""ctypes binding of libogq.so: same names and argument order as include/ogq.h."""
+"""Binding of libogq.so: same names and argument order as include/ogq.h.
+
+The data-path calls are functions of the C module `_native` (argument conversion in ctypes took longer than
+many of the kernels); the host-only helpers and the measurement helpers go through ctypes.
+"""
 from __future__ import annotations
 
 import ctypes
@@ -97,28 +101,76 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
-def _ptr(t) -> Optional[int]:
-    """Address of a torch tensor's storage, a raw integer address, or None."""
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    return t.data_ptr()
-
-
-def _stream(stream) -> Optional[int]:
-    if stream is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream
-    if isinstance(stream, int):
-        return stream
-    return stream.cuda_stream
-
-
 def _check(code: int, where: str) -> None:
     if code != 0:
         raise OgqError(code, where)
+
+
+_DATA_PATH = (
+    "ogq_levels_bingrad", "ogq_levels_bingrad_b_noalloc", "ogq_levels_orq", "ogq_quantize_pack", "ogq_unpack_sum",
+    "ogq_clip_threshold", "ogq_levels_orq_clipped", "ogq_levels_bingrad_clipped", "ogq_quant_error",
+    "ogq_expected_error", "ogq_quantize_pack_dense", "ogq_unpack_sum_dense", "ogq_quantize_pack_clipped",
+    "ogq_bucket_encode", "ogq_bucket_decode_sum",
+)
+
+
+def _attach() -> None:
+    """Gives the C module the addresses of the library's functions (before its first call)."""
+    L = lib()
+    _native_module().set_addresses({n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in _DATA_PATH})
+
+
+def _first_device() -> int:
+    """The current device, for the first call without a stream: brings torch's CUDA state up, after which the
+    C module asks torch directly."""
+    import torch
+
+    torch.cuda.current_stream()
+    _native_module().setup(_attach, _check, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+    return torch._C._cuda_getDevice()
+
+
+def _first_raw_stream(device: int) -> int:
+    import torch
+
+    return torch._C._cuda_getCurrentRawStream(device)
+
+
+def _native_module():
+    try:
+        from . import _native
+    except ImportError as e:
+        raise ImportError(
+            "the C module of the binding is missing: build it with `python -m paper_2002_11082_b200.build`; "
+            "there is no other path to the library's data-path calls"
+        ) from e
+    return _native
+
+
+def _entry(name: str):
+    try:
+        return getattr(_native_module(), name)
+    except ImportError:
+        # imported before the build: looked up again at every call
+        def late(*args, **kwargs):
+            _setup_native()
+            return getattr(_native_module(), name)(*args, **kwargs)
+
+        late.__name__ = name
+        return late
+
+
+def _setup_native() -> None:
+    _native_module().setup(_attach, _check, _first_device, _first_raw_stream)
+
+
+try:
+    _setup_native()
+except ImportError:
+    pass
+
+for _name in _DATA_PATH:
+    globals()[_name] = _entry(_name)
 
 
 def ogq_version() -> str:
@@ -141,105 +193,8 @@ def ogq_workspace_bytes(num_tensors: int, total_elems: int, max_levels: int) -> 
     return int(lib().ogq_workspace_bytes(int(num_tensors), int(total_elems), int(max_levels)))
 
 
-def ogq_levels_bingrad(d_grad, d_off, T: int, total_elems: int, variant: int, lloyd_iters: int,
-                       d_levels, d_thresh, d_status, d_ws, ws_bytes: int, stream=None) -> None:
-    _check(
-        lib().ogq_levels_bingrad(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(variant),
-                                 int(lloyd_iters), _ptr(d_levels), _ptr(d_thresh), _ptr(d_status),
-                                 _ptr(d_ws), int(ws_bytes), _stream(stream)),
-        "ogq_levels_bingrad",
-    )
-
-
-def ogq_levels_bingrad_b_noalloc(d_grad, d_off, T: int, total_elems: int, lloyd_iters: int, d_levels, d_thresh,
-                                 d_status, stream=None) -> None:
-    """BinGrad-b levels with the solver's scratch held inside the library (no workspace argument).
-
-    For callers that may not allocate device memory; at most 1024 tensors per call, and calls that
-    overlap on the GPU must be ordered because they share the one built-in scratch array."""
-    _check(
-        lib().ogq_levels_bingrad_b_noalloc(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(lloyd_iters),
-                                           _ptr(d_levels), _ptr(d_thresh), _ptr(d_status), _stream(stream)),
-        "ogq_levels_bingrad_b_noalloc",
-    )
-
-
-def ogq_levels_orq(d_grad, d_off, T: int, total_elems: int, s: int, d_levels, d_status, d_ws,
-                   ws_bytes: int, stream=None) -> None:
-    _check(
-        lib().ogq_levels_orq(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(s), _ptr(d_levels),
-                             _ptr(d_status), _ptr(d_ws), int(ws_bytes), _stream(stream)),
-        "ogq_levels_orq",
-    )
-
-
-def ogq_quantize_pack(d_grad, d_off, T: int, total_elems: int, scheme: int, s: int, d_levels, d_thresh,
-                      seed: int, stream_id: int, d_packed_off, d_packed, stream=None) -> None:
-    _check(
-        lib().ogq_quantize_pack(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(scheme), int(s),
-                                _ptr(d_levels), _ptr(d_thresh), int(seed) & 0xFFFFFFFFFFFFFFFF,
-                                int(stream_id) & 0xFFFFFFFF, _ptr(d_packed_off), _ptr(d_packed),
-                                _stream(stream)),
-        "ogq_quantize_pack",
-    )
-
-
-def ogq_unpack_sum(d_packed_k, d_levels_k, K: int, d_off, d_packed_off, T: int, total_elems: int, s: int,
-                   scale: float, d_out, stream=None) -> None:
-    _check(
-        lib().ogq_unpack_sum(_ptr(d_packed_k), _ptr(d_levels_k), int(K), _ptr(d_off), _ptr(d_packed_off),
-                             int(T), int(total_elems), int(s), float(scale), _ptr(d_out), _stream(stream)),
-        "ogq_unpack_sum",
-    )
-
-
 def ogq_bucket_packed_words(total_elems: int, d: int, bits: int) -> int:
     return int(lib().ogq_bucket_packed_words(int(total_elems), int(d), int(bits)))
-
-
-def ogq_clip_threshold(d_grad, d_off, T: int, total_elems: int, c: float, d_tau, d_status, d_ws, ws_bytes: int,
-                       stream=None) -> None:
-    _check(
-        lib().ogq_clip_threshold(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), float(c), _ptr(d_tau),
-                                 _ptr(d_status), _ptr(d_ws), int(ws_bytes), _stream(stream)),
-        "ogq_clip_threshold",
-    )
-
-
-def ogq_levels_orq_clipped(d_grad, d_off, T: int, total_elems: int, s: int, d_tau, d_levels, d_status, d_ws,
-                           ws_bytes: int, stream=None) -> None:
-    _check(
-        lib().ogq_levels_orq_clipped(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(s), _ptr(d_tau),
-                                     _ptr(d_levels), _ptr(d_status), _ptr(d_ws), int(ws_bytes), _stream(stream)),
-        "ogq_levels_orq_clipped",
-    )
-
-
-def ogq_levels_bingrad_clipped(d_grad, d_off, T: int, total_elems: int, variant: int, lloyd_iters: int, d_tau,
-                               d_levels, d_thresh, d_status, d_ws, ws_bytes: int, stream=None) -> None:
-    _check(
-        lib().ogq_levels_bingrad_clipped(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(variant),
-                                         int(lloyd_iters), _ptr(d_tau), _ptr(d_levels), _ptr(d_thresh),
-                                         _ptr(d_status), _ptr(d_ws), int(ws_bytes), _stream(stream)),
-        "ogq_levels_bingrad_clipped",
-    )
-
-
-def ogq_quant_error(d_grad, d_off, T: int, total_elems: int, s: int, d_levels, d_packed_off, d_packed, d_err,
-                    stream=None) -> None:
-    _check(
-        lib().ogq_quant_error(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(s), _ptr(d_levels),
-                              _ptr(d_packed_off), _ptr(d_packed), _ptr(d_err), _stream(stream)),
-        "ogq_quant_error",
-    )
-
-
-def ogq_expected_error(d_grad, d_off, T: int, total_elems: int, s: int, d_levels, d_err, stream=None) -> None:
-    _check(
-        lib().ogq_expected_error(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(s), _ptr(d_levels),
-                                 _ptr(d_err), _stream(stream)),
-        "ogq_expected_error",
-    )
 
 
 def ogq_dense_digits(s: int) -> int:
@@ -252,55 +207,6 @@ def ogq_dense_layout(h_off, s: int) -> np.ndarray:
     out = np.zeros_like(h)
     _check(lib().ogq_dense_layout(h.ctypes.data, h.size - 1, int(s), out.ctypes.data), "ogq_dense_layout")
     return out
-
-
-def ogq_quantize_pack_dense(d_grad, d_off, T: int, total_elems: int, s: int, d_levels, seed: int, stream_id: int,
-                            d_packed_off, d_packed, stream=None) -> None:
-    _check(
-        lib().ogq_quantize_pack_dense(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(s), _ptr(d_levels),
-                                      int(seed) & 0xFFFFFFFFFFFFFFFF, int(stream_id) & 0xFFFFFFFF,
-                                      _ptr(d_packed_off), _ptr(d_packed), _stream(stream)),
-        "ogq_quantize_pack_dense",
-    )
-
-
-def ogq_unpack_sum_dense(d_packed_k, d_levels_k, K: int, d_off, d_packed_off, T: int, total_elems: int, s: int,
-                         scale: float, d_out, stream=None) -> None:
-    _check(
-        lib().ogq_unpack_sum_dense(_ptr(d_packed_k), _ptr(d_levels_k), int(K), _ptr(d_off), _ptr(d_packed_off),
-                                   int(T), int(total_elems), int(s), float(scale), _ptr(d_out), _stream(stream)),
-        "ogq_unpack_sum_dense",
-    )
-
-
-def ogq_quantize_pack_clipped(d_grad, d_off, T: int, total_elems: int, scheme: int, s: int, d_levels, d_thresh,
-                              d_tau, seed: int, stream_id: int, d_packed_off, d_packed, stream=None) -> None:
-    _check(
-        lib().ogq_quantize_pack_clipped(_ptr(d_grad), _ptr(d_off), int(T), int(total_elems), int(scheme), int(s),
-                                        _ptr(d_levels), _ptr(d_thresh), _ptr(d_tau), int(seed) & 0xFFFFFFFFFFFFFFFF,
-                                        int(stream_id) & 0xFFFFFFFF, _ptr(d_packed_off), _ptr(d_packed),
-                                        _stream(stream)),
-        "ogq_quantize_pack_clipped",
-    )
-
-
-def ogq_bucket_encode(d_grad, total_elems: int, d: int, scheme: int, s: int, iters: int, clip_c: float, seed: int,
-                      stream_id: int, d_levels, d_thresh, d_status, d_packed, stream=None) -> None:
-    _check(
-        lib().ogq_bucket_encode(_ptr(d_grad), int(total_elems), int(d), int(scheme), int(s), int(iters), float(clip_c),
-                                int(seed) & 0xFFFFFFFFFFFFFFFF, int(stream_id) & 0xFFFFFFFF, _ptr(d_levels),
-                                _ptr(d_thresh), _ptr(d_status), _ptr(d_packed), _stream(stream)),
-        "ogq_bucket_encode",
-    )
-
-
-def ogq_bucket_decode_sum(d_packed_k, d_levels_k, K: int, total_elems: int, d: int, s: int, scale: float, d_out,
-                          stream=None) -> None:
-    _check(
-        lib().ogq_bucket_decode_sum(_ptr(d_packed_k), _ptr(d_levels_k), int(K), int(total_elems), int(d), int(s),
-                                    float(scale), _ptr(d_out), _stream(stream)),
-        "ogq_bucket_decode_sum",
-    )
 
 
 def ogq_launch_count() -> int:

@@ -1,19 +1,23 @@
 """Builds the CUDA library (libogq.so) in-tree with nvcc for sm_100a.
 
 Every .cu file is compiled to an object of its own (in parallel, and only when it or a header is
-newer than the object), then the objects are linked into the shared library.
+newer than the object), then the objects are linked into the shared library.  The CPython module with
+the data-path calls (_native, which loads the library itself) is compiled next to it with g++.
 """
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 OBJ_DIR = os.path.join(_HERE, "_build")
 LIB_PATH = os.path.join(_HERE, "libogq.so")
+NATIVE_SRC = os.path.join(CSRC, "ogq_python.cpp")
+NATIVE_PATH = os.path.join(_HERE, "_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -43,10 +47,18 @@ def _stale(target: str, deps) -> bool:
 
 
 def needs_build() -> bool:
-    return _stale(LIB_PATH, sources() + _headers())
+    return _stale(LIB_PATH, sources() + _headers()) or _stale(NATIVE_PATH, [NATIVE_SRC])
+
+
+def build_native(force: bool = False) -> str:
+    if force or _stale(NATIVE_PATH, [NATIVE_SRC]):
+        subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                        "-I", sysconfig.get_paths()["include"], NATIVE_SRC, "-o", NATIVE_PATH], check=True)
+    return NATIVE_PATH
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_native(force)
     if not force and not needs_build():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
