@@ -113,8 +113,8 @@ ogq_status ogq_levels_bingrad(const float *d_grad, const int64_t *d_off, int T, 
  *   - The call allocates and frees nothing.  The first call on each device looks up the array's
  *     device address (with that device current); make that first call outside any stream
  *     capture.
- *   - All calls on a device share the one array.  The part a call uses is cleared on `stream`
- *     before its kernels run, so leftovers of earlier calls do no harm, but two calls whose
+ *   - All calls on a device share the one array.  A call writes what it reads there, so leftovers of
+ *     earlier calls do no harm, but two calls whose
  *     work overlaps on the GPU (different streams, no ordering between them) race on it and
  *     give wrong levels.  Order such calls, or use ogq_levels_bingrad with separate scratch.
  *   - OGQ_ERR_LIMIT comes only from the tensor-count check above; a failing CUDA call is

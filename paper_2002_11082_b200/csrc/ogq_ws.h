@@ -1,4 +1,4 @@
-// Host-side layout of the caller-provided scratch buffer.
+// Host-side layout of the caller-provided scratch buffer of BinGrad-b and the clipping threshold.
 #pragma once
 
 #include <stddef.h>
@@ -8,7 +8,7 @@ namespace ogq {
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Partial sums of one split pass of the BinGrad-b solver.
+// Partial sums of one pass over one piece of a tensor.
 struct BbPart {
     double s_lo, s_hi;     // sums of {v < b_0} and {v >= b_0}
     long long c_lo, c_hi;  // their counts
@@ -18,7 +18,6 @@ struct BbWs {
     BbPart* slot_a;      // [ctas]  piece of a tensor that began before the CTA's chunk
     BbPart* slot_b;      // [ctas]  piece of a tensor that begins in the chunk and runs past it
     BbPart* direct;      // [T]     tensors that lie inside one chunk
-    unsigned* arrive;    // [T]     pieces finished in the current pass
     int* done;           // [T]     tensor needs no further pass
     long long* prev_lo;  // [T]     |{v < b_0}| of the previous pass
 };
@@ -28,7 +27,6 @@ inline size_t bb_ws_bytes(int T, int ctas)
     size_t b = 0;
     b += align_up(sizeof(BbPart) * (size_t)ctas, 256) * 2;
     b += align_up(sizeof(BbPart) * (size_t)T, 256);
-    b += align_up(sizeof(unsigned) * (size_t)T, 256);
     b += align_up(sizeof(int) * (size_t)T, 256);
     b += align_up(sizeof(long long) * (size_t)T, 256);
     return b;
@@ -41,7 +39,6 @@ inline BbWs bb_ws_carve(void* base, int T, int ctas)
     w.slot_a = (BbPart*)p; p += align_up(sizeof(BbPart) * (size_t)ctas, 256);
     w.slot_b = (BbPart*)p; p += align_up(sizeof(BbPart) * (size_t)ctas, 256);
     w.direct = (BbPart*)p; p += align_up(sizeof(BbPart) * (size_t)T, 256);
-    w.arrive = (unsigned*)p; p += align_up(sizeof(unsigned) * (size_t)T, 256);
     w.done = (int*)p; p += align_up(sizeof(int) * (size_t)T, 256);
     w.prev_lo = (long long*)p;
     return w;
