@@ -38,8 +38,8 @@ constexpr int kSelResident = 2;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelW = 16;          // binades in the fine window of round 1
 constexpr int kSelM = 7;           // log2(cells per binade) in the window
-constexpr int kSmallN = 8192;      // tensors up to this size are solved in shared memory
-constexpr int kSortN = 8192;       // candidates from which one CTA finishes a larger tensor
+constexpr int kSmallN = 16384;     // tensors up to this size are solved in shared memory
+constexpr int kSortN = 16384;      // candidates from which one CTA finishes a larger tensor
 constexpr int kAloneN = 131072;    // tensors up to this size are finished by one CTA after round 2
 constexpr int kStageCap = 320;     // per-warp staging entries for compaction
 constexpr int kParkMax = 256;      // values one warp can park between two checks in the tail of round 2 (32 lanes x 8)
@@ -882,45 +882,10 @@ __device__ __forceinline__ void flush_hist(const uint32_t* smem_hist, int ncells
     }
 }
 
-// ---------------------------------------------------------------------------
-// Block-wide exclusive scan of (count, sum) pairs in thread order (fixed order).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void block_excl_scan(unsigned long long& c, double& s, unsigned long long* sc,
-                                                double* ss, unsigned long long& tot_c, double& tot_s)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long ic = c;
-    double is = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long nc = __shfl_up_sync(0xffffffffu, ic, o);
-        const double ns = __shfl_up_sync(0xffffffffu, is, o);
-        if (lane >= o) { ic += nc; is = ns + is; }
-    }
-    const unsigned long long pc = __shfl_up_sync(0xffffffffu, ic, 1);
-    const double ps = __shfl_up_sync(0xffffffffu, is, 1);
-    __syncthreads();
-    if (lane == 31) { sc[warp] = ic; ss[warp] = is; }
-    __syncthreads();
-    unsigned long long bc = 0;
-    double bs = 0.0;
-    tot_c = 0;
-    tot_s = 0.0;
-#pragma unroll
-    for (int w = 0; w < kSelWarps; ++w) {
-        if (w < warp) { bc += sc[w]; bs += ss[w]; }
-        tot_c += sc[w];
-        tot_s += ss[w];
-    }
-    c = (lane == 0) ? bc : bc + pc;
-    s = (lane == 0) ? bs : bs + ps;
-}
-
 // The kernels from here to solver_round work on one tensor with one CTA and run their code once: what they
-// spend is the latency of barriers, of dependent loads and, most of all, of instructions that are not in the
-// instruction cache yet (about 300 cycles for every eight).  So loops stay rolled, values live in shared
-// memory instead of unrolled registers, a warp works on one level with searches spread over its lanes, and
-// fp64 division is one function.
+// spend is the latency of barriers, of dependent loads and of instructions that are not in the instruction
+// cache yet.  So loops stay rolled, values live in shared memory instead of unrolled registers, a warp works
+// on one level with searches spread over its lanes, and fp64 division is one function.
 __device__ __noinline__ double fp64_div(double a, double b) { return a / b; }
 
 struct SolverShared {
@@ -928,8 +893,8 @@ struct SolverShared {
     Interval niv[kMaxIv];
     LvInfo lv[kMaxLv];
     SolverView view;
-    unsigned long long sc[kSelWarps];
-    double ss[kSelWarps];
+    uint32_t sc[32];
+    double ss[32];
     int pb_a, pb_b, pb_c;
     int done, nm, internal, nopen;
     uint32_t offc[kMaxIv];    // per-interval shifts of the scanned prefix arrays
@@ -937,32 +902,48 @@ struct SolverShared {
     uint32_t marks[(kSlots + 31) / 32];  // candidate cells, one bit per slot
     int pa[kRefineMax], pb[kRefineMax];  // runs of candidate cells
     long long cand;           // elements inside the new intervals
-    // sorting finish
+    // finish
     uint32_t lo[kMaxIv], hi[kMaxIv];  // keys of the intervals (padded: no key lies in the surplus ones)
     uint32_t base[kMaxIv];            // first cell of the interval
     int sh[kMaxIv];                   // log2 of the keys per cell
     int start[kMaxIv + 1];            // position of the interval's first value
     double pre[kMaxIv];               // sum of the values before it
     int n_keys;
-    uint32_t below[kSelWarps];
+    uint32_t below[32];
 };
 
-// First of the ascending a[0 .. n) that exceeds pos (n if none does), by the 32 lanes of a warp: 32 probes a
-// step, three steps for 16384 entries (a binary search is fourteen dependent shared-memory reads).
-__device__ __forceinline__ int warp_upper_bound(const uint32_t* a, int n, uint32_t pos)
+// Exclusive sums of (c, s) over the CTA's threads in thread order; totals in tot_c, tot_s.  Any number of warps.
+__device__ __forceinline__ void block_excl_scan(uint32_t& c, double& s, SolverShared& S, uint32_t& tot_c, double& tot_s)
 {
-    const int lane = threadIdx.x & 31;
-    int lo = 0, hi = n;  // the answer lies in [lo, hi]
-#pragma unroll 1
-    while (lo < hi) {
-        const int step = (hi - lo + 31) >> 5;
-        const int i = lo + lane * step;
-        const int k = __popc(__ballot_sync(0xffffffffu, i < hi && a[i] <= pos));  // a prefix of the lanes
-        const int nhi = lo + k * step;
-        if (k > 0) lo += (k - 1) * step + 1;
-        if (nhi < hi) hi = nhi;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint32_t ic = c;
+    double is = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t nc = __shfl_up_sync(0xffffffffu, ic, o);
+        const double ns = __shfl_up_sync(0xffffffffu, is, o);
+        if (lane >= o) { ic += nc; is = ns + is; }
     }
-    return lo;
+    const uint32_t pc = __shfl_up_sync(0xffffffffu, ic, 1);
+    const double ps = __shfl_up_sync(0xffffffffu, is, 1);
+    __syncthreads();
+    if (lane == 31) { S.sc[warp] = ic; S.ss[warp] = is; }
+    __syncthreads();
+    uint32_t wc = lane < nw ? S.sc[lane] : 0u;
+    double ws = lane < nw ? S.ss[lane] : 0.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t nc = __shfl_up_sync(0xffffffffu, wc, o);
+        const double ns = __shfl_up_sync(0xffffffffu, ws, o);
+        if (lane >= o) { wc += nc; ws = ns + ws; }
+    }
+    tot_c = __shfl_sync(0xffffffffu, wc, 31);
+    tot_s = __shfl_sync(0xffffffffu, ws, 31);
+    const int before = warp > 0 ? warp - 1 : 0;
+    const uint32_t bc = __shfl_sync(0xffffffffu, wc, before);
+    const double bs = __shfl_sync(0xffffffffu, ws, before);
+    c = (warp > 0 ? bc : 0u) + (lane > 0 ? pc : 0u);
+    s = lane > 0 ? (warp > 0 ? bs + ps : ps) : (warp > 0 ? bs : 0.0);
 }
 
 // ---------------------------------------------------------------------------
@@ -972,91 +953,88 @@ __device__ __forceinline__ int warp_upper_bound(const uint32_t* a, int n, uint32
 // (Nothing is sorted: a level needs one rank, and the sums before it need only know which values are
 // smaller.)
 // ---------------------------------------------------------------------------
-constexpr int kChunkN = kSortN / kSelThreads;  // values per prefix sum
-
 struct CellIndex {
     float* sv;          // the values
-    uint32_t* end;      // [nc] position after the last value of every cell
-    uint16_t* cell;     // [n] cell of every value, while they are being placed
-    double* pre;        // [kSelThreads + 1] sum of the values before every kChunkN-th position
-    int n, nc;
+    uint32_t* end;      // [nc] position after the last value of every cell; nc = 1024, 2048 ... 16384
+    double* pre;        // sum of the values before every chunk-th position
+    int n, nc, chunk;   // values per prefix sum: kSortN / threads (at most 32)
 };
 
-// Shared memory: the cells, the values, their cells' numbers, the prefix sums, the list of the gathered keys.
-constexpr int kFinishCells = 16384, kSmallCells = 8192;
-template <int NC>
-constexpr size_t kIndexBytes = (size_t)NC * 4 + (size_t)kSortN * 6 + (kSelThreads + 1) * 8;
+// Shared memory: prefix sums, cells, values; then the list of the gathered keys.
+constexpr int kIndexCells = 16384;
+constexpr size_t kIndexBytes = 1032 * 8 + (size_t)kIndexCells * 4 + (size_t)kSortN * 4;
 
-__device__ __forceinline__ CellIndex index_at(unsigned char* smem, int n, int nc)
+__device__ __forceinline__ CellIndex index_at(unsigned char* smem, int n)
 {
     CellIndex X;
-    X.end = reinterpret_cast<uint32_t*>(smem);
-    X.sv = reinterpret_cast<float*>(smem + (size_t)nc * 4);
-    X.cell = reinterpret_cast<uint16_t*>(smem + (size_t)nc * 4 + (size_t)kSortN * 4);
-    X.pre = reinterpret_cast<double*>(smem + (size_t)nc * 4 + (size_t)kSortN * 6);
+    X.pre = reinterpret_cast<double*>(smem);
+    X.end = reinterpret_cast<uint32_t*>(smem + 1032 * 8);
+    X.sv = reinterpret_cast<float*>(smem + 1032 * 8 + (size_t)kIndexCells * 4);
     X.n = n;
+    X.chunk = kSortN / (int)blockDim.x;
+    int nc = 1024;  // two cells or more per value, as far as there are that many: clearing and adding up cells takes longer
+    while (nc < 2 * n && nc < kIndexCells) nc <<= 1;  // than selecting in fuller ones saves
     X.nc = nc;
     return X;
 }
 
-// fetch(i): value i of n, cell_of(i): its cell.  Called by every thread of the CTA; nc is a multiple of
-// 128 kSelWarps.
+// fetch(i): value i of n, cell_of(i): its cell.  Called by every thread of the CTA (512 or 1024).
 template <class Fetch, class CellOf>
 __device__ __forceinline__ void index_build(const CellIndex& X, SolverShared& S, Fetch fetch, CellOf cell_of)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, nt = blockDim.x;
     uint4* rows = reinterpret_cast<uint4*>(X.end);
 #pragma unroll 1
-    for (int i = tid; i < X.nc / 4; i += kSelThreads) rows[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < X.nc / 4; i += nt) rows[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 #pragma unroll 1
-    for (int i = tid; i < X.n; i += kSelThreads) {
-        const uint32_t c = cell_of(i);
-        X.cell[i] = (uint16_t)c;
-        atomicAdd(X.end + c, 1u);
-    }
+    for (int i = tid; i < X.n; i += nt) atomicAdd(X.end + cell_of(i), 1u);
     __syncthreads();
-    // exclusive sums over the cells, in place: a warp takes rows of 128 cells
-    const int nrows = X.nc / 128 / kSelWarps;
-    uint4* mine = rows + warp * nrows * 32 + lane;
-    uint32_t sum = 0u;
+    {
+        // exclusive sums over the cells, in place: a warp takes rows of 128 cells
+        const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5, nrows = X.nc >> 7, per = (nrows + nw - 1) / nw;
+        const int r0 = warp * per, r1 = r0 + per < nrows ? r0 + per : nrows;
+        uint32_t sum = 0u;
 #pragma unroll 1
-    for (int q = 0; q < nrows; ++q) {
-        const uint4 w = mine[q * 32];
-        sum += (w.x + w.y) + (w.z + w.w);
-    }
-    sum = __reduce_add_sync(0xffffffffu, sum);
-    if (lane == 0) S.below[warp] = sum;
-    __syncthreads();
-    uint32_t run = __reduce_add_sync(0xffffffffu, lane < warp ? S.below[lane & (kSelWarps - 1)] : 0u);
-#pragma unroll 1
-    for (int q = 0; q < nrows; ++q) {
-        uint4 w = mine[q * 32];
-        const uint32_t own = (w.x + w.y) + (w.z + w.w);
-        uint32_t inc = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t nb = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += nb;
+        for (int q = r0; q < r1; ++q) {
+            const uint4 w = rows[q * 32 + lane];
+            sum += (w.x + w.y) + (w.z + w.w);
         }
-        uint4 x;
-        x.x = run + inc - own; x.y = x.x + w.x; x.z = x.y + w.y; x.w = x.z + w.z;
-        run += __shfl_sync(0xffffffffu, inc, 31);
-        mine[q * 32] = x;
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0) S.below[warp] = sum;
+        __syncthreads();
+        uint32_t run = __reduce_add_sync(0xffffffffu, lane < warp ? S.below[lane] : 0u);
+#pragma unroll 1
+        for (int q = r0; q < r1; ++q) {
+            const uint4 w = rows[q * 32 + lane];
+            const uint32_t own = (w.x + w.y) + (w.z + w.w);
+            uint32_t inc = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t nb = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += nb;
+            }
+            uint4 x;
+            x.x = run + inc - own; x.y = x.x + w.x; x.z = x.y + w.y; x.w = x.z + w.z;
+            run += __shfl_sync(0xffffffffu, inc, 31);
+            rows[q * 32 + lane] = x;
+        }
     }
     __syncthreads();
 #pragma unroll 1
-    for (int i = tid; i < X.n; i += kSelThreads) X.sv[atomicAdd(X.end + X.cell[i], 1u)] = fetch(i);
+    for (int i = tid; i < X.n; i += nt) X.sv[atomicAdd(X.end + cell_of(i), 1u)] = fetch(i);
     __syncthreads();
-    // fp64 sums of the kChunkN values of every thread, scanned
-    double ls = 0.0;
+    // fp64 sums of every thread's chunk, scanned
+    double ls = 0.0, tot;
 #pragma unroll 1
-    for (int i = tid * kChunkN; i < tid * kChunkN + kChunkN && i < X.n; ++i) ls += (double)X.sv[i];
-    unsigned long long none = 0, tc;
-    double tot;
-    block_excl_scan(none, ls, S.sc, S.ss, tc, tot);
+    for (int j = 0; j < X.chunk; ++j) {
+        const int i = tid * X.chunk + (j ^ (tid & (X.chunk - 1)));  // (neighbouring threads in different banks)
+        if (i < X.n) ls += (double)X.sv[i];
+    }
+    uint32_t none = 0u, tc;
+    block_excl_scan(none, ls, S, tc, tot);
     X.pre[tid] = ls;
-    if (tid == 0) X.pre[kSelThreads] = tot;
+    if (tid == 0) X.pre[nt] = tot;
     __syncthreads();
 }
 
@@ -1069,18 +1047,21 @@ struct Ranked {
 // Sum of the values before position a (lane's share of it; add up over the warp).
 __device__ __forceinline__ double index_before_lane(const CellIndex& X, int a)
 {
-    const int lane = threadIdx.x & 31, q = a / kChunkN;
+    const int lane = threadIdx.x & 31, q = a / X.chunk;
     double x = lane == 0 ? X.pre[q] : 0.0;
-    if (q * kChunkN + lane < a) x += (double)X.sv[q * kChunkN + lane];
+    if (q * X.chunk + lane < a) x += (double)X.sv[q * X.chunk + lane];
     return x;
 }
-static_assert(kChunkN <= 32, "a lane for every value of a chunk");
 
 // The value of ascending rank p, by the 32 lanes of a warp.
 __device__ __forceinline__ Ranked index_select(const CellIndex& X, int p)
 {
     const int lane = threadIdx.x & 31;
-    const int c = warp_upper_bound(X.end, X.nc, (uint32_t)p);
+    // the cell that holds rank p: 32 probes in each of three steps
+    const int s1 = X.nc >> 5, s2 = X.nc >> 10;
+    int c = s1 * __popc(__ballot_sync(0xffffffffu, (int)X.end[(lane + 1) * s1 - 1] <= p));
+    c += s2 * __popc(__ballot_sync(0xffffffffu, (int)X.end[c + (lane + 1) * s2 - 1] <= p));
+    c += __popc(__ballot_sync(0xffffffffu, lane < s2 && (int)X.end[c + (lane & (s2 - 1))] <= p));
     const int a = c > 0 ? (int)X.end[c - 1] : 0, b = (int)X.end[c], k = p - a;
     Ranked r;
     int lt = 0, eq = 0;
@@ -1093,7 +1074,7 @@ __device__ __forceinline__ Ranked index_select(const CellIndex& X, int p)
             lt += w < v ? 1 : 0;
             eq += w == v ? 1 : 0;
         }
-        const int src = __ffs(__ballot_sync(0xffffffffu, a + lane < b && lt <= k && k < lt + eq)) - 1;
+        const int src = (__ffs(__ballot_sync(0xffffffffu, a + lane < b && lt <= k && k < lt + eq)) - 1) & 31;
         r.v = __shfl_sync(0xffffffffu, v, src);
         lt = __shfl_sync(0xffffffffu, lt, src);
         eq = __shfl_sync(0xffffffffu, eq, src);
@@ -1151,12 +1132,10 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
                 if (!(R.val > L.val)) {
                     if (lane == 0) o = L;
                 } else {
-                    const long long nseg = R.c_le - L.c_lt;
-                    const double A = (R.s_le - L.s_lt) - L.val * (double)nseg;
-                    long long k = (long long)floor(fp64_div(A, R.val - L.val));
-                    if (k < 0) k = 0;
-                    if (k > nseg - 1) k = nseg - 1;
-                    const long long p = R.c_le - 1 - k;
+                    const double nseg = (double)(R.c_le - L.c_lt);
+                    const double A = (R.s_le - L.s_lt) - L.val * nseg;
+                    const double k = fmin(fmax(floor(fp64_div(A, R.val - L.val)), 0.0), nseg - 1.0);
+                    const long long p = R.c_le - 1 - (long long)k;
                     // the interval that holds rank p: the last one that begins at or before it
                     const int j = __popc(__ballot_sync(0xffffffffu, lane < m && iv[lane].cbefore <= p)) +
                                   __popc(__ballot_sync(0xffffffffu, lane + 32 < m && iv[lane + 32].cbefore <= p)) - 1;
@@ -1185,12 +1164,13 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
         return;
     }
     // BinGrad-pb: the values with g(x) = x n - sum_{|v| >= x} |v| <= 0 come first; a warp per candidate rank
+    const int nw = blockDim.x >> 5;
     int lo = -1, hi = X.n;  // g <= 0 at lo (or lo = -1), g > 0 at hi (or hi = n)
     double b1 = fp64_div(stot - iv[0].sbefore, (double)n);  // the zero when it lies below every value of the bracket
 #pragma unroll 1
     while (true) {
         const bool last = hi - lo <= 1;
-        const int step = (hi - lo + kSelWarps - 1) / kSelWarps;
+        const int step = (hi - lo + nw - 1) / nw;
         const int i = last ? lo : lo + 1 + warp * step;
         if (last && lo < 0) break;
         bool below = false;
@@ -1208,7 +1188,7 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
         if (last) break;
         if (lane == 0) S.below[warp] = below ? 1u : 0u;
         __syncthreads();
-        const int k = __popc(__ballot_sync(0xffffffffu, lane < kSelWarps && S.below[lane & (kSelWarps - 1)]));
+        const int k = __popc(__ballot_sync(0xffffffffu, lane < nw && S.below[lane]));
         __syncthreads();
         const int nhi = lo + 1 + k * step;
         if (k > 0) lo += 1 + (k - 1) * step;
@@ -1222,29 +1202,27 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
 }
 
 // Gathers the keys of src[0 .. src_cnt) that lie inside the intervals S.niv (all of them when `filtered`),
-// indexes them and finishes the tensor from there: called when they fit kSortN.  4096 keys take about 5 us;
-// a bitonic sort in shared memory with binary searches per level took 20.
+// indexes them and finishes the tensor from there: called when they fit kSortN.
 __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s, const uint32_t* src, int src_cnt, bool filtered,
                                               float* __restrict__ levels, int32_t* __restrict__ status, unsigned char* smem,
                                               SolverShared& S)
 {
-    const int tid = threadIdx.x, lane = tid & 31;
-    uint32_t* list = reinterpret_cast<uint32_t*>(smem + kIndexBytes<kFinishCells> + 8);
+    const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
+    uint32_t* list = reinterpret_cast<uint32_t*>(smem + kIndexBytes);
+    if (tid == 0) { S.n_keys = 0; S.internal = 0; }
     __syncthreads();  // S.nm and S.niv are complete
     const int m = S.nm;
-    if (tid < kMaxIv) {
-        const bool real = tid < m;
-        const uint32_t lo = real ? S.niv[tid].klo : 0xffffffffu, hi = real ? S.niv[tid].khi : 0u;  // (no key has the value of lo: NaN)
-        S.lo[tid] = lo;
-        S.hi[tid] = hi;
-        // equal shares of the cells: an interval is a narrow slice of a binade, its values are spread evenly
-        const uint32_t share = (uint32_t)(kFinishCells / m);
-        S.sh[tid] = real ? max(0, 32 - __clz((hi - lo) / share)) : 0;
-        S.base[tid] = tid * share;
-    }
-    if (tid == 0) { S.n_keys = 0; S.internal = 0; }
     int top = 2;
     while (top < m) top <<= 1;
+    if (filtered) {
+#pragma unroll 4
+        for (int i = tid; i < src_cnt; i += nt) list[i] = __ldcg(src + i);
+    }
+    if (tid < kMaxIv) {
+        const bool real = tid < m;
+        S.lo[tid] = real ? S.niv[tid].klo : 0xffffffffu;  // (no key has this value: NaN)
+        S.hi[tid] = real ? S.niv[tid].khi : 0u;
+    }
     __syncthreads();
     auto interval = [&](uint32_t key) -> int {
         int j = 0;
@@ -1254,17 +1232,14 @@ __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s,
         return j;
     };
     int c = src_cnt;
-    if (filtered) {
-#pragma unroll 4
-        for (int i = tid; i < c; i += kSelThreads) list[i] = __ldcg(src + i);
-    } else {
+    if (!filtered) {
         constexpr int kCols = 4;  // loads in flight per thread
 #pragma unroll 1
-        for (int i0 = tid & ~31; i0 < src_cnt; i0 += kCols * kSelThreads) {
+        for (int i0 = tid & ~31; i0 < src_cnt; i0 += kCols * nt) {
             uint32_t k[kCols];
 #pragma unroll
             for (int u = 0; u < kCols; ++u) {
-                const int i = i0 + u * kSelThreads + lane;
+                const int i = i0 + u * nt + lane;
                 k[u] = i < src_cnt ? __ldcg(src + i) : 0u;
             }
             int j[kCols];
@@ -1278,7 +1253,7 @@ __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s,
             }
 #pragma unroll
             for (int u = 0; u < kCols; ++u) {
-                const bool in = i0 + u * kSelThreads + lane < src_cnt && k[u] >= S.lo[j[u]] && k[u] <= S.hi[j[u]];
+                const bool in = i0 + u * nt + lane < src_cnt && k[u] >= S.lo[j[u]] && k[u] <= S.hi[j[u]];
                 const unsigned b = __ballot_sync(0xffffffffu, in);
                 if (b) {
                     int pos = 0;
@@ -1292,15 +1267,21 @@ __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s,
         c = S.n_keys;
         if (c > kSortN) { c = kSortN; if (tid == 0) S.internal = 1; }
     }
-    const CellIndex X = index_at(smem, c, kFinishCells);
-    // (index_build begins with a barrier)
+    const CellIndex X = index_at(smem, c);
+    if (tid < m) {
+        // equal shares of the cells: an interval is a narrow slice of a binade, its values are spread evenly
+        const uint32_t share = (uint32_t)(X.nc / m);
+        S.sh[tid] = max(0, 32 - __clz((S.hi[tid] - S.lo[tid]) / share));
+        S.base[tid] = tid * share;
+    }
+    // (index_build has a barrier before the first cell is asked for)
     index_build(X, S, [&](int i) { return sel_key_to_float(list[i]); },
                 [&](int i) -> uint32_t {
                     const uint32_t key = list[i];
                     const int j = interval(key);
                     return S.base[j] + ((key - S.lo[j]) >> S.sh[j]);
                 });
-    for (int j = tid >> 5; j <= m; j += kSelWarps) {
+    for (int j = tid >> 5; j <= m; j += nt >> 5) {
         // where interval j begins: after the last value of the cell before its first
         const int a = j == m ? c : (j > 0 ? (int)X.end[S.base[j] - 1] : 0);
         const double x = warp_sum(index_before_lane(X, a));
@@ -1320,16 +1301,15 @@ __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s,
 __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool pb, int s, float* __restrict__ levels,
                              int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, float tau)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    auto value = [&](int i) -> float {
-        const float x = __ldg(src + i);
-        const float v = copysignf(fminf(fabsf(x), tau), x) + 0.0f;  // clipped, -0 counts as 0
-        return pb ? fabsf(v) : v;
-    };
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+    float* values = reinterpret_cast<float*>(smem + kIndexBytes);  // clipped, -0 as 0, magnitudes for BinGrad-pb
     uint32_t kmin = 0xffffffffu, kmax = 0u, sum = 0u;
 #pragma unroll 4
-    for (int i = tid; i < n; i += kSelThreads) {
-        const float v = value(i);
+    for (int i = tid; i < n; i += nt) {
+        const float x = __ldg(src + i);
+        float v = copysignf(fminf(fabsf(x), tau), x) + 0.0f;
+        if (pb) v = fabsf(v);
+        values[i] = v;
         const uint32_t k = float_to_key(v);
         kmin = min(kmin, k);
         kmax = max(kmax, k);
@@ -1340,9 +1320,9 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
     sum = __reduce_add_sync(0xffffffffu, sum);
     if (lane == 0) { S.lo[warp] = kmin; S.hi[warp] = kmax; S.base[warp] = sum; }
     __syncthreads();
-    kmin = __reduce_min_sync(0xffffffffu, S.lo[lane & (kSelWarps - 1)]);
-    kmax = __reduce_max_sync(0xffffffffu, S.hi[lane & (kSelWarps - 1)]);
-    sum = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? S.base[lane & (kSelWarps - 1)] : 0u);
+    kmin = __reduce_min_sync(0xffffffffu, S.lo[lane & (nw - 1)]);
+    kmax = __reduce_max_sync(0xffffffffu, S.hi[lane & (nw - 1)]);
+    sum = __reduce_add_sync(0xffffffffu, lane < nw ? S.base[lane] : 0u);
     const float vmin = key_to_float(kmin), vmax = key_to_float(kmax);
     const int nl = pb ? 2 : s;
     // (keys order Inf and NaN beyond the finite values at either end)
@@ -1353,13 +1333,21 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
         if (tid == 0) status[t] = bad ? OGQ_ST_NONFINITE : (!pb || vmax == 0.f) ? OGQ_ST_CONSTANT : 0;
         return;
     }
-    const MagnitudeCells cell((uint32_t)((float)sum / (float)n), fmaxf(fabsf(vmin), fabsf(vmax)), !pb, kSmallCells);
-    const CellIndex X = index_at(smem, n, kSmallCells);
-    index_build(X, S, value, [&](int i) { return cell(value(i)); });
+    const CellIndex X = index_at(smem, n);
+    const MagnitudeCells cell((uint32_t)((float)sum / (float)n), fmaxf(fabsf(vmin), fabsf(vmax)), !pb, (uint32_t)X.nc);
+    index_build(X, S, [&](int i) { return values[i]; }, [&](int i) { return cell(values[i]); });
+    if (warp == 0) {
+        // (the total the way index_select adds prefixes up)
+        const double x = warp_sum(index_before_lane(X, n));
+        if (lane == 0) S.offs[0] = x;
+    }
+    __syncthreads();
+    const double stot = S.offs[0];
     if (tid == 0) {
         S.internal = 0;
         S.start[0] = 0; S.start[1] = n; S.pre[0] = 0.0;
         S.niv[0].cbefore = 0; S.niv[0].sbefore = 0.0;
+        status[t] = 0;
     }
     if (tid < s) {
         LvInfo& l = S.lv[tid];
@@ -1367,11 +1355,10 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
         l.val = (double)(tid == 0 ? vmin : vmax);
         l.key = tid == 0 ? kmin : kmax;
         l.c_lt = 0; l.s_lt = 0.0;
-        l.c_le = n; l.s_le = X.pre[kSelThreads];
+        l.c_le = n; l.s_le = stot;
     }
-    if (tid == 0) status[t] = 0;
     __syncthreads();
-    levels_from_index(X, S, S.niv, 1, pb, s, n, X.pre[kSelThreads], t, levels, status);
+    levels_from_index(X, S, S.niv, 1, pb, s, n, stot, t, levels, status);
 }
 
 // Finishes a tensor whose last pass only copied the keys inside its intervals (TState::compact_only): the
@@ -1379,21 +1366,22 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
 __device__ void finish_sorted(TState* st, int t, bool pb, int s, const uint32_t* copied, float* __restrict__ levels,
                               int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, int cursor_idx)
 {
+    // (every load is issued before the first is waited for; intervals beyond st->m are not used)
+    const int tid = threadIdx.x, m = __ldcg(&st->m);
+    const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[cursor_idx]);
     __syncthreads();
-    const int m = __ldcg(&st->m);
-    if ((int)threadIdx.x < m) S.niv[threadIdx.x] = st->iv[threadIdx.x];
-    if (!pb && (int)threadIdx.x >= 64 && (int)threadIdx.x - 64 < s) {
-        const ExactLv& e = st->lv[threadIdx.x - 64];
-        LvInfo& l = S.lv[threadIdx.x - 64];
+    if (tid < kMaxIv) S.niv[tid] = st->iv[tid];
+    if (!pb && tid >= 64 && tid - 64 < s) {
+        const ExactLv& e = st->lv[tid - 64];
+        LvInfo& l = S.lv[tid - 64];
         l.exact = e.exact; l.key = e.key; l.val = (double)sel_key_to_float(e.key);
         l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
     }
-    if (threadIdx.x == 0) {
-        S.nm = m;
+    if (tid == 0) {
         S.view.n = st->n;
         S.view.stot = st->stot;
+        S.nm = m;
     }
-    const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[cursor_idx]);
     finish_from_keys(st, t, pb, s, copied, (int)src_cnt, src_cnt == cand, levels, status, smem, S);
 }
 
@@ -1403,10 +1391,8 @@ constexpr size_t kOffSlotIv = kOffSpre + kSlots * sizeof(double);
 constexpr size_t kOffRawSum = (kOffSlotIv + kSlots + 15) / 16 * 16;
 constexpr size_t kOffRawCnt = kOffRawSum + kCells * sizeof(unsigned long long);
 constexpr size_t kPrefixBytes = kOffRawCnt + kCells * sizeof(uint32_t);
-constexpr size_t kFinishBytes = kIndexBytes<kFinishCells> + 8 + kSortN * sizeof(uint32_t);
-constexpr size_t kSolveBytes = kPrefixBytes > kFinishBytes ? kPrefixBytes : kFinishBytes;
-constexpr size_t kRound3Bytes = kSolveBytes > kSmemBytes ? kSolveBytes : kSmemBytes;  // of a CTA that also streams
-static_assert(kIndexBytes<kSmallCells> <= kSmemBytes, "small tensors are solved in a streaming CTA");
+constexpr size_t kSolveBytes = kIndexBytes + (size_t)kSortN * sizeof(uint32_t);
+static_assert(kPrefixBytes <= kSolveBytes && kSmemBytes <= kSolveBytes, "the finish takes the most shared memory");
 
 // Prefix arrays over all slots of the intervals S.iv (S.view.m of them): counts and sums of the elements
 // before every slot.  A thread takes consecutive slots; a slot's cell is its index minus the number of
@@ -1419,7 +1405,7 @@ __device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* g
     uint8_t* slot_iv = smem + kOffSlotIv;
     unsigned long long* raw_sum = reinterpret_cast<unsigned long long*>(smem + kOffRawSum);
     uint32_t* raw_cnt = reinterpret_cast<uint32_t*>(smem + kOffRawCnt);
-    const int tid = threadIdx.x, m = S.view.m;
+    const int tid = threadIdx.x, nt = blockDim.x, m = S.view.m;
     const int ncells = S.iv[m - 1].cellbase + S.iv[m - 1].ncell, nslots = ncells + m;
     {
         constexpr int kC = (kCells / 4 + kSelThreads - 1) / kSelThreads, kL = (kCells / 2 + kSelThreads - 1) / kSelThreads;
@@ -1427,21 +1413,21 @@ __device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* g
         ulonglong2 l[kL];
 #pragma unroll
         for (int u = 0; u < kC; ++u)
-            if ((tid + u * kSelThreads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSelThreads);
+            if ((tid + u * nt) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * nt);
 #pragma unroll
         for (int u = 0; u < kL; ++u)
-            if ((tid + u * kSelThreads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSelThreads);
+            if ((tid + u * nt) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * nt);
         if (tid < m) S.view.slotbase[tid] = S.iv[tid].cellbase + tid;
         if (tid == 0) { S.view.slotbase[m] = nslots; S.view.nslots = nslots; }
 #pragma unroll
         for (int u = 0; u < kC; ++u)
-            if ((tid + u * kSelThreads) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * kSelThreads] = c[u];
+            if ((tid + u * nt) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * nt] = c[u];
 #pragma unroll
         for (int u = 0; u < kL; ++u)
-            if ((tid + u * kSelThreads) * 2 < ncells) reinterpret_cast<ulonglong2*>(raw_sum)[tid + u * kSelThreads] = l[u];
+            if ((tid + u * nt) * 2 < ncells) reinterpret_cast<ulonglong2*>(raw_sum)[tid + u * nt] = l[u];
     }
     __syncthreads();
-    const int per = (nslots + kSelThreads - 1) / kSelThreads;
+    const int per = (nslots + nt - 1) / nt;
     const int s0 = tid * per < nslots ? tid * per : nslots, s1 = s0 + per < nslots ? s0 + per : nslots;
     int j = 0;
     {
@@ -1449,7 +1435,7 @@ __device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* g
 #pragma unroll 1
         while (hi - j > 1) { const int mid = (j + hi) >> 1; if (S.view.slotbase[mid] <= s0) j = mid; else hi = mid; }
     }
-    unsigned long long lc = 0;
+    uint32_t lc = 0;
     double ls = 0.0;
 #pragma unroll 1
     for (int slot = s0; slot < s1; ++slot) {
@@ -1463,14 +1449,14 @@ __device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* g
         lc += n;
         ls += x;
     }
-    unsigned long long tc;
+    uint32_t tc;
     double ts;
-    block_excl_scan(lc, ls, S.sc, S.ss, tc, ts);
+    block_excl_scan(lc, ls, S, tc, ts);
 #pragma unroll 1
     for (int slot = s0; slot < s1; ++slot) {
         const uint32_t n = cpre[slot];
         const double x = spre[slot];
-        cpre[slot] = (uint32_t)lc;
+        cpre[slot] = lc;
         spre[slot] = ls;
         lc += n;
         ls += x;
@@ -1669,7 +1655,7 @@ __device__ __forceinline__ bool refine_marked(SolverShared& S)
 // keys inside the new intervals are few enough.  Called by every thread of the CTA; returns true when the
 // tensor is finished.  S.iv, S.view.m / n / stot and S.lv describe the pass that just ended.
 //   round_buf: the keys copied by the pass (null: none were), cap: words of the tensor's key region.
-__device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long long* glsum, int scheme,
+__device__ __noinline__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long long* glsum, int scheme,
                              int s, float* __restrict__ levels, int32_t* __restrict__ status,
                              unsigned* nitems, int2* items, const uint32_t* round_buf, bool enqueue,
                              unsigned char* smem, SolverShared& S, int64_t cap, int round)
@@ -1677,7 +1663,7 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
     uint32_t* cpre = reinterpret_cast<uint32_t*>(smem);
     double* spre = reinterpret_cast<double*>(smem + kOffSpre);
     const bool pb = scheme == OGQ_BINGRAD_PB;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x, nt = blockDim.x;
 
     if (tid == 0) {
         S.view.iv = S.iv;
@@ -1687,7 +1673,7 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
         S.done = 0; S.nm = -100; S.internal = 0; S.cand = 0; S.nopen = 0;
         S.pb_a = -1; S.pb_b = -1; S.pb_c = -1;
     }
-    for (int i = tid; i < (kSlots + 31) / 32; i += kSelThreads) S.marks[i] = 0u;
+    for (int i = tid; i < (kSlots + 31) / 32; i += nt) S.marks[i] = 0u;
     __syncthreads();
     solver_prefix(S, gcnt, glsum, round == 1, smem);
     const int nslots = S.view.nslots;
@@ -1734,7 +1720,7 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
         // bracket of the sign change of g, evaluated at the lower edge of every cell
         int a = -1, b = -1, cs = -1;
 #pragma unroll 1
-        for (int sl = tid; sl < nslots; sl += kSelThreads) {
+        for (int sl = tid; sl < nslots; sl += nt) {
             if (sel_is_end_slot(S.view, sl)) continue;
             double x;
             const double g = sel_pb_g(S.view, sl, &x);
@@ -1753,7 +1739,7 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
         cs = S.pb_c < a ? a : S.pb_c;
         if (cs > b) cs = b;
         bool coarse = false;  // some cell of the bracket holds more than one key
-        for (int sl = a + tid; sl <= b; sl += kSelThreads)
+        for (int sl = a + tid; sl <= b; sl += nt)
             coarse |= !sel_is_end_slot(S.view, sl) && sel_slot_shift(S.view, sl) != 0;
         coarse = __syncthreads_or(coarse);
         if (cpre[b + 1] == cpre[a]) {
@@ -1837,7 +1823,7 @@ __device__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long lo
     const bool compact_only = few && S.cand <= cap;
     const int ncells_next = S.niv[S.nm - 1].cellbase + S.niv[S.nm - 1].ncell;
     if (!compact_only) {
-        for (int i = tid; i < ncells_next; i += kSelThreads) { gcnt[i] = 0u; glsum[i] = 0ull; }
+        for (int i = tid; i < ncells_next; i += nt) { gcnt[i] = 0u; glsum[i] = 0ull; }
     }
     if (tid < S.nm) st->iv[tid] = S.niv[tid];
     if (tid == 0) {
@@ -2022,27 +2008,10 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SolverShared S;
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
-    const int nl = pb ? 2 : A.s;
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
     pdl_wait();
     pdl_launch_dependents();
-
-    if ((int)blockIdx.x < A.T) {
-        // the first T CTAs, one per tensor, settle the empty and small tensors
-        const int t = blockIdx.x;
-        const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
-        const int64_t n = tend - tbeg;
-        if (n <= 0) {
-            if (threadIdx.x < nl) A.levels[(int64_t)t * nl + threadIdx.x] = 0.f;
-            if (threadIdx.x == 0) A.status[t] = OGQ_ST_EMPTY;
-        } else if (n <= kSmallN) {
-            small_tensor(A.grad + tbeg, (int)n, t, pb, A.s, A.levels, A.status, smem, S,
-                         A.tau ? __ldcg(A.tau + t) : __int_as_float(0x7f800000));
-        }
-        return;
-    }
 
     // Flat CTAs: one chunk of the bucket each.  A piece of a tensor is streamed into the CTA's cells, which
     // are then added to the tensor's global ones.
@@ -2051,7 +2020,7 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArg
     int lo_e = 0;
     uint32_t* packed_cells = reinterpret_cast<uint32_t*>(smem + kSmemHist);
     const int ncells = pb ? kRound1Mag : kRound1Cells;
-    const int64_t lo = (int64_t)(blockIdx.x - A.T) * A.chunk;
+    const int64_t lo = (int64_t)blockIdx.x * A.chunk;
     const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
     for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
         if (tend - tbeg <= kSmallN) return;
@@ -2087,24 +2056,182 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArg
     });
 }
 
-// The first solver pass of every streamed tensor: one CTA per tensor.
-__global__ void __launch_bounds__(kSelThreads) k_sel_solve1(SelArgs A)
+// ---------------------------------------------------------------------------
+// The first solver pass: round 1's cells are the same for every tensor but for the position of the window, so
+// their keys follow from their index.
+// ---------------------------------------------------------------------------
+struct Round1Cells {
+    int lo_e;
+    bool mag;  // cells of magnitudes only
+
+    __device__ __forceinline__ int count() const { return mag ? kRound1Mag : kRound1Cells; }
+    // keys of cell c: base, log2 of their number
+    __device__ __forceinline__ uint32_t key(int c, int& sh) const
+    {
+        const bool neg = !mag && c < kRound1Mag;
+        const int mi = mag ? c : neg ? kRound1Mag - 1 - c : c - kRound1Mag;
+        const int k = mi - lo_e;
+        const bool fine = k >= 0 && k < (kSelW << kSelM);
+        sh = fine ? 23 - kSelM : 23;
+        const uint32_t bits = fine ? ((uint32_t)lo_e << 23) + ((uint32_t)k << (23 - kSelM))
+                                   : (uint32_t)(k < 0 ? mi : mi - (kSelW << kSelM) + kSelW) << 23;
+        return neg ? 0x80000000u - bits - (1u << sh) : 0x80000000u + bits;
+    }
+};
+
+// A level of the first pass: its value, or bounds of its value and the cells [sa, sb] that contain it.
+struct Level1 {
+    double vlo, vhi, s_lt, s_le;  // exact: value twice, sums before / up to it; else those of the whole range
+    uint32_t c_lt, c_le;
+    int exact, sa, sb;
+};
+
+constexpr int kCandCells = 512;  // candidate cells the first pass keeps track of
+
+struct Solve1Shared {
+    Level1 lv[kMaxLv];
+    uint32_t marks[(kRound1Cells + 31) / 32];
+    int list[kCandCells], sorted[kCandCells];
+    uint32_t starts[kCandCells / 32];   // which of the sorted candidate cells begin a run of neighbours
+    int first[kMaxIv + 1], cells_at[kMaxIv + 1];
+    int m, fail, runs;
+    uint32_t cand;
+    int pb_a, pb_b;
+};
+
+constexpr int kSolve1Threads = 1024;
+constexpr size_t kOffCells1 = ((kRound1Cells + 8) * sizeof(double) + 15) / 16 * 16;  // prefix sums, then prefix counts, then the raw cells
+constexpr size_t kOffRawSum1 = (kOffCells1 + (kRound1Cells + 8) * sizeof(uint32_t) + 15) / 16 * 16;
+constexpr size_t kOffRawCnt1 = kOffRawSum1 + kRound1Cells * sizeof(unsigned long long);
+static_assert(kOffRawCnt1 + kRound1Cells * sizeof(uint32_t) <= kIndexBytes, "the index of a small tensor takes more");
+
+// Q*(L, R) on round 1's cells by the 32 lanes of a warp; see warp_orq_solve for the bounds.
+__device__ __noinline__ void solve1_level(const Round1Cells G, const double* spre, const uint32_t* cpre, double n, const Level1* Lp,
+                                          const Level1* Rp, Level1* out)
+{
+    const int lane = threadIdx.x & 31;
+    const bool upper = lane >= 16;
+    const Level1 L = *Lp, R = *Rp;
+    const bool exact = L.exact && R.exact;
+    if (exact && !(R.vlo > L.vlo)) {
+        if (lane == 0) *out = L;
+        __syncwarp();
+        return;
+    }
+    const double floor_pos = (double)L.c_lt, ceil_pos = (double)R.c_le - 1.0;
+    double p = upper ? ceil_pos : floor_pos;
+    const double Cs = (double)(L.exact ? L.c_lt : L.c_le), Ce = (double)(R.exact ? R.c_le : R.c_lt);
+    const double Ss = L.exact ? L.s_lt : L.s_le, Se = R.exact ? R.s_le : R.s_lt;
+    const double cntM = Ce - Cs, sumM = Se - Ss;
+    if (cntM >= 0.0 && R.vlo > L.vhi) {
+        const double cntL = L.exact ? 0.0 : (double)(L.c_le - L.c_lt), cntR = R.exact ? 0.0 : (double)(R.c_le - R.c_lt);
+        // (both brackets exact: both halves compute T = (sumM - L cntM) / (R - L))
+        double num = fmax(sumM - (upper ? L.vhi : L.vlo) * cntM, 0.0);
+        num = upper ? cntR * (R.vhi - R.vlo) - num : -(cntL * (L.vhi - L.vlo) + num);
+        const double q = fp64_div(num, upper ? R.vhi - L.vhi : R.vlo - L.vlo);
+        if (exact) {
+            p = Ce - 1.0 - fmin(fmax(floor(-q), 0.0), cntM - 1.0);
+        } else {
+            const double delta = 2.0 + 1e-9 * n;
+            const double g = ceil(Ce + q + (upper ? delta : -delta)) - 1.0;
+            p = upper ? fmin(p, g) : fmax(p, g);
+        }
+    }
+    p = fmin(fmax(p, floor_pos), ceil_pos);
+    const double other = __shfl_xor_sync(0xffffffffu, p, 16);
+    if (!upper) p = fmin(p, other);
+    const uint32_t pos = __double2uint_rn(fmin(fmax(p, 0.0), n - 1.0));
+    // the cells of the two ranks: the last whose prefix does not exceed the rank
+    int lo = 0, hi = G.count() + 1;
+#pragma unroll 1
+    while (__any_sync(0xffffffffu, lo < hi)) {
+        const int step = (hi - lo + 15) >> 4;
+        const int i = lo + (lane & 15) * step;
+        const unsigned b = __ballot_sync(0xffffffffu, i < hi && cpre[i] <= pos);
+        const int k = __popc(upper ? b >> 16 : b & 0xffffu);
+        const int nhi = lo + k * step;
+        if (k > 0) lo += (k - 1) * step + 1;
+        if (nhi < hi) hi = nhi;
+    }
+    const int slot = lo - 1;
+    int sh;
+    const uint32_t key = G.key(slot, sh);
+    const double val = (double)sel_key_to_float(key + (upper ? (1u << sh) - 1u : 0u));
+    const double vhi = __shfl_sync(0xffffffffu, val, 16);
+    const int sb = __shfl_sync(0xffffffffu, slot, 16);
+    if (lane == 0) {
+        out->exact = 0;
+        out->vlo = val;
+        out->vhi = vhi;
+        out->sa = slot;
+        out->sb = sb;
+        out->c_lt = cpre[slot];
+        out->s_lt = spre[slot];
+        out->c_le = cpre[sb + 1];
+        out->s_le = spre[sb + 1];
+    }
+    __syncwarp();
+}
+
+// One CTA per tensor.  Streamed tensors: prefix sums over round 1's cells, conservative cell ranges of the
+// levels, every populated cell in them becomes an interval of round 2.  Small tensors are solved here.
+//   What bounds it: latency, 8 to 10 us for a streamed tensor and for a small one.
+__global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SolverShared S;
+    __shared__ Solve1Shared Q;
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
-    const int nl = pb ? 2 : A.s;
+    const int nl = pb ? 2 : A.s, s = A.s;
     pdl_wait();
     pdl_launch_dependents();
-    const int t = blockIdx.x;
-    const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
-    const int64_t n = tend - tbeg;
-    if (n <= kSmallN) return;
+    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // (loads first, the decision what to do with them after)
     TState* st = A.ws.st + t;
-    const int tid = threadIdx.x;
-    const uint32_t kmn = ~__ldcg(&st->kmin_inv), kmx = __ldcg(&st->kmax);
-    const int hi_e = __ldcg(&st->hi_e);
-    const bool bad = __ldcg(&st->nonfinite) != 0u, constant = !bad && !pb && kmn == kmx;
+    const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
+    const uint32_t kmn = ~__ldcg(&st->kmin_inv), kmx = __ldcg(&st->kmax), nonfinite = __ldcg(&st->nonfinite);
+    Round1Cells G;
+    G.mag = pb;
+    G.lo_e = __ldcg(&st->hi_e) - kSelW;
+    const int ncells = G.count();
+    uint32_t* gcnt = A.ws.gcnt + (size_t)t * kCells;
+    unsigned long long* glsum = A.ws.glsum + (size_t)t * kCells;
+    const int64_t n = tend - tbeg;
+    if (n <= kSmallN) {
+        if (n <= 0) {
+            if (tid < nl) A.levels[(int64_t)t * nl + tid] = 0.f;
+            if (tid == 0) A.status[t] = OGQ_ST_EMPTY;
+        } else {
+            small_tensor(A.grad + tbeg, (int)n, t, pb, s, A.levels, A.status, smem, S,
+                         A.tau ? __ldcg(A.tau + t) : __int_as_float(0x7f800000));
+        }
+        return;
+    }
+    double* spre = reinterpret_cast<double*>(smem);
+    uint32_t* cpre = reinterpret_cast<uint32_t*>(smem + kOffCells1);
+    unsigned long long* raw_sum = reinterpret_cast<unsigned long long*>(smem + kOffRawSum1);
+    uint32_t* raw_cnt = reinterpret_cast<uint32_t*>(smem + kOffRawCnt1);
+    {
+        constexpr int kC = (kRound1Cells / 4 + kSolve1Threads - 1) / kSolve1Threads,
+                      kL = (kRound1Cells / 2 + kSolve1Threads - 1) / kSolve1Threads;
+        uint4 c[kC];
+        ulonglong2 l[kL];
+#pragma unroll
+        for (int u = 0; u < kC; ++u)
+            if ((tid + u * kSolve1Threads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSolve1Threads);
+#pragma unroll
+        for (int u = 0; u < kL; ++u)
+            if ((tid + u * kSolve1Threads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSolve1Threads);
+        if (tid < (kRound1Cells + 31) / 32) Q.marks[tid] = 0u;
+        if (tid == 0) { Q.m = 0; Q.fail = 0; Q.runs = 0; Q.cand = 0u; Q.pb_a = 0; Q.pb_b = 0; }
+#pragma unroll
+        for (int u = 0; u < kC; ++u)
+            if ((tid + u * kSolve1Threads) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * kSolve1Threads] = c[u];
+#pragma unroll
+        for (int u = 0; u < kL; ++u)
+            if ((tid + u * kSolve1Threads) * 2 < ncells) reinterpret_cast<ulonglong2*>(raw_sum)[tid + u * kSolve1Threads] = l[u];
+    }
+    const bool bad = nonfinite != 0u, constant = !bad && !pb && kmn == kmx;
     if (bad || constant) {
         if (tid < nl) A.levels[(int64_t)t * nl + tid] = bad ? 0.f : sel_key_to_float(kmn);
         if (tid == 0) {
@@ -2113,24 +2240,237 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_solve1(SelArgs A)
         }
         return;
     }
-    if (tid < (pb ? 3 : 6)) S.iv[tid] = round1_interval(hi_e, pb, tid);
-    if (tid >= 64 && tid - 64 < A.s) {
-        const int q = tid - 64;
-        LvInfo& l = S.lv[q];
-        l.exact = (q == 0 || q == A.s - 1) ? 1 : 0;
-        l.key = q == 0 ? kmn : kmx;
-        l.val = l.vlo = l.vhi = (double)sel_key_to_float(l.key);
-        l.c_lt = 0; l.s_lt = 0.0; l.c_le = 0; l.s_le = 0.0;
+    __syncthreads();
+    uint32_t total;
+    double stot;
+    {
+        const int per = (ncells + kSolve1Threads - 1) / kSolve1Threads;
+        const int c0 = tid * per < ncells ? tid * per : ncells, c1 = c0 + per < ncells ? c0 + per : ncells;
+        uint32_t lc = 0u;
+        double ls = 0.0;
+#pragma unroll 1
+        for (int c = c0; c < c1; ++c) {
+            const uint32_t k = raw_cnt[c];
+            double x = 0.0;
+            if (k) {
+                int sh;
+                const uint32_t key = G.key(c, sh);
+                x = sel_cell_sum(key, sh, k, raw_sum[c]);
+            }
+            spre[c] = x;
+            lc += k;
+            ls += x;
+        }
+        block_excl_scan(lc, ls, S, total, stot);
+#pragma unroll 1
+        for (int c = c0; c < c1; ++c) {
+            const double x = spre[c];
+            cpre[c] = lc;
+            spre[c] = ls;
+            lc += raw_cnt[c];
+            ls += x;
+        }
+        // (the total is the last prefix: differences of prefixes, which decide where T falls on an integer, then carry
+        // the rounding of one chain of additions)
+        if (c0 < c1 && c1 == ncells) { cpre[ncells] = lc; spre[ncells] = ls; }
     }
+    __syncthreads();
+    stot = spre[ncells];
+    if (tid >= 64 && tid - 64 < s && !pb) {
+        const int q = tid - 64;
+        Level1& l = Q.lv[q];
+        l.exact = (q == 0 || q == s - 1) ? 1 : 0;
+        l.vlo = l.vhi = (double)sel_key_to_float(q == 0 ? kmn : kmx);
+        l.c_lt = 0u; l.s_lt = 0.0;
+        l.c_le = q == 0 ? 0u : total; l.s_le = q == 0 ? 0.0 : stot;
+        l.sa = l.sb = -1;
+    }
+    __syncthreads();
+    const bool counted = (int64_t)total == n;
+    int range_a = 0, range_b = -1;  // this warp's candidate cells
+    if (counted && !pb) {
+        static_assert(kSolve1Threads / 32 >= kMaxLv - 1, "one warp per interior level");
+#pragma unroll 1
+        for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
+            const int q = warp;
+            if (q < s - 1 && q >= stride && ((q - stride) & (2 * stride - 1)) == 0) {
+                solve1_level(G, spre, cpre, (double)n, Q.lv + q - stride, Q.lv + q + stride, Q.lv + q);
+                if (!Q.lv[q].exact) {
+                    range_a = Q.lv[q].sa;
+                    range_b = Q.lv[q].sb;
+                    if (range_a < 0 || range_a > range_b) Q.fail = 1;
+                }
+            }
+            __syncthreads();
+        }
+    } else if (counted && stot > 0.0) {
+        // bracket of the sign change of g(x) = x n - sum_{|v| >= x} |v|, evaluated at the lower edge of every cell
+        int a = 0, b = 0;
+#pragma unroll 1
+        for (int c = tid; c < ncells; c += kSolve1Threads) {
+            int sh;
+            const double x = (double)sel_key_to_float(G.key(c, sh));
+            if (!(x < INFINITY)) continue;
+            const double g = x * (double)n - (stot - spre[c]), eps = 1e-11 * (x * (double)n + stot);
+            if (g < -eps) a = c;
+            if (g <= eps) b = c;
+        }
+        a = __reduce_max_sync(0xffffffffu, a);
+        b = __reduce_max_sync(0xffffffffu, b);
+        if (lane == 0) { atomicMax(&Q.pb_a, a); atomicMax(&Q.pb_b, b); }
+        __syncthreads();
+        if (warp == 0) { range_a = Q.pb_a; range_b = max(Q.pb_a, Q.pb_b); }
+    }
+    // every populated cell of the ranges, once
+#pragma unroll 1
+    for (int c = range_a + lane; c <= range_b; c += 32) {
+        const uint32_t k = cpre[c + 1] - cpre[c], bit = 1u << (c & 31);
+        if (k && !(atomicOr(&Q.marks[c >> 5], bit) & bit)) {
+            const int i = atomicAdd(&Q.m, 1);
+            if (i < kCandCells) Q.list[i] = c;
+            atomicAdd(&Q.cand, k);
+        }
+    }
+    __syncthreads();
+    const int m = Q.m;
     if (tid == 0) {
         st->n = n;
+        st->stot = stot;
         A.status[t] = 0;
-        S.view.m = pb ? 3 : 6;
-        S.view.n = n;
-        S.view.stot = 0.0;
     }
-    solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s, A.levels, A.status,
-                 A.ws.nitems, A.ws.items, nullptr, false, smem, S, sel_region(tend) - sel_region(tbeg), 1);
+    if (!counted || Q.fail || (pb && !(stot > 0.0)) || m == 0) {
+        // all magnitudes 0, an empty bracket (g is zero between two magnitudes), or an inconsistency
+        const bool fail = !counted || !pb;
+        if (pb) {
+            const float b1 = fail || !(stot > 0.0) ? 0.f : (float)((stot - spre[Q.pb_a]) / (double)n);
+            if (tid < 2) A.levels[2 * t + tid] = tid == 0 ? -b1 : b1;
+        } else if (tid < s) {
+            A.levels[(int64_t)t * s + tid] = 0.f;
+        }
+        if (tid == 0) {
+            A.status[t] = fail ? OGQ_ST_INTERNAL : pb && !(stot > 0.0) ? OGQ_ST_CONSTANT : 0;
+            st->done = 1;
+        }
+        return;
+    }
+    const uint32_t cand = Q.cand;
+    const bool compact_only = cand <= (uint32_t)kSortN && (int64_t)cand <= sel_region(tend) - sel_region(tbeg);
+    // the candidate cells in order
+    int my_rank = 0;
+    const bool mine = tid < m && m <= kCandCells;
+    if (mine) {
+        const int c = Q.list[tid];
+#pragma unroll 4
+        for (int j = 0; j < m; ++j) my_rank += Q.list[j] < c ? 1 : 0;
+    }
+    // Intervals of round 2: one per candidate cell when there are few, else one per run of neighbouring cells (of one
+    // width); each gets the same share of the new cells.
+    const bool single = m <= kMaxIv;
+    int runs = m;
+    if (!single) {
+        if (mine) Q.sorted[my_rank] = Q.list[tid];
+        __syncthreads();
+        if (tid < kCandCells) {
+            int s0, s1;
+            bool start = false;
+            if (tid < m && m <= kCandCells) {
+                const uint32_t k1 = G.key(Q.sorted[tid], s1);
+                const uint32_t k0 = tid > 0 ? G.key(Q.sorted[tid - 1], s0) : 0u;
+                start = tid == 0 || s0 != s1 || k0 + (1u << s0) != k1;
+            }
+            const uint32_t w = __ballot_sync(0xffffffffu, start);
+            if (lane == 0) { Q.starts[warp] = w; atomicAdd(&Q.runs, __popc(w)); }
+        }
+        __syncthreads();
+        runs = m <= kCandCells ? Q.runs : kMaxIv + 1;
+    }
+    int r = runs <= kMaxIv ? 31 - __clz(kCells / runs) : 0;
+    bool fits = runs <= kMaxIv;
+    int ncells_next = runs << r;
+    if (!single && fits) {
+        // position and length of every run, then halvings so that a run keeps to its share
+        int id = -1;
+        if (tid < m) {
+            id = __popc(Q.starts[tid >> 5] & (0xffffffffu >> (31 - (tid & 31)))) - 1;
+            for (int w = 0; w < (tid >> 5); ++w) id += __popc(Q.starts[w]);
+            if ((Q.starts[tid >> 5] >> (tid & 31)) & 1u) Q.first[id] = tid;
+        }
+        if (tid == 0) Q.first[runs] = m;
+        __syncthreads();
+        const int share = kCells / runs;
+        if (tid == 0) {
+            int at = 0;
+            for (int j = 0; j < runs; ++j) {
+                const int len = Q.first[j + 1] - Q.first[j];
+                Q.cells_at[j] = at;
+                at += len <= share ? len << (31 - __clz(share / len)) : len;
+            }
+            Q.cells_at[runs] = at;
+        }
+        __syncthreads();
+        ncells_next = Q.cells_at[runs];
+        fits = ncells_next <= kCells;
+        if (fits && tid < runs) {
+            const int len = Q.first[tid + 1] - Q.first[tid], c = Q.sorted[Q.first[tid]];
+            int sh;
+            Interval iv;
+            iv.klo = G.key(c, sh);
+            iv.khi = iv.klo + ((uint32_t)len << sh) - 1u;
+            const int rr = len <= share ? 31 - __clz(share / len) : 0;
+            iv.sh = sh - rr;
+            iv.ncell = len << rr;
+            iv.cellbase = Q.cells_at[tid];
+            iv.pad = 0;
+            iv.cbefore = cpre[c];
+            iv.sbefore = spre[c];
+            st->iv[tid] = iv;
+        }
+    }
+    if (!fits) {
+        // candidates scattered over too many cells: the general pass, which joins them up
+        __syncthreads();
+        if (tid < (pb ? 3 : 6)) S.iv[tid] = round1_interval(G.lo_e + kSelW, pb, tid);
+        if (tid >= 64 && tid - 64 < s) {
+            LvInfo& l = S.lv[tid - 64];
+            l.exact = (tid == 64 || tid - 64 == s - 1) ? 1 : 0;
+            l.key = tid == 64 ? kmn : kmx;
+            l.val = l.vlo = l.vhi = (double)sel_key_to_float(l.key);
+            l.c_lt = 0; l.s_lt = 0.0; l.c_le = 0; l.s_le = 0.0;
+        }
+        if (tid == 0) { S.view.m = pb ? 3 : 6; S.view.n = n; S.view.stot = 0.0; }
+        solver_round(st, t, gcnt, glsum, A.scheme, s, A.levels, A.status, A.ws.nitems, A.ws.items, nullptr, false, smem, S,
+                     sel_region(tend) - sel_region(tbeg), 1);
+        return;
+    }
+    if (single && mine) {
+        const int c = Q.list[tid];
+        Interval iv;
+        int sh;
+        iv.klo = G.key(c, sh);
+        iv.khi = iv.klo + ((1u << sh) - 1u);
+        iv.sh = sh - r;
+        iv.ncell = 1 << r;
+        iv.cellbase = my_rank << r;
+        iv.pad = 0;
+        iv.cbefore = cpre[c];
+        iv.sbefore = spre[c];
+        st->iv[my_rank] = iv;
+    }
+    if (!pb && tid >= 64 && tid - 64 < s) {
+        const Level1& l = Q.lv[tid - 64];
+        ExactLv& e = st->lv[tid - 64];
+        e.exact = l.exact;
+        e.key = float_to_key((float)l.vlo);
+        e.c_lt = l.c_lt; e.c_le = l.c_le; e.s_lt = l.s_lt; e.s_le = l.s_le;
+    }
+    if (!compact_only)
+        for (int i = tid; i < ncells_next; i += kSolve1Threads) { gcnt[i] = 0u; glsum[i] = 0ull; }
+    if (tid == 96) {
+        st->m = runs;
+        st->cand = cand;
+        st->compact_only = compact_only ? 1 : 0;
+        st->round = 2;
+    }
 }
 
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArgs A)
@@ -2268,7 +2608,7 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
             struct { void (*kernel)(SelArgs); size_t bytes; } limits[] = {{k_sel_round1, kSmemBytes}, {k_sel_round2, kSmemBytes},
-                {k_sel_solve1, kSolveBytes}, {k_sel_solve2, kRound3Bytes}, {k_sel_round3, kRound3Bytes}};
+                {k_sel_solve1, kSolveBytes}, {k_sel_solve2, kSolveBytes}, {k_sel_round3, kSolveBytes}};
             for (auto& l : limits) {
                 e = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes);
                 if (e != cudaSuccess) return e;
@@ -2286,21 +2626,23 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
     A.scheme = scheme; A.s = s; A.levels = d_levels; A.status = d_status;
     A.ws = sel_carve(d_ws, T, total);
     cudaError_t e = cudaSuccess;
-    auto run = [&](const char* name, void (*kernel)(SelArgs), int ctas, size_t smem) {
+    auto run = [&](const char* name, void (*kernel)(SelArgs), int ctas, size_t smem, int threads = kSelThreads) {
         if (e != cudaSuccess) return;
         launch_begin(name, stream);
-        e = launch_pdl(kernel, ctas, kSelThreads, smem, stream, A);
+        e = launch_pdl(kernel, ctas, threads, smem, stream, A);
         launch_end(stream);
     };
     const bool streams = total > kSmallN;  // some tensor may be larger than one CTA settles on its own
-    if (streams) run("k_sel_prepare", k_sel_prepare, T, 0);
-    run("k_sel_round1", k_sel_round1, T + (streams ? g.ctas : 0), kSmemBytes);
     if (streams) {
-        run("k_sel_solve1", k_sel_solve1, T, kSolveBytes);
-        run("k_sel_round2", k_sel_round2, g.ctas, kSmemBytes);
-        run("k_sel_solve2", k_sel_solve2, T, kRound3Bytes);
+        run("k_sel_prepare", k_sel_prepare, T, 0);
+        run("k_sel_round1", k_sel_round1, g.ctas, kSmemBytes);
     }
-    if (total > kAloneN) run("k_sel_round3", k_sel_round3, sm_count, kRound3Bytes);
+    run("k_sel_solve1", k_sel_solve1, T, kSolveBytes, kSolve1Threads);
+    if (streams) {
+        run("k_sel_round2", k_sel_round2, g.ctas, kSmemBytes);
+        run("k_sel_solve2", k_sel_solve2, T, kSolveBytes);
+    }
+    if (total > kAloneN) run("k_sel_round3", k_sel_round3, sm_count, kSolveBytes);
     return e;
 }
 
