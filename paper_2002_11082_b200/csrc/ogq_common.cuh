@@ -40,6 +40,17 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), int ctas, int threads, 
     return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
 }
 
+// The same for a kernel whose shared memory may exceed the default limit.
+template <class... Params, class... Args>
+inline cudaError_t launch_pdl_smem(void (*kernel)(Params...), int ctas, int threads, size_t smem, cudaStream_t stream, Args... args)
+{
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(kernel, ctas, threads, smem, stream, args...);
+}
+
 // ---------------------------------------------------------------------------
 // Flat partition of the bucket: CTA c owns elements [c*chunk, (c+1)*chunk).
 // ---------------------------------------------------------------------------
@@ -101,6 +112,35 @@ __device__ __forceinline__ void for_each_piece(const int64_t* __restrict__ off, 
         }
         if (pe >= te) ++t;
     }
+}
+
+// Partition of the bucket among the warps of a grid, in runs of whole units: warps that work on their own need no barrier
+// where a run crosses from one tensor to the next.  (With a chunk per CTA every tensor cost two barriers and a chain of
+// dependent loads of 1 to 1.5 us, several times in a row where small tensors follow one another.)
+struct WarpRun {
+    int64_t lo, hi;
+};
+struct WarpRuns {
+    int64_t total, each;  // elements; elements of a run, a multiple of unit
+    int extra, unit;      // the first `extra` runs are a unit longer
+    int ctas;
+};
+
+constexpr int kRunCtas = 4;  // CTAs of such a grid on an SM: one wave; fewer where there is less than a unit for every warp
+inline WarpRuns warp_runs(int64_t total, int unit, int sm_count)
+{
+    const int64_t units = (total + unit - 1) / unit, need = (units + kWarps - 1) / kWarps, most = (int64_t)sm_count * kRunCtas;
+    const int ctas = (int)(need < 1 ? 1 : need < most ? need : most);
+    const int64_t warps = (int64_t)ctas * kWarps;
+    return WarpRuns{total, units / warps * unit, (int)(units % warps), unit, ctas};
+}
+
+__device__ __forceinline__ WarpRun warp_run(const WarpRuns& r)
+{
+    const int me = (int)blockIdx.x * kWarps + (int)(threadIdx.x >> 5);
+    const int64_t lo = me * r.each + (int64_t)(me < r.extra ? me : r.extra) * r.unit;
+    const int64_t hi = lo + r.each + (me < r.extra ? r.unit : 0);
+    return WarpRun{lo, hi < r.total ? hi : r.total};
 }
 
 // Asks L2 to fetch `bytes` (a multiple of 16) from a 16-byte aligned global address.  One thread of

@@ -102,7 +102,12 @@ __device__ __forceinline__ uint32_t entry_after_rounding(float v, uint32_t rnd, 
         if constexpr (BITS >= 3) search_step<1>(a, v, st);
     }
     float lo, w;
-    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(w) : "r"(a));
+    if constexpr (BITS == 1) {  // the only entry: a load that the compiler may move, but not past a barrier
+        const float2 e = *static_cast<const float2*>(__cvta_shared_to_generic(tab));
+        lo = e.x; w = e.y;
+    } else {
+        asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lo), "=f"(w) : "r"(a));
+    }
     const float lhs = __fmul_rn((float)(rnd >> 8), w);
     const float rhs = __fsub_rn(v, lo);
     asm("{ .reg .pred p; setp.lt.f32 p, %1, %2; @p mad.lo.u32 %0, %3, %4, %0; }"
@@ -134,9 +139,10 @@ __device__ __forceinline__ uint32_t codes_of_entries(uint32_t a0, uint32_t a1, u
     return (a0 + (a1 << BITS) + (a2 << (2 * BITS)) + (a3 << (3 * BITS)) - base) >> 3;
 }
 
-// Stores the 4*BITS-bit chunks of a warp's 128 elements at `out` (4*BITS words).  Chunks of 8 and 16 bits are
-// stored by their lanes as bytes and half-words, pairs of 4-bit chunks as bytes; 12- and 20-bit chunks are
-// assembled to words first.
+// Stores the 4*BITS-bit chunks of a warp's 128 elements at `out` (4*BITS words), as bytes or half-words: lanes whose
+// chunks are whole bytes on their own, the others after one exchange with their neighbour (a pair's 4-bit chunks make
+// one byte, its 12-bit chunks three, its 20-bit chunks five).  L2 puts the bytes together; building words of
+// 12- and 20-bit chunks first took up to four shuffles.
 template <int BITS>
 __device__ __forceinline__ void store_chunks(uint32_t* out, uint32_t chunk, int lane)
 {
@@ -144,12 +150,19 @@ __device__ __forceinline__ void store_chunks(uint32_t* out, uint32_t chunk, int 
         reinterpret_cast<uint16_t*>(out)[lane] = (uint16_t)chunk;
     } else if constexpr (BITS == 2) {
         reinterpret_cast<uint8_t*>(out)[lane] = (uint8_t)chunk;
-    } else if constexpr (BITS == 1) {
-        const uint32_t other = __shfl_xor_sync(0xffffffffu, chunk, 1);
-        if ((lane & 1) == 0) reinterpret_cast<uint8_t*>(out)[lane >> 1] = (uint8_t)(chunk | other << 4);
     } else {
-        const uint32_t word = assemble_words<BITS>(chunk, lane);
-        if (packs_word<BITS>(lane)) out[packed_word<BITS>(lane)] = word;
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, chunk, 1);
+        const bool even = (lane & 1) == 0;
+        if constexpr (BITS == 1) {
+            if (even) reinterpret_cast<uint8_t*>(out)[lane >> 1] = (uint8_t)(chunk | other << 4);
+        } else {
+            constexpr int kEven = (BITS + 1) / 2;  // bytes of the even lane; the odd lane stores the others
+            uint8_t* p = reinterpret_cast<uint8_t*>(out) + BITS * (lane >> 1) + (even ? 0 : kEven);
+            const uint32_t v = even ? chunk | other << (4 * BITS) : chunk >> 4;
+            p[0] = (uint8_t)v;
+            if (BITS == 5) p[1] = (uint8_t)(v >> 8);
+            if (even) p[BITS / 2] = (uint8_t)(v >> (8 * (BITS / 2)));
+        }
     }
 }
 
