@@ -5,16 +5,24 @@
 // this is the closest whole-word format.  Quantization itself (segment search, Philox draw, rounding
 // decision) is the one of the bit-packed path: only the packing differs.
 //
-// Unit of work: a group of U = lcm(4, M) consecutive elements of a tensor, which is a whole number of
-// 128-bit loads and Philox blocks (U / 4) and of output words (U / M).  A lane takes one group per
-// trip, a warp 32 consecutive groups; a group belongs to the CTA whose chunk holds its first element.
+// Quantizer: a group of U = lcm(4, M) consecutive elements of a tensor is a whole number of 128-bit loads and
+// Philox blocks (U / 4) and of output words (U / M).  A warp takes a tile of 32 groups: it loads and codes them 128
+// elements at a time, as the bit-packed path does, leaves the codes as bytes in shared memory, and then every lane makes the
+// words of one group.  Server: a lane takes one word of every worker, a warp 32 consecutive words, and the
+// sums go through shared memory to whole-line stores.  Groups (four words) belong to the CTA whose chunk holds their
+// first element.
 #include <math.h>
+
+#include <type_traits>
 
 #include "ogq_common.cuh"
 #include "ogq_internal.h"
 #include "ogq_quant.cuh"
+#include "ogq_unpack.cuh"
 
 namespace ogq {
+
+constexpr int kDenseUnit = 256;  // elements: granularity of the warps' runs
 
 template <int S> struct Dense;
 template <> struct Dense<3>  { static constexpr int M = 20, U = 20, BITS = 2; };
@@ -40,82 +48,138 @@ int dense_digits(int s)
     }
 }
 
+// The words of one group from its codes, four per 32-bit word x[q] as bytes: sums of four (byte) or two (16-bit weights) products
+// at a time.
 template <int S>
-__global__ void __launch_bounds__(kThreads)
-k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, int64_t total,
-                      int64_t chunk, const float* __restrict__ levels, const __grid_constant__ PhiloxKeys keys,
-                      uint32_t stream_id, const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed, const __grid_constant__ QuantSteps steps)
+__device__ __forceinline__ void dense_words(const uint32_t (&x)[Dense<S>::U / 4], uint32_t (&word)[Dense<S>::U / Dense<S>::M])
+{
+    constexpr int M = Dense<S>::M, Q = Dense<S>::U / 4, W = Dense<S>::U / M;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        word[w] = 0u;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int e = 4 * q - w * M;  // digit of the first of the four codes; those outside [0, M) are another word's
+            if (e <= -4 || e >= M) continue;
+            const int first = e < 0 ? 0 : e;
+            uint32_t c[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c[j] = e + j >= first && e + j < M ? dense_pow(S, e + j - first) : 0u;
+            uint32_t four;
+            if constexpr (S <= 5) four = __dp4a(x[q], c[0] | c[1] << 8 | c[2] << 16 | c[3] << 24, 0u);
+            else four = __dp2a_lo(c[0] | c[1] << 16, x[q], __dp2a_hi(c[2] | c[3] << 16, x[q], 0u));
+            word[w] += four * dense_pow(S, first);
+        }
+    }
+}
+
+// What bounds it: instruction issue, as the bit-packed quantizer.  One lane per group, reading its U elements itself,
+// spread each load over 32 lines and took 86 us for 25.6 M elements at s = 5.
+template <int S>
+__global__ void __launch_bounds__(kThreads, 4)
+k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, const WarpRuns runs,
+                      const float* levels, const __grid_constant__ PhiloxKeys keys,
+                      uint32_t stream_id, const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed,
+                      const __grid_constant__ QuantSteps steps)
 {
     constexpr int M = Dense<S>::M, U = Dense<S>::U, BITS = Dense<S>::BITS, W = U / M, Q = U / 4;
-    __shared__ float sh_lv[kMaxLevels];
-    __shared__ float2 sh_tab[kMaxLevels];
+    __shared__ float2 sh_tables[kWarps][kMaxLevels];
+    __shared__ uint32_t sh_codes[kWarps][32 * Q];
+    pdl_wait();
+    pdl_launch_dependents();
 
-    const int64_t lo = (int64_t)blockIdx.x * chunk;
-    const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const WarpRun run = warp_run(runs);
+    const int lane = threadIdx.x & 31;
+    float2* sh_tab = sh_tables[threadIdx.x >> 5];
+    uint32_t* codes = sh_codes[threadIdx.x >> 5];
 
-    for_each_piece(off, T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
+    for_each_piece(off, T, run.lo, run.hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + U - 1) / U, g_end = (pe - tb + U - 1) / U;
         if (g_beg >= g_end) return;
-        __syncthreads();
         bool ok = true;
-        if (threadIdx.x < S) {
-            const float cur = __ldg(levels + (int64_t)t * S + threadIdx.x);
-            const float nxt = (int)threadIdx.x + 1 < S ? __ldg(levels + (int64_t)t * S + threadIdx.x + 1) : cur;
-            sh_lv[threadIdx.x] = cur;
-            sh_tab[threadIdx.x] = quant_table_entry(cur, nxt);
+        __syncwarp();
+        if (lane < S) {
+            const float cur = __ldcg(levels + (int64_t)t * S + lane);
+            const float nxt = lane + 1 < S ? __ldcg(levels + (int64_t)t * S + lane + 1) : cur;
+            sh_tab[lane] = quant_table_entry(cur, nxt);
             ok = quant_table_scales(cur, nxt);
         }
-        const bool scales = __syncthreads_and(ok);
+        __syncwarp();
+        const bool scales = __all_sync(0xffffffffu, ok);
         const int64_t region = __ldg(packed_off + t + 1) - __ldg(packed_off + t);
         uint32_t* out = packed + __ldg(packed_off + t);
         const float* base = grad + tb;
-        const bool aligned = (tb & 3) == 0;
 
         int64_t g_rest = g_beg;
-        if (aligned && scales && n <= ((int64_t)1 << 34)) {
+        if (scales && n <= ((int64_t)1 << 34)) {
             const int64_t g_full = (n / U) < g_end ? (n / U) : g_end;
             if (g_full > g_beg) {
                 g_rest = g_full;
                 const uint32_t tabaddr = (uint32_t)__cvta_generic_to_shared(sh_tab);
                 const float mid = sh_tab[1 << (BITS - 2)].x;
                 const PhiloxHoist hz = philox_hoist(0u, (uint32_t)t, stream_id, keys);
-                for (int64_t g = g_beg + (int64_t)warp * 32 + lane; g < g_full; g += (int64_t)kWarps * 32) {
-                    const float4* src = reinterpret_cast<const float4*>(base + g * U);
-                    float4 v[Q];
+                const int ng = (int)(g_full - g_beg);
+                const float* src = base + g_beg * U + 4 * lane;
+                const uint32_t c0_first = (uint32_t)(g_beg * Q) + (uint32_t)lane;
+                auto tile = [&](int g0, auto vec, auto all) {
+                    constexpr bool whole = decltype(all)::value;  // all 32 groups are there
+                    constexpr int B = 4;  // loads in flight
+                    const int quads = whole ? 32 * Q : (ng - g0) * Q;
+                    const float* p = src + (size_t)g0 * U;
 #pragma unroll
-                    for (int q = 0; q < Q; ++q) v[q] = __ldg(src + q);
-                    uint32_t word[W];
+                    for (int q0 = 0; q0 < Q; q0 += B) {
+                        float4 v[B];
 #pragma unroll
-                    for (int w = 0; w < W; ++w) word[w] = 0u;
-                    const uint32_t c0 = (uint32_t)(g * Q);
+                        for (int u = 0; u < B; ++u) {
+                            if (q0 + u < Q && (whole || (q0 + u) * 32 + lane < quads)) {
+                                const float* a = p + (q0 + u) * 128;
+                                if constexpr (decltype(vec)::value) v[u] = __ldg(reinterpret_cast<const float4*>(a));
+                                else v[u] = make_float4(__ldg(a), __ldg(a + 1), __ldg(a + 2), __ldg(a + 3));
+                            } else {
+                                v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+                        }
 #pragma unroll
-                    for (int q = 0; q < Q; ++q) {
-                        const uint4 r = philox4x32_10_tail(c0 + (uint32_t)q, hz, keys);
-                        const float x[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-                        const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int e = 4 * q + j;  // position in the group (compile time after unrolling)
-                            const uint32_t code = (entry_after_rounding<BITS>(x[j], rw[j], tabaddr, mid, steps) - tabaddr) >> 3;
-                            word[e / M] += code * dense_pow(S, e % M);
+                        for (int u = 0; u < B; ++u) {
+                            if (q0 + u >= Q) continue;
+                            const uint4 r = philox4x32_10_tail(c0_first + (uint32_t)(g0 * Q + (q0 + u) * 32), hz, keys);
+                            codes[(q0 + u) * 32 + lane] =
+                                codes_of_entries<8>(entry_after_rounding<BITS>(v[u].x, r.x, tabaddr, mid, steps),
+                                                    entry_after_rounding<BITS>(v[u].y, r.y, tabaddr, mid, steps),
+                                                    entry_after_rounding<BITS>(v[u].z, r.z, tabaddr, mid, steps),
+                                                    entry_after_rounding<BITS>(v[u].w, r.w, tabaddr, mid, steps), tabaddr);
                         }
                     }
-                    uint32_t* dst = out + g * W;
-                    if constexpr (W == 1) dst[0] = word[0];
-                    else if constexpr (W == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(word[0], word[1]);
-                    else *reinterpret_cast<uint4*>(dst) = make_uint4(word[0], word[1], word[2], word[3]);
-                }
+                    __syncwarp();
+                    uint32_t x[Q], word[W];
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) x[q] = codes[lane * Q + q];
+                    __syncwarp();
+                    dense_words<S>(x, word);
+                    if (whole || g0 + lane < ng) {
+                        uint32_t* dst = out + (g_beg + g0 + lane) * W;
+                        if constexpr (W == 1) dst[0] = word[0];
+                        else if constexpr (W == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(word[0], word[1]);
+                        else *reinterpret_cast<uint4*>(dst) = make_uint4(word[0], word[1], word[2], word[3]);
+                    }
+                };
+                auto stream = [&](auto vec) {
+                    int g0 = 0;
+                    for (; g0 + 32 <= ng; g0 += 32) tile(g0, vec, std::true_type());
+                    if (g0 < ng) tile(g0, vec, std::false_type());
+                };
+                if ((tb & 3) == 0) stream(std::true_type());
+                else stream(std::false_type());
             }
         }
 
-        // generic path: one thread per output word, element by element (the last, partial group;
-        // everything when the tensor does not start on a 16-byte boundary)
-        // (the CTA that owns the tensor's last group also writes the zero padding of the region)
+        // generic path: one lane per output word, element by element (the last, partial group; everything when
+        // the tensor's Philox counters do not fit 32 bits or its levels are outside the range of quant_table_scales)
+        // (the warp that owns the tensor's last group also writes the zero padding of the region)
         const int64_t w_beg = g_rest * W;
         const int64_t w_end = (g_end == (n + U - 1) / U) ? region : g_end * W;
-        for (int64_t wi = w_beg + threadIdx.x; wi < w_end; wi += kThreads) {
+        for (int64_t wi = w_beg + lane; wi < w_end; wi += 32) {
             uint32_t word = 0u, p = 1u;
             for (int d = 0; d < M; ++d) {
                 const int64_t i = wi * M + d;
@@ -124,7 +188,7 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
                     const uint64_t blk = (uint64_t)i >> 2;
                     const uint4 r = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)t, stream_id, keys);
                     const uint32_t rnd = (i & 3) == 0 ? r.x : ((i & 3) == 1 ? r.y : ((i & 3) == 2 ? r.z : r.w));
-                    word += code_as_written<BITS>(x, rnd, [&](int k) { return sh_lv[k]; }) * p;
+                    word += code_as_written<BITS>(x, rnd, [&](int k) { return sh_tab[k].x; }) * p;
                 }
                 p *= (uint32_t)S;
             }
@@ -133,94 +197,143 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
     });
 }
 
+// A word w as the fraction w / S^M, in units of 2^-32: multiplied by S, its integer part is the word's highest digit and
+// the rest the fraction of the remaining word, so every further digit is one wide multiplication.  Any
+// f in [w R, (w + 1) R), R = 2^32 / S^M, gives the right digits: no multiple of a power of S lies between the two ends.  w R
+// is taken as w floor(R) + w C / 2^32 + 1, rounded down, C / 2^32 the fraction of R: for S = 5 and 17, C rounded up is
+// good enough (R > 2); for 3^20 = 9^10, R = 1.23, and C needs its first binary place behind the point, too.
 template <int S>
-__global__ void __launch_bounds__(kThreads)
+__device__ __forceinline__ uint32_t dense_fraction(uint32_t w)
+{
+    if constexpr (S == 5) return __umulhi(w, 2226670858u) + 3u * w + 1u;
+    else if constexpr (S == 17) return __umulhi(w, 2005251564u) + 10u * w + 1u;
+    else return (uint32_t)(((uint64_t)w * 995507236u + ((w >> 1) + 1u)) >> 32) + w + 1u;
+}
+
+// acc[e] += the level of digit e of w.  row: shared address of the worker's levels.
+template <int S>
+__device__ __forceinline__ void add_digits(uint32_t w, uint32_t row, float (&acc)[Dense<S>::M])
+{
+    constexpr int M = Dense<S>::M;
+    uint32_t f = dense_fraction<S>(w);
+    float v[M];
+#pragma unroll
+    for (int e = M - 1; e >= 0; --e) {
+        asm("{ .reg .b64 p; .reg .b32 d; mul.wide.u32 p, %1, %2; mov.b64 {%1, d}, p; mad.lo.u32 d, d, 4, %3; ld.shared.f32 %0, [d]; }"
+            : "=f"(v[e]), "+r"(f) : "n"(S), "r"(row));
+    }
+#pragma unroll
+    for (int e = 0; e + 1 < M; e += 2) add2(acc[e], acc[e + 1], v[e], v[e + 1]);
+    if constexpr (M & 1) acc[M - 1] = __fadd_rn(acc[M - 1], v[M - 1]);
+}
+
+// What bounds it: shared-memory reads, one per element and worker, with the instructions for the digits close behind.
+// (One lane per group with divisions by S and stores of its own, each spread over 32 lines: 119 us for 25.6 M
+// elements of 8 workers at s = 5.)  Two digits at a time through a table of pairs were no faster: a 64-bit
+// read costs as much as two.
+template <int S>
+__global__ void __launch_bounds__(kThreads, 4)
 k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
                    const int64_t* __restrict__ off, const int64_t* __restrict__ packed_off, int T, int64_t total,
                    int64_t chunk, float scale, float* __restrict__ outp)
 {
-    constexpr int M = Dense<S>::M, U = Dense<S>::U, W = U / M, Q = U / 4;
-    __shared__ float sh_lv[kMaxWorkers][kMaxLevels + 1];
+    constexpr int M = Dense<S>::M, U = 4 * M;  // U: elements of a group here (whole 16-byte lines whatever M)
+    constexpr int kTile = 32 * M;              // elements of a tile
+    constexpr int kEdgeTiles = 4;              // tensors of no more tiles in this chunk go to one warp each
+    extern __shared__ __align__(16) float sh_sums[];  // [kWarps][kTile] sums, then [kWarps + 2][K][S] level rows
     __shared__ const uint32_t* sh_pk[kMaxWorkers];
+    __shared__ const float* sh_lv[kMaxWorkers];
+    pdl_wait();
+    pdl_launch_dependents();
 
     const int64_t lo = (int64_t)blockIdx.x * chunk;
     const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((int)threadIdx.x < K) {
+        sh_pk[threadIdx.x] = packed_k[threadIdx.x];
+        sh_lv[threadIdx.x] = levels_k[threadIdx.x];
+    }
+    __syncthreads();
+    float* sum = sh_sums + warp * kTile;
+    float* all_rows = sh_sums + kWarps * kTile;
+    int turn = 0;  // the warp that takes the next small tensor
+    int set = 0;   // of the two sets of rows of larger ones: a warp that is done with one may fill the other
 
     for_each_piece(off, T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + U - 1) / U, g_end = (pe - tb + U - 1) / U;
         if (g_beg >= g_end) return;
-        __syncthreads();
-        for (int i = threadIdx.x; i < K * 32; i += kThreads) {
-            const int k = i >> 5, q = i & 31;
-            sh_lv[k][q] = __ldg(levels_k[k] + (int64_t)t * S + (q < S ? q : S - 1));
-        }
         const int64_t pofs = __ldg(packed_off + t);
-        if (threadIdx.x < K) sh_pk[threadIdx.x] = packed_k[threadIdx.x] + pofs;
-        __syncthreads();
-        float* dst = outp + tb;
-        const bool aligned = (tb & 3) == 0;
+        const int64_t w_beg = g_beg * 4;
+        const int64_t w_all = (n + M - 1) / M, w_end = g_end * 4 < w_all ? g_end * 4 : w_all;
+        const int tiles = (int)((w_end - w_beg + 31) / 32);
+        const bool vec = (reinterpret_cast<uintptr_t>(outp + tb) & 15) == 0;
 
-        int64_t g_rest = g_beg;
-        if (aligned) {
-            const int64_t g_full = (n / U) < g_end ? (n / U) : g_end;
-            if (g_full > g_beg) {
-                g_rest = g_full;
-                for (int64_t g = g_beg + (int64_t)warp * 32 + lane; g < g_full; g += (int64_t)kWarps * 32) {
-                    float acc[U];
-#pragma unroll
-                    for (int e = 0; e < U; ++e) acc[e] = 0.f;
-                    for (int k = 0; k < K; ++k) {
-                        const uint32_t* src = sh_pk[k] + g * W;
-                        uint32_t word[W];
-                        if constexpr (W == 1) word[0] = __ldg(src);
-                        else if constexpr (W == 2) { const uint2 x = __ldg(reinterpret_cast<const uint2*>(src)); word[0] = x.x; word[1] = x.y; }
-                        else { const uint4 x = __ldg(reinterpret_cast<const uint4*>(src)); word[0] = x.x; word[1] = x.y; word[2] = x.z; word[3] = x.w; }
-                        const float* row = sh_lv[k];
-#pragma unroll
-                        for (int w = 0; w < W; ++w) {
-                            uint32_t rest = word[w];
-#pragma unroll
-                            for (int d = 0; d < M; ++d) {
-                                const uint32_t qd = rest / (uint32_t)S;  // constant divisor: multiply and shift
-                                const uint32_t digit = rest - qd * (uint32_t)S;
-                                rest = qd;
-                                acc[w * M + d] = __fadd_rn(acc[w * M + d], row[digit]);
-                            }
-                        }
-                    }
-                    float4* d4 = reinterpret_cast<float4*>(dst + g * U);
-#pragma unroll
-                    for (int q = 0; q < Q; ++q)
-                        d4[q] = make_float4(__fmul_rn(acc[4 * q], scale), __fmul_rn(acc[4 * q + 1], scale),
-                                            __fmul_rn(acc[4 * q + 2], scale), __fmul_rn(acc[4 * q + 3], scale));
-                }
-            }
+        const bool small = tiles <= kEdgeTiles;
+        float* rows = all_rows + (small ? warp : kWarps + set) * K * S;
+        if (small) {
+            turn = (turn + 1) & (kWarps - 1);
+            if (turn != warp) return;
+            __syncwarp();
+            for (int i = lane; i < K * S; i += 32) rows[i] = __ldcg(sh_lv[i / S] + (int64_t)t * S + i % S);
+            __syncwarp();
+        } else {
+            set ^= 1;
+            for (int i = threadIdx.x; i < K * S; i += kThreads) rows[i] = __ldcg(sh_lv[i / S] + (int64_t)t * S + i % S);
+            __syncthreads();
         }
-
-        // generic path: one thread per element
-        const int64_t e_beg = g_rest * U;
-        int64_t e_end = g_end * U;
-        if (e_end > n) e_end = n;
-        for (int64_t i = e_beg + threadIdx.x; i < e_end; i += kThreads) {
-            const int64_t wi = i / M;
-            const int d = (int)(i - wi * M);
-            float acc = 0.f;
-            for (int k = 0; k < K; ++k) {
-                uint32_t rest = __ldg(sh_pk[k] + wi);
-                for (int q = 0; q < d; ++q) rest /= (uint32_t)S;
-                acc = __fadd_rn(acc, sh_lv[k][rest % (uint32_t)S]);
+        const uint32_t rows_addr = (uint32_t)__cvta_generic_to_shared(rows);
+        const int first = small ? 0 : warp, step = small ? 1 : kWarps;
+        for (int i = first; i < tiles; i += step) {  // a word of every worker per lane
+            const int64_t w0 = w_beg + (int64_t)i * 32;
+            const bool have = w0 + lane < w_end;
+            const int64_t at = pofs + w0 + lane;
+            // every kAhead trips the first K threads ask L2 for the workers' words of the kAhead trips after the next kAhead
+            constexpr int kAhead = 8;
+            if (((i / kWarps) & (kAhead - 1)) == 0 && (int)threadIdx.x < K && i + 2 * kAhead * kWarps <= tiles - 1)
+                prefetch_l2(sh_pk[threadIdx.x] + pofs + w_beg + (int64_t)(i / kWarps + kAhead) * kWarps * 32, kAhead * kWarps * 128u);
+            float acc[M];
+#pragma unroll
+            for (int e = 0; e < M; ++e) acc[e] = 0.f;
+            constexpr int B = M == 20 ? 2 : 4;  // workers whose words are loaded before any is used
+            int k = 0;
+            for (; k + B <= K; k += B) {
+                uint32_t w[B];
+#pragma unroll
+                for (int u = 0; u < B; ++u) w[u] = have ? __ldcg(sh_pk[k + u] + at) : 0u;
+#pragma unroll
+                for (int u = 0; u < B; ++u) add_digits<S>(w[u], rows_addr + (k + u) * (S * 4), acc);
             }
-            dst[i] = __fmul_rn(acc, scale);
+            for (; k < K; ++k) add_digits<S>(have ? __ldcg(sh_pk[k] + at) : 0u, rows_addr + k * (S * 4), acc);
+#pragma unroll
+            for (int e = 0; e < M; ++e) acc[e] = __fmul_rn(acc[e], scale);
+            float* mine = sum + lane * M;  // no bank conflicts at any of these strides and widths
+            if constexpr (M % 4 == 0) {
+#pragma unroll
+                for (int e = 0; e < M; e += 4) *reinterpret_cast<float4*>(mine + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+            } else if constexpr (M % 2 == 0) {
+#pragma unroll
+                for (int e = 0; e < M; e += 2) *reinterpret_cast<float2*>(mine + e) = make_float2(acc[e], acc[e + 1]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < M; ++e) mine[e] = acc[e];
+            }
+            __syncwarp();
+            const int64_t e0 = w0 * M, left = (w_end * M < n ? w_end * M : n) - e0;
+            float* dst = outp + tb + e0;
+            if (vec && left >= kTile) {
+#pragma unroll
+                for (int e = 0; e < kTile; e += 128)
+                    if (e + 128 <= kTile || e + 4 * lane < kTile)
+                        *reinterpret_cast<float4*>(dst + e + 4 * lane) = *reinterpret_cast<const float4*>(sum + e + 4 * lane);
+            } else {
+#pragma unroll 4
+                for (int e = lane; e < kTile; e += 32)
+                    if (e < left) dst[e] = sum[e];
+            }
+            __syncwarp();
         }
     });
-}
-
-static int dense_flat_target(int sm_count)
-{
-    int t = sm_count * 8;
-    return t < kMaxFlatCtas ? t : kMaxFlatCtas;
 }
 
 cudaError_t launch_quantize_pack_dense(const float* d_grad, const int64_t* d_off, int T, int64_t total, int s,
@@ -228,12 +341,13 @@ cudaError_t launch_quantize_pack_dense(const float* d_grad, const int64_t* d_off
                                        const int64_t* d_packed_off, uint32_t* d_packed, int sm_count,
                                        cudaStream_t stream)
 {
-    FlatGrid g = make_flat_grid(total, dense_flat_target(sm_count), 16640);  // a multiple of every group length
+    const WarpRuns runs = warp_runs(total, kDenseUnit, sm_count);
     const PhiloxKeys keys = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
+    cudaError_t e = cudaErrorInvalidValue;
     launch_begin("k_quantize_pack_dense", stream);
 #define OGQ_LAUNCH_D(SS)                                                                                     \
-    k_quantize_pack_dense<SS><<<g.ctas, kThreads, 0, stream>>>(d_grad, d_off, T, total, g.chunk, d_levels,  \
-                                                               keys, stream_id, d_packed_off, d_packed, quant_steps())
+    e = launch_pdl(k_quantize_pack_dense<SS>, runs.ctas, kThreads, 0, stream, d_grad, d_off, T, runs, d_levels, \
+                   keys, stream_id, d_packed_off, d_packed, quant_steps())
     switch (s) {
         case 3: OGQ_LAUNCH_D(3); break;
         case 5: OGQ_LAUNCH_D(5); break;
@@ -243,18 +357,20 @@ cudaError_t launch_quantize_pack_dense(const float* d_grad, const int64_t* d_off
     }
 #undef OGQ_LAUNCH_D
     launch_end(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_unpack_sum_dense(const uint32_t* const* d_packed_k, const float* const* d_levels_k, int K,
                                     const int64_t* d_off, const int64_t* d_packed_off, int T, int64_t total, int s,
                                     float scale, float* d_out, int sm_count, cudaStream_t stream)
 {
-    FlatGrid g = make_flat_grid(total, dense_flat_target(sm_count), 16640);
+    const FlatGrid g = make_flat_grid(total, sm_count * kRunCtas, 4096);
+    cudaError_t e = cudaErrorInvalidValue;
     launch_begin("k_unpack_sum_dense", stream);
 #define OGQ_LAUNCH_UD(SS)                                                                                       \
-    k_unpack_sum_dense<SS><<<g.ctas, kThreads, 0, stream>>>(d_packed_k, d_levels_k, K, d_off, d_packed_off, T, \
-                                                            total, g.chunk, scale, d_out)
+    e = launch_pdl_smem(k_unpack_sum_dense<SS>, g.ctas, kThreads, \
+                        (kWarps * 32 * Dense<SS>::M + (kWarps + 2) * K * SS) * sizeof(float), stream, d_packed_k, d_levels_k, K, d_off, d_packed_off, T, \
+                   total, g.chunk, scale, d_out)
     switch (s) {
         case 3: OGQ_LAUNCH_UD(3); break;
         case 5: OGQ_LAUNCH_UD(5); break;
@@ -264,7 +380,7 @@ cudaError_t launch_unpack_sum_dense(const uint32_t* const* d_packed_k, const flo
     }
 #undef OGQ_LAUNCH_UD
     launch_end(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace ogq
