@@ -16,6 +16,7 @@
 #include "ogq_internal.h"
 #include "ogq_quant.cuh"
 #include "ogq_sort.cuh"
+#include "ogq_unpack.cuh"
 
 namespace ogq {
 
@@ -296,6 +297,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_bucket_encode(BktArgs A, size_t 
     constexpr int kTeams = WARP ? kBktWarpsPerCta : 1;
     __shared__ BktShared sh_team[kTeams];
     __shared__ TeamScratch<WARP> scratch;
+    pdl_wait();
+    pdl_launch_dependents();
     const int team = WARP ? (int)(threadIdx.x >> 5) : 0;
     const int P = KPT * (WARP ? 32 : (int)blockDim.x);
     const int step = (int)gridDim.x * kTeams;
@@ -310,73 +313,68 @@ __global__ void __launch_bounds__(MAXT, MINB) k_bucket_encode(BktArgs A, size_t 
 
 // Server step for fixed-length buckets: out[i] = scale * sum_k levels_k[i / d][code_k[i]].  Because d is
 // a multiple of 128, the packed codes of consecutive buckets form one contiguous bit stream (only the
-// last, shorter bucket is padded), so a warp takes 128 consecutive elements of the flat gradient at a
-// time and only has to fetch the level rows of the bucket they lie in.  Same additions in the same
-// (worker) order as ogq_unpack_sum with offsets j * d.
-constexpr int kDecWorkers = 8;  // workers per batch: their level rows and packed words are loaded before any is used
-
+// last, shorter bucket is padded).  A warp takes a run of consecutive groups of 256 elements, eight per lane, and keeps the
+// workers' level rows of the group's one or two buckets (two: lanes 16 ... 31 are in the second) in shared
+// memory until the bucket changes.  Same additions in the same (worker) order as ogq_unpack_sum with offsets j * d.
 template <int BITS>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_bucket_decode_sum(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
-                    int64_t total, int d, int s, int64_t total_words, float scale, float* __restrict__ outp)
+                    int64_t total, int d, int nb, int s, int64_t total_words, float scale, float* __restrict__ outp)
 {
-    __shared__ float sh_lv[kWarps][kDecWorkers][kMaxLevels];
+    extern __shared__ float sh_rows[];  // [kWarps][2][K][kRowStride]
     __shared__ const uint32_t* sh_pk[kMaxWorkers];
     __shared__ const float* sh_lp[kMaxWorkers];
+    constexpr int R = kRowStride<BITS>, kWords = 8 * BITS;
+    pdl_wait();
+    pdl_launch_dependents();
     for (int k = threadIdx.x; k < K; k += kThreads) { sh_pk[k] = packed_k[k]; sh_lp[k] = levels_k[k]; }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr uint32_t kMask4 = (BITS * 4 >= 32) ? 0xffffffffu : ((1u << (BITS * 4)) - 1u);
-    constexpr uint32_t kMask1 = (1u << BITS) - 1u;
-    const int64_t ngroups = (total + 127) >> 7;
-    for (int64_t g = (int64_t)blockIdx.x * kWarps + warp; g < ngroups; g += (int64_t)gridDim.x * kWarps) {
-        const int64_t i0 = (g << 7) + 4 * lane;
-        const int64_t j = (g << 7) / d;  // the bucket of this group
-        const int64_t bit = i0 * BITS;
-        const int64_t wi = bit >> 5;
-        const int sh = (int)(bit & 31);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int k0 = 0; k0 < K; k0 += kDecWorkers) {
-            const int kn = (K - k0 < kDecWorkers) ? K - k0 : kDecWorkers;
-            // all loads of the batch first (level rows: every code a BITS-bit field can hold gets an entry)
-            float row[kDecWorkers];
-            uint32_t w_lo[kDecWorkers], w_hi[kDecWorkers];
-            const bool straddle = sh + 4 * BITS > 32;
-#pragma unroll
-            for (int u = 0; u < kDecWorkers; ++u) {
-                row[u] = 0.f; w_lo[u] = 0u; w_hi[u] = 0u;
-                if (u < kn) {
-                    row[u] = __ldg(sh_lp[k0 + u] + j * s + (lane < s ? lane : s - 1));
-                    if (i0 < total) {
-                        const uint32_t* p = sh_pk[k0 + u];
-                        if (wi < total_words) w_lo[u] = __ldg(p + wi);
-                        if (straddle && wi + 1 < total_words) w_hi[u] = __ldg(p + wi + 1);
-                    }
-                }
+    const int64_t ngroups = (total + 255) >> 8, full = total >> 8;
+    const int64_t nw = (int64_t)gridDim.x * kWarps, me = (int64_t)blockIdx.x * kWarps + warp;
+    const int64_t g_beg = me * ngroups / nw, g_end = (me + 1) * ngroups / nw;
+    if (g_beg >= g_end) return;
+    float* rows = sh_rows + warp * 2 * K * R;
+    const int shift = (int)((reinterpret_cast<uintptr_t>(outp) >> 2) & 3);
+    int j = (int)((g_beg << 8) / d), at = (int)((g_beg << 8) - (int64_t)j * d);  // bucket of the group, first element in it
+    int j_rows = -1, two_rows = 0;                                               // buckets the rows are of
+    for (int64_t g = g_beg; g < g_end; ++g) {
+        const int two = at + 128 >= d && j + 1 < nb;
+        if (j != j_rows || two > two_rows) {
+            __syncwarp();
+            for (int i = lane; i < (K * R << two); i += 32) {
+                const int q = i % R, kk = i / R, second = kk >= K;
+                rows[i] = __ldcg(sh_lp[second ? kk - K : kk] + (int64_t)(j + second) * s + (q < s ? q : s - 1));
             }
             __syncwarp();
+            j_rows = j; two_rows = two;
+        }
+        const float* mine = rows + (two && lane >= 16 ? K * R : 0);
+        const int64_t w0 = g * kWords;
+        if (g < full) {
+            float a[1][8];
+            sum_workers<BITS, 1, false>(K, lane, nullptr, mine, [&](int k, int) { return sh_pk[k] + w0; }, a);
 #pragma unroll
-            for (int u = 0; u < kDecWorkers; ++u)
-                if (u < kn) sh_lv[warp][u][lane] = row[u];
-            __syncwarp();
+            for (int e = 0; e < 8; ++e) a[0][e] = __fmul_rn(a[0][e], scale);
+            store8(outp + (g << 8) + 8 * lane, shift, lane, a[0]);
+        } else {  // the last, partial group
+            const int64_t i0 = (g << 8) + 8 * lane, wi = (i0 * BITS) >> 5;
+            if (i0 < total) {
+                const int sh = (int)(i0 * BITS) & 31;
+                const bool more = sh + 8 * BITS > 32 && wi + 1 < total_words;
+                float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int k = 0; k < K; ++k) {
+                    const uint32_t lo = __ldcg(sh_pk[k] + wi), hi = more ? __ldcg(sh_pk[k] + wi + 1) : 0u;
+                    const uint64_t codes = ((uint64_t)hi << 32 | lo) >> sh;
 #pragma unroll
-            for (int u = 0; u < kDecWorkers; ++u) {
-                if (u < kn) {
-                    const uint32_t bits4 = __funnelshift_r(w_lo[u], w_hi[u], sh) & kMask4;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        acc[e] = __fadd_rn(acc[e], sh_lv[warp][u][(bits4 >> (e * BITS)) & kMask1]);
+                    for (int e = 0; e < 8; ++e) a[e] = __fadd_rn(a[e], mine[k * R + ((int)(codes >> (e * BITS)) & (R - 1))]);
                 }
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (i0 + e < total) outp[i0 + e] = __fmul_rn(a[e], scale);
             }
         }
-        if (i0 + 3 < total) {
-            *reinterpret_cast<float4*>(outp + i0) = make_float4(__fmul_rn(acc[0], scale), __fmul_rn(acc[1], scale),
-                                                                __fmul_rn(acc[2], scale), __fmul_rn(acc[3], scale));
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (i0 + e < total) outp[i0 + e] = __fmul_rn(acc[e], scale);
-        }
+        for (at += 256; at >= d; at -= d) ++j;
     }
 }
 
@@ -388,13 +386,20 @@ cudaError_t launch_bucket_decode_sum(const uint32_t* const* d_packed_k, const fl
     const int64_t nb = (total + d - 1) / d;
     const int64_t last = total - (nb - 1) * d;
     const int64_t total_words = (nb - 1) * ((int64_t)d * bits / 32) + ((last * bits + 31) / 32 + 3) / 4 * 4;
-    const int64_t ngroups = (total + 127) >> 7;
+    const int64_t ngroups = (total + 255) >> 8;
     int64_t ctas = (ngroups + kWarps - 1) / kWarps;
-    if (ctas > (int64_t)sm_count * 8) ctas = (int64_t)sm_count * 8;
+    if (ctas > (int64_t)sm_count * 4) ctas = (int64_t)sm_count * 4;
+    const size_t rows = (size_t)kWarps * 2 * K * (sizeof(float) << bits);
+    cudaError_t e = cudaSuccess;
     launch_begin("k_bucket_decode_sum", stream);
 #define OGQ_LAUNCH_BD(B)                                                                                        \
-    k_bucket_decode_sum<B><<<(int)ctas, kThreads, 0, stream>>>(d_packed_k, d_levels_k, K, total, d, s, total_words, \
-                                                               scale, d_out)
+    do {                                                                                                        \
+        if (rows > 40 * 1024)                                                                                   \
+            e = cudaFuncSetAttribute(k_bucket_decode_sum<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); \
+        if (e == cudaSuccess)                                                                                   \
+            e = launch_pdl(k_bucket_decode_sum<B>, (int)ctas, kThreads, rows, stream, d_packed_k, d_levels_k, K, total, d, \
+                           (int)nb, s, total_words, scale, d_out);                                              \
+    } while (0)
     switch (bits) {
         case 1: OGQ_LAUNCH_BD(1); break;
         case 2: OGQ_LAUNCH_BD(2); break;
@@ -405,7 +410,7 @@ cudaError_t launch_bucket_decode_sum(const uint32_t* const* d_packed_k, const fl
     }
 #undef OGQ_LAUNCH_BD
     launch_end(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 static int bkt_pow2(int d)
@@ -455,9 +460,9 @@ static cudaError_t bkt_launch(const BktArgs& A, const PhiloxKeys& pk, int sm_cou
     const int64_t need = ((int64_t)A.nb + teams - 1) / teams;
     if (ctas > need) ctas = need;
     launch_begin("k_bucket_encode", stream);
-    kernel<<<(int)ctas, team_threads * teams, smem, stream>>>(A, team_bytes, pk);
+    e = launch_pdl(kernel, (int)ctas, team_threads * teams, smem, stream, A, team_bytes, pk);
     launch_end(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 // Values per thread: a bucket of up to 512 elements is one warp's (4, 8 or 16 per lane: its barriers are
