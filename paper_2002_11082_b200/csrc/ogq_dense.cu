@@ -22,8 +22,6 @@
 
 namespace ogq {
 
-constexpr int kDenseUnit = 256;  // elements: granularity of the warps' runs
-
 template <int S> struct Dense;
 template <> struct Dense<3>  { static constexpr int M = 20, U = 20, BITS = 2; };
 template <> struct Dense<5>  { static constexpr int M = 13, U = 52, BITS = 3; };
@@ -77,7 +75,7 @@ __device__ __forceinline__ void dense_words(const uint32_t (&x)[Dense<S>::U / 4]
 // spread each load over 32 lines and took 86 us for 25.6 M elements at s = 5.
 template <int S>
 __global__ void __launch_bounds__(kThreads, 4)
-k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, const WarpRuns runs,
+k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, int64_t total, int64_t chunk,
                       const float* levels, const __grid_constant__ PhiloxKeys keys,
                       uint32_t stream_id, const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed,
                       const __grid_constant__ QuantSteps steps)
@@ -88,15 +86,24 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
     pdl_wait();
     pdl_launch_dependents();
 
-    const WarpRun run = warp_run(runs);
-    const int lane = threadIdx.x & 31;
-    float2* sh_tab = sh_tables[threadIdx.x >> 5];
-    uint32_t* codes = sh_codes[threadIdx.x >> 5];
+    const int64_t lo = (int64_t)blockIdx.x * chunk;
+    const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float2* sh_tab = sh_tables[warp];
+    uint32_t* codes = sh_codes[warp];
+    int turn = 0;  // the warp that takes the first tile of the next piece
 
-    for_each_piece(off, T, run.lo, run.hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
+    for_each_piece(off, T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + U - 1) / U, g_end = (pe - tb + U - 1) / U;
         if (g_beg >= g_end) return;
+        const int64_t g_full = (n / U) < g_end ? (n / U) : g_end;  // groups wholly inside the tensor
+        const int ng = (int)(g_full - g_beg);
+        // the warps take tiles in turn, the words of a partial group or of the padding count as one more; no barriers
+        const bool last = g_end == (n + U - 1) / U;
+        const int tiles = (ng + 31) / 32, all = tiles + (last ? 1 : 0), first = (warp - turn) & (kWarps - 1);
+        turn = (turn + all) & (kWarps - 1);
+        if (first >= all) return;
         bool ok = true;
         __syncwarp();
         if (lane < S) {
@@ -111,15 +118,13 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
         uint32_t* out = packed + __ldg(packed_off + t);
         const float* base = grad + tb;
 
-        int64_t g_rest = g_beg;
+        int i_rest = first;
         if (scales && n <= ((int64_t)1 << 34)) {
-            const int64_t g_full = (n / U) < g_end ? (n / U) : g_end;
-            if (g_full > g_beg) {
-                g_rest = g_full;
+            if (first < tiles) {
+                i_rest = first + (tiles - first + kWarps - 1) / kWarps * kWarps;  // this warp's first tile that is not done
                 const uint32_t tabaddr = (uint32_t)__cvta_generic_to_shared(sh_tab);
                 const float mid = sh_tab[1 << (BITS - 2)].x;
                 const PhiloxHoist hz = philox_hoist(0u, (uint32_t)t, stream_id, keys);
-                const int ng = (int)(g_full - g_beg);
                 const float* src = base + g_beg * U + 4 * lane;
                 const uint32_t c0_first = (uint32_t)(g_beg * Q) + (uint32_t)lane;
                 auto tile = [&](int g0, auto vec, auto all) {
@@ -165,8 +170,8 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
                     }
                 };
                 auto stream = [&](auto vec) {
-                    int g0 = 0;
-                    for (; g0 + 32 <= ng; g0 += 32) tile(g0, vec, std::true_type());
+                    int g0 = first * 32;
+                    for (; g0 + 32 <= ng; g0 += kWarps * 32) tile(g0, vec, std::true_type());
                     if (g0 < ng) tile(g0, vec, std::false_type());
                 };
                 if ((tb & 3) == 0) stream(std::true_type());
@@ -176,10 +181,11 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
 
         // generic path: one lane per output word, element by element (the last, partial group; everything when
         // the tensor's Philox counters do not fit 32 bits or its levels are outside the range of quant_table_scales)
-        // (the warp that owns the tensor's last group also writes the zero padding of the region)
-        const int64_t w_beg = g_rest * W;
-        const int64_t w_end = (g_end == (n + U - 1) / U) ? region : g_end * W;
-        for (int64_t wi = w_beg + lane; wi < w_end; wi += 32) {
+        // (the warp that takes the last tile also writes the zero padding of the region)
+        for (; i_rest < all; i_rest += kWarps) {
+          const int64_t w_beg = (i_rest < tiles ? g_beg + (int64_t)i_rest * 32 : g_full) * W;
+          const int64_t w_end = i_rest >= tiles ? region : (i_rest * 32 + 32 < ng ? w_beg + 32 * W : g_full * W);
+          for (int64_t wi = w_beg + lane; wi < w_end; wi += 32) {
             uint32_t word = 0u, p = 1u;
             for (int d = 0; d < M; ++d) {
                 const int64_t i = wi * M + d;
@@ -193,6 +199,7 @@ k_quantize_pack_dense(const float* __restrict__ grad, const int64_t* __restrict_
                 p *= (uint32_t)S;
             }
             out[wi] = word;
+          }
         }
     });
 }
@@ -341,12 +348,12 @@ cudaError_t launch_quantize_pack_dense(const float* d_grad, const int64_t* d_off
                                        const int64_t* d_packed_off, uint32_t* d_packed, int sm_count,
                                        cudaStream_t stream)
 {
-    const WarpRuns runs = warp_runs(total, kDenseUnit, sm_count);
+    const FlatGrid g = make_flat_grid(total, sm_count * kRunCtas, 4096);
     const PhiloxKeys keys = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     cudaError_t e = cudaErrorInvalidValue;
     launch_begin("k_quantize_pack_dense", stream);
 #define OGQ_LAUNCH_D(SS)                                                                                     \
-    e = launch_pdl(k_quantize_pack_dense<SS>, runs.ctas, kThreads, 0, stream, d_grad, d_off, T, runs, d_levels, \
+    e = launch_pdl(k_quantize_pack_dense<SS>, g.ctas, kThreads, 0, stream, d_grad, d_off, T, total, g.chunk, d_levels, \
                    keys, stream_id, d_packed_off, d_packed, quant_steps())
     switch (s) {
         case 3: OGQ_LAUNCH_D(3); break;
