@@ -35,7 +35,7 @@ struct BbArgs {
 // clamped to [-tau, tau].
 template <bool CLIP>
 __device__ __forceinline__ PartSum bb_split(const float* __restrict__ grad, int64_t pb, int64_t pe, float b0, float tau,
-                                            double* sh_d, long long* sh_l)
+                                            double* sh_d, long long* sh_l, bool down = false)
 {
     PartSum r = {0.0, 0.0, 0, 0};
     int below = 0;
@@ -46,7 +46,7 @@ __device__ __forceinline__ PartSum bb_split(const float* __restrict__ grad, int6
         r.s_lo += b ? d : 0.0;
         r.s_hi += b ? 0.0 : d;
         below += b ? 1 : 0;
-    });
+    }, down);
     r.s_lo = block_sum(r.s_lo, sh_d);
     r.s_hi = block_sum(r.s_hi, sh_d);
     r.c_lo = block_sum((long long)below, sh_l);
@@ -158,16 +158,17 @@ __global__ void __launch_bounds__(kThreads) k_bb_pass(BbArgs A, int flat_ctas, i
 
     const int64_t lo = (int64_t)blockIdx.x * A.chunk;
     const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
+    const bool down = ((pass & 1) != 0) != CLIP;  // the passes go up and down in turn, after the clipping threshold's upward one
     for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         if (te - tb <= kSoloN || (pass > 0 && __ldcg(A.ws.done + t))) return;
         const float b0 = pass == 0 ? -INFINITY : __ldcg(A.thresh + t);
-        const PartSum a = bb_split<CLIP>(A.grad, pb, pe, b0, CLIP ? __ldcg(A.tau + t) : 0.f, sh_d, sh_l);
+        const PartSum a = bb_split<CLIP>(A.grad, pb, pe, b0, CLIP ? __ldcg(A.tau + t) : 0.f, sh_d, sh_l, down);
         if (threadIdx.x == 0) {
             BbPart p;
             p.s_lo = a.s_lo; p.s_hi = a.s_hi; p.c_lo = a.c_lo; p.c_hi = a.c_hi;
             *part_slot(A.ws, t, tb, te, A.chunk) = p;
         }
-    });
+    }, down);
 }
 
 // One CTA per tensor: adds up the partial sums of the pass before.

@@ -1,9 +1,10 @@
 // Quantize + bit-pack, and unpack + dequantize + sum over K workers.
 //
-// Inside a tensor the unit of work is a group of 128 (quantizer) or 256 (server) consecutive elements (tensor-relative),
-// which fills a whole number of words.  The quantizer gives every warp a run of consecutive elements of the flat
-// bucket, the server step every CTA a chunk; a group belongs to the run or chunk that holds its first element, so no
-// two warps ever touch the same word.  Quantizer: lane l handles elements 4l..4l+3 (one 128-bit load, one Philox block).
+// Both kernels give every CTA a chunk of the flat bucket.  Inside a tensor the unit of work is a group of 128
+// (quantizer) or 256 (server) consecutive elements (tensor-relative), which fills a whole number of words; a group belongs
+// to the CTA whose chunk holds its first element, so no two ever touch the same word.  Quantizer: lane l
+// handles elements 4l..4l+3 (one 128-bit load, one Philox block).  (Runs and level tables of their own for the warps, without
+// barriers, were 2 us faster where many small tensors follow one another and 8 to 12 % slower in tensors of 100 M elements.)
 #include <math.h>
 
 #include <type_traits>
@@ -18,21 +19,22 @@ namespace ogq {
 // CLIP: every value is first clamped to [-tau_arr[t], tau_arr[t]] (gradient clipping).
 template <int BITS, bool THRESHOLD, bool CLIP>
 __global__ void __launch_bounds__(kThreads, 4)
-k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, const WarpRuns runs,
-                int s, const float* levels, const float* thresh, const float* tau_arr,
+k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, int64_t total,
+                int64_t chunk, int s, const float* levels, const float* thresh, const float* tau_arr,
                 const __grid_constant__ PhiloxKeys keys, uint32_t stream_id,
                 const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed, const __grid_constant__ QuantSteps steps)
 {
-    __shared__ float2 sh_tables[kWarps][kMaxLevels];
+    __shared__ float sh_lv[kMaxLevels];
+    __shared__ float2 sh_tab[kMaxLevels];
     pdl_wait();
     pdl_launch_dependents();
 
-    const WarpRun run = warp_run(runs);
-    const int lane = threadIdx.x & 31;
-    float2* sh_tab = sh_tables[threadIdx.x >> 5];
+    const int64_t lo = (int64_t)blockIdx.x * chunk;
+    const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWords = 4 * BITS;  // words of a group
 
-    for_each_piece(off, T, run.lo, run.hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
+    for_each_piece(off, T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + 127) >> 7, g_end = (pe - tb + 127) >> 7;
         if (g_beg >= g_end) return;
@@ -43,16 +45,16 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
         if (THRESHOLD) {
             b0 = __ldcg(thresh + t);
         } else {
+            __syncthreads();
             bool ok = true;
-            __syncwarp();
-            if (lane < s) {
-                const float cur = __ldcg(levels + (int64_t)t * s + lane);
-                const float nxt = lane + 1 < s ? __ldcg(levels + (int64_t)t * s + lane + 1) : cur;
-                sh_tab[lane] = quant_table_entry(cur, nxt);
+            if (threadIdx.x < s) {
+                const float cur = __ldcg(levels + (int64_t)t * s + threadIdx.x);
+                const float nxt = (int)threadIdx.x + 1 < s ? __ldcg(levels + (int64_t)t * s + threadIdx.x + 1) : cur;
+                sh_lv[threadIdx.x] = cur;
+                sh_tab[threadIdx.x] = quant_table_entry(cur, nxt);
                 ok = quant_table_scales(cur, nxt);
             }
-            __syncwarp();
-            scales = __all_sync(0xffffffffu, ok);
+            scales = __syncthreads_and(ok);
         }
         const int64_t region = __ldg(packed_off + t + 1) - __ldg(packed_off + t);
         uint32_t* out = packed + __ldg(packed_off + t);
@@ -100,26 +102,29 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
                         if constexpr (decltype(vec)::value) return __ldg(reinterpret_cast<const float4*>(p));
                         else return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
                     };
-                    int gl = 0;
-                    for (; gl + kU <= ng; gl += kU) {
-                        // L2 is asked for the block (kU groups, 512 bytes each) two trips ahead: the random-rounding
+                    const int rest = ng - warp - (kU - 1) * kWarps - 1;
+                    const int trips = rest >= 0 ? rest / (kU * kWarps) + 1 : 0;
+                    constexpr int kStep = CLIP ? -kU * kWarps : kU * kWarps;
+                    int gl = warp + (CLIP ? (trips - 1) * kU * kWarps : 0);
+                    for (int k = 0; k < trips; ++k, gl += kStep) {
+                        // L2 is asked for the block (kU kWarps groups, 512 bytes each) two trips ahead: the random-rounding
                         // variants compute long enough between their loads for it to pay
-                        if (!THRESHOLD && lane == 0 && gl + 3 * kU <= ng)
-                            prefetch_l2(src - (tb & 3) + (size_t)(gl + 2 * kU) * 128, kU * 512u);
+                        if (!THRESHOLD && threadIdx.x == 0 && (CLIP ? k + 2 < trips : gl + 3 * kU * kWarps <= ng))
+                            prefetch_l2(src - (tb & 3) + (int64_t)(gl + 2 * kStep) * 128, kU * kWarps * 512u);
                         float4 v[kU];
 #pragma unroll
-                        for (int u = 0; u < kU; ++u) v[u] = load4(gl + u);
+                        for (int u = 0; u < kU; ++u) v[u] = load4(gl + u * kWarps);
 #pragma unroll
-                        for (int u = 0; u < kU; ++u) code4(v[u], gl + u);
+                        for (int u = 0; u < kU; ++u) code4(v[u], gl + u * kWarps);
                     }
-                    for (; gl < ng; ++gl) code4(load4(gl), gl);
+                    for (gl = warp + trips * kU * kWarps; gl < ng; gl += kWarps) code4(load4(gl), gl);
                 };
                 if (aligned) stream(std::true_type());
                 else stream(std::false_type());
             }
         }
 
-        for (int64_t g = g_rest; g < g_end; ++g) {
+        for (int64_t g = g_rest + warp; g < g_end; g += kWarps) {
             const int64_t i0 = (g << 7) + 4 * lane;
             float x[4];
             if (aligned && i0 + 3 < n) {
@@ -142,7 +147,7 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
                 const uint4 r = philox4x32_10((uint32_t)q, (uint32_t)(q >> 32), (uint32_t)t, stream_id, keys);
                 const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) c[j] = code_as_written<BITS>(x[j], rw[j], [&](int k) { return sh_tab[k].x; });
+                for (int j = 0; j < 4; ++j) c[j] = code_as_written<BITS>(x[j], rw[j], [&](int k) { return sh_lv[k]; });
             }
             if (i0 + 3 >= n) {
 #pragma unroll
@@ -153,7 +158,7 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
             const int64_t widx = g * kWords + packed_word<BITS>(lane);
             if (packs_word<BITS>(lane) && widx < region) out[widx] = word;
         }
-    });
+    }, CLIP);  // clipped: the threshold's pass went up, the solver's two down and up
 }
 
 // Server step.  A CTA takes a chunk of the flat bucket, its warps the groups in turn: with a run of its own for every warp
@@ -163,7 +168,7 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
 // warp each, without a barrier, and read their levels from global memory: 0.6 us of set-up a tensor is what the
 // smallest ones took longest for.
 template <int BITS>
-__global__ void __launch_bounds__(kThreads, kRunCtas)
+__global__ void __launch_bounds__(kThreads, kStreamCtas)
 k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
              const int64_t* __restrict__ off, const int64_t* __restrict__ packed_off, int T, int64_t total,
              int64_t chunk, int s, float scale, float* __restrict__ outp)
@@ -265,12 +270,15 @@ cudaError_t launch_quantize_pack(const float* d_grad, const int64_t* d_off, int 
                                  const int64_t* d_packed_off, uint32_t* d_packed, int sm_count,
                                  cudaStream_t stream)
 {
-    const WarpRuns runs = warp_runs(total, 128, sm_count);
+    // One wave for the threshold quantizer, whose CTAs then begin where a pass over the same chunks left the data in L2 (97 -> 91 us
+    // for 143.7 M elements); three waves for the random ones, which are bound by instruction issue and gain more from
+    // an even finish (203, 195, 191, 193, 196 us with one, two, three, four, eight).
+    const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas * (scheme == OGQ_BINGRAD_B ? 1 : 3), 8192);
     const PhiloxKeys keys = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     const int bits = ogq_bits_for_levels(s);
     cudaError_t e = cudaErrorInvalidValue;
 #define OGQ_LAUNCH_QC(B, TH, CL)                                                                        \
-    e = launch_pdl(k_quantize_pack<B, TH, CL>, runs.ctas, kThreads, 0, stream, d_grad, d_off, T, runs, s, \
+    e = launch_pdl(k_quantize_pack<B, TH, CL>, g.ctas, kThreads, 0, stream, d_grad, d_off, T, total, g.chunk, s, \
                    d_levels, d_thresh, d_tau, keys, stream_id, d_packed_off, d_packed, quant_steps())
 #define OGQ_LAUNCH_Q(B, TH)                    \
     do {                                       \
@@ -300,7 +308,7 @@ cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* co
                               const int64_t* d_off, const int64_t* d_packed_off, int T, int64_t total,
                               int s, float scale, float* d_out, int sm_count, cudaStream_t stream)
 {
-    const FlatGrid g = make_flat_grid(total, sm_count * kRunCtas, 4096);
+    const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas, 4096);
     const int bits = ogq_bits_for_levels(s);
     cudaError_t e = cudaErrorInvalidValue;
 #define OGQ_LAUNCH_U(B)                                                                               \

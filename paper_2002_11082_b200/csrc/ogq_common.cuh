@@ -95,12 +95,25 @@ __device__ __forceinline__ int find_tensor(const int64_t* __restrict__ off, int 
 }
 
 // Calls f(t, tensor_begin, tensor_end, piece_begin, piece_end) for every non-empty
-// intersection of the flat range [lo, hi) with a tensor, in ascending order.
+// intersection of the flat range [lo, hi) with a tensor, in ascending order, or in descending order
+// when `down`.
+//   The passes that one encode makes over the gradient go up and down in turn: what a pass read last is still in L2 when
+// the next one begins with it.  (All of them upwards, a bucket larger than L2 is fetched from DRAM in full by every one.)
 template <class F>
 __device__ __forceinline__ void for_each_piece(const int64_t* __restrict__ off, int T, int64_t lo,
-                                               int64_t hi, F f)
+                                               int64_t hi, F f, bool down = false)
 {
     if (lo >= hi || T <= 0) return;
+    if (down) {
+        int64_t pos = hi;
+        for (int t = find_tensor(off, T, hi - 1); t >= 0 && pos > lo; --t) {
+            const int64_t tb = __ldg(off + t), te = __ldg(off + t + 1);
+            const int64_t pb = tb > lo ? tb : lo, pe = te < pos ? te : pos;
+            if (pe > pb) f(t, tb, te, pb, pe);
+            pos = pb < pos ? pb : pos;
+        }
+        return;
+    }
     int t = find_tensor(off, T, lo);
     int64_t pos = lo;
     while (pos < hi && t < T) {
@@ -114,34 +127,7 @@ __device__ __forceinline__ void for_each_piece(const int64_t* __restrict__ off, 
     }
 }
 
-// Partition of the bucket among the warps of a grid, in runs of whole units: warps that work on their own need no barrier
-// where a run crosses from one tensor to the next.  (With a chunk per CTA every tensor cost two barriers and a chain of
-// dependent loads of 1 to 1.5 us, several times in a row where small tensors follow one another.)
-struct WarpRun {
-    int64_t lo, hi;
-};
-struct WarpRuns {
-    int64_t total, each;  // elements; elements of a run, a multiple of unit
-    int extra, unit;      // the first `extra` runs are a unit longer
-    int ctas;
-};
-
-constexpr int kRunCtas = 4;  // CTAs of such a grid on an SM: one wave; fewer where there is less than a unit for every warp
-inline WarpRuns warp_runs(int64_t total, int unit, int sm_count)
-{
-    const int64_t units = (total + unit - 1) / unit, need = (units + kWarps - 1) / kWarps, most = (int64_t)sm_count * kRunCtas;
-    const int ctas = (int)(need < 1 ? 1 : need < most ? need : most);
-    const int64_t warps = (int64_t)ctas * kWarps;
-    return WarpRuns{total, units / warps * unit, (int)(units % warps), unit, ctas};
-}
-
-__device__ __forceinline__ WarpRun warp_run(const WarpRuns& r)
-{
-    const int me = (int)blockIdx.x * kWarps + (int)(threadIdx.x >> 5);
-    const int64_t lo = me * r.each + (int64_t)(me < r.extra ? me : r.extra) * r.unit;
-    const int64_t hi = lo + r.each + (me < r.extra ? r.unit : 0);
-    return WarpRun{lo, hi < r.total ? hi : r.total};
-}
+constexpr int kStreamCtas = 4;  // CTAs per SM of the server step and the dense kernels: one wave, 64 registers a thread
 
 // Asks L2 to fetch `bytes` (a multiple of 16) from a 16-byte aligned global address.  One thread of
 // a CTA issues it for the block the CTA will read a couple of loop trips later: the loads then find
@@ -154,9 +140,9 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
 }
 
 // Block-cooperative visit of grad[pb, pe): 128-bit loads on the aligned body,
-// scalar loads on the ragged head and tail.  f(float) is called once per element.
+// scalar loads on the ragged head and tail; downwards when `down`.  f(float) is called once per element.
 template <class F>
-__device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int64_t pb, int64_t pe, F f)
+__device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int64_t pb, int64_t pe, F f, bool down = false)
 {
     int64_t a = (pb + 3) & ~(int64_t)3;
     if (a > pe) a = pe;
@@ -166,8 +152,11 @@ __device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int6
     if (tid < (int)(a - pb)) f(__ldg(grad + pb + tid));
     if (tid < (int)(pe - b)) f(__ldg(grad + b + tid));
     const float4* g4 = reinterpret_cast<const float4*>(grad);
-    int64_t i = (a >> 2) + tid, e = b >> 2;
-    for (; i + 3 * kThreads < e; i += 4 * kThreads) {
+    const int64_t first = (a >> 2) + tid, e = b >> 2;
+    const int64_t trips = first + 3 * kThreads < e ? (e - first - 3 * kThreads - 1) / (4 * kThreads) + 1 : 0;
+    const int64_t step = down ? -4 * kThreads : 4 * kThreads;
+    int64_t i = down ? first + (trips - 1) * 4 * kThreads : first;
+    for (int64_t k = 0; k < trips; ++k, i += step) {
         float4 x0 = __ldg(g4 + i);
         float4 x1 = __ldg(g4 + i + kThreads);
         float4 x2 = __ldg(g4 + i + 2 * kThreads);
@@ -177,7 +166,7 @@ __device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int6
         f(x2.x); f(x2.y); f(x2.z); f(x2.w);
         f(x3.x); f(x3.y); f(x3.z); f(x3.w);
     }
-    for (; i < e; i += kThreads) {
+    for (i = first + trips * 4 * kThreads; i < e; i += kThreads) {
         float4 x = __ldg(g4 + i);
         f(x.x); f(x.y); f(x.z); f(x.w);
     }

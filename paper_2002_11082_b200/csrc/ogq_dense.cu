@@ -348,7 +348,7 @@ cudaError_t launch_quantize_pack_dense(const float* d_grad, const int64_t* d_off
                                        const int64_t* d_packed_off, uint32_t* d_packed, int sm_count,
                                        cudaStream_t stream)
 {
-    const FlatGrid g = make_flat_grid(total, sm_count * kRunCtas, 4096);
+    const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas, 4096);
     const PhiloxKeys keys = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     cudaError_t e = cudaErrorInvalidValue;
     launch_begin("k_quantize_pack_dense", stream);
@@ -371,7 +371,7 @@ cudaError_t launch_unpack_sum_dense(const uint32_t* const* d_packed_k, const flo
                                     const int64_t* d_off, const int64_t* d_packed_off, int T, int64_t total, int s,
                                     float scale, float* d_out, int sm_count, cudaStream_t stream)
 {
-    const FlatGrid g = make_flat_grid(total, sm_count * kRunCtas, 4096);
+    const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas, 4096);
     cudaError_t e = cudaErrorInvalidValue;
     launch_begin("k_unpack_sum_dense", stream);
 #define OGQ_LAUNCH_UD(SS)                                                                                       \

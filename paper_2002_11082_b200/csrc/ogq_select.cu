@@ -525,21 +525,22 @@ __device__ __noinline__ void stream_round1(const float* __restrict__ grad, int64
     const int64_t first = a >> 2, e = b >> 2;
     const int64_t ntrips = (e - first) / (4 * kSelThreads);  // full trips: the same for every thread
     constexpr int kNp = MAG ? kPackedPerSign : kPackedCells;
-    const float4* src = g4 + first + tid;                                              // this thread's next load
-    const float4* pfp = g4 + first + (int64_t)kPrefetchTrips * 4 * kSelThreads;       // next block to ask L2 for
-    const float4* const pf_end = g4 + e - 4 * kSelThreads;
+    // upwards; downwards behind the clipping threshold's pass, which went up
+    constexpr int kStep = CLIP ? -4 * kSelThreads : 4 * kSelThreads;
+    const float4* src = g4 + first + tid + (CLIP ? (ntrips - 1) * 4 * kSelThreads : 0);  // this thread's next load
+    int64_t pf_left = ntrips - kPrefetchTrips;                                           // blocks L2 is still to be asked for
     for (int64_t t0 = 0; t0 < ntrips; t0 += kPackTrips) {
         const int nt = (int)((ntrips - t0 < kPackTrips) ? ntrips - t0 : kPackTrips);
         if (tid == 0) { sh_coarse = 0u; sh_total = 0u; }
         __syncthreads();
         const float4* const period = src;
         for (int tt = 0; tt < nt; ++tt) {
-            if (tid == 0 && pfp <= pf_end) prefetch_l2(pfp, kTripBytes);
-            pfp += 4 * kSelThreads;
+            if (tid == 0 && pf_left > 0) prefetch_l2(src + kPrefetchTrips * kStep, kTripBytes);
+            --pf_left;
             float4 x[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) x[u] = __ldg(src + u * kSelThreads);
-            src += 4 * kSelThreads;
+            src += kStep;
 #pragma unroll
             for (int u = 0; u < 4; ++u) f.template four<true>(x[u]);
         }
@@ -584,7 +585,7 @@ __device__ __noinline__ void stream_round1(const float* __restrict__ grad, int64
             for (int tt = 0; tt < nt; ++tt) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const float4 x = __ldg(period + (tt * 4 + u) * kSelThreads);
+                    const float4 x = __ldg(period + tt * kStep + u * kSelThreads);
                     const float vv[4] = {f.canon(x.x), f.canon(x.y), f.canon(x.z), f.canon(x.w)};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -730,7 +731,7 @@ template <bool CLIP>
 __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64_t pb, int64_t pe,
                                               bool magnitude_only, const Table& tb, uint32_t* cnt, uint32_t* lo,
                                               uint32_t* hi, uint32_t* stage, uint32_t* dst, int64_t cap,
-                                              unsigned long long* cursor, int* overflow, bool nohist, float tau)
+                                              unsigned long long* cursor, int* overflow, bool nohist, float tau, bool down)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ Round2Ctx ctx;
@@ -778,12 +779,16 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
     // hits in one go (nearly every trip has a hit in some lane, so the divergent parking code is
     // paid once per trip, not once per few values).  `fill` mirrors the stage's fill counter in a
     // register: it is the same in all lanes, so whether to drain first is a uniform decision.
-    int64_t pf = (a >> 2) + (int64_t)kPrefetchTrips * 4 * kSelThreads;
+    const int64_t rest = e - i0 - 3 * kSelThreads - 32;
+    const int64_t trips = rest >= 0 ? rest / (4 * kSelThreads) + 1 : 0, after = i0 + trips * 4 * kSelThreads;
+    const int64_t step = down ? -4 * kSelThreads : 4 * kSelThreads;
+    if (down) i0 += (trips - 1) * 4 * kSelThreads;
+    // blocks to ask for: thread 0's trips, but for one upwards that the CTA's last warps do not have
+    int64_t pf_left = trips - kPrefetchTrips - (!down && after > e ? 1 : 0);
     __syncwarp();
     int fill = *(volatile int*)&fills[warp];
-    for (; i0 + 3 * kSelThreads + 32 <= e; i0 += 4 * kSelThreads) {
-        if (threadIdx.x == 0 && pf + 4 * kSelThreads <= e) prefetch_l2(g4 + pf, kTripBytes);
-        pf += 4 * kSelThreads;
+    for (int64_t k = 0; k < trips; ++k, i0 += step) {
+        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(g4 + i0 + kPrefetchTrips * step, kTripBytes);
         float4 x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = __ldg(g4 + i0 + lane + u * kSelThreads);
@@ -814,6 +819,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
             hits &= 0xffu;
         }
     }
+    i0 = after;
     if (i0 < e) {
         check();  // the trips above may have left the stage nearly full
 #pragma unroll
@@ -1893,7 +1899,8 @@ struct SelArgs {
 // already built in tb): the values inside the intervals are copied to key buffer k (what fits the
 // tensor's region) and, unless copy_only, counted on the cells.
 __device__ __forceinline__ void grad_pass(const SelArgs& A, int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_,
-                                          int k, const Table& tb, uint32_t* hist, unsigned char* smem, bool copy_only)
+                                          int k, const Table& tb, uint32_t* hist, unsigned char* smem, bool copy_only,
+                                          bool down = false)
 {
     TState* st = A.ws.st + t;
     uint32_t* stage = reinterpret_cast<uint32_t*>(smem + kSmemHist) + (threadIdx.x >> 5) * kStageCap;
@@ -1902,10 +1909,10 @@ __device__ __forceinline__ void grad_pass(const SelArgs& A, int t, int64_t tbeg,
     const bool mag = A.scheme == OGQ_BINGRAD_PB;
     if (A.tau)
         stream_round2<true>(A.grad, pb_, pe_, mag, tb, hist, hist + kCells, hist + 2 * kCells, stage, dst, cap,
-                            &st->cursor[k], &st->overflow, copy_only, __ldcg(A.tau + t));
+                            &st->cursor[k], &st->overflow, copy_only, __ldcg(A.tau + t), down);
     else
         stream_round2<false>(A.grad, pb_, pe_, mag, tb, hist, hist + kCells, hist + 2 * kCells, stage, dst, cap,
-                             &st->cursor[k], &st->overflow, copy_only, 0.f);
+                             &st->cursor[k], &st->overflow, copy_only, 0.f, down);
 }
 
 // Continues the rounds of one tensor on a single CTA until it is finished (the working set is
@@ -2053,7 +2060,7 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArg
             atomicMax(&st->kmax, kmax);
             if (anynf) atomicOr(&st->nonfinite, 1u);
         }
-    });
+    }, A.tau != nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -2486,6 +2493,7 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
     // one sort), adds the cells to the tensor's global ones.
     const int64_t lo = (int64_t)blockIdx.x * A.chunk;
     const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
+    const bool down = A.tau == nullptr;  // against round 1's direction
     for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
         if (tend - tbeg <= kSmallN) return;
         TState* st = A.ws.st + t;
@@ -2497,10 +2505,10 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
         const bool copy_only = __ldcg(&st->compact_only) != 0;
         if (!copy_only) zero_hist(hist, tb.ncells);
         __syncthreads();
-        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, tb, hist, smem, copy_only);
+        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, tb, hist, smem, copy_only, down);
         __syncthreads();
         if (!copy_only) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
-    });
+    }, down);
 }
 
 // What follows round 2, one CTA per tensor: the sorting finish when round 2 only copied, else a solver pass;
