@@ -190,25 +190,6 @@ __device__ __forceinline__ Interval round1_interval(int hi_e, bool magnitude_onl
     return x;
 }
 
-// Round-1 cell of a value, computed directly (same layout as round1_intervals produces):
-// magnitude cells ascend with |v|; negative values mirror them below, non-negative ones above.
-__device__ __forceinline__ void round1_cell(uint32_t bits, int lo_e, bool magnitude_only, int& cell,
-                                            uint32_t& lowkey)
-{
-    const uint32_t mag = bits & 0x7fffffffu;
-    const uint32_t rel = mag - ((uint32_t)lo_e << 23);
-    const int e = (int)(mag >> 23);
-    const bool fine = rel < ((uint32_t)kSelW << 23);
-    const int mi = fine ? lo_e + (int)(rel >> (23 - kSelM)) : ((e < lo_e) ? e : e - kSelW + (kSelW << kSelM));
-    const uint32_t mask = fine ? ((1u << (23 - kSelM)) - 1u) : 0x7fffffu;
-    const uint32_t low = mag & mask;
-    if (magnitude_only) { cell = mi; lowkey = low; }
-    else if (bits >> 31) { cell = kRound1Mag - 1 - mi; lowkey = mask - low; }
-    else { cell = kRound1Mag + mi; lowkey = low; }
-}
-
-__device__ __forceinline__ uint32_t key_to_bits(uint32_t k) { return (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k; }
-
 __device__ __forceinline__ bool classify(const Table& tb, uint32_t key, int& cell, uint32_t& low, int& sh)
 {
     int idx = 0;
@@ -312,38 +293,6 @@ struct Stager {  // per-warp compaction stage
         if (fill > kStageCap - 128) flush();
     }
 };
-
-// Block-cooperative visit of grad[pb, pe) without warp collectives: 128-bit loads on the aligned
-// body (four in flight per thread), scalar loads on the ragged head and tail.
-template <class F>
-__device__ __forceinline__ void visit_plain(const float* __restrict__ grad, int64_t pb, int64_t pe, F f)
-{
-    int64_t a = (pb + 3) & ~(int64_t)3;
-    if (a > pe) a = pe;
-    int64_t b = pe & ~(int64_t)3;
-    if (b < a) b = a;
-    const int tid = threadIdx.x;
-    if (tid < (int)(a - pb)) f(__ldg(grad + pb + tid));
-    if (tid < (int)(pe - b)) f(__ldg(grad + b + tid));
-    const float4* g4 = reinterpret_cast<const float4*>(grad);
-    int64_t i = (a >> 2) + tid;
-    const int64_t e = b >> 2;
-    for (; i + 3 * kSelThreads < e; i += 4 * kSelThreads) {
-        const float4 x0 = __ldg(g4 + i);
-        const float4 x1 = __ldg(g4 + i + kSelThreads);
-        const float4 x2 = __ldg(g4 + i + 2 * kSelThreads);
-        const float4 x3 = __ldg(g4 + i + 3 * kSelThreads);
-        f(x0.x); f(x0.y); f(x0.z); f(x0.w);
-        f(x1.x); f(x1.y); f(x1.z); f(x1.w);
-        f(x2.x); f(x2.y); f(x2.z); f(x2.w);
-        f(x3.x); f(x3.y); f(x3.z); f(x3.w);
-    }
-    for (; i < e; i += kSelThreads) {
-        const float4 x = __ldg(g4 + i);
-        f(x.x); f(x.y); f(x.z); f(x.w);
-    }
-}
-
 
 __device__ __forceinline__ float min3f(float a, float b, float c)
 {
@@ -836,33 +785,26 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
     round2_drain(&tb, &ctx, stage, *(volatile int*)&fills[warp]);
 }
 
-// Streams one piece of a tensor's working set: histogram of the keys inside the intervals,
-// optional copy of those keys, and (round 1) min / max / non-finite tracking.
-template <bool FIRST, bool FROM_GRAD, bool COMPACT>
-__device__ __forceinline__ void stream_piece(const void* __restrict__ src, int64_t pb, int64_t pe,
-                                             bool magnitude_only, const Table& tb, uint32_t* cnt,
-                                             uint32_t* lo, uint32_t* hi, Stager& stg, uint32_t& kmin,
-                                             uint32_t& kmax, uint32_t& nonfinite, bool nohist = false)
+// Streams copied keys [pb, pe) of a tensor: counts those inside the intervals on the cells (unless nohist) and copies
+// them on.
+__device__ __forceinline__ void stream_piece(const uint32_t* __restrict__ src, int64_t pb, int64_t pe, const Table& tb,
+                                             uint32_t* cnt, uint32_t* lo, uint32_t* hi, Stager& stg, bool nohist)
 {
-    auto handle = [&](uint32_t key, uint32_t* kk, int& c) {
-        int cell, sh;
-        uint32_t low;
-        if (classify(tb, key, cell, low, sh)) {
-            if (!nohist) hist_add(cnt, lo, hi, cell, low);
-            if (COMPACT) kk[c++] = key;
-        }
-    };
-    static_assert(!FROM_GRAD && !FIRST, "fp32 input goes through stream_round1 / stream_round2");
-    {
-        warp_visit4<uint4, uint32_t>((const uint32_t*)src, pb, pe, [&](const uint32_t* x, int nv) {
-            uint32_t kk[4];
-            int c = 0;
+    warp_visit4<uint4, uint32_t>(src, pb, pe, [&](const uint32_t* x, int nv) {
+        uint32_t kk[4];
+        int c = 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (j < nv) handle(x[j], kk, c);
-            if (COMPACT) stg.append(kk, c);
-        });
-    }
+        for (int j = 0; j < 4; ++j) {
+            if (j >= nv) continue;
+            int cell, sh;
+            uint32_t low;
+            if (classify(tb, x[j], cell, low, sh)) {
+                if (!nohist) hist_add(cnt, lo, hi, cell, low);
+                kk[c++] = x[j];
+            }
+        }
+        stg.append(kk, c);
+    });
 }
 
 __device__ __forceinline__ void zero_hist(uint32_t* smem_hist, int ncells)
@@ -1944,9 +1886,7 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
             stg.dst = A.ws.buf[round & 1] + sel_region(tbeg);
             stg.cursor = &st->cursor[round & 1];
             stg.fill = 0;
-            uint32_t kmin = 0, kmax = 0, nf = 0;
-            stream_piece<false, false, true>(src, sel_region(tbeg), sel_region(tbeg) + cnt, false, tb, hist, hist + kCells,
-                                             hist + 2 * kCells, stg, kmin, kmax, nf, copy_only);
+            stream_piece(src, sel_region(tbeg), sel_region(tbeg) + cnt, tb, hist, hist + kCells, hist + 2 * kCells, stg, copy_only);
             stg.flush();
         }
         __syncthreads();
@@ -2577,9 +2517,7 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
             stg.dst = A.ws.buf[1] + sel_region(tbeg);
             stg.cursor = &st->cursor[1];
             stg.fill = 0;
-            uint32_t kmin = 0, kmax = 0, nf = 0;
-            stream_piece<false, false, true>(A.ws.buf[0], sel_region(tbeg) + pb_, sel_region(tbeg) + pe_, false, tb, hist,
-                                             hist + kCells, hist + 2 * kCells, stg, kmin, kmax, nf, copy_only);
+            stream_piece(A.ws.buf[0], sel_region(tbeg) + pb_, sel_region(tbeg) + pe_, tb, hist, hist + kCells, hist + 2 * kCells, stg, copy_only);
             stg.flush();
         }
         __syncthreads();

@@ -138,12 +138,6 @@ OGQ_HD int sel_slot_shift(const SolverView& v, int slot)
 
 OGQ_HD double sel_slot_vlo(const SolverView& v, int slot) { return (double)sel_key_to_float(sel_slot_kbase(v, slot)); }
 
-OGQ_HD double sel_slot_vhi(const SolverView& v, int slot)
-{
-    const int sh = sel_slot_shift(v, slot);
-    return (double)sel_key_to_float(sel_slot_kbase(v, slot) + ((sh > 0) ? ((1u << sh) - 1u) : 0u));
-}
-
 // First slot whose prefix count exceeds pos.
 OGQ_HD int sel_upper_bound(const SolverView& v, long long pos)
 {
@@ -182,81 +176,6 @@ struct LvInfo {
     int sa, sb;       // cell-slot range when not exact
     double vlo, vhi;  // value bounds of that range
 };
-
-OGQ_HD void sel_make_exact_from_slot(const SolverView& v, int slot, LvInfo& o)
-{
-    o.exact = 1;
-    o.key = sel_slot_kbase(v, slot);
-    o.val = (double)sel_key_to_float(o.key);
-    o.c_lt = v.cpre[slot];
-    o.c_le = v.cpre[slot + 1];
-    o.s_lt = v.spre[slot];
-    o.s_le = v.spre[slot + 1];
-    o.sa = o.sb = slot;
-    o.vlo = o.vhi = o.val;
-}
-
-OGQ_HD void sel_make_range(const SolverView& v, int sa, int sb, LvInfo& o)
-{
-    o.exact = 0;
-    o.sa = sa;
-    o.sb = sb;
-    o.vlo = sel_slot_vlo(v, sa);
-    o.vhi = sel_slot_vhi(v, sb);
-}
-
-// Ranks [pos_lo, pos_hi] that are certain to contain Q*(L, R) when L or R is only known to lie in a range of
-// cells.
-OGQ_HD void sel_orq_range(const SolverView& v, const LvInfo& L, const LvInfo& R, long long& pos_lo, long long& pos_hi)
-{
-    // prefix state right after L's part and right before R's part
-    const long long Cs = L.exact ? L.c_lt : (long long)v.cpre[L.sb + 1];
-    const double Ss = L.exact ? L.s_lt : v.spre[L.sb + 1];
-    const long long Ce = R.exact ? R.c_le : (long long)v.cpre[R.sa];
-    const double Se = R.exact ? R.s_le : v.spre[R.sa];
-    const double Llo = L.exact ? L.val : L.vlo, Lhi = L.exact ? L.val : L.vhi;
-    const double Rlo = R.exact ? R.val : R.vlo, Rhi = R.exact ? R.val : R.vhi;
-    const long long cntL = L.exact ? 0 : (long long)v.cpre[L.sb + 1] - (long long)v.cpre[L.sa];
-    const long long cntR = R.exact ? 0 : (long long)v.cpre[R.sb + 1] - (long long)v.cpre[R.sa];
-    const long long floor_pos = L.exact ? L.c_lt : (long long)v.cpre[L.sa];
-    const long long ceil_pos = (R.exact ? R.c_le : (long long)v.cpre[R.sb + 1]) - 1;
-    pos_lo = floor_pos;
-    pos_hi = ceil_pos;
-    // With M the elements strictly between L's cells and R's cells (count cntM, sum sumM, all of
-    // them inside [Lhi, Rlo]), T = [t_L + (sumM - L cntM) + t_R] / (R - L), where t_L and t_R are
-    // the contributions of the elements of L's and R's own cells.  f(L, R) = (sumM - L cntM)/(R - L)
-    // decreases in L and in R, so its extremes are taken at matching corners, which stays tight
-    // even when a bracket is only known to lie somewhere in a sparse stretch of cells.
-    const double den_lo = Rlo - Lhi;
-    const long long cntM = Ce - Cs;
-    if (cntM >= 0 && den_lo > 0.0) {
-        const double sumM = Se - Ss;
-        double num_lo = sumM - Lhi * (double)cntM, num_hi = sumM - Llo * (double)cntM;
-        if (num_lo < 0.0) num_lo = 0.0;
-        if (num_hi < 0.0) num_hi = 0.0;
-        const double mid_lo = num_lo / (Rhi - Lhi), mid_hi = num_hi / (Rlo - Llo);
-        const double eps_l = (double)cntL * (Lhi - Llo) / (Rlo - Llo);
-        const double eps_r = (double)cntR * (Rhi - Rlo) / (Rhi - Lhi);
-        const double g_lo = (double)Ce - eps_l - mid_hi;
-        const double g_hi = (double)Ce + eps_r - mid_lo;
-        const double delta = 2.0 + 1e-9 * (double)v.n;
-        const double p_lo = ceil(g_lo - delta) - 1.0, p_hi = ceil(g_hi + delta) - 1.0;
-        if (p_lo > (double)pos_lo) pos_lo = (long long)p_lo;
-        if (p_hi < (double)pos_hi) pos_hi = (long long)p_hi;
-        if (pos_lo > ceil_pos) pos_lo = ceil_pos;
-        if (pos_hi < floor_pos) pos_hi = floor_pos;
-        if (pos_lo > pos_hi) pos_lo = pos_hi;
-    }
-    if (pos_lo < 0) pos_lo = 0;
-    if (pos_hi > v.n - 1) pos_hi = v.n - 1;
-}
-
-OGQ_HD int sel_floor_log2(long long x)
-{
-    int r = 0;
-    while ((x >> (r + 1)) > 0) ++r;
-    return r;
-}
 
 // Turns open slot ranges into the intervals of the next round.
 //
