@@ -4,8 +4,8 @@ solvers, quantize + bit-pack, unpack + sum, behind a C ABI (``include/ogq.h``).
 This package is a thin binding over ``libogq.so`` (a C module for the data-path
 calls, ctypes for the helpers): it only marshals arguments (torch tensors supply
 device memory and streams); every step of the path runs in the library's CUDA
-kernels.  There is no CPU fallback: importing
-the binding fails if the library has not been built.
+kernels.  There is no CPU fallback: the first
+call fails if the library has not been built.
 """
 from .binding import (  # noqa: F401
     OGQ_BINGRAD_PB,

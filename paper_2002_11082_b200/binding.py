@@ -53,44 +53,12 @@ def lib() -> ctypes.CDLL:
         L.ogq_packed_layout.argtypes = [vp, i32, i32, vp]
         L.ogq_workspace_bytes.restype = sz
         L.ogq_workspace_bytes.argtypes = [i32, i64, i32]
-        L.ogq_levels_bingrad.restype = i32
-        L.ogq_levels_bingrad.argtypes = [vp, vp, i32, i64, i32, i32, vp, vp, vp, vp, sz, vp]
-        L.ogq_levels_bingrad_b_noalloc.restype = i32
-        L.ogq_levels_bingrad_b_noalloc.argtypes = [vp, vp, i32, i64, i32, vp, vp, vp, vp]
-        L.ogq_levels_orq.restype = i32
-        L.ogq_levels_orq.argtypes = [vp, vp, i32, i64, i32, vp, vp, vp, sz, vp]
-        L.ogq_quantize_pack.restype = i32
-        L.ogq_quantize_pack.argtypes = [vp, vp, i32, i64, i32, i32, vp, vp, ctypes.c_uint64, ctypes.c_uint32, vp, vp, vp]
-        L.ogq_unpack_sum.restype = i32
-        L.ogq_unpack_sum.argtypes = [vp, vp, i32, vp, vp, i32, i64, i32, ctypes.c_float, vp, vp]
         L.ogq_bucket_packed_words.restype = i64
         L.ogq_bucket_packed_words.argtypes = [i64, i32, i32]
-        L.ogq_bucket_encode.restype = i32
-        L.ogq_bucket_encode.argtypes = [vp, i64, i32, i32, i32, i32, ctypes.c_float, ctypes.c_uint64, ctypes.c_uint32,
-                                        vp, vp, vp, vp, vp]
-        L.ogq_clip_threshold.restype = i32
-        L.ogq_clip_threshold.argtypes = [vp, vp, i32, i64, ctypes.c_float, vp, vp, vp, sz, vp]
-        L.ogq_levels_orq_clipped.restype = i32
-        L.ogq_levels_orq_clipped.argtypes = [vp, vp, i32, i64, i32, vp, vp, vp, vp, sz, vp]
-        L.ogq_quant_error.restype = i32
-        L.ogq_quant_error.argtypes = [vp, vp, i32, i64, i32, vp, vp, vp, vp, vp]
-        L.ogq_expected_error.restype = i32
-        L.ogq_expected_error.argtypes = [vp, vp, i32, i64, i32, vp, vp, vp]
         L.ogq_dense_digits.restype = i32
         L.ogq_dense_digits.argtypes = [i32]
         L.ogq_dense_layout.restype = i32
         L.ogq_dense_layout.argtypes = [vp, i32, i32, vp]
-        L.ogq_quantize_pack_dense.restype = i32
-        L.ogq_quantize_pack_dense.argtypes = [vp, vp, i32, i64, i32, vp, ctypes.c_uint64, ctypes.c_uint32, vp, vp, vp]
-        L.ogq_unpack_sum_dense.restype = i32
-        L.ogq_unpack_sum_dense.argtypes = [vp, vp, i32, vp, vp, i32, i64, i32, ctypes.c_float, vp, vp]
-        L.ogq_quantize_pack_clipped.restype = i32
-        L.ogq_quantize_pack_clipped.argtypes = [vp, vp, i32, i64, i32, i32, vp, vp, vp, ctypes.c_uint64, ctypes.c_uint32,
-                                                vp, vp, vp]
-        L.ogq_levels_bingrad_clipped.restype = i32
-        L.ogq_levels_bingrad_clipped.argtypes = [vp, vp, i32, i64, i32, i32, vp, vp, vp, vp, vp, sz, vp]
-        L.ogq_bucket_decode_sum.restype = i32
-        L.ogq_bucket_decode_sum.argtypes = [vp, vp, i32, i64, i32, i32, ctypes.c_float, vp, vp]
         L.ogq_launch_count.restype = ctypes.c_ulonglong
         L.ogq_launch_count.argtypes = []
         L.ogq_profile_enable.restype = i32

@@ -18,8 +18,8 @@ constexpr int kChunkAlign = 1024;   // flat chunk boundaries are multiples of th
 // finished and its writes are visible.  The launch latency of every kernel of a chain so overlaps with the
 // kernel before it.  Every kernel launched with launch_pdl calls pdl_wait() in all its threads, so
 // completion passes from kernel to kernel, and only then allows its own successor to be launched: at most
-// two kernels of a chain are on the device.  What one kernel of a chain writes and a later one reads goes
-// through L2 (__ldcg), never through the read-only path, whose loads the compiler may move.
+// two kernels of a chain are on the device.  What one kernel of a chain writes and a later one reads is
+// loaded plainly or from L2 (__ldcg), never through the read-only path, whose loads the compiler may move.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -80,8 +80,7 @@ inline QuantSteps quant_steps() { return QuantSteps{1u, 8u, 16u, 32u}; }
 // Segment search and rounding decision of one element.  `tab` is the shared address of the table, `mid` its
 // middle level.  Returns the address of the entry whose index is the element's
 // code: the entry of the segment's lower level, or the next one when the element rounds up.
-//   What bounds the quantizer is instruction issue (32 instructions per element at s = 9, ten of them Philox)
-// with the integer / logic pipe close behind, so the conditional steps are multiply-adds, which go to the
+//   28 instructions per element at s = 9, ten of them Philox; the integer / logic pipe is the busiest, so the conditional steps are multiply-adds, which go to the
 // other pipe; both factors are parameters (1 and the distance), a plain addition or a known power of two
 // would become an integer-pipe instruction.
 template <int STEP>

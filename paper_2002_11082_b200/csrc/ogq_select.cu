@@ -218,9 +218,7 @@ __device__ __forceinline__ void hist_add(uint32_t* cnt, uint32_t* lo, uint32_t* 
 
 // Warp-uniform visit of base[pb, pe): every lane of a warp calls f(x, nvalid) the same number of
 // times (nvalid = 0, 1 or 4), so f may use warp collectives.  128-bit loads on the aligned body.
-__device__ __forceinline__ float4 ld4(const float4* p) { return __ldg(p); }
 __device__ __forceinline__ uint4 ld4(const uint4* p) { return __ldcg(p); }
-__device__ __forceinline__ float ld1(const float* p) { return __ldg(p); }
 __device__ __forceinline__ uint32_t ld1(const uint32_t* p) { return __ldcg(p); }
 
 template <class E4, class E, class F>
@@ -1835,7 +1833,7 @@ struct SelArgs {
     const int64_t* off;
     int T;
     int64_t total, chunk;
-    int flat_ctas, scheme, s;
+    int scheme, s;
     float* levels;
     int32_t* status;
     SelWs ws;
@@ -2126,7 +2124,8 @@ __device__ __noinline__ void solve1_level(const Round1Cells G, const double* spr
 
 // One CTA per tensor.  Streamed tensors: prefix sums over round 1's cells, conservative cell ranges of the
 // levels, every populated cell in them becomes an interval of round 2.  Small tensors are solved here.
-//   What bounds it: latency, 8 to 10 us for a streamed tensor and for a small one.
+//   What bounds it: latency and, with several small tensors on an SM, their shared memory (one CTA per SM): 22 us for the 161
+// tensors of the ResNet-50 bucket, 13 for the 38 of VGG-19.
 __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -2572,7 +2571,7 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
     const int target = wave < kMaxFlatCtas ? (int)wave : kMaxFlatCtas;
     FlatGrid g = make_flat_grid(total, target, 16384);
     SelArgs A;
-    A.grad = d_grad; A.tau = d_tau; A.off = d_off; A.T = T; A.total = total; A.chunk = g.chunk; A.flat_ctas = g.ctas;
+    A.grad = d_grad; A.tau = d_tau; A.off = d_off; A.T = T; A.total = total; A.chunk = g.chunk;
     A.scheme = scheme; A.s = s; A.levels = d_levels; A.status = d_status;
     A.ws = sel_carve(d_ws, T, total);
     cudaError_t e = cudaSuccess;

@@ -12,20 +12,12 @@
 //   - a conservative range of cells that must contain it,
 // and turns the ranges into the (narrower, finer) intervals of the next round.
 //
-// Everything here is plain single-threaded code that compiles for the host as
-// well, so it can be exercised without a GPU; the kernels call it from one
-// thread after building the prefix arrays in parallel.
+// Everything here is plain single-threaded device code; the kernels call it
+// from one thread after building the prefix arrays in parallel.
 #pragma once
 
 #include <math.h>
 #include <stdint.h>
-#include <string.h>
-
-#ifdef __CUDACC__
-#define OGQ_HD __host__ __device__ __forceinline__
-#else
-#define OGQ_HD inline
-#endif
 
 namespace ogq {
 
@@ -52,21 +44,15 @@ struct ExactLv {
     double s_lt, s_le;     // sums of those elements
 };
 
-OGQ_HD float sel_key_to_float(uint32_t k)
+__device__ __forceinline__ float sel_key_to_float(uint32_t k)
 {
     uint32_t b = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
-    float f;
-#ifdef __CUDA_ARCH__
-    f = __uint_as_float(b);
-#else
-    memcpy(&f, &b, 4);
-#endif
-    return f;
+    return __uint_as_float(b);
 }
 
 // Exact sum of the fp32 values of a cell [kbase, kbase + 2^sh) holding cnt elements whose
 // low key bits (key - kbase) add up to lsum.  The cell lies in one binade and one sign.
-OGQ_HD double sel_cell_sum(uint32_t kbase, int sh, unsigned long long cnt, unsigned long long lsum)
+__device__ __forceinline__ double sel_cell_sum(uint32_t kbase, int sh, unsigned long long cnt, unsigned long long lsum)
 {
     if (cnt == 0) return 0.0;
     unsigned long long magsum;
@@ -86,12 +72,8 @@ OGQ_HD double sel_cell_sum(uint32_t kbase, int sh, unsigned long long cnt, unsig
     // value = mant * 2^(max(e,1) - 150); for e = 0 (subnormals) mant is the plain sum of magnitudes
     const unsigned long long mant = (e == 0) ? magsum : magsum - cnt * ((unsigned long long)(e - 1) << 23);
     const int ee = (e == 0) ? 1 : e;
-#ifdef __CUDA_ARCH__
     const double scale = __hiloint2double((ee + 873) << 20, 0);  // 2^(ee - 150), exact
     return sign * (__ull2double_rn(mant) * scale);
-#else
-    return sign * ldexp((double)mant, ee - 150);
-#endif
 }
 
 // Prefix arrays over "slots": interval j owns slots [slotbase[j], slotbase[j] + ncell_j]; slot
@@ -108,7 +90,7 @@ struct SolverView {
     double stot;
 };
 
-OGQ_HD int sel_interval_of_slot(const SolverView& v, int slot)
+__device__ __forceinline__ int sel_interval_of_slot(const SolverView& v, int slot)
 {
     if (v.slot_iv) return v.slot_iv[slot];
     int lo = 0, hi = v.m;  // last interval whose first slot is <= slot
@@ -119,27 +101,27 @@ OGQ_HD int sel_interval_of_slot(const SolverView& v, int slot)
     return lo;
 }
 
-OGQ_HD bool sel_is_end_slot(const SolverView& v, int slot)
+__device__ __forceinline__ bool sel_is_end_slot(const SolverView& v, int slot)
 {
     const int j = sel_interval_of_slot(v, slot);
     return slot == v.slotbase[j] + v.iv[j].ncell;
 }
 
-OGQ_HD uint32_t sel_slot_kbase(const SolverView& v, int slot)
+__device__ __forceinline__ uint32_t sel_slot_kbase(const SolverView& v, int slot)
 {
     const int j = sel_interval_of_slot(v, slot);
     return v.iv[j].klo + ((uint32_t)(slot - v.slotbase[j]) << v.iv[j].sh);
 }
 
-OGQ_HD int sel_slot_shift(const SolverView& v, int slot)
+__device__ __forceinline__ int sel_slot_shift(const SolverView& v, int slot)
 {
     return v.iv[sel_interval_of_slot(v, slot)].sh;
 }
 
-OGQ_HD double sel_slot_vlo(const SolverView& v, int slot) { return (double)sel_key_to_float(sel_slot_kbase(v, slot)); }
+__device__ __forceinline__ double sel_slot_vlo(const SolverView& v, int slot) { return (double)sel_key_to_float(sel_slot_kbase(v, slot)); }
 
 // First slot whose prefix count exceeds pos.
-OGQ_HD int sel_upper_bound(const SolverView& v, long long pos)
+__device__ __forceinline__ int sel_upper_bound(const SolverView& v, long long pos)
 {
     int lo = 0, hi = v.nslots;
     while (lo < hi) {
@@ -152,7 +134,7 @@ OGQ_HD int sel_upper_bound(const SolverView& v, long long pos)
 // Cell slot that holds the element of ascending rank pos (0-based).  If pos falls between two
 // intervals, round_up selects the first cell after the gap, otherwise the last cell before it.
 // Returns -1 when there is no such cell.
-OGQ_HD int sel_locate(const SolverView& v, long long pos, bool round_up, bool* in_gap)
+__device__ __forceinline__ int sel_locate(const SolverView& v, long long pos, bool round_up, bool* in_gap)
 {
     const int u = sel_upper_bound(v, pos);
     *in_gap = false;
@@ -187,7 +169,7 @@ struct LvInfo {
 // and their level becomes exact quickly; this is what lets the levels that depend on it tighten
 // in the next round.  The spare cell budget is then handed out narrow intervals first.
 // Returns the number of new intervals, or a negative code if no refinement is possible.
-OGQ_HD int sel_refine(const SolverView& v, int nr, const int* ra_in, const int* rb_in, bool trim_empty,
+__device__ __forceinline__ int sel_refine(const SolverView& v, int nr, const int* ra_in, const int* rb_in, bool trim_empty,
                       Interval* out, long long* total_elems_out)
 {
     constexpr int kTight = 8;
@@ -372,7 +354,7 @@ OGQ_HD int sel_refine(const SolverView& v, int nr, const int* ra_in, const int* 
 
 // ------------------------------------------------------------------ BinGrad-pb
 // g(x) = x n - sum_{|v| >= x} |v| at the lower edge of a cell slot (keys are magnitudes here).
-OGQ_HD double sel_pb_g(const SolverView& v, int slot, double* x_out)
+__device__ __forceinline__ double sel_pb_g(const SolverView& v, int slot, double* x_out)
 {
     const double x = sel_slot_vlo(v, slot);
     *x_out = x;
@@ -383,7 +365,7 @@ OGQ_HD double sel_pb_g(const SolverView& v, int slot, double* x_out)
 // change of g lies in [x_c, next key).  With P_up the sum of all magnitudes above x_c: if the
 // zero P_up / n of the piece above x_c is larger than x_c it is the answer, otherwise g jumps
 // across zero at the data value x_c itself.
-OGQ_HD double sel_pb_final(const SolverView& v, int slot)
+__device__ __forceinline__ double sel_pb_final(const SolverView& v, int slot)
 {
     const double x = sel_slot_vlo(v, slot);
     const double stat_up = (v.stot - v.spre[slot + 1]) / (double)v.n;

@@ -109,7 +109,7 @@ template <int BITS>
 __device__ __forceinline__ void table_indices(const uint32_t (&c)[kTableWorkers<BITS>], uint32_t (&x)[2])
 {
     if constexpr (BITS == 1) {
-        // 8 x 8 bit transpose
+        // 8 x 8 bit transpose by three rounds of exchanges (Warren, Hacker's Delight, section 7-3)
         uint32_t lo = c[0] | c[1] << 8 | c[2] << 16 | c[3] << 24, hi = c[4] | c[5] << 8 | c[6] << 16 | c[7] << 24, t;
         t = (lo ^ (lo >> 7)) & 0x00aa00aau; lo ^= t ^ (t << 7);
         t = (hi ^ (hi >> 7)) & 0x00aa00aau; hi ^= t ^ (t << 7);
