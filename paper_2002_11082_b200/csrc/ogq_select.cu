@@ -40,11 +40,11 @@ constexpr int kSelThreads = 512;    // two CTAs are resident per SM: a CTA in a 
                                     // set-up phase leaves the other half of the SM streaming
 constexpr int kSelResident = 2;
 constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSolveThreads = 1024;  // of the solver launches
 constexpr int kSelW = 16;          // binades in the fine window of round 1
 constexpr int kSelM = 7;           // log2(cells per binade) in the window
 constexpr int kSmallN = 16384;     // tensors up to this size are solved in shared memory
 constexpr int kSortN = 16384;      // candidates from which one CTA finishes a larger tensor
-constexpr int kAloneN = 131072;    // tensors up to this size are finished by one CTA after round 2
 constexpr int kStageCap = 320;     // per-warp staging entries for compaction
 constexpr int kParkMax = 256;      // values one warp can park between two checks in the tail of round 2 (32 lanes x 8)
 constexpr int kMaxSlices = 64;     // CTAs that share one tensor's copied keys in round 3
@@ -125,6 +125,19 @@ constexpr size_t kSmemHist = 3 * kCells * sizeof(uint32_t);
 constexpr size_t kSmemStage = kSelWarps * kStageCap * sizeof(uint32_t);
 constexpr size_t kSmemBytes = kSmemHist + kSmemStage;
 
+// Every structure in shared memory that a function which is not inlined uses lies in the dynamic shared memory and is reached
+// through this symbol: through a reference it would be read by generic loads.
+extern __shared__ __align__(16) unsigned char smem[];
+
+struct Round2Ctx {  // per-CTA constants of round 2, kept in shared memory to spare registers
+    uint32_t* dst;
+    unsigned long long* cursor;
+    uint32_t clear;  // 0x7fffffff when only magnitudes count
+    int nohist;      // copy the keys inside the intervals without counting them
+    unsigned long long cap;  // words of the tensor's region in the destination buffer
+    int* overflow;           // set when a copy did not fit
+};
+
 struct Table {  // interval lookup table of the tensor being streamed
     uint32_t klo[kMaxIv];
     uint32_t khi[kMaxIv];
@@ -133,27 +146,16 @@ struct Table {  // interval lookup table of the tensor being streamed
     int m, ncells;
     int lo_e;                                      // bottom binade of the round-1 fine window
     uint32_t coarse[1024];                         // one bit per block of 2^17 keys that touches an interval
+    Round2Ctx ctx;
+    int fills[kSelWarps];                          // values parked per warp
 };
+constexpr size_t kStreamBytes = kSmemBytes + sizeof(Table);
+__device__ __forceinline__ Table& sel_table() { return *reinterpret_cast<Table*>(smem + kSmemBytes); }
+__device__ __forceinline__ uint32_t* sel_hist() { return reinterpret_cast<uint32_t*>(smem); }
+__device__ __forceinline__ uint32_t* sel_stage() { return reinterpret_cast<uint32_t*>(smem + kSmemHist); }
 
+// By the first kMaxIv threads of the CTA (called by all threads; the caller synchronises afterwards).
 __device__ __forceinline__ void table_from_intervals(Table& tb, const Interval* iv, int m)
-{
-    // called by one thread
-    int nc = 0;
-    for (int j = 0; j < kMaxIv; ++j) {
-        if (j < m) {
-            tb.klo[j] = iv[j].klo; tb.khi[j] = iv[j].khi; tb.sh[j] = iv[j].sh; tb.cellbase[j] = iv[j].cellbase;
-            nc = iv[j].cellbase + iv[j].ncell;
-        } else {
-            tb.klo[j] = 0xffffffffu; tb.khi[j] = 0u; tb.sh[j] = 0; tb.cellbase[j] = 0;
-        }
-    }
-    tb.m = m;
-    tb.ncells = nc;
-}
-
-// The same, spread over the first kMaxIv threads of the CTA (called by all threads; the caller
-// synchronises afterwards).
-__device__ __forceinline__ void table_from_intervals_cta(Table& tb, const Interval* iv, int m)
 {
     const int j = threadIdx.x;
     if (j < kMaxIv) {
@@ -194,7 +196,12 @@ __device__ __forceinline__ Interval round1_interval(int hi_e, bool magnitude_onl
     return x;
 }
 
-__device__ __forceinline__ bool classify(const Table& tb, uint32_t key, int& cell, uint32_t& low, int& sh)
+// A pass that only copies keys writes them as interval (top bits) and distance from its lowest key, so that the finish need not
+// search for the interval again (it took 18,000 of 40,000 cycles for 14,000 keys): intervals of at most 2^kRelBits keys.
+constexpr int kRelBits = 26;
+static_assert(kMaxIv <= 1 << (32 - kRelBits), "an interval's number fits the top bits");
+
+__device__ __forceinline__ bool classify(const Table& tb, uint32_t key, int& cell, uint32_t& low, int& sh, uint32_t& packed)
 {
     int idx = 0;
 #pragma unroll
@@ -202,6 +209,7 @@ __device__ __forceinline__ bool classify(const Table& tb, uint32_t key, int& cel
         if (tb.klo[idx + step] <= key) idx += step;
     sh = tb.sh[idx];
     const uint32_t rel = key - tb.klo[idx];
+    packed = (uint32_t)idx << kRelBits | (rel & ((1u << kRelBits) - 1u));
     cell = tb.cellbase[idx] + (int)(rel >> sh);
     low = rel & ((1u << sh) - 1u);
     return key >= tb.klo[idx] && key <= tb.khi[idx];
@@ -448,13 +456,17 @@ struct Round1Body {
 // Round1Body::fine), folded into the wide counters every kPackTrips loop trips; the sum of the folded
 // counts is checked against the number of values that went in, and a mismatch (a cell took 256 values
 // or more within the trips: heavily repeated values) redoes those trips with the two-add path.
-// packed: kPackedCells zeroed words of shared memory, zero again on return.
+// The packed cells (the compaction stages) are zero before, and zero again on return.
+struct Round1Out {
+    float vmin, vmax;
+    uint32_t nonfinite;
+};
+
 template <bool MAG, bool CLIP>
-__device__ __noinline__ void stream_round1(const float* __restrict__ grad, int64_t pb, int64_t pe, int lo_e,
-                                              uint32_t* hist, uint32_t* packed, float& vmin, float& vmax,
-                                              uint32_t& nonfinite, float tau)
+__device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, int64_t pb, int64_t pe, int lo_e, float tau)
 {
     __shared__ uint32_t sh_coarse, sh_total;
+    uint32_t *hist = sel_hist(), *packed = sel_stage();
     Round1Body<MAG, CLIP> f;
     f.tau = tau;
     f.lo23 = (uint32_t)lo_e << 23;
@@ -464,7 +476,7 @@ __device__ __noinline__ void stream_round1(const float* __restrict__ grad, int64
     f.cnt = (uint32_t)__cvta_generic_to_shared(hist + (MAG ? 0 : kRound1Mag));
     f.pk = (uint32_t)__cvta_generic_to_shared(packed);
     f.coarse = (uint32_t)__cvta_generic_to_shared(&sh_coarse);
-    f.mn = vmin; f.mx = vmax; f.nonfinite = nonfinite;
+    f.mn = __int_as_float(0x7f800000); f.mx = __int_as_float(0xff800000); f.nonfinite = 0u;
     int64_t a = (pb + 3) & ~(int64_t)3;
     if (a > pe) a = pe;
     int64_t b = pe & ~(int64_t)3;
@@ -551,7 +563,7 @@ __device__ __noinline__ void stream_round1(const float* __restrict__ grad, int64
     }
     __syncthreads();
     for (int64_t i = first + ntrips * 4 * kSelThreads + tid; i < e; i += kSelThreads) f.template four<false>(__ldg(g4 + i));
-    vmin = f.mn; vmax = f.mx; nonfinite = f.nonfinite;
+    return Round1Out{f.mn, f.mx, f.nonfinite};
 }
 
 // Round 2 over grad[pb, pe).  Phase A: a one-bit-per-2^17-bit-patterns test on the raw fp32 bits
@@ -559,20 +571,14 @@ __device__ __noinline__ void stream_round1(const float* __restrict__ grad, int64
 // yet).  Phase B, whenever the stage fills up: the parked values are turned into keys and classified
 // exactly 32 at a time, so that the expensive part runs with all lanes busy; keys inside an interval
 // are histogrammed and copied out.
-struct Round2Ctx {  // per-CTA constants of round 2, kept in shared memory to spare registers
-    uint32_t *cnt, *lo, *hi;
-    uint32_t* dst;
-    unsigned long long* cursor;
-    uint32_t clear;  // 0x7fffffff when only magnitudes count
-    int nohist;      // copy the keys inside the intervals without counting them
-    unsigned long long cap;  // words of the tensor's region in the destination buffer
-    int* overflow;           // set when a copy did not fit
-};
-
 // Phase B of round 2 for one warp: classifies `fill` parked values 32 at a time.  A free function
 // taking values, so that the caller's per-warp state can stay in registers.
-__device__ __noinline__ void round2_drain(const Table* tb, const Round2Ctx* ctx, const uint32_t* stage, int fill)
+__device__ __noinline__ void round2_drain(int fill)
 {
+    const Table* tb = &sel_table();
+    const Round2Ctx* ctx = &tb->ctx;
+    uint32_t* hist = sel_hist();
+    const uint32_t* stage = sel_stage() + (threadIdx.x >> 5) * kStageCap;
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const uint32_t clear = ctx->clear;
@@ -586,9 +592,10 @@ __device__ __noinline__ void round2_drain(const Table* tb, const Round2Ctx* ctx,
             if (bits == 0x80000000u) bits = 0u;
             key = bits ^ ((uint32_t)((int)bits >> 31) | 0x80000000u);
             int cell, sh;
-            uint32_t low;
-            in = classify(*tb, key, cell, low, sh);
-            if (in && !ctx->nohist) hist_add(ctx->cnt, ctx->lo, ctx->hi, cell, low);
+            uint32_t low, packed;
+            in = classify(*tb, key, cell, low, sh, packed);
+            if (ctx->nohist) key = packed;
+            else if (in) hist_add(hist, hist + kCells, hist + 2 * kCells, cell, low);
         }
         const uint32_t m2 = __ballot_sync(0xffffffffu, in);
         if (m2) {
@@ -680,16 +687,15 @@ struct Round2Warp {
 
 template <bool CLIP>
 __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64_t pb, int64_t pe,
-                                              bool magnitude_only, const Table& tb, uint32_t* cnt, uint32_t* lo,
-                                              uint32_t* hi, uint32_t* stage, uint32_t* dst, int64_t cap,
-                                              unsigned long long* cursor, int* overflow, bool nohist, float tau, bool down)
+                                              bool magnitude_only, uint32_t* dst, int64_t cap, unsigned long long* cursor, int* overflow, bool nohist, float tau, bool down)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ Round2Ctx ctx;
-    __shared__ int fills[kSelWarps];
+    Table& tb = sel_table();
+    Round2Ctx& ctx = tb.ctx;
+    int* fills = tb.fills;
     __syncthreads();
     if (threadIdx.x == 0) {
-        ctx.cnt = cnt; ctx.lo = lo; ctx.hi = hi; ctx.dst = dst; ctx.cursor = cursor;
+        ctx.dst = dst; ctx.cursor = cursor;
         ctx.clear = magnitude_only ? 0x7fffffffu : 0xffffffffu;
         ctx.nohist = nohist ? 1 : 0;
         ctx.cap = (unsigned long long)cap;
@@ -700,7 +706,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
     Round2Warp<CLIP> w;
     w.tau = tau;
     w.coarse = (uint32_t)__cvta_generic_to_shared(tb.coarse);
-    w.stage = (uint32_t)__cvta_generic_to_shared(stage);
+    w.stage = (uint32_t)__cvta_generic_to_shared(sel_stage() + warp * kStageCap);
     w.fillp = (uint32_t)__cvta_generic_to_shared(&fills[warp]);
     int64_t a = (pb + 3) & ~(int64_t)3;
     if (a > pe) a = pe;
@@ -716,7 +722,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
         __syncwarp();
         const int f = *(volatile int*)&fills[warp];
         if (f > kStageCap - kParkMax) {
-            round2_drain(&tb, &ctx, stage, f);
+            round2_drain(f);
             if (lane == 0) fills[warp] = 0;
             __syncwarp();
         }
@@ -757,7 +763,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
                 break;
             }
             if (fill) {
-                round2_drain(&tb, &ctx, stage, fill);
+                round2_drain(fill);
                 if (lane == 0) fills[warp] = 0;
                 __syncwarp();
                 fill = 0;
@@ -784,11 +790,11 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
         }
     }
     __syncwarp();
-    round2_drain(&tb, &ctx, stage, *(volatile int*)&fills[warp]);
+    round2_drain(*(volatile int*)&fills[warp]);
 }
 
-// Streams copied keys [pb, pe) of a tensor: counts those inside the intervals on the cells (unless nohist) and copies
-// them on.
+// Streams copied keys [pb, pe) of a tensor: counts those inside the intervals on the cells and copies them on, or copies them
+// on as interval and distance (nohist).
 __device__ __forceinline__ void stream_piece(const uint32_t* __restrict__ src, int64_t pb, int64_t pe, const Table& tb,
                                              uint32_t* cnt, uint32_t* lo, uint32_t* hi, Stager& stg, bool nohist)
 {
@@ -799,10 +805,10 @@ __device__ __forceinline__ void stream_piece(const uint32_t* __restrict__ src, i
         for (int j = 0; j < 4; ++j) {
             if (j >= nv) continue;
             int cell, sh;
-            uint32_t low;
-            if (classify(tb, x[j], cell, low, sh)) {
+            uint32_t low, packed;
+            if (classify(tb, x[j], cell, low, sh, packed)) {
                 if (!nohist) hist_add(cnt, lo, hi, cell, low);
-                kk[c++] = x[j];
+                kk[c++] = nohist ? packed : x[j];
             }
         }
         stg.append(kk, c);
@@ -838,7 +844,7 @@ __device__ __forceinline__ void flush_hist(const uint32_t* smem_hist, int ncells
 // on one level with searches spread over its lanes, and fp64 division is one function.
 __device__ __noinline__ double fp64_div(double a, double b) { return a / b; }
 
-struct SolverShared {
+struct __align__(16) SolverShared {
     Interval iv[kMaxIv];
     Interval niv[kMaxIv];
     LvInfo lv[kMaxLv];
@@ -853,14 +859,15 @@ struct SolverShared {
     int pa[kRefineMax], pb[kRefineMax];  // runs of candidate cells
     long long cand;           // elements inside the new intervals
     // finish
-    uint32_t lo[kMaxIv], hi[kMaxIv];  // keys of the intervals (padded: no key lies in the surplus ones)
-    uint32_t base[kMaxIv];            // first cell of the interval
-    int sh[kMaxIv];                   // log2 of the keys per cell
-    int start[kMaxIv + 1];            // position of the interval's first value
-    double pre[kMaxIv];               // sum of the values before it
+    uint4 place[kMaxIv];        // of the intervals: lowest and highest key (padded: no key lies in the surplus ones), first cell, log2 of the keys per cell
+    uint32_t before[kMaxIv];    // elements of the tensor below the interval (surplus ones: more than there are)
+    int start[kMaxIv + 1];      // position of the interval's first value
+    double pre[kMaxIv];         // sum of the values before it
     int n_keys;
     uint32_t below[32];
 };
+
+__device__ __forceinline__ SolverShared& sel_state();
 
 // Exclusive sums of (c, s) over the CTA's threads in thread order; totals in tot_c, tot_s.  Any number of warps.
 __device__ __forceinline__ void block_excl_scan(uint32_t& c, double& s, SolverShared& S, uint32_t& tot_c, double& tot_s)
@@ -904,89 +911,155 @@ __device__ __forceinline__ void block_excl_scan(uint32_t& c, double& s, SolverSh
 // smaller.)
 // ---------------------------------------------------------------------------
 struct CellIndex {
-    float* sv;          // the values
-    uint32_t* end;      // [nc] position after the last value of every cell; nc = 1024, 2048 ... 16384
-    double* pre;        // sum of the values before every chunk-th position
-    int n, nc, chunk;   // values per prefix sum: kSortN / threads (at most 32)
+    float* sv;      // the values, at padded positions
+    uint32_t* end;  // [nc] position after the last value of every cell; nc = 1024, 2048 ... 16384
+    double* pre;    // [i] sum of the first i << chunk values
+    int n, nc, chunk;
 };
 
-// Shared memory: prefix sums, cells, values; then the list of the gathered keys.
-constexpr int kIndexCells = 16384;
-constexpr size_t kIndexBytes = 1032 * 8 + (size_t)kIndexCells * 4 + (size_t)kSortN * 4;
+// Position i of the values: two words of padding after every sixteen, so that threads that read runs of eight or sixteen
+// values side by side meet in no bank.
+__device__ __forceinline__ int index_at_word(int i) { return i + ((i >> 4) << 1); }
 
-__device__ __forceinline__ CellIndex index_at(unsigned char* smem, int n)
+// Shared memory: the list of the keys, later the prefix sums in its place; cells; values.
+constexpr int kIndexCells = 16384;
+constexpr size_t kOffIndexEnd = (size_t)kSortN * 4 + 16;
+constexpr size_t kOffIndexValues = kOffIndexEnd + (size_t)kIndexCells * 4;
+constexpr size_t kIndexBytes = kOffIndexValues + ((size_t)kSortN / 16 * 18) * 4;
+
+__device__ __forceinline__ CellIndex index_at(int n)
 {
     CellIndex X;
     X.pre = reinterpret_cast<double*>(smem);
-    X.end = reinterpret_cast<uint32_t*>(smem + 1032 * 8);
-    X.sv = reinterpret_cast<float*>(smem + 1032 * 8 + (size_t)kIndexCells * 4);
+    X.end = reinterpret_cast<uint32_t*>(smem + kOffIndexEnd);
+    X.sv = reinterpret_cast<float*>(smem + kOffIndexValues);
     X.n = n;
-    X.chunk = kSortN / (int)blockDim.x;
-    int nc = 1024;  // two cells or more per value, as far as there are that many: clearing and adding up cells takes longer
-    while (nc < 2 * n && nc < kIndexCells) nc <<= 1;  // than selecting in fuller ones saves
-    X.nc = nc;
+    // two cells or more per value, as far as there are that many (a power of two from 1024 on): clearing and adding up cells
+    // takes longer than selecting in fuller ones saves
+    X.nc = min(max(1 << (32 - __clz(2 * n - 1)), 1024), kIndexCells);
+    X.chunk = max(32 - __clz((n - 1) / (int)blockDim.x), 1);
     return X;
 }
 
-// fetch(i): value i of n, cell_of(i): its cell.  Called by every thread of the CTA (512 or 1024).
-template <class Fetch, class CellOf>
-__device__ __forceinline__ void index_build(const CellIndex& X, SolverShared& S, Fetch fetch, CellOf cell_of)
+// cells(i, c, v): cells and values of the four values i[0..3] of n, which may lie where the prefix sums go.  Called by every
+// thread of the CTA.
+//   What bounds it: the latency of its six barriers and of instructions run once.  So four values of a thread are
+// in flight at a time, the cells are added up without a loop, and only the positions that there are are summed (a fixed
+// 16,384 positions took 2.3 us of the 13 us for 300 values).
+constexpr int kIndexCols = 4;  // values of a thread in flight
+
+template <class Cells>
+__device__ __forceinline__ void index_build(const CellIndex& X, SolverShared& S, Cells cells)
 {
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     uint4* rows = reinterpret_cast<uint4*>(X.end);
-#pragma unroll 1
     for (int i = tid; i < X.nc / 4; i += nt) rows[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
+    constexpr int kCols = kIndexCols;
+    auto four = [&](int i0, uint32_t (&c)[kCols], float (&v)[kCols]) {
+        int i[kCols];
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) i[u] = min(i0 + u * nt, X.n - 1);
+        cells(i, c, v);
+    };
 #pragma unroll 1
-    for (int i = tid; i < X.n; i += nt) atomicAdd(X.end + cell_of(i), 1u);
+    for (int i0 = tid; i0 < X.n; i0 += kCols * nt) {
+        uint32_t c[kCols];
+        float v[kCols];
+        four(i0, c, v);
+#pragma unroll
+        for (int u = 0; u < kCols; ++u)
+            if (i0 + u * nt < X.n) atomicAdd(X.end + c[u], 1u);
+    }
     __syncthreads();
     {
-        // exclusive sums over the cells, in place: a warp takes rows of 128 cells
-        const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5, nrows = X.nc >> 7, per = (nrows + nw - 1) / nw;
-        const int r0 = warp * per, r1 = r0 + per < nrows ? r0 + per : nrows;
-        uint32_t sum = 0u;
+        // exclusive sums over the cells, in place: a warp takes consecutive rows of 128 cells, kRows at a time
+        constexpr int kRows = 4;
+        const int nrows = X.nc >> 7, per = (nrows + nw - 1) / nw;
+        const int r0 = min(warp * per, nrows), r1 = min(r0 + per, nrows);
+        uint32_t mine = 0u;
 #pragma unroll 1
         for (int q = r0; q < r1; ++q) {
             const uint4 w = rows[q * 32 + lane];
-            sum += (w.x + w.y) + (w.z + w.w);
+            mine += (w.x + w.y) + (w.z + w.w);
         }
-        sum = __reduce_add_sync(0xffffffffu, sum);
-        if (lane == 0) S.below[warp] = sum;
+        mine = __reduce_add_sync(0xffffffffu, mine);
+        if (lane == 0) S.below[warp] = mine;
         __syncthreads();
         uint32_t run = __reduce_add_sync(0xffffffffu, lane < warp ? S.below[lane] : 0u);
 #pragma unroll 1
-        for (int q = r0; q < r1; ++q) {
-            const uint4 w = rows[q * 32 + lane];
-            const uint32_t own = (w.x + w.y) + (w.z + w.w);
-            uint32_t inc = own;
+        for (int q = r0; q < r1; q += kRows) {
+            uint4 w[kRows];
+            uint32_t own[kRows], inc[kRows];
+#pragma unroll
+            for (int u = 0; u < kRows; ++u) {
+                w[u] = q + u < r1 ? rows[(q + u) * 32 + lane] : make_uint4(0u, 0u, 0u, 0u);
+                own[u] = inc[u] = (w[u].x + w[u].y) + (w[u].z + w[u].w);
+            }
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t nb = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += nb;
+#pragma unroll
+                for (int u = 0; u < kRows; ++u) {
+                    const uint32_t nb = __shfl_up_sync(0xffffffffu, inc[u], o);
+                    if (lane >= o) inc[u] += nb;
+                }
             }
-            uint4 x;
-            x.x = run + inc - own; x.y = x.x + w.x; x.z = x.y + w.y; x.w = x.z + w.z;
-            run += __shfl_sync(0xffffffffu, inc, 31);
-            rows[q * 32 + lane] = x;
+#pragma unroll
+            for (int u = 0; u < kRows; ++u) {
+                uint4 x;
+                x.x = run + inc[u] - own[u]; x.y = x.x + w[u].x; x.z = x.y + w[u].y; x.w = x.z + w[u].z;
+                run += __shfl_sync(0xffffffffu, inc[u], 31);
+                if (q + u < r1) rows[(q + u) * 32 + lane] = x;
+            }
         }
     }
     __syncthreads();
 #pragma unroll 1
-    for (int i = tid; i < X.n; i += nt) X.sv[atomicAdd(X.end + cell_of(i), 1u)] = fetch(i);
-    __syncthreads();
-    // fp64 sums of every thread's chunk, scanned
-    double ls = 0.0, tot;
-#pragma unroll 1
-    for (int j = 0; j < X.chunk; ++j) {
-        const int i = tid * X.chunk + (j ^ (tid & (X.chunk - 1)));  // (neighbouring threads in different banks)
-        if (i < X.n) ls += (double)X.sv[i];
+    for (int i0 = tid; i0 < X.n; i0 += kCols * nt) {
+        uint32_t c[kCols], at[kCols];
+        float v[kCols];
+        four(i0, c, v);
+#pragma unroll
+        for (int u = 0; u < kCols; ++u)
+            if (i0 + u * nt < X.n) at[u] = atomicAdd(X.end + c[u], 1u);
+#pragma unroll
+        for (int u = 0; u < kCols; ++u)
+            if (i0 + u * nt < X.n) X.sv[index_at_word((int)at[u])] = v[u];
     }
-    uint32_t none = 0u, tc;
-    block_excl_scan(none, ls, S, tc, tot);
-    X.pre[tid] = ls;
-    if (tid == 0) X.pre[nt] = tot;
+    __syncthreads();
+    // fp64 sums before every run of 2^chunk positions, one run a thread
+    const int p0 = tid << X.chunk;
+    double ls = 0.0;
+    if (p0 < X.n) {
+#pragma unroll 1
+        for (int i = p0; i < min(p0 + (1 << X.chunk), X.n); i += 2) {
+            const float2 w = *reinterpret_cast<const float2*>(X.sv + index_at_word(i));
+            ls += (double)w.x;
+            if (i + 1 < X.n) ls += (double)w.y;
+        }
+    }
+    const int used = (X.n + (32 << X.chunk) - 1) >> (5 + X.chunk);  // warps that have any
+    if (warp < used) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double nb = __shfl_up_sync(0xffffffffu, ls, o);
+            if (lane >= o) ls = nb + ls;
+        }
+        if (lane == 31) S.ss[warp] = ls;
+    }
+    __syncthreads();
+    if (warp < used) {
+        const double up = __shfl_up_sync(0xffffffffu, ls, 1);
+        const double before = warp > 0 ? warp_sum(lane < warp ? S.ss[lane] : 0.0) : 0.0;
+        X.pre[tid] = lane > 0 ? before + up : before;
+        if (lane == 31 && warp == used - 1) X.pre[tid + 1] = before + ls;
+    }
     __syncthreads();
 }
+
+constexpr size_t kSolveBytes = kIndexBytes + sizeof(SolverShared);
+static_assert(kIndexBytes % 16 == 0 && sizeof(SolverShared) % 16 == 0, "structures in the dynamic shared memory are aligned");
+__device__ __forceinline__ SolverShared& sel_state() { return *reinterpret_cast<SolverShared*>(smem + kIndexBytes); }
 
 struct Ranked {
     float v;
@@ -994,41 +1067,47 @@ struct Ranked {
     double s_lt, s_le; // their sums
 };
 
-// Sum of the values before position a (lane's share of it; add up over the warp).
-__device__ __forceinline__ double index_before_lane(const CellIndex& X, int a)
+// Sum of the values before position a <= n, by the 32 lanes of a warp.
+__device__ __forceinline__ double index_before(const CellIndex& X, int a)
 {
-    const int lane = threadIdx.x & 31, q = a / X.chunk;
-    double x = lane == 0 ? X.pre[q] : 0.0;
-    if (q * X.chunk + lane < a) x += (double)X.sv[q * X.chunk + lane];
-    return x;
+    const int lane = threadIdx.x & 31, q = a >> X.chunk, first = q << X.chunk;
+    double x = first + lane < a ? (double)X.sv[index_at_word(first + lane)] : 0.0;
+    for (int o = (1 << X.chunk) >> 1; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return __shfl_sync(0xffffffffu, x, 0) + X.pre[q];
 }
 
 // The value of ascending rank p, by the 32 lanes of a warp.
 __device__ __forceinline__ Ranked index_select(const CellIndex& X, int p)
 {
     const int lane = threadIdx.x & 31;
-    // the cell that holds rank p: 32 probes in each of three steps
+    // the cell that holds rank p: 32 probes in each of three steps (the first ones shifted so that they lie in different banks)
     const int s1 = X.nc >> 5, s2 = X.nc >> 10;
-    int c = s1 * __popc(__ballot_sync(0xffffffffu, (int)X.end[(lane + 1) * s1 - 1] <= p));
-    c += s2 * __popc(__ballot_sync(0xffffffffu, (int)X.end[c + (lane + 1) * s2 - 1] <= p));
-    c += __popc(__ballot_sync(0xffffffffu, lane < s2 && (int)X.end[c + (lane & (s2 - 1))] <= p));
+    const int k1 = __popc(__ballot_sync(0xffffffffu, (int)X.end[(lane + 1) * s1 - 1 - lane] <= p));
+    int c = k1 > 0 ? k1 * s1 - k1 + 1 : 0;
+    const int i2 = c + (lane + 1) * s2 - 1;
+    c += s2 * __popc(__ballot_sync(0xffffffffu, i2 < X.nc && (int)X.end[min(i2, X.nc - 1)] <= p));
+    if (s2 > 1) c += __popc(__ballot_sync(0xffffffffu, lane < s2 && (int)X.end[min(c + lane, X.nc - 1)] <= p));
     const int a = c > 0 ? (int)X.end[c - 1] : 0, b = (int)X.end[c], k = p - a;
     Ranked r;
     int lt = 0, eq = 0;
-    double s = index_before_lane(X, a);
+    const double before = index_before(X, a);
+    double s = 0.0;
     if (b - a <= 32) {
-        const float v = a + lane < b ? X.sv[a + lane] : __int_as_float(0x7f800000);
+        const float v = a + lane < b ? X.sv[index_at_word(a + lane)] : __int_as_float(0x7f800000);
 #pragma unroll 1
         for (int j = 0; j < b - a; ++j) {
             const float w = __shfl_sync(0xffffffffu, v, j);
-            lt += w < v ? 1 : 0;
+            if (w < v) {
+                ++lt;
+                s += (double)w;
+            }
             eq += w == v ? 1 : 0;
         }
         const int src = (__ffs(__ballot_sync(0xffffffffu, a + lane < b && lt <= k && k < lt + eq)) - 1) & 31;
         r.v = __shfl_sync(0xffffffffu, v, src);
         lt = __shfl_sync(0xffffffffu, lt, src);
         eq = __shfl_sync(0xffffffffu, eq, src);
-        if (v < r.v) s += (double)v;
+        s = __shfl_sync(0xffffffffu, s, src);
     } else {
         // a crowded cell (mostly one value many times over): its keys are bisected bit by bit
         uint32_t key = 0u;
@@ -1038,70 +1117,76 @@ __device__ __forceinline__ Ranked index_select(const CellIndex& X, int p)
             int n_lt = 0, n_eq = 0;
 #pragma unroll 1
             for (int i = a + lane; i < b; i += 32) {
-                const uint32_t w = float_to_key(X.sv[i]);
-                n_lt += w < cand ? 1 : 0;
-                n_eq += w == cand ? 1 : 0;
+                const float w = X.sv[index_at_word(i)];
+                const uint32_t wk = float_to_key(w);
+                n_lt += wk < cand ? 1 : 0;
+                if (bit < 0) {
+                    n_eq += wk == cand ? 1 : 0;
+                    if (wk < cand) s += (double)w;
+                }
             }
-            n_lt = __reduce_add_sync(0xffffffffu, n_lt);
+            n_lt = (int)__reduce_add_sync(0xffffffffu, (uint32_t)n_lt);
             if (bit >= 0) {
                 if (n_lt <= k) key = cand;
             } else {
                 lt = n_lt;
-                eq = __reduce_add_sync(0xffffffffu, n_eq);
+                eq = (int)__reduce_add_sync(0xffffffffu, (uint32_t)n_eq);
             }
         }
         r.v = key_to_float(key);
-#pragma unroll 1
-        for (int i = a + lane; i < b; i += 32)
-            if (X.sv[i] < r.v) s += (double)X.sv[i];
+        s = warp_sum(s);
     }
     r.i_lt = a + lt;
     r.i_le = a + lt + eq;
-    r.s_lt = warp_sum(s);
+    r.s_lt = before + s;
     r.s_le = r.s_lt + (double)r.v * (double)eq;
     return r;
 }
 
-// Levels from the indexed values: those of the m intervals iv (S.start, S.pre: where each begins), whose
-// cbefore and sbefore tie them to the whole tensor of n elements with sum stot.  ORQ: the open levels of
+// Levels from the indexed values: those of m intervals, which begin at positions S.start with sum S.pre before them and have
+// S.before elements of the whole tensor (n of them, sum stot) below them, sum iv[].sbefore.  ORQ: the open levels of
 // S.lv, one warp per level, one depth of Algorithm 1 at a time.  BinGrad-pb: the sign change of g.
 // Called by every thread of the CTA.
-__device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared& S, const Interval* iv, int m, bool pb, int s,
-                                               long long n, double stot, int t, float* __restrict__ levels,
+__device__ __noinline__ void levels_from_index(int values, int m, bool pb, int s,
+                                               double n, double stot, int t, float* __restrict__ levels,
                                                int32_t* __restrict__ status)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    SolverShared& S = sel_state();
+    const Interval* iv = S.niv;
+    const CellIndex X = index_at(values);  // (made again: a reference would put it into local memory)
     if (!pb) {
         static_assert(kSelWarps >= kMaxLv - 1, "one warp per interior level");
+        const int q = warp;
 #pragma unroll 1
         for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
-            const int q = warp;
             if (q < s - 1 && q >= stride && ((q - stride) & (2 * stride - 1)) == 0 && !S.lv[q].exact) {
                 const LvInfo &L = S.lv[q - stride], &R = S.lv[q + stride];
                 LvInfo& o = S.lv[q];
-                if (!(R.val > L.val)) {
+                const double lval = L.val, width = R.val - lval;
+                const uint32_t le = (uint32_t)R.c_le, lt = (uint32_t)L.c_lt;
+                if (!(width > 0.0)) {
                     if (lane == 0) o = L;
                 } else {
-                    const double nseg = (double)(R.c_le - L.c_lt);
-                    const double A = (R.s_le - L.s_lt) - L.val * nseg;
-                    const double k = fmin(fmax(floor(fp64_div(A, R.val - L.val)), 0.0), nseg - 1.0);
-                    const long long p = R.c_le - 1 - (long long)k;
+                    const double nseg = (double)(le - lt);
+                    const double A = (R.s_le - L.s_lt) - lval * nseg;
+                    const uint32_t k = (uint32_t)fmin(fmax(floor(A / width), 0.0), nseg - 1.0), p = le - 1u - k;
                     // the interval that holds rank p: the last one that begins at or before it
-                    const int j = __popc(__ballot_sync(0xffffffffu, lane < m && iv[lane].cbefore <= p)) +
-                                  __popc(__ballot_sync(0xffffffffu, lane + 32 < m && iv[lane + 32].cbefore <= p)) - 1;
-                    const long long i = j >= 0 ? S.start[j] + (p - iv[j].cbefore) : -1;
+                    int j = __popc(__ballot_sync(0xffffffffu, S.before[lane] <= p)) - 1;
+                    if (m > 32) j += __popc(__ballot_sync(0xffffffffu, S.before[lane + 32] <= p));
+                    const int i = j >= 0 ? S.start[j] + (int)(p - S.before[j]) : -1;
                     if (i < 0 || i >= S.start[j + 1]) {
                         if (lane == 0) { o = L; S.internal = 1; }
                     } else {
-                        const Ranked r = index_select(X, (int)i);
+                        const Ranked r = index_select(X, i);
                         if (lane == 0) {
-                            o.exact = 1;
+                            const uint32_t cb = S.before[j] - (uint32_t)S.start[j];
+                            const double sb = iv[j].sbefore, pre = S.pre[j];
                             o.val = (double)r.v;
-                            o.key = float_to_key(r.v);
-                            o.c_lt = iv[j].cbefore + (r.i_lt - S.start[j]);
-                            o.c_le = iv[j].cbefore + (r.i_le - S.start[j]);
-                            o.s_lt = iv[j].sbefore + (r.s_lt - S.pre[j]);
-                            o.s_le = iv[j].sbefore + (r.s_le - S.pre[j]);
+                            o.c_lt = cb + (uint32_t)r.i_lt;
+                            o.c_le = cb + (uint32_t)r.i_le;
+                            o.s_lt = sb + (r.s_lt - pre);
+                            o.s_le = sb + (r.s_le - pre);
                         }
                     }
                 }
@@ -1116,7 +1201,7 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
     // BinGrad-pb: the values with g(x) = x n - sum_{|v| >= x} |v| <= 0 come first; a warp per candidate rank
     const int nw = blockDim.x >> 5;
     int lo = -1, hi = X.n;  // g <= 0 at lo (or lo = -1), g > 0 at hi (or hi = n)
-    double b1 = fp64_div(stot - iv[0].sbefore, (double)n);  // the zero when it lies below every value of the bracket
+    double b1 = fp64_div(stot - iv[0].sbefore, n);  // the zero when it lies below every value of the bracket
 #pragma unroll 1
     while (true) {
         const bool last = hi - lo <= 1;
@@ -1129,9 +1214,9 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
             const int j = __popc(__ballot_sync(0xffffffffu, lane < m && S.start[lane] <= i)) +
                           __popc(__ballot_sync(0xffffffffu, lane + 32 < m && S.start[lane + 32] <= i)) - 1;
             const double x = (double)r.v, before = iv[j].sbefore + (r.s_lt - S.pre[j]);
-            below = x * (double)n - (stot - before) <= 0.0;
+            below = x * n - (stot - before) <= 0.0;
             if (last) {
-                const double up = fp64_div(stot - (iv[j].sbefore + (r.s_le - S.pre[j])), (double)n);
+                const double up = fp64_div(stot - (iv[j].sbefore + (r.s_le - S.pre[j])), n);
                 b1 = up > x ? up : x;
             }
         }
@@ -1151,39 +1236,36 @@ __device__ __noinline__ void levels_from_index(const CellIndex& X, SolverShared&
     }
 }
 
-// Gathers the keys of src[0 .. src_cnt) that lie inside the intervals S.niv (all of them when `filtered`),
-// indexes them and finishes the tensor from there: called when they fit kSortN.
-__device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s, const uint32_t* src, int src_cnt, bool filtered,
-                                              float* __restrict__ levels, int32_t* __restrict__ status, unsigned char* smem,
-                                              SolverShared& S)
+// Finishes the tensor from the keys inside the intervals S.niv, which fit kSortN: src[0 .. src_cnt) are these keys as a copy-only pass
+// wrote them (packed; src is 16-byte aligned and readable to the end of its last 16 bytes), or keys among which they are.
+__device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s, const uint32_t* src, int src_cnt, bool packed,
+                                              float* __restrict__ levels, int32_t* __restrict__ status)
 {
     const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
-    uint32_t* list = reinterpret_cast<uint32_t*>(smem + kIndexBytes);
-    if (tid == 0) { S.n_keys = 0; S.internal = 0; }
-    __syncthreads();  // S.nm and S.niv are complete
+    SolverShared& S = sel_state();
+    uint32_t* list = reinterpret_cast<uint32_t*>(smem);
+    __syncthreads();  // S.nm and S.niv are complete; the shared memory is free
     const int m = S.nm;
-    int top = 2;
-    while (top < m) top <<= 1;
-    if (filtered) {
-#pragma unroll 4
-        for (int i = tid; i < src_cnt; i += nt) list[i] = __ldcg(src + i);
+    int c = src_cnt;
+    if (packed) {
+        const uint32_t to = (uint32_t)__cvta_generic_to_shared(list);
+#pragma unroll 1
+        for (int i = tid; i < (src_cnt + 3) / 4; i += nt)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(to + 16u * (uint32_t)i), "l"(src + 4 * (size_t)i) : "memory");
     }
     if (tid < kMaxIv) {
         const bool real = tid < m;
-        S.lo[tid] = real ? S.niv[tid].klo : 0xffffffffu;  // (no key has this value: NaN)
-        S.hi[tid] = real ? S.niv[tid].khi : 0u;
+        S.place[tid].x = real ? S.niv[tid].klo : 0xffffffffu;  // (no key has this value: NaN)
+        S.place[tid].y = real ? S.niv[tid].khi : 0u;
+        S.before[tid] = real ? (uint32_t)S.niv[tid].cbefore : 0xffffffffu;
     }
+    if (tid == 0) { S.n_keys = 0; S.internal = 0; }
+    if (packed) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    auto interval = [&](uint32_t key) -> int {
-        int j = 0;
-#pragma unroll 1
-        for (int step = top >> 1; step >= 1; step >>= 1)
-            if (S.lo[j + step] <= key) j += step;
-        return j;
-    };
-    int c = src_cnt;
-    if (!filtered) {
-        constexpr int kCols = 4;  // loads in flight per thread
+    constexpr int kCols = kIndexCols;
+    if (!packed) {
+        int top = 1;
+        while (top < m) top <<= 1;
 #pragma unroll 1
         for (int i0 = tid & ~31; i0 < src_cnt; i0 += kCols * nt) {
             uint32_t k[kCols];
@@ -1199,17 +1281,18 @@ __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s,
             for (int step = top >> 1; step >= 1; step >>= 1) {
 #pragma unroll
                 for (int u = 0; u < kCols; ++u)
-                    if (S.lo[j[u] + step] <= k[u]) j[u] += step;
+                    if (S.place[j[u] + step].x <= k[u]) j[u] += step;
             }
 #pragma unroll
             for (int u = 0; u < kCols; ++u) {
-                const bool in = i0 + u * nt + lane < src_cnt && k[u] >= S.lo[j[u]] && k[u] <= S.hi[j[u]];
+                const uint4 at = S.place[j[u]];
+                const bool in = i0 + u * nt + lane < src_cnt && k[u] >= at.x && k[u] <= at.y;
                 const unsigned b = __ballot_sync(0xffffffffu, in);
                 if (b) {
                     int pos = 0;
                     if (lane == 0) pos = atomicAdd(&S.n_keys, __popc(b));
                     pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(b & ((1u << lane) - 1u));
-                    if (in && pos < kSortN) list[pos] = k[u];
+                    if (in && pos < kSortN) list[pos] = (uint32_t)j[u] << kRelBits | ((k[u] - at.x) & ((1u << kRelBits) - 1u));
                 }
             }
         }
@@ -1217,46 +1300,64 @@ __device__ __noinline__ void finish_from_keys(TState* st, int t, bool pb, int s,
         c = S.n_keys;
         if (c > kSortN) { c = kSortN; if (tid == 0) S.internal = 1; }
     }
-    const CellIndex X = index_at(smem, c);
+    const CellIndex X = index_at(c);
     if (tid < m) {
         // equal shares of the cells: an interval is a narrow slice of a binade, its values are spread evenly
         const uint32_t share = (uint32_t)(X.nc / m);
-        S.sh[tid] = max(0, 32 - __clz((S.hi[tid] - S.lo[tid]) / share));
-        S.base[tid] = tid * share;
+        S.place[tid].z = tid * share;
+        S.place[tid].w = (uint32_t)max(0, 32 - __clz((S.place[tid].y - S.place[tid].x) / share));
     }
     // (index_build has a barrier before the first cell is asked for)
-    index_build(X, S, [&](int i) { return sel_key_to_float(list[i]); },
-                [&](int i) -> uint32_t {
-                    const uint32_t key = list[i];
-                    const int j = interval(key);
-                    return S.base[j] + ((key - S.lo[j]) >> S.sh[j]);
-                });
+    index_build(X, S, [&](const int (&i)[kCols], uint32_t (&cell)[kCols], float (&v)[kCols]) {
+        uint32_t k[kCols];
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) k[u] = list[i[u]];
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) {
+            const uint4 at = S.place[k[u] >> kRelBits];
+            const uint32_t rel = k[u] & ((1u << kRelBits) - 1u);
+            cell[u] = at.z + (rel >> at.w);
+            v[u] = sel_key_to_float(at.x + rel);
+        }
+    });
     for (int j = tid >> 5; j <= m; j += nt >> 5) {
         // where interval j begins: after the last value of the cell before its first
-        const int a = j == m ? c : (j > 0 ? (int)X.end[S.base[j] - 1] : 0);
-        const double x = warp_sum(index_before_lane(X, a));
+        const int a = j == m ? c : (j > 0 ? (int)X.end[S.place[j].z - 1u] : 0);
+        const double x = index_before(X, a);
         if (lane == 0) {
             S.start[j] = a;
             if (j < m) S.pre[j] = x;
         }
     }
     __syncthreads();
-    levels_from_index(X, S, S.niv, m, pb, s, S.view.n, S.view.stot, t, levels, status);
+    levels_from_index(c, m, pb, s, (double)S.view.n, S.view.stot, t, levels, status);
     if (tid == 0) st->done = 1;
-    __threadfence();
-    __syncthreads();
 }
 
 // Small tensors: all values indexed, the definitions applied directly.
 __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool pb, int s, float* __restrict__ levels,
-                             int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, float tau)
+                             int32_t* __restrict__ status, float tau)
 {
+    SolverShared& S = sel_state();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
-    float* values = reinterpret_cast<float*>(smem + kIndexBytes);  // clipped, -0 as 0, magnitudes for BinGrad-pb
+    float* values = reinterpret_cast<float*>(smem);  // clipped, -0 as 0, magnitudes for BinGrad-pb
     uint32_t kmin = 0xffffffffu, kmax = 0u, sum = 0u;
+    constexpr int kCols = kIndexCols;
+    // (asynchronous copies: one latency of DRAM for all of a thread's values; four at a time in registers, 16,384 values took
+    // 17,000 cycles to load)
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(values);
+    const int whole = ((uintptr_t)src & 15) == 0 ? n & ~3 : 0;
+#pragma unroll 1
+    for (int i = 4 * tid; i < whole; i += 4 * nt)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(to + 4u * (uint32_t)i), "l"(src + i) : "memory");
+#pragma unroll 1
+    for (int i = whole + tid; i < n; i += nt)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(to + 4u * (uint32_t)i), "l"(src + i) : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 #pragma unroll 4
     for (int i = tid; i < n; i += nt) {
-        const float x = __ldg(src + i);
+        const float x = values[i];
         float v = copysignf(fminf(fabsf(x), tau), x) + 0.0f;
         if (pb) v = fabsf(v);
         values[i] = v;
@@ -1268,11 +1369,12 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
     kmin = __reduce_min_sync(0xffffffffu, kmin);
     kmax = __reduce_max_sync(0xffffffffu, kmax);
     sum = __reduce_add_sync(0xffffffffu, sum);
-    if (lane == 0) { S.lo[warp] = kmin; S.hi[warp] = kmax; S.base[warp] = sum; }
+    if (lane == 0) S.place[warp] = make_uint4(kmin, kmax, sum, 0u);
     __syncthreads();
-    kmin = __reduce_min_sync(0xffffffffu, S.lo[lane & (nw - 1)]);
-    kmax = __reduce_max_sync(0xffffffffu, S.hi[lane & (nw - 1)]);
-    sum = __reduce_add_sync(0xffffffffu, lane < nw ? S.base[lane] : 0u);
+    const uint4 w = S.place[lane & (nw - 1)];
+    kmin = __reduce_min_sync(0xffffffffu, w.x);
+    kmax = __reduce_max_sync(0xffffffffu, w.y);
+    sum = __reduce_add_sync(0xffffffffu, lane < nw ? w.z : 0u);
     const float vmin = key_to_float(kmin), vmax = key_to_float(kmax);
     const int nl = pb ? 2 : s;
     // (keys order Inf and NaN beyond the finite values at either end)
@@ -1283,20 +1385,22 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
         if (tid == 0) status[t] = bad ? OGQ_ST_NONFINITE : (!pb || vmax == 0.f) ? OGQ_ST_CONSTANT : 0;
         return;
     }
-    const CellIndex X = index_at(smem, n);
+    const CellIndex X = index_at(n);
     const MagnitudeCells cell((uint32_t)((float)sum / (float)n), fmaxf(fabsf(vmin), fabsf(vmax)), !pb, (uint32_t)X.nc);
-    index_build(X, S, [&](int i) { return values[i]; }, [&](int i) { return cell(values[i]); });
-    if (warp == 0) {
-        // (the total the way index_select adds prefixes up)
-        const double x = warp_sum(index_before_lane(X, n));
-        if (lane == 0) S.offs[0] = x;
-    }
-    __syncthreads();
-    const double stot = S.offs[0];
+    index_build(X, S, [&](const int (&i)[kCols], uint32_t (&c)[kCols], float (&v)[kCols]) {
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) {
+            v[u] = values[i[u]];
+            c[u] = cell(v[u]);
+        }
+    });
+    // (the total the way index_select adds prefixes up)
+    const double stot = index_before(X, n);
+    if (tid < kMaxIv) S.before[tid] = tid == 0 ? 0u : 0xffffffffu;
     if (tid == 0) {
         S.internal = 0;
         S.start[0] = 0; S.start[1] = n; S.pre[0] = 0.0;
-        S.niv[0].cbefore = 0; S.niv[0].sbefore = 0.0;
+        S.niv[0].sbefore = 0.0;
         status[t] = 0;
     }
     if (tid < s) {
@@ -1308,18 +1412,15 @@ __device__ void small_tensor(const float* __restrict__ src, int n, int t, bool p
         l.c_le = n; l.s_le = stot;
     }
     __syncthreads();
-    levels_from_index(X, S, S.niv, 1, pb, s, n, stot, t, levels, status);
+    levels_from_index(n, 1, pb, s, (double)n, stot, t, levels, status);
 }
 
-// Finishes a tensor whose last pass only copied the keys inside its intervals (TState::compact_only): the
-// solver state the previous pass left in global memory is loaded back.  Called by every thread of the CTA.
-__device__ void finish_sorted(TState* st, int t, bool pb, int s, const uint32_t* copied, float* __restrict__ levels,
-                              int32_t* __restrict__ status, unsigned char* smem, SolverShared& S, int cursor_idx)
+// What the finish of a tensor needs from its state, for a tensor whose last pass only copied the keys inside its intervals
+// (TState::compact_only).  Called by every thread of the CTA; every load is issued before the first is waited for.
+// Intervals beyond st->m are not used.
+__device__ __forceinline__ void finish_load(const TState* st, bool pb, int s, SolverShared& S)
 {
-    // (every load is issued before the first is waited for; intervals beyond st->m are not used)
-    const int tid = threadIdx.x, m = __ldcg(&st->m);
-    const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[cursor_idx]);
-    __syncthreads();
+    const int tid = threadIdx.x;
     if (tid < kMaxIv) S.niv[tid] = st->iv[tid];
     if (!pb && tid >= 64 && tid - 64 < s) {
         const ExactLv& e = st->lv[tid - 64];
@@ -1327,12 +1428,21 @@ __device__ void finish_sorted(TState* st, int t, bool pb, int s, const uint32_t*
         l.exact = e.exact; l.key = e.key; l.val = (double)sel_key_to_float(e.key);
         l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
     }
-    if (tid == 0) {
+    if (tid == 96) {
         S.view.n = st->n;
         S.view.stot = st->stot;
-        S.nm = m;
+        S.nm = st->m;
     }
-    finish_from_keys(st, t, pb, s, copied, (int)src_cnt, src_cnt == cand, levels, status, smem, S);
+}
+
+// Finishes such a tensor.
+__device__ void finish_sorted(TState* st, int t, bool pb, int s, const uint32_t* copied, float* __restrict__ levels,
+                              int32_t* __restrict__ status, int cursor_idx)
+{
+    const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[cursor_idx]);
+    __syncthreads();
+    finish_load(st, pb, s, sel_state());
+    finish_from_keys(st, t, pb, s, copied, (int)min(src_cnt, cand), true, levels, status);
 }
 
 // Shared memory of a solver pass: the prefix arrays over the slots, and the raw cells as they come from L2.
@@ -1341,14 +1451,12 @@ constexpr size_t kOffSlotIv = kOffSpre + kSlots * sizeof(double);
 constexpr size_t kOffRawSum = (kOffSlotIv + kSlots + 15) / 16 * 16;
 constexpr size_t kOffRawCnt = kOffRawSum + kCells * sizeof(unsigned long long);
 constexpr size_t kPrefixBytes = kOffRawCnt + kCells * sizeof(uint32_t);
-constexpr size_t kSolveBytes = kIndexBytes + (size_t)kSortN * sizeof(uint32_t);
-static_assert(kPrefixBytes <= kSolveBytes && kSmemBytes <= kSolveBytes, "the finish takes the most shared memory");
+static_assert(kPrefixBytes <= kIndexBytes && kStreamBytes <= kIndexBytes, "the index takes the most shared memory");
 
 // Prefix arrays over all slots of the intervals S.iv (S.view.m of them): counts and sums of the elements
 // before every slot.  A thread takes consecutive slots; a slot's cell is its index minus the number of
 // intervals before it (every interval has one end slot).
-__device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* gcnt, const unsigned long long* glsum, bool first,
-                                              unsigned char* smem)
+__device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* gcnt, const unsigned long long* glsum, bool first)
 {
     uint32_t* cpre = reinterpret_cast<uint32_t*>(smem);
     double* spre = reinterpret_cast<double*>(smem + kOffSpre);
@@ -1436,8 +1544,12 @@ __device__ __forceinline__ void solver_prefix(SolverShared& S, const uint32_t* g
 // L cntM) + t_R] / (R - L), t_L and t_R the contributions of the elements of L's and R's own cells.
 // (sumM - L cntM) / (R - L) decreases in L and in R, so its extremes are taken at matching corners, which
 // stays tight even when a bracket is only known to lie somewhere in a sparse stretch of cells.
-__device__ __noinline__ bool warp_orq_solve(const SolverView& v, const LvInfo& L, const LvInfo& R, LvInfo& out)
+__device__ __noinline__ bool warp_orq_solve(int q, int stride)
 {
+    SolverShared& S = sel_state();
+    const SolverView& v = S.view;
+    const LvInfo &L = S.lv[q - stride], &R = S.lv[q + stride];
+    LvInfo& out = S.lv[q];
     const int lane = threadIdx.x & 31;
     const bool upper = lane >= 16;
     if (L.exact && R.exact && !(R.val > L.val)) {
@@ -1607,9 +1719,9 @@ __device__ __forceinline__ bool refine_marked(SolverShared& S)
 //   round_buf: the keys copied by the pass (null: none were), cap: words of the tensor's key region.
 __device__ __noinline__ bool solver_round(TState* st, int t, uint32_t* gcnt, unsigned long long* glsum, int scheme,
                              int s, float* __restrict__ levels, int32_t* __restrict__ status,
-                             unsigned* nitems, int2* items, const uint32_t* round_buf, bool enqueue,
-                             unsigned char* smem, SolverShared& S, int64_t cap, int round)
+                             unsigned* nitems, int2* items, const uint32_t* round_buf, bool enqueue, int64_t cap, int round)
 {
+    SolverShared& S = sel_state();
     uint32_t* cpre = reinterpret_cast<uint32_t*>(smem);
     double* spre = reinterpret_cast<double*>(smem + kOffSpre);
     const bool pb = scheme == OGQ_BINGRAD_PB;
@@ -1625,7 +1737,7 @@ __device__ __noinline__ bool solver_round(TState* st, int t, uint32_t* gcnt, uns
     }
     for (int i = tid; i < (kSlots + 31) / 32; i += nt) S.marks[i] = 0u;
     __syncthreads();
-    solver_prefix(S, gcnt, glsum, round == 1, smem);
+    solver_prefix(S, gcnt, glsum, round == 1);
     const int nslots = S.view.nslots;
     if (round == 1) {
         if (tid == 0) {
@@ -1649,7 +1761,7 @@ __device__ __noinline__ bool solver_round(TState* st, int t, uint32_t* gcnt, uns
         for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
             const int q = warp;
             if (q < s - 1 && q >= stride && ((q - stride) & (2 * stride - 1)) == 0 && !S.lv[q].exact) {
-                const bool ok = warp_orq_solve(S.view, S.lv[q - stride], S.lv[q + stride], S.lv[q]);
+                const bool ok = warp_orq_solve(q, stride);
                 __syncwarp();
                 if (!ok) {
                     if (lane == 0) S.internal = 1;
@@ -1759,11 +1871,11 @@ __device__ __noinline__ bool solver_round(TState* st, int t, uint32_t* gcnt, uns
     }
     // (the copies of the pass that just ended are complete unless it overflowed its region)
     const bool incomplete = round >= 2 && __ldcg(&st->overflow) != 0;
-    const bool few = S.cand <= kSortN;
+    const bool few = __syncthreads_and(tid >= S.nm || S.niv[tid].khi - S.niv[tid].klo < (1u << kRelBits)) && S.cand <= kSortN;
     if (round >= 2 && few && round_buf != nullptr && !incomplete) {
         const long long src_cnt = (long long)__ldcg(&st->cursor[round & 1]);
         if (src_cnt <= (enqueue ? kScanMax : kScanMaxAlone)) {
-            finish_from_keys(st, t, pb, s, round_buf, (int)src_cnt, src_cnt == S.cand, levels, status, smem, S);
+            finish_from_keys(st, t, pb, s, round_buf, (int)src_cnt, false, levels, status);
             return true;
         }
     }
@@ -1843,30 +1955,31 @@ struct SelArgs {
 // already built in tb): the values inside the intervals are copied to key buffer k (what fits the
 // tensor's region) and, unless copy_only, counted on the cells.
 __device__ __forceinline__ void grad_pass(const SelArgs& A, int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_,
-                                          int k, const Table& tb, uint32_t* hist, unsigned char* smem, bool copy_only,
+                                          int k, bool copy_only,
                                           bool down = false)
 {
     TState* st = A.ws.st + t;
-    uint32_t* stage = reinterpret_cast<uint32_t*>(smem + kSmemHist) + (threadIdx.x >> 5) * kStageCap;
     uint32_t* dst = A.ws.buf[k] + sel_region(tbeg);
     const int64_t cap = sel_region(tend) - sel_region(tbeg);
     const bool mag = A.scheme == OGQ_BINGRAD_PB;
     if (A.tau)
-        stream_round2<true>(A.grad, pb_, pe_, mag, tb, hist, hist + kCells, hist + 2 * kCells, stage, dst, cap,
+        stream_round2<true>(A.grad, pb_, pe_, mag, dst, cap,
                             &st->cursor[k], &st->overflow, copy_only, __ldcg(A.tau + t), down);
     else
-        stream_round2<false>(A.grad, pb_, pe_, mag, tb, hist, hist + kCells, hist + 2 * kCells, stage, dst, cap,
+        stream_round2<false>(A.grad, pb_, pe_, mag, dst, cap,
                              &st->cursor[k], &st->overflow, copy_only, 0.f, down);
 }
 
 // Continues the rounds of one tensor on a single CTA until it is finished (the working set is
 // tiny by then).  Called by the CTA that completed round >= 3.
-__device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table& tb, SolverShared& S)
+__device__ void finish_alone(const SelArgs& A, int t)
 {
+    SolverShared& S = sel_state();
+    Table& tb = sel_table();
     TState* st = A.ws.st + t;
     uint32_t* gcnt = A.ws.gcnt + (size_t)t * kCells;
     unsigned long long* glsum = A.ws.glsum + (size_t)t * kCells;
-    uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+    uint32_t* hist = sel_hist();
     const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
     for (int guard = 0; guard < kMaxRounds; ++guard) {
         const int round = __ldcg(&st->round);
@@ -1874,17 +1987,17 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
         const int64_t cnt = (int64_t)__ldcg(&st->cursor[(round - 1) & 1]);
         const bool copy_only = st->compact_only != 0;
         __syncthreads();
-        if (threadIdx.x == 0) table_from_intervals(tb, st->iv, st->m);
+        table_from_intervals(tb, st->iv, st->m);
         __syncthreads();
         if (!copy_only) zero_hist(hist, tb.ncells);
         __syncthreads();
         if (st->from_grad) {
             // the previous pass's copies did not fit: this pass reads the tensor itself again
             build_prefilter(tb, A.scheme == OGQ_BINGRAD_PB);
-            grad_pass(A, t, tbeg, tend, tbeg, tend, round & 1, tb, hist, smem, copy_only);
+            grad_pass(A, t, tbeg, tend, tbeg, tend, round & 1, copy_only);
         } else {
             Stager stg;
-            stg.stage = reinterpret_cast<uint32_t*>(smem + kSmemHist) + (threadIdx.x >> 5) * kStageCap;
+            stg.stage = sel_stage() + (threadIdx.x >> 5) * kStageCap;
             stg.dst = A.ws.buf[round & 1] + sel_region(tbeg);
             stg.cursor = &st->cursor[round & 1];
             stg.fill = 0;
@@ -1895,7 +2008,7 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
         if (copy_only) {
             __threadfence();
             __syncthreads();
-            finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[round & 1] + sel_region(tbeg), A.levels, A.status, smem, S, round & 1);
+            finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[round & 1] + sel_region(tbeg), A.levels, A.status, round & 1);
             return;
         }
         flush_hist(hist, tb.ncells, gcnt, glsum);
@@ -1903,7 +2016,7 @@ __device__ void finish_alone(const SelArgs& A, int t, unsigned char* smem, Table
         solver_load(st, S, A.scheme == OGQ_BINGRAD_PB, A.s);
         __syncthreads();
         if (solver_round(st, t, gcnt, glsum, A.scheme, A.s, A.levels, A.status, A.ws.nitems, A.ws.items,
-                         A.ws.buf[round & 1] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg), round))
+                         A.ws.buf[round & 1] + sel_region(tbeg), false, sel_region(tend) - sel_region(tbeg), round))
             return;
     }
     if (threadIdx.x == 0) {
@@ -1956,47 +2069,41 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
 
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArgs A)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
-    uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+    uint32_t* hist = sel_hist();
     pdl_wait();
     pdl_launch_dependents();
 
     // Flat CTAs: one chunk of the bucket each.  A piece of a tensor is streamed into the CTA's cells, which
     // are then added to the tensor's global ones.
-    float vmin = 0.f, vmax = 0.f, tau = 0.f;
-    uint32_t nf = 0u;
-    int lo_e = 0;
-    uint32_t* packed_cells = reinterpret_cast<uint32_t*>(smem + kSmemHist);
+    uint32_t* packed_cells = sel_stage();
     const int ncells = pb ? kRound1Mag : kRound1Cells;
     const int64_t lo = (int64_t)blockIdx.x * A.chunk;
     const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
     for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
         if (tend - tbeg <= kSmallN) return;
         TState* st = A.ws.st + t;
-        lo_e = __ldcg(&st->hi_e) - kSelW;
-        tau = A.tau ? __ldcg(A.tau + t) : 0.f;
-        vmin = __int_as_float(0x7f800000);
-        vmax = __int_as_float(0xff800000);
-        nf = 0u;
+        const int lo_e = __ldcg(&st->hi_e) - kSelW;
+        const float tau = A.tau ? __ldcg(A.tau + t) : 0.f;
         __syncthreads();
         zero_hist(hist, ncells);
         for (int i = threadIdx.x; i < kPackedCells; i += kSelThreads) packed_cells[i] = 0u;
         __syncthreads();
         const bool clip = A.tau != nullptr;
+        Round1Out r;
         if (pb) {
-            if (clip) stream_round1<true, true>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
-            else stream_round1<true, false>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
+            if (clip) r = stream_round1<true, true>(A.grad, pb_, pe_, lo_e, tau);
+            else r = stream_round1<true, false>(A.grad, pb_, pe_, lo_e, tau);
         } else {
-            if (clip) stream_round1<false, true>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
-            else stream_round1<false, false>(A.grad, pb_, pe_, lo_e, hist, packed_cells, vmin, vmax, nf, tau);
+            if (clip) r = stream_round1<false, true>(A.grad, pb_, pe_, lo_e, tau);
+            else r = stream_round1<false, false>(A.grad, pb_, pe_, lo_e, tau);
         }
         __syncthreads();
         flush_hist(hist, ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
         // min / max / non-finite: one atomic per warp
-        const uint32_t kmin = __reduce_min_sync(0xffffffffu, float_to_key(vmin));  // +Inf / -Inf when the
-        const uint32_t kmax = __reduce_max_sync(0xffffffffu, float_to_key(vmax));  // thread saw nothing
-        const bool anynf = __any_sync(0xffffffffu, nf != 0u);
+        const uint32_t kmin = __reduce_min_sync(0xffffffffu, float_to_key(r.vmin));  // +Inf / -Inf when the
+        const uint32_t kmax = __reduce_max_sync(0xffffffffu, float_to_key(r.vmax));  // thread saw nothing
+        const bool anynf = __any_sync(0xffffffffu, r.nonfinite != 0u);
         if ((threadIdx.x & 31) == 0) {
             atomicMax(&st->kmin_inv, ~kmin);
             atomicMax(&st->kmax, kmax);
@@ -2026,6 +2133,21 @@ struct Round1Cells {
                                    : (uint32_t)(k < 0 ? mi : mi - (kSelW << kSelM) + kSelW) << 23;
         return neg ? 0x80000000u - bits - (1u << sh) : 0x80000000u + bits;
     }
+    // exact sum of the cell's values: sel_cell_sum for these cells
+    __device__ __forceinline__ double sum(int c, uint32_t cnt, unsigned long long lsum) const
+    {
+        const bool neg = !mag && c < kRound1Mag;
+        const int mi = mag ? c : neg ? kRound1Mag - 1 - c : c - kRound1Mag;
+        const int k = mi - lo_e;
+        const bool fine = (unsigned)k < (unsigned)(kSelW << kSelM);
+        const int e = fine ? lo_e + (k >> kSelM) : k < 0 ? mi : mi - (kSelW << kSelM) + kSelW;
+        const uint32_t first = (e > 0 ? 1u << 23 : 0u) + (fine ? (uint32_t)(k & ((1 << kSelM) - 1)) << (23 - kSelM) : 0u);
+        const uint32_t last = fine ? (1u << (23 - kSelM)) - 1u : (1u << 23) - 1u;
+        // mantissas in units of 2^(max(e, 1) - 150); negative cells have their low bits mirrored
+        const unsigned long long mant = (unsigned long long)cnt * first + (neg ? (unsigned long long)cnt * last - lsum : lsum);
+        const double x = __ull2double_rn(mant) * __hiloint2double((max(e, 1) + 873) << 20, 0);
+        return neg ? -x : x;
+    }
 };
 
 // A level of the first pass: its value, or bounds of its value and the cells [sa, sb] that contain it.
@@ -2037,7 +2159,7 @@ struct Level1 {
 
 constexpr int kCandCells = 512;  // candidate cells the first pass keeps track of
 
-struct Solve1Shared {
+struct __align__(16) Solve1Shared {
     Level1 lv[kMaxLv];
     uint32_t marks[(kRound1Cells + 31) / 32];
     int list[kCandCells], sorted[kCandCells];
@@ -2048,19 +2170,24 @@ struct Solve1Shared {
     int pb_a, pb_b;
 };
 
-constexpr int kSolve1Threads = 1024;
 constexpr size_t kOffCells1 = ((kRound1Cells + 8) * sizeof(double) + 15) / 16 * 16;  // prefix sums, then prefix counts, then the raw cells
 constexpr size_t kOffRawSum1 = (kOffCells1 + (kRound1Cells + 8) * sizeof(uint32_t) + 15) / 16 * 16;
 constexpr size_t kOffRawCnt1 = kOffRawSum1 + kRound1Cells * sizeof(unsigned long long);
 static_assert(kOffRawCnt1 + kRound1Cells * sizeof(uint32_t) <= kIndexBytes, "the index of a small tensor takes more");
 
+constexpr size_t kSolve1Bytes = kSolveBytes + sizeof(Solve1Shared);
+__device__ __forceinline__ Solve1Shared& sel_state1() { return *reinterpret_cast<Solve1Shared*>(smem + kSolveBytes); }
+
 // Q*(L, R) on round 1's cells by the 32 lanes of a warp; see warp_orq_solve for the bounds.
-__device__ __noinline__ void solve1_level(const Round1Cells G, const double* spre, const uint32_t* cpre, double n, const Level1* Lp,
-                                          const Level1* Rp, Level1* out)
+__device__ __noinline__ void solve1_level(int lo_e, double n, int q, int stride)
 {
+    const Round1Cells G{lo_e, false};
+    const double* spre = reinterpret_cast<const double*>(smem);
+    const uint32_t* cpre = reinterpret_cast<const uint32_t*>(smem + kOffCells1);
+    Level1* out = sel_state1().lv + q;
     const int lane = threadIdx.x & 31;
     const bool upper = lane >= 16;
-    const Level1 L = *Lp, R = *Rp;
+    const Level1 L = out[-stride], R = out[stride];
     const bool exact = L.exact && R.exact;
     if (exact && !(R.vlo > L.vlo)) {
         if (lane == 0) *out = L;
@@ -2126,11 +2253,10 @@ __device__ __noinline__ void solve1_level(const Round1Cells G, const double* spr
 // levels, every populated cell in them becomes an interval of round 2.  Small tensors are solved here.
 //   What bounds it: latency and, with several small tensors on an SM, their shared memory (one CTA per SM): 22 us for the 161
 // tensors of the ResNet-50 bucket, 13 for the 38 of VGG-19.
-__global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
+__global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SolverShared S;
-    __shared__ Solve1Shared Q;
+    SolverShared& S = sel_state();
+    Solve1Shared& Q = sel_state1();
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
     const int nl = pb ? 2 : A.s, s = A.s;
     pdl_wait();
@@ -2152,7 +2278,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
             if (tid < nl) A.levels[(int64_t)t * nl + tid] = 0.f;
             if (tid == 0) A.status[t] = OGQ_ST_EMPTY;
         } else {
-            small_tensor(A.grad + tbeg, (int)n, t, pb, s, A.levels, A.status, smem, S,
+            small_tensor(A.grad + tbeg, (int)n, t, pb, s, A.levels, A.status,
                          A.tau ? __ldcg(A.tau + t) : __int_as_float(0x7f800000));
         }
         return;
@@ -2162,24 +2288,24 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
     unsigned long long* raw_sum = reinterpret_cast<unsigned long long*>(smem + kOffRawSum1);
     uint32_t* raw_cnt = reinterpret_cast<uint32_t*>(smem + kOffRawCnt1);
     {
-        constexpr int kC = (kRound1Cells / 4 + kSolve1Threads - 1) / kSolve1Threads,
-                      kL = (kRound1Cells / 2 + kSolve1Threads - 1) / kSolve1Threads;
+        constexpr int kC = (kRound1Cells / 4 + kSolveThreads - 1) / kSolveThreads,
+                      kL = (kRound1Cells / 2 + kSolveThreads - 1) / kSolveThreads;
         uint4 c[kC];
         ulonglong2 l[kL];
 #pragma unroll
         for (int u = 0; u < kC; ++u)
-            if ((tid + u * kSolve1Threads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSolve1Threads);
+            if ((tid + u * kSolveThreads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSolveThreads);
 #pragma unroll
         for (int u = 0; u < kL; ++u)
-            if ((tid + u * kSolve1Threads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSolve1Threads);
+            if ((tid + u * kSolveThreads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSolveThreads);
         if (tid < (kRound1Cells + 31) / 32) Q.marks[tid] = 0u;
         if (tid == 0) { Q.m = 0; Q.fail = 0; Q.runs = 0; Q.cand = 0u; Q.pb_a = 0; Q.pb_b = 0; }
 #pragma unroll
         for (int u = 0; u < kC; ++u)
-            if ((tid + u * kSolve1Threads) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * kSolve1Threads] = c[u];
+            if ((tid + u * kSolveThreads) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * kSolveThreads] = c[u];
 #pragma unroll
         for (int u = 0; u < kL; ++u)
-            if ((tid + u * kSolve1Threads) * 2 < ncells) reinterpret_cast<ulonglong2*>(raw_sum)[tid + u * kSolve1Threads] = l[u];
+            if ((tid + u * kSolveThreads) * 2 < ncells) reinterpret_cast<ulonglong2*>(raw_sum)[tid + u * kSolveThreads] = l[u];
     }
     const bool bad = nonfinite != 0u, constant = !bad && !pb && kmn == kmx;
     if (bad || constant) {
@@ -2194,7 +2320,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
     uint32_t total;
     double stot;
     {
-        const int per = (ncells + kSolve1Threads - 1) / kSolve1Threads;
+        const int per = (ncells + kSolveThreads - 1) / kSolveThreads;
         const int c0 = tid * per < ncells ? tid * per : ncells, c1 = c0 + per < ncells ? c0 + per : ncells;
         uint32_t lc = 0u;
         double ls = 0.0;
@@ -2202,11 +2328,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
         for (int c = c0; c < c1; ++c) {
             const uint32_t k = raw_cnt[c];
             double x = 0.0;
-            if (k) {
-                int sh;
-                const uint32_t key = G.key(c, sh);
-                x = sel_cell_sum(key, sh, k, raw_sum[c]);
-            }
+            if (k) x = G.sum(c, k, raw_sum[c]);
             spre[c] = x;
             lc += k;
             ls += x;
@@ -2239,12 +2361,12 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
     const bool counted = (int64_t)total == n;
     int range_a = 0, range_b = -1;  // this warp's candidate cells
     if (counted && !pb) {
-        static_assert(kSolve1Threads / 32 >= kMaxLv - 1, "one warp per interior level");
+        static_assert(kSolveThreads / 32 >= kMaxLv - 1, "one warp per interior level");
 #pragma unroll 1
         for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
             const int q = warp;
             if (q < s - 1 && q >= stride && ((q - stride) & (2 * stride - 1)) == 0) {
-                solve1_level(G, spre, cpre, (double)n, Q.lv + q - stride, Q.lv + q + stride, Q.lv + q);
+                solve1_level(G.lo_e, (double)n, q, stride);
                 if (!Q.lv[q].exact) {
                     range_a = Q.lv[q].sa;
                     range_b = Q.lv[q].sb;
@@ -2257,7 +2379,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
         // bracket of the sign change of g(x) = x n - sum_{|v| >= x} |v|, evaluated at the lower edge of every cell
         int a = 0, b = 0;
 #pragma unroll 1
-        for (int c = tid; c < ncells; c += kSolve1Threads) {
+        for (int c = tid; c < ncells; c += kSolveThreads) {
             int sh;
             const double x = (double)sel_key_to_float(G.key(c, sh));
             if (!(x < INFINITY)) continue;
@@ -2304,7 +2426,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
         return;
     }
     const uint32_t cand = Q.cand;
-    const bool compact_only = cand <= (uint32_t)kSortN && (int64_t)cand <= sel_region(tend) - sel_region(tbeg);
+    bool compact_only = cand <= (uint32_t)kSortN && (int64_t)cand <= sel_region(tend) - sel_region(tbeg);
     // the candidate cells in order
     int my_rank = 0;
     const bool mine = tid < m && m <= kCandCells;
@@ -2360,12 +2482,14 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
         __syncthreads();
         ncells_next = Q.cells_at[runs];
         fits = ncells_next <= kCells;
+        bool narrow = true;
         if (fits && tid < runs) {
             const int len = Q.first[tid + 1] - Q.first[tid], c = Q.sorted[Q.first[tid]];
             int sh;
             Interval iv;
             iv.klo = G.key(c, sh);
             iv.khi = iv.klo + ((uint32_t)len << sh) - 1u;
+            narrow = (unsigned long long)len << sh <= 1ull << kRelBits;
             const int rr = len <= share ? 31 - __clz(share / len) : 0;
             iv.sh = sh - rr;
             iv.ncell = len << rr;
@@ -2375,6 +2499,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
             iv.sbefore = spre[c];
             st->iv[tid] = iv;
         }
+        compact_only = __syncthreads_and(narrow) && compact_only;
     }
     if (!fits) {
         // candidates scattered over too many cells: the general pass, which joins them up
@@ -2388,8 +2513,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
             l.c_lt = 0; l.s_lt = 0.0; l.c_le = 0; l.s_le = 0.0;
         }
         if (tid == 0) { S.view.m = pb ? 3 : 6; S.view.n = n; S.view.stot = 0.0; }
-        solver_round(st, t, gcnt, glsum, A.scheme, s, A.levels, A.status, A.ws.nitems, A.ws.items, nullptr, false, smem, S,
-                     sel_region(tend) - sel_region(tbeg), 1);
+        solver_round(st, t, gcnt, glsum, A.scheme, s, A.levels, A.status, A.ws.nitems, A.ws.items, nullptr, false, sel_region(tend) - sel_region(tbeg), 1);
         return;
     }
     if (single && mine) {
@@ -2414,7 +2538,7 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
         e.c_lt = l.c_lt; e.c_le = l.c_le; e.s_lt = l.s_lt; e.s_le = l.s_le;
     }
     if (!compact_only)
-        for (int i = tid; i < ncells_next; i += kSolve1Threads) { gcnt[i] = 0u; glsum[i] = 0ull; }
+        for (int i = tid; i < ncells_next; i += kSolveThreads) { gcnt[i] = 0u; glsum[i] = 0ull; }
     if (tid == 96) {
         st->m = runs;
         st->cand = cand;
@@ -2425,10 +2549,9 @@ __global__ void __launch_bounds__(kSolve1Threads) k_sel_solve1(SelArgs A)
 
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArgs A)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ Table tb;
+    Table& tb = sel_table();
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
-    uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+    uint32_t* hist = sel_hist();
     pdl_wait();
     pdl_launch_dependents();
     // Second pass over a piece: builds the tensor's interval table and prefilter, clears the CTA's cells,
@@ -2442,52 +2565,49 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
         TState* st = A.ws.st + t;
         if (__ldcg(&st->done)) return;  // settled in round 1
         __syncthreads();
-        table_from_intervals_cta(tb, st->iv, __ldcg(&st->m));
+        table_from_intervals(tb, st->iv, __ldcg(&st->m));
         __syncthreads();
         build_prefilter(tb, pb);
         const bool copy_only = __ldcg(&st->compact_only) != 0;
         if (!copy_only) zero_hist(hist, tb.ncells);
         __syncthreads();
-        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, tb, hist, smem, copy_only, down);
+        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, copy_only, down);
         __syncthreads();
         if (!copy_only) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
     }, down);
 }
 
-// What follows round 2, one CTA per tensor: the sorting finish when round 2 only copied, else a solver pass;
-// tensors of up to kAloneN elements that are then still open are taken to the end here, larger ones get
+// What follows round 2, one CTA per tensor: the finish from the copied keys when round 2 only copied, else a solver pass and
 // work items of the round-3 kernel.
-__global__ void __launch_bounds__(kSelThreads) k_sel_solve2(SelArgs A)
+__global__ void __launch_bounds__(kSolveThreads) k_sel_solve2(SelArgs A)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ Table tb;
-    __shared__ SolverShared S;
+    SolverShared& S = sel_state();
     pdl_wait();
     pdl_launch_dependents();
     const int t = blockIdx.x;
     const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
     const int64_t n = tend - tbeg;
     TState* st = A.ws.st + t;
-    if (n <= kSmallN || __ldcg(&st->done)) return;
-    if (__ldcg(&st->compact_only) != 0) {
-        finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[0] + sel_region(tbeg), A.levels, A.status, smem, S, 0);
+    const int done = __ldcg(&st->done), compact_only = __ldcg(&st->compact_only);
+    const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[0]);
+    finish_load(st, A.scheme == OGQ_BINGRAD_PB, A.s, S);  // (all loads in one go, the decision what to do with them after)
+    if (n <= kSmallN || done) return;
+    if (compact_only != 0) {
+        finish_from_keys(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[0] + sel_region(tbeg), (int)min(src_cnt, cand), true,
+                         A.levels, A.status);
         return;
     }
-    const bool alone = n <= kAloneN;
     const int round = solver_load(st, S, A.scheme == OGQ_BINGRAD_PB, A.s);
-    if (solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s, A.levels, A.status,
-                     A.ws.nitems, A.ws.items, A.ws.buf[0] + sel_region(tbeg), !alone, smem, S, sel_region(tend) - sel_region(tbeg), round))
-        return;
-    if (alone) finish_alone(A, t, smem, tb, S);
+    solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s, A.levels, A.status,
+                 A.ws.nitems, A.ws.items, A.ws.buf[0] + sel_region(tbeg), true, sel_region(tend) - sel_region(tbeg), round);
 }
 
 __global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ Table tb;
-    __shared__ SolverShared S;
+    Table& tb = sel_table();
+    SolverShared& S = sel_state();
     __shared__ int sh_last;
-    uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+    uint32_t* hist = sel_hist();
     pdl_wait();
     pdl_launch_dependents();
     const unsigned nitems = __ldcg(A.ws.nitems);
@@ -2506,17 +2626,17 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
         if (pb_ > cnt) pb_ = cnt;
         if (pe_ > cnt) pe_ = cnt;
         __syncthreads();
-        if (threadIdx.x == 0) table_from_intervals(tb, st->iv, __ldcg(&st->m));
+        table_from_intervals(tb, st->iv, __ldcg(&st->m));
         const bool copy_only = __ldcg(&st->compact_only) != 0;
         __syncthreads();
         if (!copy_only) zero_hist(hist, tb.ncells);
         __syncthreads();
         if (from_grad) {
             build_prefilter(tb, A.scheme == OGQ_BINGRAD_PB);
-            grad_pass(A, t, tbeg, tend, tbeg + pb_, tbeg + pe_, 1, tb, hist, smem, copy_only);
+            grad_pass(A, t, tbeg, tend, tbeg + pb_, tbeg + pe_, 1, copy_only);
         } else {
             Stager stg;
-            stg.stage = reinterpret_cast<uint32_t*>(smem + kSmemHist) + (threadIdx.x >> 5) * kStageCap;
+            stg.stage = sel_stage() + (threadIdx.x >> 5) * kStageCap;
             stg.dst = A.ws.buf[1] + sel_region(tbeg);
             stg.cursor = &st->cursor[1];
             stg.fill = 0;
@@ -2535,13 +2655,13 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
         if (!sh_last) continue;
         __threadfence();
         if (copy_only) {
-            finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[1] + sel_region(tbeg), A.levels, A.status, smem, S, 1);
+            finish_sorted(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[1] + sel_region(tbeg), A.levels, A.status, 1);
             continue;
         }
         const int round = solver_load(st, S, A.scheme == OGQ_BINGRAD_PB, A.s);
         if (!solver_round(st, t, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells, A.scheme, A.s,
-                          A.levels, A.status, A.ws.nitems, A.ws.items, A.ws.buf[1] + sel_region(tbeg), false, smem, S, sel_region(tend) - sel_region(tbeg), round))
-            finish_alone(A, t, smem, tb, S);
+                          A.levels, A.status, A.ws.nitems, A.ws.items, A.ws.buf[1] + sel_region(tbeg), false, sel_region(tend) - sel_region(tbeg), round))
+            finish_alone(A, t);
     }
 }
 
@@ -2556,8 +2676,8 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
-            struct { void (*kernel)(SelArgs); size_t bytes; } limits[] = {{k_sel_round1, kSmemBytes}, {k_sel_round2, kSmemBytes},
-                {k_sel_solve1, kSolveBytes}, {k_sel_solve2, kSolveBytes}, {k_sel_round3, kSolveBytes}};
+            struct { void (*kernel)(SelArgs); size_t bytes; } limits[] = {{k_sel_round1, kSmemBytes}, {k_sel_round2, kStreamBytes},
+                {k_sel_solve1, kSolve1Bytes}, {k_sel_solve2, kSolveBytes}, {k_sel_round3, kSolveBytes}};
             for (auto& l : limits) {
                 e = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes);
                 if (e != cudaSuccess) return e;
@@ -2586,12 +2706,12 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         run("k_sel_prepare", k_sel_prepare, T, 0);
         run("k_sel_round1", k_sel_round1, g.ctas, kSmemBytes);
     }
-    run("k_sel_solve1", k_sel_solve1, T, kSolveBytes, kSolve1Threads);
+    run("k_sel_solve1", k_sel_solve1, T, kSolve1Bytes, kSolveThreads);
     if (streams) {
-        run("k_sel_round2", k_sel_round2, g.ctas, kSmemBytes);
-        run("k_sel_solve2", k_sel_solve2, T, kSolveBytes);
+        run("k_sel_round2", k_sel_round2, g.ctas, kStreamBytes);
+        run("k_sel_solve2", k_sel_solve2, T, kSolveBytes, kSolveThreads);
+        run("k_sel_round3", k_sel_round3, sm_count, kSolveBytes);
     }
-    if (total > kAloneN) run("k_sel_round3", k_sel_round3, sm_count, kSolveBytes);
     return e;
 }
 
