@@ -26,6 +26,9 @@
 // last, took 89 and 125 us for the two rounds of that bucket instead of 61 and 61.
 #include <math.h>
 
+#include <stddef.h>
+
+#include <algorithm>
 #include <atomic>
 
 #include "ogq_common.cuh"
@@ -61,8 +64,9 @@ static_assert(kRound1Cells <= kCells, "round-1 cells exceed the budget");
 struct TState {
     int done, round, m, hi_e;
     unsigned kmin_inv, kmax, nonfinite, arrive;
-    unsigned expected;
-    int compact_only;  // the next pass only copies the keys inside the intervals: they fit one sort
+    unsigned expected;  // CTAs that work on the tensor in round 3; the candidate cells of a tensor copied in their order
+    int compact_only;  // 1: the next pass only copies the keys inside the intervals: they fit one sort.  2: it copies them in order of
+                       // round 1's cells, for k_sel_round3 to select among one cell's at a time
     int overflow;      // the current pass dropped copies that did not fit the tensor's region
     int from_grad;     // the current pass (round >= 3) reads the gradient, not the previous pass's copies
     unsigned long long cursor[2];
@@ -77,8 +81,8 @@ struct SelWs {
     TState* st;                  // [T]
     uint32_t* gcnt;              // [T][kCells]
     unsigned long long* glsum;   // [T][kCells]
-    unsigned* nitems;            // [1] work items of round 3
-    int2* items;                 // [T * kMaxSlices]
+    unsigned* nitems;            // [2] work items of round 3
+    int2* items;                 // [T * kMaxSlices], from the end on: tensors copied in order of their cells (nitems[1] of them)
     uint32_t* buf[2];            // [total / kBufDiv] copied keys: tensor t owns [sel_region(off[t]), sel_region(off[t+1]))
 };
 
@@ -123,17 +127,30 @@ static SelWs sel_carve(void* base, int T, int64_t total)
 // ---------------------------------------------------------------------------
 constexpr size_t kSmemHist = 3 * kCells * sizeof(uint32_t);
 constexpr size_t kSmemStage = kSelWarps * kStageCap * sizeof(uint32_t);
-constexpr size_t kSmemBytes = kSmemHist + kSmemStage;
 
 // Every structure in shared memory that a function which is not inlined uses lies in the dynamic shared memory and is reached
 // through this symbol: through a reference it would be read by generic loads.
 extern __shared__ __align__(16) unsigned char smem[];
 
+// A candidate cell of round 1 of a tensor whose keys are copied in order of these cells; the table lies where the tensor's finer
+// cells would have their sums, the cursors of the cells where they would have their counts.
+constexpr int kCandCells = 512;  // at most
+constexpr int kCellBits = 23;    // log2 of the keys of the widest cell
+static_assert(kCandCells <= 1 << (32 - kCellBits), "a cell's number fits above its keys");
+struct CandCell {
+    double sbefore;      // sum of the elements below it
+    uint32_t cbefore, n; // number of these, and of its own
+    uint32_t klo, base;  // lowest key; where its own begin in the tensor's region (a multiple of four)
+    int sh, pad;         // log2 of the keys
+};
+static_assert(sizeof(CandCell) * kCandCells <= sizeof(unsigned long long) * kCells, "the table fits");
+
 struct Round2Ctx {  // per-CTA constants of round 2, kept in shared memory to spare registers
     uint32_t* dst;
     unsigned long long* cursor;
     uint32_t clear;  // 0x7fffffff when only magnitudes count
-    int nohist;      // copy the keys inside the intervals without counting them
+    int mode;        // TState::compact_only: whether, and in what order, keys are copied without counting them
+    uint32_t* cursors;       // of the candidate cells
     unsigned long long cap;  // words of the tensor's region in the destination buffer
     int* overflow;           // set when a copy did not fit
 };
@@ -147,12 +164,23 @@ struct Table {  // interval lookup table of the tensor being streamed
     int lo_e;                                      // bottom binade of the round-1 fine window
     uint32_t coarse[1024];                         // one bit per block of 2^17 keys that touches an interval
     Round2Ctx ctx;
-    int fills[kSelWarps];                          // values parked per warp
+    int fills[kSolveThreads / 32];                 // values parked per warp
+    int cta_fill;                                  // mode 2: keys in the CTA's buffer
 };
-constexpr size_t kStreamBytes = kSmemBytes + sizeof(Table);
-__device__ __forceinline__ Table& sel_table() { return *reinterpret_cast<Table*>(smem + kSmemBytes); }
+// Mode 2 counts nothing: in place of the cells lie, for every candidate cell, where its keys begin and this CTA's number of
+// them (then their place), and the CTA's buffer.
+struct Partition {
+    uint32_t base[kCandCells], cnt[kCandCells];
+    uint32_t buffer[kSmemHist / sizeof(uint32_t) - 2 * kCandCells];
+};
+constexpr int kCtaBuffer = (int)(kSmemHist / sizeof(uint32_t)) - 2 * kCandCells;
+__device__ __forceinline__ Partition& sel_partition() { return *reinterpret_cast<Partition*>(smem); }
+// the cells, the table, the stages (of the streaming kernels' sixteen warps, or of round 3's 32)
+constexpr size_t kOffStage = kSmemHist + (sizeof(Table) + 15) / 16 * 16;
+constexpr size_t kStreamBytes = kOffStage + kSmemStage;
+__device__ __forceinline__ Table& sel_table() { return *reinterpret_cast<Table*>(smem + kSmemHist); }
 __device__ __forceinline__ uint32_t* sel_hist() { return reinterpret_cast<uint32_t*>(smem); }
-__device__ __forceinline__ uint32_t* sel_stage() { return reinterpret_cast<uint32_t*>(smem + kSmemHist); }
+__device__ __forceinline__ uint32_t* sel_stage() { return reinterpret_cast<uint32_t*>(smem + kOffStage); }
 
 // By the first kMaxIv threads of the CTA (called by all threads; the caller synchronises afterwards).
 __device__ __forceinline__ void table_from_intervals(Table& tb, const Interval* iv, int m)
@@ -236,7 +264,7 @@ __device__ __forceinline__ void warp_visit4(const E* __restrict__ base, int64_t 
     if (a > pe) a = pe;
     int64_t b = pe & ~(int64_t)3;
     if (b < a) b = a;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nt = blockDim.x;
     if (warp == 0) {
         E x[4];
         int nv = 0;
@@ -246,12 +274,12 @@ __device__ __forceinline__ void warp_visit4(const E* __restrict__ base, int64_t 
     }
     const E4* b4 = reinterpret_cast<const E4*>(base);
     const int64_t e = b >> 2;
-    for (int64_t i0 = (a >> 2) + warp * 32; i0 < e; i0 += 4 * kSelThreads) {
+    for (int64_t i0 = (a >> 2) + warp * 32; i0 < e; i0 += 4 * nt) {
         E x[4][4];
         int nx[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + (int64_t)u * kSelThreads + lane;
+            const int64_t i = i0 + (int64_t)u * nt + lane;
             nx[u] = 0;
             if (i < e) {
                 const E4 v = ld4(b4 + i);
@@ -261,7 +289,7 @@ __device__ __forceinline__ void warp_visit4(const E* __restrict__ base, int64_t 
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (i0 + (int64_t)u * kSelThreads < e) f(x[u], nx[u]);
+            if (i0 + (int64_t)u * nt < e) f(x[u], nx[u]);
     }
 }
 
@@ -571,11 +599,37 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
 // yet).  Phase B, whenever the stage fills up: the parked values are turned into keys and classified
 // exactly 32 at a time, so that the expensive part runs with all lanes busy; keys inside an interval
 // are histogrammed and copied out.
+// A key copied in order of the candidate cells: to position `at` of the tensor's region, as its distance from the cell's lowest key.
+__device__ __forceinline__ void partition_store(const Table& tb, uint32_t code, uint32_t at)
+{
+    if (at < tb.ctx.cap) tb.ctx.dst[at] = code & ((1u << kCellBits) - 1u);
+}
+
+// The CTA's buffer to the cells' places, which it reserves with one addition per cell.  Called by every thread.
+__device__ __forceinline__ void partition_flush()
+{
+    Table& tb = sel_table();
+    Partition& part = sel_partition();
+    __syncthreads();
+    const int n = min(tb.cta_fill, kCtaBuffer);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&part.cnt[part.buffer[i] >> kCellBits], 1u);
+    __syncthreads();
+    for (int c = threadIdx.x; c < kCandCells; c += blockDim.x)
+        if (part.cnt[c]) part.cnt[c] = part.base[c] + atomicAdd(tb.ctx.cursors + c, part.cnt[c]);
+    __syncthreads();
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint32_t code = part.buffer[i];
+        partition_store(tb, code, atomicAdd(&part.cnt[code >> kCellBits], 1u));
+    }
+}
+
 // Phase B of round 2 for one warp: classifies `fill` parked values 32 at a time.  A free function
 // taking values, so that the caller's per-warp state can stay in registers.
 __device__ __noinline__ void round2_drain(int fill)
 {
-    const Table* tb = &sel_table();
+    Table* tb = &sel_table();
     const Round2Ctx* ctx = &tb->ctx;
     uint32_t* hist = sel_hist();
     const uint32_t* stage = sel_stage() + (threadIdx.x >> 5) * kStageCap;
@@ -594,11 +648,20 @@ __device__ __noinline__ void round2_drain(int fill)
             int cell, sh;
             uint32_t low, packed;
             in = classify(*tb, key, cell, low, sh, packed);
-            if (ctx->nohist) key = packed;
+            if (ctx->mode == 1) key = packed;
+            else if (ctx->mode == 2) key = (uint32_t)cell << kCellBits | low;
             else if (in) hist_add(hist, hist + kCells, hist + 2 * kCells, cell, low);
         }
         const uint32_t m2 = __ballot_sync(0xffffffffu, in);
-        if (m2) {
+        if (ctx->mode == 2) {
+            // into the CTA's buffer; what that does not hold goes to its cell's place at once
+            int pos = 0;
+            if (lane == 0 && m2) pos = atomicAdd(&tb->cta_fill, __popc(m2));
+            pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m2 & lt);
+            Partition& part = sel_partition();
+            if (in && pos < kCtaBuffer) part.buffer[pos] = key;
+            else if (in) partition_store(*tb, key, part.base[key >> kCellBits] + atomicAdd(ctx->cursors + (key >> kCellBits), 1u));
+        } else if (m2) {
             unsigned long long pos = 0;
             if (lane == 0) pos = atomicAdd(ctx->cursor, (unsigned long long)__popc(m2));
             pos = __shfl_sync(0xffffffffu, pos, 0);
@@ -619,7 +682,7 @@ __device__ __noinline__ void round2_drain(int fill)
 // a left shift by the block index brings its bit to the top of the word.
 __device__ __forceinline__ void build_prefilter(Table& tb, bool magnitude_only)
 {
-    for (int i = threadIdx.x; i < 1024; i += kSelThreads) tb.coarse[i] = 0u;
+    for (int i = threadIdx.x; i < 1024; i += blockDim.x) tb.coarse[i] = 0u;
     __syncthreads();
     if ((int)threadIdx.x < tb.m) {
         const uint32_t ba = tb.klo[threadIdx.x] >> 17, bb = tb.khi[threadIdx.x] >> 17;
@@ -685,24 +748,17 @@ struct Round2Warp {
     }
 };
 
-template <bool CLIP>
-__device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64_t pb, int64_t pe,
-                                              bool magnitude_only, uint32_t* dst, int64_t cap, unsigned long long* cursor, int* overflow, bool nohist, float tau, bool down)
+// NT: threads of the CTA; DOWN: from the end of the piece to its beginning.  The table and its Round2Ctx are complete.
+// Inlined: as a function of its own, with what its callers' limits leave it, a pass over 143.7 M elements took 135 us
+// instead of 113.
+template <bool CLIP, int NT, bool DOWN>
+__device__ __forceinline__ void stream_round2(const float* __restrict__ grad, int64_t pb, int64_t pe, float tau)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     Table& tb = sel_table();
-    Round2Ctx& ctx = tb.ctx;
     int* fills = tb.fills;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ctx.dst = dst; ctx.cursor = cursor;
-        ctx.clear = magnitude_only ? 0x7fffffffu : 0xffffffffu;
-        ctx.nohist = nohist ? 1 : 0;
-        ctx.cap = (unsigned long long)cap;
-        ctx.overflow = overflow;
-    }
     if (lane == 0) fills[warp] = 0;
-    __syncthreads();
+    __syncwarp();
     Round2Warp<CLIP> w;
     w.tau = tau;
     w.coarse = (uint32_t)__cvta_generic_to_shared(tb.coarse);
@@ -730,25 +786,25 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
     const float4* g4 = reinterpret_cast<const float4*>(grad);
     const int64_t e = b >> 2;
     int64_t i0 = (a >> 2) + warp * 32;  // the trip counts below are warp-uniform
-    // Trips of 4 x kSelThreads float4 (one contiguous block of kTripBytes per CTA).  One thread asks
+    // Trips of 4 x NT float4 (one contiguous block of 64 NT bytes per CTA).  One thread asks
     // L2 for the block kPrefetchTrips ahead, so that the loads below find their lines there.
     // A lane tests its sixteen values of a trip without branching; the warp then parks the trip's
     // hits in one go (nearly every trip has a hit in some lane, so the divergent parking code is
     // paid once per trip, not once per few values).  `fill` mirrors the stage's fill counter in a
     // register: it is the same in all lanes, so whether to drain first is a uniform decision.
-    const int64_t rest = e - i0 - 3 * kSelThreads - 32;
-    const int64_t trips = rest >= 0 ? rest / (4 * kSelThreads) + 1 : 0, after = i0 + trips * 4 * kSelThreads;
-    const int64_t step = down ? -4 * kSelThreads : 4 * kSelThreads;
-    if (down) i0 += (trips - 1) * 4 * kSelThreads;
+    const int64_t rest = e - i0 - 3 * NT - 32;
+    const int64_t trips = rest >= 0 ? rest / (4 * NT) + 1 : 0, after = i0 + trips * 4 * NT;
+    constexpr int64_t step = DOWN ? -4 * NT : 4 * NT;
+    if (DOWN) i0 += (trips - 1) * 4 * NT;
     // blocks to ask for: thread 0's trips, but for one upwards that the CTA's last warps do not have
-    int64_t pf_left = trips - kPrefetchTrips - (!down && after > e ? 1 : 0);
+    int64_t pf_left = trips - kPrefetchTrips - (!DOWN && after > e ? 1 : 0);
     __syncwarp();
     int fill = *(volatile int*)&fills[warp];
     for (int64_t k = 0; k < trips; ++k, i0 += step) {
-        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(g4 + i0 + kPrefetchTrips * step, kTripBytes);
+        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(g4 + i0 + kPrefetchTrips * step, 4u * NT * 16u);
         float4 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = __ldg(g4 + i0 + lane + u * kSelThreads);
+        for (int u = 0; u < 4; ++u) x[u] = __ldg(g4 + i0 + lane + u * NT);
         uint32_t hits = 0u;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -758,7 +814,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
             const int tot = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(hits));
             if (tot == 0) break;
             if (fill + tot <= kStageCap) {
-                if (hits) w.park_hits(hits, g4 + i0 + lane, kSelThreads);
+                if (hits) w.park_hits(hits, g4 + i0 + lane, NT);
                 fill += tot;
                 break;
             }
@@ -771,7 +827,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
             }
             // more hits in one trip than the empty stage holds: the first eight values of every lane now
             const uint32_t first = hits & 0xff00u;
-            if (first) w.park_hits(first, g4 + i0 + lane, kSelThreads);
+            if (first) w.park_hits(first, g4 + i0 + lane, NT);
             fill = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(first));
             hits &= 0xffu;
         }
@@ -781,7 +837,7 @@ __device__ __noinline__ void stream_round2(const float* __restrict__ grad, int64
         check();  // the trips above may have left the stage nearly full
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + lane + (int64_t)u * kSelThreads;
+            const int64_t i = i0 + lane + (int64_t)u * NT;
             if (i < e) {
                 const float4 x = __ldg(g4 + i);
                 w.one(x.x); w.one(x.y); w.one(x.z); w.one(x.w);
@@ -817,7 +873,7 @@ __device__ __forceinline__ void stream_piece(const uint32_t* __restrict__ src, i
 
 __device__ __forceinline__ void zero_hist(uint32_t* smem_hist, int ncells)
 {
-    for (int i = threadIdx.x; i < ncells; i += kSelThreads) {
+    for (int i = threadIdx.x; i < ncells; i += blockDim.x) {
         smem_hist[i] = 0u;
         smem_hist[kCells + i] = 0u;
         smem_hist[2 * kCells + i] = 0u;
@@ -827,7 +883,7 @@ __device__ __forceinline__ void zero_hist(uint32_t* smem_hist, int ncells)
 __device__ __forceinline__ void flush_hist(const uint32_t* smem_hist, int ncells, uint32_t* gcnt,
                                            unsigned long long* glsum)
 {
-    for (int i = threadIdx.x; i < ncells; i += kSelThreads) {
+    for (int i = threadIdx.x; i < ncells; i += blockDim.x) {
         const uint32_t c = smem_hist[i];
         if (c) {
             atomicAdd(gcnt + i, c);
@@ -1451,7 +1507,7 @@ constexpr size_t kOffSlotIv = kOffSpre + kSlots * sizeof(double);
 constexpr size_t kOffRawSum = (kOffSlotIv + kSlots + 15) / 16 * 16;
 constexpr size_t kOffRawCnt = kOffRawSum + kCells * sizeof(unsigned long long);
 constexpr size_t kPrefixBytes = kOffRawCnt + kCells * sizeof(uint32_t);
-static_assert(kPrefixBytes <= kIndexBytes && kStreamBytes <= kIndexBytes, "the index takes the most shared memory");
+static_assert(kPrefixBytes <= kIndexBytes && kOffStage + 2 * kSmemStage <= kIndexBytes, "the index takes the most shared memory");
 
 // Prefix arrays over all slots of the intervals S.iv (S.view.m of them): counts and sums of the elements
 // before every slot.  A thread takes consecutive slots; a slot's cell is its index minus the number of
@@ -1953,21 +2009,26 @@ struct SelArgs {
 
 // One pass over grad[pb_, pe_) of tensor t with the tensor's current intervals (table and prefilter
 // already built in tb): the values inside the intervals are copied to key buffer k (what fits the
-// tensor's region) and, unless copy_only, counted on the cells.
+// tensor's region) and, in mode 0, counted on the cells.
+template <int NT>
 __device__ __forceinline__ void grad_pass(const SelArgs& A, int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_,
-                                          int k, bool copy_only,
-                                          bool down = false)
+                                          int k, int mode)
 {
     TState* st = A.ws.st + t;
-    uint32_t* dst = A.ws.buf[k] + sel_region(tbeg);
-    const int64_t cap = sel_region(tend) - sel_region(tbeg);
-    const bool mag = A.scheme == OGQ_BINGRAD_PB;
-    if (A.tau)
-        stream_round2<true>(A.grad, pb_, pe_, mag, dst, cap,
-                            &st->cursor[k], &st->overflow, copy_only, __ldcg(A.tau + t), down);
-    else
-        stream_round2<false>(A.grad, pb_, pe_, mag, dst, cap,
-                             &st->cursor[k], &st->overflow, copy_only, 0.f, down);
+    Round2Ctx& ctx = sel_table().ctx;
+    if (threadIdx.x == 0) {
+        ctx.dst = A.ws.buf[k] + sel_region(tbeg);
+        ctx.cap = (unsigned long long)(sel_region(tend) - sel_region(tbeg));
+        ctx.cursor = &st->cursor[k];
+        ctx.overflow = &st->overflow;
+        ctx.cursors = A.ws.gcnt + (size_t)t * kCells;
+        ctx.clear = A.scheme == OGQ_BINGRAD_PB ? 0x7fffffffu : 0xffffffffu;
+        ctx.mode = mode;
+    }
+    __syncthreads();
+    // (round 2 itself goes against round 1's direction)
+    if (A.tau) stream_round2<true, NT, false>(A.grad, pb_, pe_, __ldcg(A.tau + t));
+    else stream_round2<false, NT, NT == kSelThreads>(A.grad, pb_, pe_, 0.f);
 }
 
 // Continues the rounds of one tensor on a single CTA until it is finished (the working set is
@@ -1994,7 +2055,7 @@ __device__ void finish_alone(const SelArgs& A, int t)
         if (st->from_grad) {
             // the previous pass's copies did not fit: this pass reads the tensor itself again
             build_prefilter(tb, A.scheme == OGQ_BINGRAD_PB);
-            grad_pass(A, t, tbeg, tend, tbeg, tend, round & 1, copy_only);
+            grad_pass<kSolveThreads>(A, t, tbeg, tend, tbeg, tend, round & 1, copy_only);
         } else {
             Stager stg;
             stg.stage = sel_stage() + (threadIdx.x >> 5) * kStageCap;
@@ -2033,7 +2094,7 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
     pdl_launch_dependents();
     const int t = blockIdx.x;
     const int64_t tbeg = __ldg(A.off + t), n = __ldg(A.off + t + 1) - tbeg;
-    if (t == 0 && threadIdx.x == 0) *A.ws.nitems = 0u;
+    if (t == 0 && threadIdx.x == 0) { A.ws.nitems[0] = 0u; A.ws.nitems[1] = 0u; }
     if (n <= kSmallN) return;
     // Anchor of the fine window: largest binade among strided samples, plus two.
     int e = (int)((__float_as_uint(__ldg(A.grad + tbeg + (int64_t)threadIdx.x * n / kSelThreads)) >> 23) & 255u);
@@ -2157,8 +2218,6 @@ struct Level1 {
     int exact, sa, sb;
 };
 
-constexpr int kCandCells = 512;  // candidate cells the first pass keeps track of
-
 struct __align__(16) Solve1Shared {
     Level1 lv[kMaxLv];
     uint32_t marks[(kRound1Cells + 31) / 32];
@@ -2253,7 +2312,7 @@ __device__ __noinline__ void solve1_level(int lo_e, double n, int q, int stride)
 // levels, every populated cell in them becomes an interval of round 2.  Small tensors are solved here.
 //   What bounds it: latency and, with several small tensors on an SM, their shared memory (one CTA per SM): 22 us for the 161
 // tensors of the ResNet-50 bucket, 13 for the 38 of VGG-19.
-__global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
+__global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
 {
     SolverShared& S = sel_state();
     Solve1Shared& Q = sel_state1();
@@ -2429,11 +2488,16 @@ __global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
     bool compact_only = cand <= (uint32_t)kSortN && (int64_t)cand <= sel_region(tend) - sel_region(tbeg);
     // the candidate cells in order
     int my_rank = 0;
+    uint32_t my_base = 0u;  // elements of those before, each rounded up to whole 128-bit words
     const bool mine = tid < m && m <= kCandCells;
     if (mine) {
         const int c = Q.list[tid];
 #pragma unroll 4
-        for (int j = 0; j < m; ++j) my_rank += Q.list[j] < c ? 1 : 0;
+        for (int j = 0; j < m; ++j) {
+            const bool less = Q.list[j] < c;
+            my_rank += less ? 1 : 0;
+            if (cand > (uint32_t)kSortN && less) my_base += (cpre[Q.list[j] + 1] - cpre[Q.list[j]] + 3u) & ~3u;
+        }
     }
     // Intervals of round 2: one per candidate cell when there are few, else one per run of neighbouring cells (of one
     // width); each gets the same share of the new cells.
@@ -2456,7 +2520,10 @@ __global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
         __syncthreads();
         runs = m <= kCandCells ? Q.runs : kMaxIv + 1;
     }
-    int r = runs <= kMaxIv ? 31 - __clz(kCells / runs) : 0;
+    // More candidates than one CTA's index holds, but not more than the copies have room for: round 2 copies them in order of
+    // these cells and k_sel_round3 selects among one cell's at a time.
+    const bool ordered = !pb && cand > (uint32_t)kSortN && (int64_t)cand + 3 * m <= sel_region(tend) - sel_region(tbeg) && runs <= kMaxIv;
+    int r = runs <= kMaxIv && !ordered ? 31 - __clz(kCells / runs) : 0;
     bool fits = runs <= kMaxIv;
     int ncells_next = runs << r;
     if (!single && fits) {
@@ -2475,7 +2542,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
             for (int j = 0; j < runs; ++j) {
                 const int len = Q.first[j + 1] - Q.first[j];
                 Q.cells_at[j] = at;
-                at += len <= share ? len << (31 - __clz(share / len)) : len;
+                at += len <= share && !ordered ? len << (31 - __clz(share / len)) : len;
             }
             Q.cells_at[runs] = at;
         }
@@ -2490,7 +2557,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
             iv.klo = G.key(c, sh);
             iv.khi = iv.klo + ((uint32_t)len << sh) - 1u;
             narrow = (unsigned long long)len << sh <= 1ull << kRelBits;
-            const int rr = len <= share ? 31 - __clz(share / len) : 0;
+            const int rr = len <= share && !ordered ? 31 - __clz(share / len) : 0;
             iv.sh = sh - rr;
             iv.ncell = len << rr;
             iv.cellbase = Q.cells_at[tid];
@@ -2537,12 +2604,28 @@ __global__ void __launch_bounds__(kSolveThreads) k_sel_solve1(SelArgs A)
         e.key = float_to_key((float)l.vlo);
         e.c_lt = l.c_lt; e.c_le = l.c_le; e.s_lt = l.s_lt; e.s_le = l.s_le;
     }
-    if (!compact_only)
+    if (ordered) {
+        if (mine) {
+            const int c = Q.list[tid];
+            CandCell x;
+            x.sbefore = spre[c];
+            x.cbefore = cpre[c];
+            x.n = cpre[c + 1] - cpre[c];
+            x.klo = G.key(c, x.sh);
+            x.base = my_base;
+            x.pad = 0;
+            reinterpret_cast<CandCell*>(glsum)[my_rank] = x;
+            gcnt[tid] = 0u;
+        }
+        if (tid == 0) A.ws.items[(size_t)A.T * kMaxSlices - 1 - atomicAdd(A.ws.nitems + 1, 1u)].x = t;
+    } else if (!compact_only) {
         for (int i = tid; i < ncells_next; i += kSolveThreads) { gcnt[i] = 0u; glsum[i] = 0ull; }
+    }
     if (tid == 96) {
         st->m = runs;
         st->cand = cand;
-        st->compact_only = compact_only ? 1 : 0;
+        if (ordered) st->expected = (unsigned)m;
+        st->compact_only = ordered ? 2 : compact_only ? 1 : 0;
         st->round = 2;
     }
 }
@@ -2568,30 +2651,40 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
         table_from_intervals(tb, st->iv, __ldcg(&st->m));
         __syncthreads();
         build_prefilter(tb, pb);
-        const bool copy_only = __ldcg(&st->compact_only) != 0;
-        if (!copy_only) zero_hist(hist, tb.ncells);
+        const int mode = __ldcg(&st->compact_only);
+        if (mode == 0) zero_hist(hist, tb.ncells);
+        if (mode == 2) {
+            const CandCell* cells = reinterpret_cast<const CandCell*>(A.ws.glsum + (size_t)t * kCells);
+            const int m = (int)__ldcg(&st->expected);
+            for (int i = threadIdx.x; i < kCandCells; i += kSelThreads) {
+                sel_partition().base[i] = i < m ? __ldcg(&cells[i].base) : 0u;
+                sel_partition().cnt[i] = 0u;
+            }
+            if (threadIdx.x == 0) tb.cta_fill = 0;
+        }
         __syncthreads();
-        grad_pass(A, t, tbeg, tend, pb_, pe_, 0, copy_only, down);
+        grad_pass<kSelThreads>(A, t, tbeg, tend, pb_, pe_, 0, mode);
+        if (mode == 2) partition_flush();
         __syncthreads();
-        if (!copy_only) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
+        if (mode == 0) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
     }, down);
 }
 
 // What follows round 2, one CTA per tensor: the finish from the copied keys when round 2 only copied, else a solver pass and
 // work items of the round-3 kernel.
-__global__ void __launch_bounds__(kSolveThreads) k_sel_solve2(SelArgs A)
+__global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve2(SelArgs A)
 {
-    SolverShared& S = sel_state();
     pdl_wait();
     pdl_launch_dependents();
     const int t = blockIdx.x;
+    SolverShared& S = sel_state();
     const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
     const int64_t n = tend - tbeg;
     TState* st = A.ws.st + t;
     const int done = __ldcg(&st->done), compact_only = __ldcg(&st->compact_only);
     const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[0]);
     finish_load(st, A.scheme == OGQ_BINGRAD_PB, A.s, S);  // (all loads in one go, the decision what to do with them after)
-    if (n <= kSmallN || done) return;
+    if (n <= kSmallN || done || compact_only == 2) return;
     if (compact_only != 0) {
         finish_from_keys(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[0] + sel_region(tbeg), (int)min(src_cnt, cand), true,
                          A.levels, A.status);
@@ -2602,7 +2695,247 @@ __global__ void __launch_bounds__(kSolveThreads) k_sel_solve2(SelArgs A)
                  A.ws.nitems, A.ws.items, A.ws.buf[0] + sel_region(tbeg), true, sel_region(tend) - sel_region(tbeg), round);
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
+// ---------------------------------------------------------------------------
+// Tensors with more candidates than one CTA's index holds: their keys lie in order of round 1's candidate cells, whose
+// exact counts and sums are known.  The exact rank of a level, known when its two brackets are, tells the cell; the level is
+// selected among that cell's keys alone, by counts on their upper and then on their lower bits.  A cluster per tensor;
+// the CTAs share out the levels of a depth of Algorithm 1, and where there are fewer levels than CTAs, the keys of a cell.
+//   What bounds it: the latency of a depth, two reads of a cell's keys (80,000 of 50 M values) and three cluster barriers.
+// It takes the place of a finer histogram in round 2, a solver pass on it and a third round.
+// ---------------------------------------------------------------------------
+constexpr int kCluster = 8;     // CTAs: the levels of the last depth of 17
+constexpr int kUpperBits = 11;  // of a key, in the first count
+
+struct __align__(16) CellSelect {
+    uint32_t upper[1 << kUpperBits], lower[1 << (kCellBits - kUpperBits)];
+    LvInfo lv[kMaxLv];
+    unsigned long long part[32], sum;  // of the keys below the upper bits' range, this CTA's share
+    uint32_t warp_n[32];
+    int cell, open, fail;    // the rank's cell, -1: none has it; whether there is a rank (the brackets differ)
+    uint32_t rank;           // of the level
+    uint32_t bin, below, n;  // what bin_of_rank found
+    CandCell cells[kCandCells];
+};
+static_assert(sizeof(CellSelect) <= kIndexBytes, "fits the solver's shared memory");
+
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_address(const void* p, int rank)
+{
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(a) : "r"(rank));
+    return a;
+}
+
+// The bin that holds rank r, from the counts of `group` CTAs from rank `first` on: to Q.bin, Q.below (elements before it) and
+// Q.n (its own).  PER: bins of a thread; c: their counts on return.  Called by every thread; ends with a barrier.
+template <int PER>
+__device__ __forceinline__ void bin_of_rank(CellSelect& Q, const uint32_t* bins, int nbins, int first, int group, uint32_t r, uint32_t (&c)[PER])
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) c[j] = 0u;
+    if (tid * PER < nbins) {
+        static_assert(PER % 2 == 0, "two bins a load");
+        uint32_t x[kCluster][PER];
+#pragma unroll
+        for (int g = 0; g < kCluster; ++g) {  // (all loads before the first is used: one at a time, this took 13,000 cycles)
+#pragma unroll
+            for (int j = 0; j < PER; j += 2) {
+                x[g][j] = x[g][j + 1] = 0u;
+                if (g < group)
+                    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(x[g][j]), "=r"(x[g][j + 1])
+                                 : "r"(cluster_address(bins + tid * PER + j, first + g)));
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < kCluster; ++g)
+#pragma unroll
+            for (int j = 0; j < PER; ++j) c[j] += x[g][j];
+    }
+    uint32_t own = 0u;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) own += c[j];
+    uint32_t inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t nb = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += nb;
+    }
+    if (lane == 31) Q.warp_n[warp] = inc;
+    __syncthreads();
+    uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? Q.warp_n[lane] : 0u) + inc - own;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (before <= r && r - before < c[j]) { Q.bin = (uint32_t)(tid * PER + j); Q.below = before; Q.n = c[j]; }
+        before += c[j];
+    }
+    __syncthreads();
+}
+
+// Sum over the CTA's threads, valid in all of them.
+__device__ __forceinline__ unsigned long long cta_sum(CellSelect& Q, unsigned long long x)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    x = (unsigned long long)warp_sum((long long)x);
+    if (lane == 0) Q.part[warp] = x;
+    __syncthreads();
+    return (unsigned long long)warp_sum((long long)Q.part[lane]);
+}
+
+// Tensor t by the CTAs of a cluster, all of which call this.
+__device__ __noinline__ void tensor_from_cells(const SelArgs& A, int t, int rank)
+{
+    CellSelect& Q = *reinterpret_cast<CellSelect*>(smem);
+    const int tid = threadIdx.x, s = A.s;
+    TState* st = A.ws.st + t;
+    const CandCell* cells = reinterpret_cast<const CandCell*>(A.ws.glsum + (size_t)t * kCells);
+    const uint32_t* keys = A.ws.buf[0] + sel_region(__ldg(A.off + t));
+    uint32_t cb = 0xffffffffu, cn = 0u;  // the candidate cell of this thread
+    static_assert(kCandCells <= kSolveThreads, "a thread per candidate cell");
+    if (tid < kCandCells) {
+        const CandCell x = cells[tid];  // (those beyond the last are not cells)
+        if (tid < (int)__ldcg(&st->expected)) {
+            Q.cells[tid] = x;
+            cb = x.cbefore;
+            cn = x.n;
+        }
+    }
+    if (tid < s) {
+        const ExactLv& e = st->lv[tid];
+        LvInfo& l = Q.lv[tid];
+        l.val = (double)sel_key_to_float(e.key);
+        l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
+    }
+    if (tid == 0) Q.fail = 0;
+    cluster_sync_all();  // (nobody writes into a CTA that is not here yet)
+#pragma unroll 1
+    for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
+        const int group = kCluster * 2 * stride / (s - 1), first = rank / group * group;  // the CTAs that share this one's level
+        const int q = stride * (2 * (rank / group) + 1);
+        const LvInfo &L = Q.lv[q - stride], &R = Q.lv[q + stride];
+        if (tid < 32) {  // (by one warp: the fp64 unit is the bottleneck when all compute the same)
+            const double width = R.val - L.val, nseg = (double)((uint32_t)R.c_le - (uint32_t)L.c_lt);
+            const double a = (R.s_le - L.s_lt) - L.val * nseg;
+            const bool open = width > 0.0;
+            if (tid == 0) {
+                Q.cell = -1;
+                Q.open = open ? 1 : 0;
+                Q.rank = open ? (uint32_t)R.c_le - 1u - (uint32_t)fmin(fmax(floor(a / width), 0.0), nseg - 1.0) : 0u;
+            }
+        }
+        __syncthreads();
+        const bool open = Q.open != 0;
+        const uint32_t p = Q.rank;
+        if (open && cb <= p && p - cb < cn) Q.cell = tid;
+        __syncthreads();
+        const int c = Q.cell;
+        // this CTA's share of the cell's keys
+        int share = 0, sh = kUpperBits;
+        const uint4* src = nullptr;
+        CandCell cell = {};
+        if (c >= 0) {
+            cell = Q.cells[c];
+            sh = cell.sh;
+            const int per = (((int)cell.n + group - 1) / group + 3) & ~3, begin = min((rank - first) * per, (int)cell.n);
+            share = min(per, (int)cell.n - begin);
+            src = reinterpret_cast<const uint4*>(keys + cell.base + begin);
+        }
+        const int low = sh - kUpperBits;  // lower bits
+        auto each = [&](auto f) {
+            constexpr int kCols = 4;  // loads in flight
+#pragma unroll 1
+            for (int i0 = tid; 4 * i0 < share; i0 += kCols * kSolveThreads) {
+                uint4 k[kCols];
+#pragma unroll
+                for (int u = 0; u < kCols; ++u)
+                    if (4 * (i0 + u * kSolveThreads) < share) k[u] = __ldcg(src + i0 + u * kSolveThreads);
+#pragma unroll
+                for (int u = 0; u < kCols; ++u) {
+                    const int left = share - 4 * (i0 + u * kSolveThreads);
+                    if (left > 0) f(k[u].x);
+                    if (left > 1) f(k[u].y);
+                    if (left > 2) f(k[u].z);
+                    if (left > 3) f(k[u].w);
+                }
+            }
+        };
+        for (int i = tid; i < 1 << kUpperBits; i += kSolveThreads) Q.upper[i] = 0u;
+        for (int i = tid; i < 1 << low; i += kSolveThreads) Q.lower[i] = 0u;
+        __syncthreads();
+        each([&](uint32_t k) { atomicAdd(&Q.upper[(k >> low) & ((1u << kUpperBits) - 1u)], 1u); });
+        cluster_sync_all();
+        uint32_t below = 0u, bin = 0u;
+        if (c >= 0) {
+            uint32_t n2[(1 << kUpperBits) / kSolveThreads];
+            bin_of_rank(Q, Q.upper, 1 << kUpperBits, first, group, p - cell.cbefore, n2);
+            below = Q.below;
+            bin = Q.bin;
+        }
+        unsigned long long sum = 0ull;
+        each([&](uint32_t k) {
+            if (k >> low == bin) atomicAdd(&Q.lower[k & ((1u << low) - 1u)], 1u);
+            else if (k >> low < bin) sum += k;
+        });
+        sum = cta_sum(Q, sum);
+        if (tid == 0) Q.sum = sum;
+        cluster_sync_all();
+        if (rank == first) {
+            uint32_t n_lt = 0u;
+            if (c >= 0) {
+                constexpr int kPer = (1 << (kCellBits - kUpperBits)) / kSolveThreads;
+                uint32_t n4[kPer];
+                bin_of_rank(Q, Q.lower, 1 << low, first, group, p - cell.cbefore - below, n4);
+                // the keys of the range that are smaller, from their counts
+                sum = 0ull;
+#pragma unroll
+                for (int j = 0; j < kPer; ++j)
+                    if ((uint32_t)(tid * kPer + j) < Q.bin) sum += (unsigned long long)n4[j] * ((bin << low) + (uint32_t)(tid * kPer + j));
+                if (tid < group) {
+                    unsigned long long x;
+                    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(x) : "r"(cluster_address(&Q.sum, first + tid)));
+                    sum += x;
+                }
+                sum = cta_sum(Q, sum);
+                n_lt = below + Q.below;
+            }
+            if (tid < kCluster) {
+                LvInfo o = L;
+                if (c >= 0) {
+                    o.val = (double)sel_key_to_float(cell.klo + (bin << low) + Q.bin);
+                    o.c_lt = (long long)cell.cbefore + n_lt;
+                    o.c_le = o.c_lt + Q.n;
+                    o.s_lt = cell.sbefore + sel_cell_sum(cell.klo, sh, n_lt, sum);
+                    o.s_le = o.s_lt + o.val * (double)Q.n;
+                }
+                const uint32_t to = cluster_address(&Q.lv[q], tid);
+                auto put = [&](size_t at, auto x) {
+                    asm volatile("st.shared::cluster.b64 [%0], %1;" :: "r"(to + (uint32_t)at), "l"(x) : "memory");
+                };
+                put(offsetof(LvInfo, val), __double_as_longlong(o.val));
+                put(offsetof(LvInfo, c_lt), o.c_lt);
+                put(offsetof(LvInfo, c_le), o.c_le);
+                put(offsetof(LvInfo, s_lt), __double_as_longlong(o.s_lt));
+                put(offsetof(LvInfo, s_le), __double_as_longlong(o.s_le));
+                if (c < 0 && open)  // no candidate cell holds the rank: an inconsistency
+                    asm volatile("st.shared::cluster.b32 [%0], %1;" :: "r"(cluster_address(&Q.fail, tid)), "r"(1) : "memory");
+            }
+        }
+        cluster_sync_all();
+    }
+    if (rank == 0) {
+        if (tid < s) A.levels[(int64_t)t * s + tid] = Q.fail ? 0.f : (float)Q.lv[tid].val;
+        if (tid == 0) {
+            if (Q.fail) A.status[t] |= OGQ_ST_INTERNAL;
+            st->done = 1;
+        }
+    }
+    __syncthreads();
+}
+
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kSolveThreads, 1) k_sel_round3(SelArgs A)
 {
     Table& tb = sel_table();
     SolverShared& S = sel_state();
@@ -2610,7 +2943,9 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
     uint32_t* hist = sel_hist();
     pdl_wait();
     pdl_launch_dependents();
-    const unsigned nitems = __ldcg(A.ws.nitems);
+    const unsigned nitems = __ldcg(A.ws.nitems), ncells = __ldcg(A.ws.nitems + 1);
+    for (unsigned w = blockIdx.x / kCluster; w < ncells; w += gridDim.x / kCluster)
+        tensor_from_cells(A, __ldcg(&A.ws.items[(size_t)A.T * kMaxSlices - 1 - w].x), (int)(blockIdx.x % kCluster));
 
     for (unsigned w = blockIdx.x; w < nitems; w += gridDim.x) {
         const int2 it = A.ws.items[w];
@@ -2633,7 +2968,7 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_round3(SelArgs A)
         __syncthreads();
         if (from_grad) {
             build_prefilter(tb, A.scheme == OGQ_BINGRAD_PB);
-            grad_pass(A, t, tbeg, tend, tbeg + pb_, tbeg + pe_, 1, copy_only);
+            grad_pass<kSolveThreads>(A, t, tbeg, tend, tbeg + pb_, tbeg + pe_, 1, copy_only);
         } else {
             Stager stg;
             stg.stage = sel_stage() + (threadIdx.x >> 5) * kStageCap;
@@ -2676,7 +3011,7 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
-            struct { void (*kernel)(SelArgs); size_t bytes; } limits[] = {{k_sel_round1, kSmemBytes}, {k_sel_round2, kStreamBytes},
+            struct { void (*kernel)(SelArgs); size_t bytes; } limits[] = {{k_sel_round1, kStreamBytes}, {k_sel_round2, kStreamBytes},
                 {k_sel_solve1, kSolve1Bytes}, {k_sel_solve2, kSolveBytes}, {k_sel_round3, kSolveBytes}};
             for (auto& l : limits) {
                 e = cudaFuncSetAttribute(l.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes);
@@ -2704,13 +3039,13 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
     const bool streams = total > kSmallN;  // some tensor may be larger than one CTA settles on its own
     if (streams) {
         run("k_sel_prepare", k_sel_prepare, T, 0);
-        run("k_sel_round1", k_sel_round1, g.ctas, kSmemBytes);
+        run("k_sel_round1", k_sel_round1, g.ctas, kStreamBytes);
     }
     run("k_sel_solve1", k_sel_solve1, T, kSolve1Bytes, kSolveThreads);
     if (streams) {
         run("k_sel_round2", k_sel_round2, g.ctas, kStreamBytes);
         run("k_sel_solve2", k_sel_solve2, T, kSolveBytes, kSolveThreads);
-        run("k_sel_round3", k_sel_round3, sm_count, kSolveBytes);
+        run("k_sel_round3", k_sel_round3, kMaxSlices, kSolveBytes, kSolveThreads);
     }
     return e;
 }
