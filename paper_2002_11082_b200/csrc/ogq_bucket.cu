@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 k_bucket_decode_sum(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
                     int64_t total, int d, int nb, int s, int64_t total_words, float scale, float* __restrict__ outp)
 {
-    extern __shared__ float sh_rows[];  // [kWarps][2][K][kRowStride]
+    extern __shared__ __align__(256) unsigned char sh_rows[];  // [kWarps][2][row_bytes(K)]
     __shared__ const uint32_t* sh_pk[kMaxWorkers];
     __shared__ const float* sh_lp[kMaxWorkers];
     constexpr int R = kRowStride<BITS>, kWords = 8 * BITS;
@@ -334,7 +334,9 @@ k_bucket_decode_sum(const uint32_t* const* __restrict__ packed_k, const float* c
     const int64_t nw = (int64_t)gridDim.x * kWarps, me = (int64_t)blockIdx.x * kWarps + warp;
     const int64_t g_beg = me * ngroups / nw, g_end = (me + 1) * ngroups / nw;
     if (g_beg >= g_end) return;
-    float* rows = sh_rows + warp * 2 * K * R;
+    const uint32_t rb = row_bytes<BITS>(K);
+    unsigned char* rows = sh_rows + (size_t)warp * 2 * rb;
+    const uint32_t rows_at = (uint32_t)__cvta_generic_to_shared(rows);
     const int shift = (int)((reinterpret_cast<uintptr_t>(outp) >> 2) & 3);
     int j = (int)((g_beg << 8) / d), at = (int)((g_beg << 8) - (int64_t)j * d);  // bucket of the group, first element in it
     int j_rows = -1, two_rows = 0;                                               // buckets the rows are of
@@ -344,16 +346,17 @@ k_bucket_decode_sum(const uint32_t* const* __restrict__ packed_k, const float* c
             __syncwarp();
             for (int i = lane; i < (K * R << two); i += 32) {
                 const int q = i % R, kk = i / R, second = kk >= K;
-                rows[i] = __ldcg(sh_lp[second ? kk - K : kk] + (int64_t)(j + second) * s + (q < s ? q : s - 1));
+                const int k = second ? kk - K : kk;
+                reinterpret_cast<float*>(rows + (second ? rb : 0u))[k * R + q] = __ldcg(sh_lp[k] + (int64_t)(j + second) * s + (q < s ? q : s - 1));
             }
             __syncwarp();
             j_rows = j; two_rows = two;
         }
-        const float* mine = rows + (two && lane >= 16 ? K * R : 0);
+        const uint32_t other = two && lane >= 16 ? rb : 0u;
         const int64_t w0 = g * kWords;
         if (g < full) {
             float a[1][8];
-            sum_workers<BITS, 1, false>(K, lane, nullptr, mine, [&](int k, int) { return sh_pk[k] + w0; }, a);
+            sum_workers<BITS, 1, false>(K, lane, 0u, rows_at + other, [&](int k, int) { return sh_pk[k] + w0; }, a);
 #pragma unroll
             for (int e = 0; e < 8; ++e) a[0][e] = __fmul_rn(a[0][e], scale);
             store8(outp + (g << 8) + 8 * lane, shift, lane, a[0]);
@@ -362,6 +365,7 @@ k_bucket_decode_sum(const uint32_t* const* __restrict__ packed_k, const float* c
             if (i0 < total) {
                 const int sh = (int)(i0 * BITS) & 31;
                 const bool more = sh + 8 * BITS > 32 && wi + 1 < total_words;
+                const float* mine = reinterpret_cast<const float*>(rows + other);
                 float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 for (int k = 0; k < K; ++k) {
                     const uint32_t lo = __ldcg(sh_pk[k] + wi), hi = more ? __ldcg(sh_pk[k] + wi + 1) : 0u;
@@ -389,11 +393,12 @@ cudaError_t launch_bucket_decode_sum(const uint32_t* const* d_packed_k, const fl
     const int64_t ngroups = (total + 255) >> 8;
     int64_t ctas = (ngroups + kWarps - 1) / kWarps;
     if (ctas > (int64_t)sm_count * 4) ctas = (int64_t)sm_count * 4;
-    const size_t rows = (size_t)kWarps * 2 * K * (sizeof(float) << bits);
+    size_t rows = 0;
     cudaError_t e = cudaSuccess;
     launch_begin("k_bucket_decode_sum", stream);
 #define OGQ_LAUNCH_BD(B)                                                                                        \
     do {                                                                                                        \
+        rows = (size_t)kWarps * 2 * row_bytes<B>(K);                                                            \
         if (rows > 40 * 1024)                                                                                   \
             e = cudaFuncSetAttribute(k_bucket_decode_sum<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024); \
         if (e == cudaSuccess)                                                                                   \

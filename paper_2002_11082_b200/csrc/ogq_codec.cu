@@ -7,6 +7,7 @@
 // barriers, were 2 us faster where many small tensors follow one another and 8 to 12 % slower in tensors of 100 M elements.)
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "ogq_common.cuh"
@@ -161,24 +162,26 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
     }, CLIP);  // clipped: the threshold's pass went up, the solver's two down and up
 }
 
+constexpr size_t kRowsBytes = 16 * 1024;  // level rows of the server step's tensors: 32 tensors of eight workers of nine levels, two of the most
+constexpr int kMaxTables = 8;             // and tables of sums
+
 // Server step.  A CTA takes a chunk of the flat bucket, its warps the groups in turn: with a run of its own for every warp
 // the workers' streams were read in pieces too short for DRAM (62 instead of 52 us for 25.6 M elements of eight workers,
-// nine levels).  Tensors of more than kEdgeGroups groups in this CTA's chunk go through
-// the CTA's tables in shared memory; the groups of smaller ones, and a tensor's last, partial group, go to one
-// warp each, without a barrier, and read their levels from global memory: 0.6 us of set-up a tensor is what the
-// smallest ones took longest for.
+// nine levels).  The level rows (and tables of sums) of the next `batch` tensors of the chunk are in shared memory at a
+// time: their levels lie one after the other in every worker's array, so they come with one wait, and the groups of
+// these tensors are gone through without barriers.  (Rows of one tensor at a time, with two barriers and a wait for L2 each,
+// and small tensors' levels read from L2 per element: 62 instead of 55 us for nine levels, eight workers and the 161 tensors of the ResNet-50 bucket, 82 instead of 61 for five levels.)
 template <int BITS>
 __global__ void __launch_bounds__(kThreads, kStreamCtas)
 k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
              const int64_t* __restrict__ off, const int64_t* __restrict__ packed_off, int T, int64_t total,
-             int64_t chunk, int s, float scale, float* __restrict__ outp)
+             int64_t chunk, int s, int batch, float scale, float* __restrict__ outp)
 {
+    extern __shared__ __align__(1024) unsigned char sh_mem[];  // tables of sums [kMaxTables][256], then level rows [batch][row_bytes(K)]
     __shared__ const uint32_t* sh_pk[kMaxWorkers];
     __shared__ const float* sh_lv[kMaxWorkers];
-    __shared__ float sh_table[kTableFloats<BITS> ? kTableFloats<BITS> : 1];
-    __shared__ float sh_rows[kMaxWorkers * kRowStride<BITS>];
-    constexpr int kEdgeGroups = 4;
     constexpr int kWords = 8 * BITS;  // words of a group
+    constexpr bool kTable = kTableFloats<BITS> > 0;
     pdl_wait();
     pdl_launch_dependents();
 
@@ -190,76 +193,96 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
         sh_lv[threadIdx.x] = levels_k[threadIdx.x];
     }
     __syncthreads();
-    int turn = 0;  // the warp that takes the next edge group
+    const uint32_t rb = row_bytes<BITS>(K);
+    float* tables = reinterpret_cast<float*>(sh_mem);
+    unsigned char* rows = sh_mem + (kTable ? kMaxTables * 1024 : 0);
+    int t_first = -1;  // the first tensor whose rows are here
+    int turn = 0;      // the warp that takes the next group
 
     for_each_piece(off, T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + 255) >> 8, g_end = (pe - tb + 255) >> 8;
         if (g_beg >= g_end) return;
-        const int64_t pofs = __ldg(packed_off + t);
-        float* dst = outp + tb;
-        // codes above s - 1 (never produced by the quantizer) read the top level
-        auto level = [&](int k, int code) -> float { return __ldcg(sh_lv[k] + (int64_t)t * s + (code < s ? code : s - 1)); };
-
-        const int64_t g_full = (n >> 8) < g_end ? (n >> 8) : g_end;
-        int64_t g_edge = g_beg;
-        if (g_full - g_beg > kEdgeGroups) {
-            g_edge = g_full;
-            __syncthreads();
-            if constexpr (kTableFloats<BITS> > 0)
-                for (int i = threadIdx.x; i < kTableFloats<BITS>; i += kThreads) sh_table[i] = table_entry<BITS>(i, K, level);
-            for (int i = threadIdx.x + (kTableWorkers<BITS> << BITS); i < (K << BITS); i += kThreads)
-                sh_rows[i] = level(i >> BITS, i & ((1 << BITS) - 1));
-            __syncthreads();
-            const int shift = (int)((reinterpret_cast<uintptr_t>(dst) >> 2) & 3);  // floats above a 16-byte boundary
-            const int64_t w0 = pofs + g_beg * kWords;
-            float* dst8 = dst + (g_beg << 8) + 8 * lane;
-            const int ng = (int)(g_full - g_beg);
-            auto write = [&](int gl, float (&a)[8]) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) a[j] = __fmul_rn(a[j], scale);
-                store8(dst8 + (size_t)gl * 256, shift, lane, a);
-            };
-            constexpr int G = 2;       // groups per warp and trip
-            constexpr int kAhead = 8;  // trips between two prefetch requests
-            constexpr int kTrip = G * kWarps;
-            int gl = warp;
-            for (int trip = 0; gl + kWarps < ng; gl += kTrip, ++trip) {
-                // every kAhead trips K threads ask L2 for the workers' words of the kAhead trips after the next
-                // kAhead (no gain at one bit per code)
-                if (BITS >= 2 && (trip & (kAhead - 1)) == 0 && (int)threadIdx.x < K && (trip + 2 * kAhead) * kTrip <= ng)
-                    prefetch_l2(sh_pk[threadIdx.x] + w0 + (int64_t)(trip + kAhead) * kTrip * kWords, kAhead * kTrip * kWords * 4u);
-                float a[G][8];
-                sum_workers<BITS, G, true>(K, lane, sh_table, sh_rows,
-                                     [&](int k, int g) { return sh_pk[k] + w0 + (int64_t)(gl + g * kWarps) * kWords; }, a);
-#pragma unroll
-                for (int g = 0; g < G; ++g) write(gl + g * kWarps, a[g]);
+        if (t_first < 0 || t >= t_first + batch) {
+            if (t_first >= 0) __syncthreads();
+            t_first = t;
+            // row entry `code` of worker k in tensor t + i; codes above s - 1 (never produced by the quantizer) read the top level
+            // (of the tensors that begin in this chunk; batch <= 32)
+            const int nt = __popc(__ballot_sync(0xffffffffu, lane < batch && t + lane < T && __ldg(off + min(t + lane, T)) < hi));
+            for (int i = threadIdx.x; i < (nt * K << BITS); i += kThreads) {
+                const int code = i & ((1 << BITS) - 1), q = i >> BITS, k = q % K, j = q / K;
+                reinterpret_cast<float*>(rows + (size_t)j * rb)[(k << BITS) + code] =
+                    __ldcg(sh_lv[k] + (int64_t)(t + j) * s + (code < s ? code : s - 1));
             }
-            if (gl < ng) {
-                float a[1][8];
-                sum_workers<BITS, 1, true>(K, lane, sh_table, sh_rows, [&](int k, int) { return sh_pk[k] + w0 + (int64_t)gl * kWords; }, a);
-                write(gl, a[0]);
+            __syncthreads();
+            if constexpr (kTable) {
+                for (int i = threadIdx.x; i < nt * 256; i += kThreads) {
+                    const float* row = reinterpret_cast<const float*>(rows + (size_t)(i >> 8) * rb);
+                    tables[i] = table_entry<BITS>(i & 255, K, [&](int k, int code) { return row[(k << BITS) + code]; });
+                }
+                __syncthreads();
             }
         }
+        const int64_t pofs = __ldg(packed_off + t);
+        float* dst = outp + tb;
+        const int slot = t - t_first;
+        const uint32_t row = (uint32_t)__cvta_generic_to_shared(rows) + (uint32_t)slot * rb,
+                       table = (uint32_t)__cvta_generic_to_shared(tables) + (uint32_t)slot * 1024u;
+        const int64_t g_full = (n >> 8) < g_end ? (n >> 8) : g_end;
+        const int ng = g_full > g_beg ? (int)(g_full - g_beg) : 0, all = (int)(g_end - g_beg);
+        const int first = (warp - turn) & (kWarps - 1);
+        turn = (turn + all) & (kWarps - 1);
+        const int shift = (int)((reinterpret_cast<uintptr_t>(dst) >> 2) & 3);  // floats above a 16-byte boundary
+        const int64_t w0 = pofs + g_beg * kWords;
+        float* dst8 = dst + (g_beg << 8) + 8 * lane;
+        auto write = [&](int gl, float (&a)[8]) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) a[j] = __fmul_rn(a[j], scale);
+            store8(dst8 + (size_t)gl * 256, shift, lane, a);
+        };
+        constexpr int G = 2;       // groups per warp and trip
+        constexpr int kAhead = 8;  // trips between two prefetch requests
+        constexpr int kTrip = G * kWarps;
+        int gl = first;
+        for (int trip = 0; gl + kWarps < ng; gl += kTrip, ++trip) {
+            // every kAhead trips K threads ask L2 for the workers' words of the kAhead trips after the next
+            // kAhead (no gain at one bit per code)
+            if (BITS >= 2 && (trip & (kAhead - 1)) == 0 && (int)threadIdx.x < K && (trip + 2 * kAhead) * kTrip <= ng)
+                prefetch_l2(sh_pk[threadIdx.x] + w0 + (int64_t)(trip + kAhead) * kTrip * kWords, kAhead * kTrip * kWords * 4u);
+            float a[G][8];
+            sum_workers<BITS, G, true>(K, lane, table, row,
+                                 [&](int k, int g) { return sh_pk[k] + w0 + (int64_t)(gl + g * kWarps) * kWords; }, a);
+#pragma unroll
+            for (int g = 0; g < G; ++g) write(gl + g * kWarps, a[g]);
+        }
+        if (gl < ng) {
+            float a[1][8];
+            sum_workers<BITS, 1, true>(K, lane, table, row, [&](int k, int) { return sh_pk[k] + w0 + (int64_t)gl * kWords; }, a);
+            write(gl, a[0]);
+        }
 
-        const int64_t region = __ldg(packed_off + t + 1) - pofs;
-        for (int64_t g = g_edge; g < g_end; ++g, turn = (turn + 1) & (kWarps - 1)) {
-            const int64_t i0 = (g << 8) + 8 * lane;
-            if (turn != warp || i0 >= n) continue;
-            const int64_t wi = (i0 * BITS) >> 5;
-            const int sh = (int)(i0 * BITS) & 31;
-            const bool two = sh + 8 * BITS > 32 && wi + 1 < region;
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            for (int k = 0; k < K; ++k) {
-                const uint32_t* p = sh_pk[k] + pofs + wi;
-                const uint32_t a = __ldcg(p), b = two ? __ldcg(p + 1) : 0u;
-                const uint64_t codes = ((uint64_t)b << 32 | a) >> sh;
+        // the tensor's last, partial group
+        if (all > ng && ((ng - first) & (kWarps - 1)) == 0) {
+            const int64_t i0 = (g_full << 8) + 8 * lane;
+            if (i0 < n) {
+                const int64_t region = __ldg(packed_off + t + 1) - pofs, wi = (i0 * BITS) >> 5;
+                const int sh = (int)(i0 * BITS) & 31;
+                const bool two = sh + 8 * BITS > 32 && wi + 1 < region;
+                const float* mine = reinterpret_cast<const float*>(rows + (size_t)slot * rb);
+                float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+                for (int k = 0; k < K; ++k) {
+                    const uint32_t* p = sh_pk[k] + pofs + wi;
+                    const uint32_t a = __ldcg(p), b = two ? __ldcg(p + 1) : 0u;
+                    const uint64_t codes = ((uint64_t)b << 32 | a) >> sh;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[j] = __fadd_rn(acc[j], level(k, (int)(codes >> (j * BITS)) & ((1 << BITS) - 1)));
+                    for (int j = 0; j < 8; ++j)
+                        acc[j] = __fadd_rn(acc[j], mine[(k << BITS) + ((int)(codes >> (j * BITS)) & ((1 << BITS) - 1))]);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (i0 + j < n) dst[i0 + j] = __fmul_rn(acc[j], scale);
             }
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (i0 + j < n) dst[i0 + j] = __fmul_rn(acc[j], scale);
         }
     });
 }
@@ -312,8 +335,12 @@ cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* co
     const int bits = ogq_bits_for_levels(s);
     cudaError_t e = cudaErrorInvalidValue;
 #define OGQ_LAUNCH_U(B)                                                                               \
-    e = launch_pdl(k_unpack_sum<B>, g.ctas, kThreads, 0, stream, d_packed_k, d_levels_k, K, d_off, d_packed_off, T, \
-                   total, g.chunk, s, scale, d_out)
+    {                                                                                                 \
+        const size_t each = row_bytes<B>(K), tables = kTableFloats<B> > 0 ? kMaxTables * 1024 : 0;       \
+        const int batch = (int)std::min<size_t>(std::max<size_t>(kRowsBytes / each, 1), (size_t)(tables ? kMaxTables : 32)); \
+        e = launch_pdl(k_unpack_sum<B>, g.ctas, kThreads, tables + each * batch, stream, d_packed_k, d_levels_k, K, d_off, \
+                       d_packed_off, T, total, g.chunk, s, batch, scale, d_out);                      \
+    }
     launch_begin("k_unpack_sum", stream);
     switch (bits) {
         case 1: OGQ_LAUNCH_U(1); break;

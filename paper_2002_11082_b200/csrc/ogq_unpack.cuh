@@ -54,16 +54,17 @@ __device__ __forceinline__ EightCodes<BITS> load_codes(const uint32_t* __restric
     return c;
 }
 
-// Byte offsets into a level row of the eight codes.
+// Shared addresses of the levels of the eight codes in the row at `row`, a multiple of the row's size (4-bit codes: of 256): it
+// comes in with the instruction that isolates the code.
 template <int BITS>
-__device__ __forceinline__ void code_offsets(const EightCodes<BITS>& c, uint32_t (&o)[8])
+__device__ __forceinline__ void code_addresses(const EightCodes<BITS>& c, uint32_t row, uint32_t (&o)[8])
 {
     if constexpr (BITS == 4) {
         const uint32_t even = (c.lo << 2) & 0x3c3c3c3cu, odd = (c.lo >> 2) & 0x3c3c3c3cu;  // one byte per code, times 4
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            o[2 * j] = __byte_perm(even, 0u, 0x4440 + j);
-            o[2 * j + 1] = __byte_perm(odd, 0u, 0x4440 + j);
+            o[2 * j] = __byte_perm(even, row, 0x7650 + j);
+            o[2 * j + 1] = __byte_perm(odd, row, 0x7650 + j);
         }
     } else {
         constexpr uint32_t mask = ((1u << BITS) - 1u) << 2;
@@ -75,9 +76,17 @@ __device__ __forceinline__ void code_offsets(const EightCodes<BITS>& c, uint32_t
             else if (b + BITS <= 32) x = c.lo >> (b - 2);
             else if (b < 32) x = __funnelshift_r(c.lo, c.hi, b - 2);
             else x = b - 32 < 2 ? c.hi << (2 - (b - 32)) : c.hi >> (b - 34);
-            o[j] = x & mask;
+            o[j] = (x & mask) | row;
         }
     }
+}
+
+template <int OFFSET>
+__device__ __forceinline__ float load_level(uint32_t at)
+{
+    float x;
+    asm("ld.shared.f32 %0, [%1+%2];" : "=f"(x) : "r"(at), "n"(OFFSET));
+    return x;
 }
 
 // Two fp32 additions in one instruction (each rounded to nearest): (a0, a1) += (b0, b1).
@@ -90,16 +99,27 @@ __device__ __forceinline__ void add2(float& a0, float& a1, float b0, float b1)
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a0), "=f"(a1) : "l"(a));
 }
 
-// acc += the levels of one worker's codes; row: its level row.
-template <int BITS>
-__device__ __forceinline__ void add_levels(const EightCodes<BITS>& c, const float* row, float (&acc)[8])
+// acc += the levels of the codes of worker u of those whose rows begin at `row`.
+template <int BITS, int U>
+__device__ __forceinline__ void add_levels(const EightCodes<BITS>& c, uint32_t row, float (&acc)[8])
 {
     uint32_t o[8];
-    code_offsets<BITS>(c, o);
-    const char* r = reinterpret_cast<const char*>(row);
+    code_addresses<BITS>(c, row, o);
 #pragma unroll
     for (int j = 0; j < 8; j += 2)
-        add2(acc[j], acc[j + 1], *reinterpret_cast<const float*>(r + o[j]), *reinterpret_cast<const float*>(r + o[j + 1]));
+        add2(acc[j], acc[j + 1], load_level<U * kRowStride<BITS> * 4>(o[j]), load_level<U * kRowStride<BITS> * 4>(o[j + 1]));
+}
+
+// The workers from U on of a batch of B.
+template <int BITS, int G, int B, int U = 0>
+__device__ __forceinline__ void add_batch(const EightCodes<BITS> (&c)[G][B], int workers, uint32_t row, float (&acc)[G][8])
+{
+    if constexpr (U < B) {
+        if (U >= workers) return;
+#pragma unroll
+        for (int g = 0; g < G; ++g) add_levels<BITS, U>(c[g][U], row, acc[g]);
+        add_batch<BITS, G, B, U + 1>(c, workers, row, acc);
+    }
 }
 
 // Table indices of eight elements from the codes of the kTableWorkers workers of a table (workers that do not
@@ -148,26 +168,30 @@ __device__ __forceinline__ float table_entry(int i, int K, Level level)
     return a;
 }
 
-// The table's sums for eight elements.
-__device__ __forceinline__ void read_table(const uint32_t (&x)[2], const float* table, float (&acc)[8])
+// The table's sums for eight elements; table: its shared address, a multiple of its size.
+__device__ __forceinline__ void read_table(const uint32_t (&x)[2], uint32_t table, float (&acc)[8])
 {
-    const char* r = reinterpret_cast<const char*>(table);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const uint32_t w = x[j >> 2];
         const int b = 8 * (j & 3);
-        acc[j] = *reinterpret_cast<const float*>(r + ((b == 0 ? w << 2 : w >> (b - 2)) & 0x3fcu));
+        acc[j] = load_level<0>(((b == 0 ? w << 2 : w >> (b - 2)) & 0x3fcu) | table);
     }
 }
 
+// Bytes of the level rows of K workers: rows begin at multiples of 256 bytes (see code_addresses).
+template <int BITS>
+__host__ __device__ constexpr uint32_t row_bytes(int K) { return ((uint32_t)K * kRowStride<BITS> * 4u + 255u) & ~255u; }
+
 // Sums of the G groups of 256 elements at word(k, g) (worker k's first word of group g), eight elements of each for
-// this lane.  table (not read unless TABLE), rows: in shared memory.  The words of several workers are loaded before any
+// this lane.  table (not read unless TABLE), rows: shared addresses.  The words of several workers are loaded before any
 // is used.
 template <int BITS, int G, bool TABLE, class Word>
-__device__ __forceinline__ void sum_workers(int K, int lane, const float* table, const float* rows, Word word, float (&acc)[G][8])
+__device__ __forceinline__ void sum_workers(int K, int lane, uint32_t table, uint32_t rows, Word word, float (&acc)[G][8])
 {
     constexpr int W = TABLE ? kTableWorkers<BITS> : 0;
     constexpr int B = BITS == 4 ? 8 : 4;  // workers per batch
+    static_assert(BITS != 4 || B * kRowStride<BITS> * 4 % 256 == 0, "a batch's rows begin at a multiple of 256 bytes");
     int k0 = 0;
     if constexpr (W > 0) {
         uint32_t c[G][W], x[2];
@@ -188,22 +212,21 @@ __device__ __forceinline__ void sum_workers(int K, int lane, const float* table,
             for (int j = 0; j < 8; ++j) acc[g][j] = 0.f;
     }
     for (; k0 < K; k0 += B) {
-        const float* r = rows + k0 * kRowStride<BITS>;
+        const uint32_t r = rows + (uint32_t)k0 * (kRowStride<BITS> * 4u);
+        EightCodes<BITS> c[G][B];
         if (k0 + B <= K) {
-            EightCodes<BITS> c[G][B];
 #pragma unroll
             for (int g = 0; g < G; ++g)
 #pragma unroll
                 for (int u = 0; u < B; ++u) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
-#pragma unroll
-            for (int g = 0; g < G; ++g)
-#pragma unroll
-                for (int u = 0; u < B; ++u) add_levels<BITS>(c[g][u], r + u * kRowStride<BITS>, acc[g]);
+            add_batch<BITS, G, B>(c, B, r, acc);
         } else {
-            for (int k = k0; k < K; ++k, r += kRowStride<BITS>) {
 #pragma unroll
-                for (int g = 0; g < G; ++g) add_levels<BITS>(load_codes<BITS>(word(k, g), lane), r, acc[g]);
-            }
+            for (int u = 0; u < B; ++u)
+                if (k0 + u < K)
+#pragma unroll
+                    for (int g = 0; g < G; ++g) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
+            add_batch<BITS, G, B>(c, K - k0, r, acc);
         }
     }
 }
