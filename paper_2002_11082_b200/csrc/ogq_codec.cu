@@ -163,7 +163,7 @@ k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off,
 }
 
 constexpr size_t kRowsBytes = 16 * 1024;  // level rows of the server step's tensors: 32 tensors of eight workers of nine levels, two of the most
-constexpr int kMaxTables = 8;             // and tables of sums
+constexpr int kMaxTables = 16;            // and tables of sums
 
 // Server step.  A CTA takes a chunk of the flat bucket, its warps the groups in turn: with a run of its own for every warp
 // the workers' streams were read in pieces too short for DRAM (62 instead of 52 us for 25.6 M elements of eight workers,
@@ -180,6 +180,7 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
     extern __shared__ __align__(1024) unsigned char sh_mem[];  // tables of sums [kMaxTables][256], then level rows [batch][row_bytes(K)]
     __shared__ const uint32_t* sh_pk[kMaxWorkers];
     __shared__ const float* sh_lv[kMaxWorkers];
+    static_assert(kThreads == 256, "a thread per entry of a table");
     constexpr int kWords = 8 * BITS;  // words of a group
     constexpr bool kTable = kTableFloats<BITS> > 0;
     pdl_wait();
@@ -203,35 +204,39 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
         const int64_t n = te - tb;
         const int64_t g_beg = (pb - tb + 255) >> 8, g_end = (pe - tb + 255) >> 8;
         if (g_beg >= g_end) return;
+        const int64_t pofs = __ldg(packed_off + t);  // (asked for before the rows are waited for)
         if (t_first < 0 || t >= t_first + batch) {
             if (t_first >= 0) __syncthreads();
             t_first = t;
             // row entry `code` of worker k in tensor t + i; codes above s - 1 (never produced by the quantizer) read the top level
             // (of the tensors that begin in this chunk; batch <= 32)
-            const int nt = __popc(__ballot_sync(0xffffffffu, lane < batch && t + lane < T && __ldg(off + min(t + lane, T)) < hi));
-            for (int i = threadIdx.x; i < (nt * K << BITS); i += kThreads) {
-                const int code = i & ((1 << BITS) - 1), q = i >> BITS, k = q % K, j = q / K;
-                reinterpret_cast<float*>(rows + (size_t)j * rb)[(k << BITS) + code] =
-                    __ldcg(sh_lv[k] + (int64_t)(t + j) * s + (code < s ? code : s - 1));
+            const int most = batch < T - t ? batch : T - t;
+            const int nt = most == 1 ? 1 : __popc(__ballot_sync(0xffffffffu, lane < most && __ldg(off + t + (lane < most ? lane : 0)) < hi));
+            const int width = 32 - __clz(K - 1) + BITS;  // log2 of the entries per tensor, rounded up (K = 1: BITS)
+#pragma unroll 4
+            for (int i = threadIdx.x; i < nt << width; i += kThreads) {
+                const int j = i >> width, q = i & ((1 << width) - 1), k = q >> BITS, code = q & ((1 << BITS) - 1);
+                if (k < K)
+                    reinterpret_cast<float*>(rows + (size_t)j * rb)[q] = __ldcg(sh_lv[k] + (int64_t)(t + j) * s + (code < s ? code : s - 1));
             }
             __syncthreads();
             if constexpr (kTable) {
-                for (int i = threadIdx.x; i < nt * 256; i += kThreads) {
-                    const float* row = reinterpret_cast<const float*>(rows + (size_t)(i >> 8) * rb);
-                    tables[i] = table_entry<BITS>(i & 255, K, [&](int k, int code) { return row[(k << BITS) + code]; });
+                for (int j = 0; j < nt; ++j) {
+                    const float* row = reinterpret_cast<const float*>(rows + (size_t)j * rb);
+                    tables[j * 256 + threadIdx.x] = table_entry<BITS>(threadIdx.x, K, [&](int k, int code) { return row[(k << BITS) + code]; });
                 }
                 __syncthreads();
             }
         }
-        const int64_t pofs = __ldg(packed_off + t);
+        const int all = (int)(g_end - g_beg), first = (warp - turn) & (kWarps - 1);
+        turn = (turn + all) & (kWarps - 1);
+        if (first >= all) return;
         float* dst = outp + tb;
         const int slot = t - t_first;
         const uint32_t row = (uint32_t)__cvta_generic_to_shared(rows) + (uint32_t)slot * rb,
                        table = (uint32_t)__cvta_generic_to_shared(tables) + (uint32_t)slot * 1024u;
         const int64_t g_full = (n >> 8) < g_end ? (n >> 8) : g_end;
-        const int ng = g_full > g_beg ? (int)(g_full - g_beg) : 0, all = (int)(g_end - g_beg);
-        const int first = (warp - turn) & (kWarps - 1);
-        turn = (turn + all) & (kWarps - 1);
+        const int ng = g_full > g_beg ? (int)(g_full - g_beg) : 0;
         const int shift = (int)((reinterpret_cast<uintptr_t>(dst) >> 2) & 3);  // floats above a 16-byte boundary
         const int64_t w0 = pofs + g_beg * kWords;
         float* dst8 = dst + (g_beg << 8) + 8 * lane;
@@ -337,7 +342,7 @@ cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* co
 #define OGQ_LAUNCH_U(B)                                                                               \
     {                                                                                                 \
         const size_t each = row_bytes<B>(K), tables = kTableFloats<B> > 0 ? kMaxTables * 1024 : 0;       \
-        const int batch = (int)std::min<size_t>(std::max<size_t>(kRowsBytes / each, 1), (size_t)(tables ? kMaxTables : 32)); \
+        const int batch = (int)std::min<size_t>(std::max<size_t>(kRowsBytes / each, 1), (size_t)std::min(T, tables ? kMaxTables : 32)); \
         e = launch_pdl(k_unpack_sum<B>, g.ctas, kThreads, tables + each * batch, stream, d_packed_k, d_levels_k, K, d_off, \
                        d_packed_off, T, total, g.chunk, s, batch, scale, d_out);                      \
     }

@@ -220,6 +220,11 @@ __device__ __forceinline__ void sum_workers(int K, int lane, uint32_t table, uin
 #pragma unroll
                 for (int u = 0; u < B; ++u) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
             add_batch<BITS, G, B>(c, B, r, acc);
+        } else if (W == 0 && k0 + 1 == K) {  // (the last one alone, often the only one: few instructions to fetch)
+#pragma unroll
+            for (int g = 0; g < G; ++g) c[g][0] = load_codes<BITS>(word(k0, g), lane);
+#pragma unroll
+            for (int g = 0; g < G; ++g) add_levels<BITS, 0>(c[g][0], r, acc[g]);
         } else {
 #pragma unroll
             for (int u = 0; u < B; ++u)
