@@ -1117,6 +1117,15 @@ constexpr size_t kSolveBytes = kIndexBytes + sizeof(SolverShared);
 static_assert(kIndexBytes % 16 == 0 && sizeof(SolverShared) % 16 == 0, "structures in the dynamic shared memory are aligned");
 __device__ __forceinline__ SolverShared& sel_state() { return *reinterpret_cast<SolverShared*>(smem + kIndexBytes); }
 
+// floor(T), T = sum_{L <= v <= R} (v - L) / (R - L) from the prefix sums s_r and s_l at the ends of a segment of nseg values.  Where T is
+// an integer (always one where nothing lies between L and R), the rounding of the sums may put it a little below:
+// what is within their rounding of the next integer counts as that.
+__device__ __forceinline__ double floor_of_t(double s_r, double s_l, double lval, double width, double nseg)
+{
+    const double low = lval * nseg, a = (s_r - s_l) - low, k = floor(a / width);
+    return (k + 1.0) * width - a <= 0x1p-49 * (fabs(s_r) + fabs(s_l) + fabs(low)) ? k + 1.0 : k;
+}
+
 struct Ranked {
     float v;
     int i_lt, i_le;    // #{values < v}, #{values <= v}
@@ -1225,8 +1234,7 @@ __device__ __noinline__ void levels_from_index(int values, int m, bool pb, int s
                     if (lane == 0) o = L;
                 } else {
                     const double nseg = (double)(le - lt);
-                    const double A = (R.s_le - L.s_lt) - lval * nseg;
-                    const uint32_t k = (uint32_t)fmin(fmax(floor(A / width), 0.0), nseg - 1.0), p = le - 1u - k;
+                    const uint32_t k = (uint32_t)fmin(fmax(floor_of_t(R.s_le, L.s_lt, lval, width, nseg), 0.0), nseg - 1.0), p = le - 1u - k;
                     // the interval that holds rank p: the last one that begins at or before it
                     int j = __popc(__ballot_sync(0xffffffffu, S.before[lane] <= p)) - 1;
                     if (m > 32) j += __popc(__ballot_sync(0xffffffffu, S.before[lane + 32] <= p));
@@ -1619,8 +1627,7 @@ __device__ __noinline__ bool warp_orq_solve(int q, int stride)
     long long pos;
     if (exact) {
         const long long nseg = R.c_le - L.c_lt;
-        const double A = (R.s_le - L.s_lt) - L.val * (double)nseg;
-        long long k = (long long)floor(fp64_div(A, R.val - L.val));
+        long long k = (long long)floor_of_t(R.s_le, L.s_lt, L.val, R.val - L.val, (double)nseg);
         if (k < 0) k = 0;
         if (k > nseg - 1) k = nseg - 1;
         pos = R.c_le - 1 - k;
@@ -2818,12 +2825,11 @@ __device__ __noinline__ void tensor_from_cells(const SelArgs& A, int t, int rank
         const LvInfo &L = Q.lv[q - stride], &R = Q.lv[q + stride];
         if (tid < 32) {  // (by one warp: the fp64 unit is the bottleneck when all compute the same)
             const double width = R.val - L.val, nseg = (double)((uint32_t)R.c_le - (uint32_t)L.c_lt);
-            const double a = (R.s_le - L.s_lt) - L.val * nseg;
             const bool open = width > 0.0;
             if (tid == 0) {
                 Q.cell = -1;
                 Q.open = open ? 1 : 0;
-                Q.rank = open ? (uint32_t)R.c_le - 1u - (uint32_t)fmin(fmax(floor(a / width), 0.0), nseg - 1.0) : 0u;
+                Q.rank = open ? (uint32_t)R.c_le - 1u - (uint32_t)fmin(fmax(floor_of_t(R.s_le, L.s_lt, L.val, width, nseg), 0.0), nseg - 1.0) : 0u;
             }
         }
         __syncthreads();
