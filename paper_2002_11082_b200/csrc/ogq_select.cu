@@ -925,38 +925,42 @@ struct __align__(16) SolverShared {
 
 __device__ __forceinline__ SolverShared& sel_state();
 
-// Exclusive sums of (c, s) over the CTA's threads in thread order; totals in tot_c, tot_s.  Any number of warps.
+// Exclusive sums of (c, s) over the CTA's threads in thread order; totals in tot_c, tot_s.  Any number of warps.  (The warps'
+// sums are added up by one warp: by all of them for themselves, the shuffles of 32 warps took 3200 cycles in all.)
 __device__ __forceinline__ void block_excl_scan(uint32_t& c, double& s, SolverShared& S, uint32_t& tot_c, double& tot_s)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    auto scan = [&](uint32_t& x, double& y) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t nc = __shfl_up_sync(0xffffffffu, x, o);
+            const double ns = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) { x += nc; y = ns + y; }
+        }
+    };
     uint32_t ic = c;
     double is = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t nc = __shfl_up_sync(0xffffffffu, ic, o);
-        const double ns = __shfl_up_sync(0xffffffffu, is, o);
-        if (lane >= o) { ic += nc; is = ns + is; }
-    }
+    scan(ic, is);
     const uint32_t pc = __shfl_up_sync(0xffffffffu, ic, 1);
     const double ps = __shfl_up_sync(0xffffffffu, is, 1);
     __syncthreads();
     if (lane == 31) { S.sc[warp] = ic; S.ss[warp] = is; }
     __syncthreads();
-    uint32_t wc = lane < nw ? S.sc[lane] : 0u;
-    double ws = lane < nw ? S.ss[lane] : 0.0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t nc = __shfl_up_sync(0xffffffffu, wc, o);
-        const double ns = __shfl_up_sync(0xffffffffu, ws, o);
-        if (lane >= o) { wc += nc; ws = ns + ws; }
+    if (warp == 0) {
+        uint32_t wc = lane < nw ? S.sc[lane] : 0u;
+        double ws = lane < nw ? S.ss[lane] : 0.0;
+        scan(wc, ws);
+        __syncwarp();
+        S.sc[lane] = wc;
+        S.ss[lane] = ws;
     }
-    tot_c = __shfl_sync(0xffffffffu, wc, 31);
-    tot_s = __shfl_sync(0xffffffffu, ws, 31);
-    const int before = warp > 0 ? warp - 1 : 0;
-    const uint32_t bc = __shfl_sync(0xffffffffu, wc, before);
-    const double bs = __shfl_sync(0xffffffffu, ws, before);
-    c = (warp > 0 ? bc : 0u) + (lane > 0 ? pc : 0u);
-    s = lane > 0 ? (warp > 0 ? bs + ps : ps) : (warp > 0 ? bs : 0.0);
+    __syncthreads();
+    tot_c = S.sc[31];
+    tot_s = S.ss[31];
+    const uint32_t bc = warp > 0 ? S.sc[warp - 1] : 0u;
+    const double bs = warp > 0 ? S.ss[warp - 1] : 0.0;
+    c = bc + (lane > 0 ? pc : 0u);
+    s = lane > 0 ? (warp > 0 ? bs + ps : ps) : bs;
 }
 
 // ---------------------------------------------------------------------------
@@ -968,7 +972,7 @@ __device__ __forceinline__ void block_excl_scan(uint32_t& c, double& s, SolverSh
 // ---------------------------------------------------------------------------
 struct CellIndex {
     float* sv;      // the values, at padded positions
-    uint32_t* end;  // [nc] position after the last value of every cell; nc = 1024, 2048 ... 16384
+    uint32_t* end;  // [nc] position after the last value of every cell; nc = 1024, 2048 ... 8192
     double* pre;    // [i] sum of the first i << chunk values
     int n, nc, chunk;
 };
@@ -978,7 +982,7 @@ struct CellIndex {
 __device__ __forceinline__ int index_at_word(int i) { return i + ((i >> 4) << 1); }
 
 // Shared memory: the list of the keys, later the prefix sums in its place; cells; values.
-constexpr int kIndexCells = 16384;
+constexpr int kIndexCells = 8192;
 constexpr size_t kOffIndexEnd = (size_t)kSortN * 4 + 16;
 constexpr size_t kOffIndexValues = kOffIndexEnd + (size_t)kIndexCells * 4;
 constexpr size_t kIndexBytes = kOffIndexValues + ((size_t)kSortN / 16 * 18) * 4;
@@ -990,8 +994,8 @@ __device__ __forceinline__ CellIndex index_at(int n)
     X.end = reinterpret_cast<uint32_t*>(smem + kOffIndexEnd);
     X.sv = reinterpret_cast<float*>(smem + kOffIndexValues);
     X.n = n;
-    // two cells or more per value, as far as there are that many (a power of two from 1024 on): clearing and adding up cells
-    // takes longer than selecting in fuller ones saves
+    // two cells or more per value, as far as there are that many (a power of two from 1024 on): clearing and adding up more cells
+    // takes longer than selecting in fuller ones saves (ResNet-50 bucket 147.6 us with 16,384, 146.2 with 8192 and with 4096)
     X.nc = min(max(1 << (32 - __clz(2 * n - 1)), 1024), kIndexCells);
     X.chunk = max(32 - __clz((n - 1) / (int)blockDim.x), 1);
     return X;
@@ -2283,24 +2287,26 @@ __device__ __noinline__ void solve1_level(int lo_e, double n, int q, int stride)
     const double other = __shfl_xor_sync(0xffffffffu, p, 16);
     if (!upper) p = fmin(p, other);
     const uint32_t pos = __double2uint_rn(fmin(fmax(p, 0.0), n - 1.0));
-    // the cells of the two ranks: the last whose prefix does not exceed the rank
-    int lo = 0, hi = G.count() + 1;
-#pragma unroll 1
-    while (__any_sync(0xffffffffu, lo < hi)) {
-        const int step = (hi - lo + 15) >> 4;
-        const int i = lo + (lane & 15) * step;
-        const unsigned b = __ballot_sync(0xffffffffu, i < hi && cpre[i] <= pos);
-        const int k = __popc(upper ? b >> 16 : b & 0xffffu);
-        const int nhi = lo + k * step;
-        if (k > 0) lo += (k - 1) * step + 1;
-        if (nhi < hi) hi = nhi;
-    }
-    const int slot = lo - 1;
+    // the cells of the two ranks: the last whose prefix does not exceed the rank, by 32 probes in each of three steps
+    const uint32_t pos_a = __shfl_sync(0xffffffffu, pos, 0), pos_b = __shfl_sync(0xffffffffu, pos, 16);
+    constexpr int kStep1 = 161, kStep2 = 6;  // (an odd stride: different banks)
+    static_assert(32 * kStep1 > kRound1Cells && 26 * kStep2 + 5 >= kStep1, "the probes reach every cell");
+    const int nc = G.count();
+    int sa = 0, sb = 0;
+    auto probe = [&](int step, int probes) {
+        const int ia = sa + (lane + 1) * step, ib = sb + (lane + 1) * step;
+        const bool a = lane < probes && ia <= nc && cpre[min(ia, nc)] <= pos_a, b = lane < probes && ib <= nc && cpre[min(ib, nc)] <= pos_b;
+        sa += step * __popc(__ballot_sync(0xffffffffu, a));
+        sb += step * __popc(__ballot_sync(0xffffffffu, b));
+    };
+    probe(kStep1, 32);
+    probe(kStep2, 26);
+    probe(1, 5);
+    const int slot = upper ? sb : sa;
     int sh;
     const uint32_t key = G.key(slot, sh);
     const double val = (double)sel_key_to_float(key + (upper ? (1u << sh) - 1u : 0u));
     const double vhi = __shfl_sync(0xffffffffu, val, 16);
-    const int sb = __shfl_sync(0xffffffffu, slot, 16);
     if (lane == 0) {
         out->exact = 0;
         out->vlo = val;
@@ -2349,21 +2355,20 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
         }
         return;
     }
+    constexpr int kC = (kRound1Cells / 4 + kSolveThreads - 1) / kSolveThreads, kL = (kRound1Cells / 2 + kSolveThreads - 1) / kSolveThreads;
+    uint4 c[kC];
+    ulonglong2 l[kL];
+#pragma unroll
+    for (int u = 0; u < kC; ++u)
+        if ((tid + u * kSolveThreads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSolveThreads);
+#pragma unroll
+    for (int u = 0; u < kL; ++u)
+        if ((tid + u * kSolveThreads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSolveThreads);
     double* spre = reinterpret_cast<double*>(smem);
     uint32_t* cpre = reinterpret_cast<uint32_t*>(smem + kOffCells1);
     unsigned long long* raw_sum = reinterpret_cast<unsigned long long*>(smem + kOffRawSum1);
     uint32_t* raw_cnt = reinterpret_cast<uint32_t*>(smem + kOffRawCnt1);
     {
-        constexpr int kC = (kRound1Cells / 4 + kSolveThreads - 1) / kSolveThreads,
-                      kL = (kRound1Cells / 2 + kSolveThreads - 1) / kSolveThreads;
-        uint4 c[kC];
-        ulonglong2 l[kL];
-#pragma unroll
-        for (int u = 0; u < kC; ++u)
-            if ((tid + u * kSolveThreads) * 4 < ncells) c[u] = __ldcg(reinterpret_cast<const uint4*>(gcnt) + tid + u * kSolveThreads);
-#pragma unroll
-        for (int u = 0; u < kL; ++u)
-            if ((tid + u * kSolveThreads) * 2 < ncells) l[u] = __ldcg(reinterpret_cast<const ulonglong2*>(glsum) + tid + u * kSolveThreads);
         if (tid < (kRound1Cells + 31) / 32) Q.marks[tid] = 0u;
         if (tid == 0) { Q.m = 0; Q.fail = 0; Q.runs = 0; Q.cand = 0u; Q.pb_a = 0; Q.pb_b = 0; }
 #pragma unroll
@@ -2461,13 +2466,18 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
     }
     // every populated cell of the ranges, once
 #pragma unroll 1
-    for (int c = range_a + lane; c <= range_b; c += 32) {
-        const uint32_t k = cpre[c + 1] - cpre[c], bit = 1u << (c & 31);
-        if (k && !(atomicOr(&Q.marks[c >> 5], bit) & bit)) {
-            const int i = atomicAdd(&Q.m, 1);
-            if (i < kCandCells) Q.list[i] = c;
-            atomicAdd(&Q.cand, k);
+    for (int base = range_a; base <= range_b; base += 32) {
+        const int c = base + lane;
+        const uint32_t k = c <= range_b ? cpre[c + 1] - cpre[c] : 0u, bit = 1u << (c & 31);
+        const bool fresh = k && !(atomicOr(&Q.marks[c >> 5], bit) & bit);
+        const uint32_t b = __ballot_sync(0xffffffffu, fresh), sum = __reduce_add_sync(0xffffffffu, fresh ? k : 0u);
+        int i = 0;
+        if (lane == 0 && b) {
+            i = atomicAdd(&Q.m, __popc(b));
+            atomicAdd(&Q.cand, sum);
         }
+        i = __shfl_sync(0xffffffffu, i, 0) + __popc(b & ((1u << lane) - 1u));
+        if (fresh && i < kCandCells) Q.list[i] = c;
     }
     __syncthreads();
     const int m = Q.m;
@@ -3051,7 +3061,10 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
     if (streams) {
         run("k_sel_round2", k_sel_round2, g.ctas, kStreamBytes);
         run("k_sel_solve2", k_sel_solve2, T, kSolveBytes, kSolveThreads);
-        run("k_sel_round3", k_sel_round3, kMaxSlices, kSolveBytes, kSolveThreads);
+        // a cluster per tensor that may have that many candidates (its copies have room for an eighth of it); an empty launch of
+        // eight clusters takes 2.9 us, of one 1.5
+        const int64_t clusters = std::min<int64_t>(std::min<int64_t>(T, total / (kBufDiv * kSortN)), kMaxSlices / kCluster);
+        run("k_sel_round3", k_sel_round3, (int)std::max<int64_t>(clusters, 1) * kCluster, kSolveBytes, kSolveThreads);
     }
     return e;
 }
