@@ -212,6 +212,12 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
             // (of the tensors that begin in this chunk; batch <= 32)
             const int most = batch < T - t ? batch : T - t;
             const int nt = most == 1 ? 1 : __popc(__ballot_sync(0xffffffffu, lane < most && __ldg(off + t + (lane < most ? lane : 0)) < hi));
+            if constexpr (kTable) {
+                if (nt == 1)  // one tensor: its table from L2 as well, without a barrier in between
+                    tables[threadIdx.x] = table_entry<BITS>(threadIdx.x, K, [&](int k, int code) {
+                        return __ldcg(sh_lv[k] + (int64_t)t * s + (code < s ? code : s - 1));
+                    });
+            }
             const int width = 32 - __clz(K - 1) + BITS;  // log2 of the entries per tensor, rounded up (K = 1: BITS)
 #pragma unroll 4
             for (int i = threadIdx.x; i < nt << width; i += kThreads) {
@@ -221,11 +227,13 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
             }
             __syncthreads();
             if constexpr (kTable) {
-                for (int j = 0; j < nt; ++j) {
-                    const float* row = reinterpret_cast<const float*>(rows + (size_t)j * rb);
-                    tables[j * 256 + threadIdx.x] = table_entry<BITS>(threadIdx.x, K, [&](int k, int code) { return row[(k << BITS) + code]; });
+                if (nt > 1) {
+                    for (int j = 0; j < nt; ++j) {
+                        const float* row = reinterpret_cast<const float*>(rows + (size_t)j * rb);
+                        tables[j * 256 + threadIdx.x] = table_entry<BITS>(threadIdx.x, K, [&](int k, int code) { return row[(k << BITS) + code]; });
+                    }
+                    __syncthreads();
                 }
-                __syncthreads();
             }
         }
         const int all = (int)(g_end - g_beg), first = (warp - turn) & (kWarps - 1);

@@ -6,24 +6,27 @@
 // count and an exact integer sum of the low key bits.  A launch with one CTA
 // per tensor then solves on the cell prefix sums and leaves a few narrow
 // candidate intervals.  Round 2 streams the bucket again, against round 1's
-// direction, copies the few percent of elements inside the intervals to scratch
-// and histograms them on a finer grid; another launch per tensor solves again, and
-// round 3 and later work on the copied keys only, until every level's rank falls
-// into a single-key cell.  As soon as the elements still in question fit one CTA's
-// sort (kSortN), the next pass only copies them and the tensor is finished from
-// the sorted keys.  Tensors of at most kSmallN elements are not streamed: the
-// first solver launch sorts them in shared memory.  The key buffers hold one eighth
-// of the bucket: a pass whose copies do not fit is repeated on the gradient with
+// direction, and copies the few percent of elements inside the intervals to scratch.  What follows depends on their
+// number:
+//   up to kSortN            round 2 only copies them; one CTA indexes the copied keys and finishes the tensor.
+//   ORQ, more, and room     round 2 copies them in order of round 1's cells; a cluster of CTAs selects every
+//                           level among the keys of the cell that holds its rank (k_sel_round3).
+//   otherwise               round 2 counts them on a finer grid as well; another launch per tensor solves again, and round
+//                           3 and later work on the copied keys only, until every level's rank falls into a single-key
+//                           cell or one CTA's index holds the rest.
+// Tensors of at most kSmallN elements are not streamed: the first solver launch indexes them in shared memory.  The key
+// buffers hold one eighth of the bucket: a pass whose copies do not fit is repeated on the gradient with
 // the narrower intervals.
 //
-// All cross-CTA accumulation is integer (atomic adds, min, max), and the
-// per-tensor prefix sums are built in a fixed order, so results are
-// bit-reproducible.  No kernel waits on another CTA; only round 3, whose slices of
-// a tensor are counted off by an atomic, has its last CTA go on with the solver.
-//   What bounds it: the rounds stream at 4.4 to 4.9 TB/s from DRAM, bound by the latency of their loads at 64 registers a
-// thread and by the integer pipe; the solver launches are bound by the latency of one CTA's fp64 chains and barriers
-// (ResNet-50 bucket, nine levels: 22 and 28 us of 169).  Solving in the streaming kernels, by the CTA that arrived
-// last, took 89 and 125 us for the two rounds of that bucket instead of 61 and 61.
+// All cross-CTA accumulation is integer (atomic adds, min, max), and a rank does not depend on the order in which
+// values reach their cells: counts are exact, sums of what one cell holds are exact but for values of many
+// binades, and an integer T is recognised within their rounding (floor_of_t).  No kernel waits on another CTA but for the
+// clusters of round 3; the slices of a tensor there are counted off by an atomic, and the last CTA goes on with the solver.
+//   What bounds it: the rounds stream at 4.6 to 5.0 TB/s from DRAM, bound by the integer pipe (with every load pinned to one
+// block in the cache round 1 of 143.7 M elements takes 133 us, with its own loads 125); the solver launches are bound by
+// the latency of one CTA's barriers and of code that runs once (ResNet-50 bucket, nine levels: about 21 and 17 of 147 us).
+// Solving in the streaming kernels, by the CTA that arrived last, took 89 and 125 us for the two rounds of that bucket
+// instead of 61 and 61.
 #include <math.h>
 
 #include <stddef.h>
@@ -2323,8 +2326,8 @@ __device__ __noinline__ void solve1_level(int lo_e, double n, int q, int stride)
 
 // One CTA per tensor.  Streamed tensors: prefix sums over round 1's cells, conservative cell ranges of the
 // levels, every populated cell in them becomes an interval of round 2.  Small tensors are solved here.
-//   What bounds it: latency and, with several small tensors on an SM, their shared memory (one CTA per SM): 22 us for the 161
-// tensors of the ResNet-50 bucket, 13 for the 38 of VGG-19.
+//   What bounds it: latency; for the ResNet-50 bucket (21 us, 161 tensors) that of its largest small tensors, whose 16,384 values take
+// 32,000 cycles, a streamed tensor 23,000.
 __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
 {
     SolverShared& S = sel_state();
