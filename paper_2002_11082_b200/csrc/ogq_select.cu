@@ -52,7 +52,6 @@ constexpr int kSelM = 7;           // log2(cells per binade) in the window
 constexpr int kSmallN = 16384;     // tensors up to this size are solved in shared memory
 constexpr int kSortN = 16384;      // candidates from which one CTA finishes a larger tensor
 constexpr int kStageCap = 320;     // per-warp staging entries for compaction
-constexpr int kParkMax = 256;      // values one warp can park between two checks in the tail of round 2 (32 lanes x 8)
 constexpr int kMaxSlices = 64;     // CTAs that share one tensor's copied keys in round 3
 constexpr int kSliceElems = 16384;
 constexpr int kMaxRounds = 32;
@@ -517,14 +516,14 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
     if (tid < (int)(pe - b)) f.one(__ldg(grad + b + tid));
     const float4* g4 = reinterpret_cast<const float4*>(grad);
     const int64_t first = a >> 2, e = b >> 2;
-    const int64_t ntrips = (e - first) / (4 * kSelThreads);  // full trips: the same for every thread
+    const int ntrips = (int)((e - first) / (4 * kSelThreads));  // full trips: the same for every thread
     constexpr int kNp = MAG ? kPackedPerSign : kPackedCells;
     // upwards; downwards behind the clipping threshold's pass, which went up
     constexpr int kStep = CLIP ? -4 * kSelThreads : 4 * kSelThreads;
     const float4* src = g4 + first + tid + (CLIP ? (ntrips - 1) * 4 * kSelThreads : 0);  // this thread's next load
-    int64_t pf_left = ntrips - kPrefetchTrips;                                           // blocks L2 is still to be asked for
-    for (int64_t t0 = 0; t0 < ntrips; t0 += kPackTrips) {
-        const int nt = (int)((ntrips - t0 < kPackTrips) ? ntrips - t0 : kPackTrips);
+    int pf_left = ntrips - kPrefetchTrips;
+    for (int t0 = 0; t0 < ntrips; t0 += kPackTrips) {
+        const int nt = min(ntrips - t0, kPackTrips);
         if (tid == 0) { sh_coarse = 0u; sh_total = 0u; }
         __syncthreads();
         const float4* const period = src;
@@ -593,7 +592,7 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
         __syncthreads();  // everyone has read the totals before they are reset
     }
     __syncthreads();
-    for (int64_t i = first + ntrips * 4 * kSelThreads + tid; i < e; i += kSelThreads) f.template four<false>(__ldg(g4 + i));
+    for (int64_t i = first + (int64_t)ntrips * 4 * kSelThreads + tid; i < e; i += kSelThreads) f.template four<false>(__ldg(g4 + i));
     return Round1Out{f.mn, f.mx, f.nonfinite};
 }
 
@@ -776,16 +775,6 @@ __device__ __forceinline__ void stream_round2(const float* __restrict__ grad, in
         else if (lane >= 4 && lane - 4 < (int)(pe - b)) w.one(__ldg(grad + b + lane - 4));
         __syncwarp();
     }
-    // The tail below parks at most kParkMax values between two checks of the stage's fill.
-    auto check = [&]() {
-        __syncwarp();
-        const int f = *(volatile int*)&fills[warp];
-        if (f > kStageCap - kParkMax) {
-            round2_drain(f);
-            if (lane == 0) fills[warp] = 0;
-            __syncwarp();
-        }
-    };
     const float4* g4 = reinterpret_cast<const float4*>(grad);
     const int64_t e = b >> 2;
     int64_t i0 = (a >> 2) + warp * 32;  // the trip counts below are warp-uniform
@@ -803,21 +792,12 @@ __device__ __forceinline__ void stream_round2(const float* __restrict__ grad, in
     int64_t pf_left = trips - kPrefetchTrips - (!DOWN && after > e ? 1 : 0);
     __syncwarp();
     int fill = *(volatile int*)&fills[warp];
-    for (int64_t k = 0; k < trips; ++k, i0 += step) {
-        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(g4 + i0 + kPrefetchTrips * step, 4u * NT * 16u);
-        float4 x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = __ldg(g4 + i0 + lane + u * NT);
-        uint32_t hits = 0u;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            w.test(x[u].x, hits); w.test(x[u].y, hits); w.test(x[u].z, hits); w.test(x[u].w, hits);
-        }
+    auto park = [&](uint32_t hits, const float4* p) {
         for (;;) {  // one turn, unless the stage has to be drained to make room
             const int tot = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(hits));
             if (tot == 0) break;
             if (fill + tot <= kStageCap) {
-                if (hits) w.park_hits(hits, g4 + i0 + lane, NT);
+                if (hits) w.park_hits(hits, p, NT);
                 fill += tot;
                 break;
             }
@@ -830,24 +810,38 @@ __device__ __forceinline__ void stream_round2(const float* __restrict__ grad, in
             }
             // more hits in one trip than the empty stage holds: the first eight values of every lane now
             const uint32_t first = hits & 0xff00u;
-            if (first) w.park_hits(first, g4 + i0 + lane, NT);
+            if (first) w.park_hits(first, p, NT);
             fill = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(first));
             hits &= 0xffu;
         }
-    }
-    i0 = after;
-    if (i0 < e) {
-        check();  // the trips above may have left the stage nearly full
+    };
+    auto last_trip = [&]() {  // the float4 after the whole trips, some of the four
+        if (after >= e) return;
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = after + lane + u * NT < e ? __ldg(g4 + after + lane + u * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t hits = 0u;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + lane + (int64_t)u * NT;
-            if (i < e) {
-                const float4 x = __ldg(g4 + i);
-                w.one(x.x); w.one(x.y); w.one(x.z); w.one(x.w);
-            }
-            if (u & 1) check();
+            w.test(x[u].x, hits); w.test(x[u].y, hits); w.test(x[u].z, hits); w.test(x[u].w, hits);
+            if (after + lane + u * NT >= e) hits &= ~15u;
         }
+        park(hits, g4 + after + lane);
+    };
+    if (DOWN) last_trip();
+    for (int64_t k = 0; k < trips; ++k, i0 += step) {
+        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(g4 + i0 + kPrefetchTrips * step, 4u * NT * 16u);
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = __ldg(g4 + i0 + lane + u * NT);
+        uint32_t hits = 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            w.test(x[u].x, hits); w.test(x[u].y, hits); w.test(x[u].z, hits); w.test(x[u].w, hits);
+        }
+        park(hits, g4 + i0 + lane);
     }
+    if (!DOWN) last_trip();
     __syncwarp();
     round2_drain(*(volatile int*)&fills[warp]);
 }
@@ -1269,32 +1263,59 @@ __device__ __noinline__ void levels_from_index(int values, int m, bool pb, int s
         if (threadIdx.x == 0 && fail) status[t] |= OGQ_ST_INTERNAL;
         return;
     }
-    // BinGrad-pb: the values with g(x) = x n - sum_{|v| >= x} |v| <= 0 come first; a warp per candidate rank
+    // BinGrad-pb: the values with g(x) = x n - sum_{|v| >= x} |v| <= 0 come first.  Two ranks that enclose the last of them, from the
+    // first value w of every run of positions: what lies below w's cell has at least the sum of the whole runs before
+    // that cell, what lies below w at most that of the runs up to the cell's end.  Then a warp per candidate rank.
+    // (The ranks by rounds of 32 candidates alone took 16,000 cycles for 16,384 values: three rounds and a last selection.)
     const int nw = blockDim.x >> 5;
     int lo = -1, hi = X.n;  // g <= 0 at lo (or lo = -1), g > 0 at hi (or hi = n)
-    double b1 = fp64_div(stot - iv[0].sbefore, n);  // the zero when it lies below every value of the bracket
+    {
+        const int i = (int)threadIdx.x << X.chunk;
+        if (i < X.n) {
+            const double w = (double)X.sv[index_at_word(i)];
+            int c = 0;  // w's cell: the first that ends after i
+#pragma unroll 1
+            for (int step = X.nc >> 1; step >= 1; step >>= 1)
+                if ((int)X.end[c + step - 1] <= i) c += step;
+            const int a = c > 0 ? (int)X.end[c - 1] : 0, b = (int)X.end[c], j = c / (X.nc / m);
+            const double shift = stot - (iv[j].sbefore - S.pre[j]), x = w * n, eps = 1e-11 * (x + stot);
+            if (x - (shift - X.pre[(b + (1 << X.chunk) - 1) >> X.chunk]) < -eps) lo = a;
+            if (x - (shift - X.pre[a >> X.chunk]) > eps) hi = b - 1;
+        }
+        lo = __reduce_max_sync(0xffffffffu, lo);
+        hi = __reduce_min_sync(0xffffffffu, hi);
+        if (lane == 0) { S.sc[warp] = (uint32_t)lo; S.below[warp] = (uint32_t)hi; }
+        __syncthreads();
+        lo = __reduce_max_sync(0xffffffffu, lane < nw ? (int)S.sc[lane] : -1);
+        hi = __reduce_min_sync(0xffffffffu, lane < nw ? (int)S.below[lane] : X.n);
+        __syncthreads();
+    }
+    double b1 = 0.0;
 #pragma unroll 1
     while (true) {
-        const bool last = hi - lo <= 1;
-        const int step = (hi - lo + nw - 1) / nw;
-        const int i = last ? lo : lo + 1 + warp * step;
-        if (last && lo < 0) break;
-        bool below = false;
-        if (i < hi && (!last || warp == 0)) {
+        const bool last = hi - lo <= nw;
+        const int step = last ? 1 : (hi - lo + nw - 1) / nw, i = (last ? lo : lo + 1) + warp * step;
+        bool below = i < 0;
+        if (below) {
+            b1 = fp64_div(stot - iv[0].sbefore, n);  // the zero when it lies below every value of the bracket
+        } else if (i < hi) {
             const Ranked r = index_select(X, i);
             const int j = __popc(__ballot_sync(0xffffffffu, lane < m && S.start[lane] <= i)) +
                           __popc(__ballot_sync(0xffffffffu, lane + 32 < m && S.start[lane + 32] <= i)) - 1;
             const double x = (double)r.v, before = iv[j].sbefore + (r.s_lt - S.pre[j]);
-            below = x * n - (stot - before) <= 0.0;
+            below = x * n - (stot - before) <= 0.0 || (last && warp == 0);  // (at lo, known)
             if (last) {
                 const double up = fp64_div(stot - (iv[j].sbefore + (r.s_le - S.pre[j])), n);
                 b1 = up > x ? up : x;
             }
         }
-        if (last) break;
-        if (lane == 0) S.below[warp] = below ? 1u : 0u;
+        if (lane == 0) { S.below[warp] = below ? 1u : 0u; S.ss[warp] = b1; }
         __syncthreads();
         const int k = __popc(__ballot_sync(0xffffffffu, lane < nw && S.below[lane]));
+        if (last) {
+            b1 = S.ss[k - 1];
+            break;
+        }
         __syncthreads();
         const int nhi = lo + 1 + k * step;
         if (k > 0) lo += 1 + (k - 1) * step;
@@ -2014,7 +2035,8 @@ struct SelArgs {
     const float* tau;  // per-tensor clipping thresholds, or null
     const int64_t* off;
     int T;
-    int64_t total, chunk;
+    int64_t total, chunk;  // chunk 0: shares of equal work (streamed_share)
+    int first;             // the small tensors' launch is the first of the call
     int scheme, s;
     float* levels;
     int32_t* status;
@@ -2100,7 +2122,109 @@ __device__ void finish_alone(const SelArgs& A, int t)
     }
 }
 
-// Clears what the passes over tensor t add to and fixes the tensor's window: one CTA per tensor.
+// The part [lo, hi) of the bucket that this CTA streams.  A piece of a tensor costs its elements and what its set-up and the
+// flush of its cells take, as much as kPieceCost elements; tensors of at most kSmallN elements cost nothing.  Every CTA gets the same
+// share of that sum.  (Equal chunks of the bucket instead: on the ResNet-50 bucket the CTAs of round 1 ended 23 to 40 us after its start, in
+// the median 32, because some had three pieces and some mostly small tensors.)  Worked out by every CTA for itself, from the
+// offsets alone, while the launch before is still running; with more than kMaxShared tensors chunks of the bucket are used.
+constexpr int kPieceCost = 24576;
+constexpr int kMaxShared = 8 * kSelThreads;
+constexpr int kMinShare = 4 * kSelThreads * 4;  // elements per CTA of a small bucket: one trip of the streaming loops
+
+__device__ __forceinline__ void streamed_share(const SelArgs& A, int64_t& lo, int64_t& hi)
+{
+    __shared__ long long sh_sum[kSelWarps], sh_at[2];
+    if (A.chunk > 0) {
+        lo = (int64_t)blockIdx.x * A.chunk;
+        hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
+        return;
+    }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = (A.T + kSelThreads - 1) / kSelThreads, t0 = min(tid * per, A.T), t1 = min(t0 + per, A.T);
+    auto cost = [&](int t) -> long long {
+        const long long n = __ldg(A.off + t + 1) - __ldg(A.off + t);
+        return n <= kSmallN ? 0 : t > 0 ? n + kPieceCost : n;
+    };
+    long long own = 0;
+    for (int t = t0; t < t1; ++t) own += cost(t);
+    long long inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long nb = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += nb;
+    }
+    if (lane == 31) sh_sum[warp] = inc;
+    if (tid < 2) sh_at[tid] = A.total;  // (a share that ends, or begins, behind the last streamed tensor)
+    __syncthreads();
+    const long long all = lane < kSelWarps ? sh_sum[lane] : 0;
+    long long pos = warp_sum(lane < warp ? all : 0ll) + inc - own;
+    const long long total = warp_sum(all), len = (total + gridDim.x - 1) / gridDim.x;
+    for (int t = t0; t < t1; ++t) {
+        const long long c = cost(t), tb = __ldg(A.off + t);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const long long x = ((long long)blockIdx.x + j) * len - pos;
+            if (x >= 0 && x < c) {
+                const long long lead = t > 0 ? kPieceCost : 0;
+                sh_at[j] = x <= lead ? tb : max(tb, (tb + x - lead) & ~63ll);
+            }
+        }
+        pos += c;
+    }
+    __syncthreads();
+    lo = sh_at[0];
+    hi = sh_at[1];
+}
+
+// Calls f(t, tensor_begin, tensor_end, piece_begin, piece_end) for the pieces of streamed tensors in [lo, hi), in ascending order
+// or, when `down`, in descending order.  Called by all threads of a CTA; small tensors are passed over 32 at a time.
+template <class F>
+__device__ __forceinline__ void for_each_streamed(const SelArgs& A, int64_t lo, int64_t hi, F f, bool down)
+{
+    if (lo >= hi || A.T <= 0) return;
+    const int lane = threadIdx.x & 31, dir = down ? -1 : 1;
+    int t = find_tensor(A.off, A.T, down ? hi - 1 : lo);
+    while (true) {
+        const int mine = t + dir * lane;
+        int64_t tb = 0, te = 0;
+        bool in = false;
+        if (mine >= 0 && mine < A.T) {
+            tb = __ldg(A.off + mine);
+            te = __ldg(A.off + mine + 1);
+            in = tb < hi && te > lo;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in && te - tb > kSmallN);
+        if (!m) {
+            if (!__shfl_sync(0xffffffffu, (int)(mine >= 0 && mine < A.T && (down ? te > lo : tb < hi)), 31)) return;
+            t += 32 * dir;
+            continue;
+        }
+        const int src = __ffs(m) - 1;
+        const int64_t b = __shfl_sync(0xffffffffu, tb, src), e = __shfl_sync(0xffffffffu, te, src);
+        t += dir * src;
+        f(t, b, e, b > lo ? b : lo, e < hi ? e : hi);
+        t += dir;
+    }
+}
+
+// Anchor of a tensor's fine window in round 1: the largest binade among kSelThreads strided samples, plus two.  Called by every
+// thread of a CTA, with this thread's sample; ends without a barrier (sh: kSelWarps values).
+__device__ __forceinline__ float window_sample(const float* __restrict__ grad, int64_t tbeg, int64_t n)
+{
+    return __ldg(grad + tbeg + (int64_t)threadIdx.x * n / kSelThreads);
+}
+__device__ __forceinline__ int window_top(float sample, int* sh)
+{
+    int e = (int)((__float_as_uint(sample) >> 23) & 255u);
+    if (e == 255) e = 0;
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
+    __syncthreads();
+    const int top = __reduce_max_sync(0xffffffffu, sh[threadIdx.x & (kSelWarps - 1)]) + 2;
+    return min(max(top, kSelW), 255);  // binade 255 (Inf / NaN) always stays outside the fine window
+}
+
+// Clears what the passes over tensor t add to: one CTA per tensor.  Round 1 runs meanwhile and waits for it before it adds its cells.
 __global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
 {
     __shared__ int sh_i[kSelWarps];
@@ -2110,23 +2234,14 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
     const int64_t tbeg = __ldg(A.off + t), n = __ldg(A.off + t + 1) - tbeg;
     if (t == 0 && threadIdx.x == 0) { A.ws.nitems[0] = 0u; A.ws.nitems[1] = 0u; }
     if (n <= kSmallN) return;
-    // Anchor of the fine window: largest binade among strided samples, plus two.
-    int e = (int)((__float_as_uint(__ldg(A.grad + tbeg + (int64_t)threadIdx.x * n / kSelThreads)) >> 23) & 255u);
-    if (e == 255) e = 0;
+    const float sample = window_sample(A.grad, tbeg, n);
     const int ncells = A.scheme == OGQ_BINGRAD_PB ? kRound1Mag : kRound1Cells;
     uint4* cnt = reinterpret_cast<uint4*>(A.ws.gcnt + (size_t)t * kCells);
     uint4* sum = reinterpret_cast<uint4*>(A.ws.glsum + (size_t)t * kCells);
     for (int i = threadIdx.x; i < ncells / 4; i += kSelThreads) cnt[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int i = threadIdx.x; i < ncells / 2; i += kSelThreads) sum[i] = make_uint4(0u, 0u, 0u, 0u);
-    e = __reduce_max_sync(0xffffffffu, e);
-    if ((threadIdx.x & 31) == 0) sh_i[threadIdx.x >> 5] = e;
-    __syncthreads();
+    const int hi_e = window_top(sample, sh_i);
     if (threadIdx.x == 0) {
-        int hi_e = 0;
-        for (int w = 0; w < kSelWarps; ++w) hi_e = max(hi_e, sh_i[w]);
-        hi_e += 2;
-        if (hi_e < kSelW) hi_e = kSelW;
-        if (hi_e > 255) hi_e = 255;  // binade 255 (Inf / NaN) always stays outside the fine window
         TState* st = A.ws.st + t;
         st->hi_e = hi_e;
         st->done = 0;
@@ -2142,28 +2257,27 @@ __global__ void __launch_bounds__(kSelThreads) k_sel_prepare(SelArgs A)
     }
 }
 
+// Flat CTAs: a share of the bucket each.  A piece of a tensor is streamed into the CTA's cells, which are then added to the
+// tensor's global ones.  What it reads is the call's input, so it streams while the launch before still clears the global
+// cells: that one has waited for everything earlier in the stream before it let this one start.
 __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArgs A)
 {
+    __shared__ int sh_top[kSelWarps];
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
     uint32_t* hist = sel_hist();
-    pdl_wait();
     pdl_launch_dependents();
-
-    // Flat CTAs: one chunk of the bucket each.  A piece of a tensor is streamed into the CTA's cells, which
-    // are then added to the tensor's global ones.
     uint32_t* packed_cells = sel_stage();
     const int ncells = pb ? kRound1Mag : kRound1Cells;
-    const int64_t lo = (int64_t)blockIdx.x * A.chunk;
-    const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
-    for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
-        if (tend - tbeg <= kSmallN) return;
+    int64_t lo, hi;
+    streamed_share(A, lo, hi);
+    for_each_streamed(A, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
         TState* st = A.ws.st + t;
-        const int lo_e = __ldcg(&st->hi_e) - kSelW;
+        const float sample = window_sample(A.grad, tbeg, tend - tbeg);
         const float tau = A.tau ? __ldcg(A.tau + t) : 0.f;
         __syncthreads();
         zero_hist(hist, ncells);
         for (int i = threadIdx.x; i < kPackedCells; i += kSelThreads) packed_cells[i] = 0u;
-        __syncthreads();
+        const int lo_e = window_top(sample, sh_top) - kSelW;  // (with a barrier)
         const bool clip = A.tau != nullptr;
         Round1Out r;
         if (pb) {
@@ -2173,6 +2287,7 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArg
             if (clip) r = stream_round1<false, true>(A.grad, pb_, pe_, lo_e, tau);
             else r = stream_round1<false, false>(A.grad, pb_, pe_, lo_e, tau);
         }
+        pdl_wait();
         __syncthreads();
         flush_hist(hist, ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
         // min / max / non-finite: one atomic per warp
@@ -2185,6 +2300,7 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round1(SelArg
             if (anynf) atomicOr(&st->nonfinite, 1u);
         }
     }, A.tau != nullptr);
+    pdl_wait();  // (a CTA without a piece: completion passes from kernel to kernel)
 }
 
 // ---------------------------------------------------------------------------
@@ -2324,22 +2440,26 @@ __device__ __noinline__ void solve1_level(int lo_e, double n, int q, int stride)
     __syncwarp();
 }
 
-// One CTA per tensor.  Streamed tensors: prefix sums over round 1's cells, conservative cell ranges of the
-// levels, every populated cell in them becomes an interval of round 2.  Small tensors are solved here.
-//   What bounds it: latency; for the ResNet-50 bucket (21 us, 161 tensors) that of its largest small tensors, whose 16,384 values take
-// 32,000 cycles, a streamed tensor 23,000.
+// One CTA per streamed tensor: prefix sums over round 1's cells, conservative cell ranges of the levels, every populated cell in
+// them becomes an interval of round 2.
+//   What bounds it: latency, 20,000 cycles of barriers, dependent loads and code that runs once.
 __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
 {
     SolverShared& S = sel_state();
     Solve1Shared& Q = sel_state1();
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
     const int nl = pb ? 2 : A.s, s = A.s;
+    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
+    const int64_t n = tend - tbeg;
+    if (n <= kSmallN) {
+        if (t == 0) pdl_wait();  // (one CTA at least: completion passes from kernel to kernel)
+        return;
+    }
     pdl_wait();
     pdl_launch_dependents();
-    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // (loads first, the decision what to do with them after)
     TState* st = A.ws.st + t;
-    const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
     const uint32_t kmn = ~__ldcg(&st->kmin_inv), kmx = __ldcg(&st->kmax), nonfinite = __ldcg(&st->nonfinite);
     Round1Cells G;
     G.mag = pb;
@@ -2347,17 +2467,6 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
     const int ncells = G.count();
     uint32_t* gcnt = A.ws.gcnt + (size_t)t * kCells;
     unsigned long long* glsum = A.ws.glsum + (size_t)t * kCells;
-    const int64_t n = tend - tbeg;
-    if (n <= kSmallN) {
-        if (n <= 0) {
-            if (tid < nl) A.levels[(int64_t)t * nl + tid] = 0.f;
-            if (tid == 0) A.status[t] = OGQ_ST_EMPTY;
-        } else {
-            small_tensor(A.grad + tbeg, (int)n, t, pb, s, A.levels, A.status,
-                         A.tau ? __ldcg(A.tau + t) : __int_as_float(0x7f800000));
-        }
-        return;
-    }
     constexpr int kC = (kRound1Cells / 4 + kSolveThreads - 1) / kSolveThreads, kL = (kRound1Cells / 2 + kSolveThreads - 1) / kSolveThreads;
     uint4 c[kC];
     ulonglong2 l[kL];
@@ -2655,16 +2764,15 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
     Table& tb = sel_table();
     const bool pb = A.scheme == OGQ_BINGRAD_PB;
     uint32_t* hist = sel_hist();
+    int64_t lo, hi;
+    streamed_share(A, lo, hi);
     pdl_wait();
     pdl_launch_dependents();
     // Second pass over a piece: builds the tensor's interval table and prefilter, clears the CTA's cells,
     // copies the values inside the intervals and counts them on the finer cells (unless they already fit
     // one sort), adds the cells to the tensor's global ones.
-    const int64_t lo = (int64_t)blockIdx.x * A.chunk;
-    const int64_t hi = (lo + A.chunk < A.total) ? lo + A.chunk : A.total;
     const bool down = A.tau == nullptr;  // against round 1's direction
-    for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
-        if (tend - tbeg <= kSmallN) return;
+    for_each_streamed(A, lo, hi, [&](int t, int64_t tbeg, int64_t tend, int64_t pb_, int64_t pe_) {
         TState* st = A.ws.st + t;
         if (__ldcg(&st->done)) return;  // settled in round 1
         __syncthreads();
@@ -2691,20 +2799,35 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
 }
 
 // What follows round 2, one CTA per tensor: the finish from the copied keys when round 2 only copied, else a solver pass and
-// work items of the round-3 kernel.
+// work items of the round-3 kernel.  Small tensors are solved here, from the call's input alone, so before the rounds are waited
+// for: in the first solver pass, whose launch they made longer (ResNet-50 bucket: 161 CTAs on 148 SMs, 21 us instead of 10), they
+// stood in the way of the streamed tensors.
 __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve2(SelArgs A)
 {
-    pdl_wait();
-    pdl_launch_dependents();
+    if (A.first) pdl_wait();
     const int t = blockIdx.x;
     SolverShared& S = sel_state();
     const int64_t tbeg = __ldg(A.off + t), tend = __ldg(A.off + t + 1);
     const int64_t n = tend - tbeg;
+    if (n <= kSmallN) {
+        const bool pb = A.scheme == OGQ_BINGRAD_PB;
+        const int nl = pb ? 2 : A.s;
+        if (n <= 0) {
+            if ((int)threadIdx.x < nl) A.levels[(int64_t)t * nl + threadIdx.x] = 0.f;
+            if (threadIdx.x == 0) A.status[t] = OGQ_ST_EMPTY;
+        } else {
+            small_tensor(A.grad + tbeg, (int)n, t, pb, A.s, A.levels, A.status, A.tau ? __ldcg(A.tau + t) : __int_as_float(0x7f800000));
+        }
+        if (t == 0) pdl_wait();  // (one CTA at least: completion passes from kernel to kernel)
+        return;
+    }
+    pdl_wait();
+    pdl_launch_dependents();
     TState* st = A.ws.st + t;
     const int done = __ldcg(&st->done), compact_only = __ldcg(&st->compact_only);
     const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[0]);
     finish_load(st, A.scheme == OGQ_BINGRAD_PB, A.s, S);  // (all loads in one go, the decision what to do with them after)
-    if (n <= kSmallN || done || compact_only == 2) return;
+    if (done || compact_only == 2) return;
     if (compact_only != 0) {
         finish_from_keys(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[0] + sel_region(tbeg), (int)min(src_cnt, cand), true,
                          A.levels, A.status);
@@ -3040,12 +3163,12 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         }
     }
     // Flat streaming CTAs: one wave (kSelResident per SM).  Each CTA pays a set-up and a flush of its
-    // cells per tensor piece, so larger chunks stream more of the time.
+    // cells per tensor piece, so larger shares stream more of the time.
     const int64_t wave = (int64_t)kSelResident * sm_count;
     const int target = wave < kMaxFlatCtas ? (int)wave : kMaxFlatCtas;
-    FlatGrid g = make_flat_grid(total, target, 16384);
+    FlatGrid g = make_flat_grid(total, target, T > kMaxShared ? 16384 : kMinShare);
     SelArgs A;
-    A.grad = d_grad; A.tau = d_tau; A.off = d_off; A.T = T; A.total = total; A.chunk = g.chunk;
+    A.grad = d_grad; A.tau = d_tau; A.off = d_off; A.T = T; A.total = total; A.chunk = T > kMaxShared ? g.chunk : 0;
     A.scheme = scheme; A.s = s; A.levels = d_levels; A.status = d_status;
     A.ws = sel_carve(d_ws, T, total);
     cudaError_t e = cudaSuccess;
@@ -3055,15 +3178,16 @@ cudaError_t launch_levels_select(const float* d_grad, const int64_t* d_off, int 
         e = launch_pdl(kernel, ctas, threads, smem, stream, A);
         launch_end(stream);
     };
+    A.first = total > kSmallN ? 0 : 1;
     const bool streams = total > kSmallN;  // some tensor may be larger than one CTA settles on its own
     if (streams) {
         run("k_sel_prepare", k_sel_prepare, T, 0);
         run("k_sel_round1", k_sel_round1, g.ctas, kStreamBytes);
-    }
-    run("k_sel_solve1", k_sel_solve1, T, kSolve1Bytes, kSolveThreads);
-    if (streams) {
+        run("k_sel_solve1", k_sel_solve1, T, kSolve1Bytes, kSolveThreads);
         run("k_sel_round2", k_sel_round2, g.ctas, kStreamBytes);
-        run("k_sel_solve2", k_sel_solve2, T, kSolveBytes, kSolveThreads);
+    }
+    run("k_sel_solve2", k_sel_solve2, T, kSolveBytes, kSolveThreads);
+    if (streams) {
         // a cluster per tensor that may have that many candidates (its copies have room for an eighth of it); an empty launch of
         // eight clusters takes 2.9 us, of one 1.5
         const int64_t clusters = std::min<int64_t>(std::min<int64_t>(T, total / (kBufDiv * kSortN)), kMaxSlices / kCluster);
