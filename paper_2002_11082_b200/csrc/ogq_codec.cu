@@ -171,7 +171,7 @@ constexpr int kMaxTables = 16;            // and tables of sums
 // time: their levels lie one after the other in every worker's array, so they come with one wait, and the groups of
 // these tensors are gone through without barriers.  (Rows of one tensor at a time, with two barriers and a wait for L2 each,
 // and small tensors' levels read from L2 per element: 62 instead of 55 us for nine levels, eight workers and the 161 tensors of the ResNet-50 bucket, 82 instead of 61 for five levels.)
-template <int BITS>
+template <int BITS, int REST>
 __global__ void __launch_bounds__(kThreads, kStreamCtas)
 k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
              const int64_t* __restrict__ off, const int64_t* __restrict__ packed_off, int T, int64_t total,
@@ -251,7 +251,7 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
         auto write = [&](int gl, float (&a)[8]) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) a[j] = __fmul_rn(a[j], scale);
-            store8(dst8 + (size_t)gl * 256, shift, lane, a);
+            store8<(BITS > 1)>(dst8 + (size_t)gl * 256, shift, lane, a);
         };
         constexpr int G = 2;       // groups per warp and trip
         constexpr int kAhead = 8;  // trips between two prefetch requests
@@ -263,14 +263,14 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
             if (BITS >= 2 && (trip & (kAhead - 1)) == 0 && (int)threadIdx.x < K && (trip + 2 * kAhead) * kTrip <= ng)
                 prefetch_l2(sh_pk[threadIdx.x] + w0 + (int64_t)(trip + kAhead) * kTrip * kWords, kAhead * kTrip * kWords * 4u);
             float a[G][8];
-            sum_workers<BITS, G, true>(K, lane, table, row,
+            sum_workers<BITS, G, true, REST>(K, lane, table, row,
                                  [&](int k, int g) { return sh_pk[k] + w0 + (int64_t)(gl + g * kWarps) * kWords; }, a);
 #pragma unroll
             for (int g = 0; g < G; ++g) write(gl + g * kWarps, a[g]);
         }
         if (gl < ng) {
             float a[1][8];
-            sum_workers<BITS, 1, true>(K, lane, table, row, [&](int k, int) { return sh_pk[k] + w0 + (int64_t)gl * kWords; }, a);
+            sum_workers<BITS, 1, true, REST>(K, lane, table, row, [&](int k, int) { return sh_pk[k] + w0 + (int64_t)gl * kWords; }, a);
             write(gl, a[0]);
         }
 
@@ -353,7 +353,7 @@ k_unpack_one(const uint32_t* const* __restrict__ packed_k, const float* const* _
                 if (gl + g * kWarps >= ng) break;
                 float a[8];
                 look_up(c[g], a);
-                store8(dst8 + (size_t)(gl + g * kWarps) * 256, shift, lane, a);
+                store8<(BITS > 1)>(dst8 + (size_t)(gl + g * kWarps) * 256, shift, lane, a);
             }
         }
         // the tensor's last, partial group
@@ -429,8 +429,10 @@ cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* co
     } else {                                                                                          \
         const size_t each = row_bytes<B>(K), tables = kTableFloats<B> > 0 ? kMaxTables * 1024 : 0;       \
         const int batch = (int)std::min<size_t>(std::max<size_t>(kRowsBytes / each, 1), (size_t)std::min(T, tables ? kMaxTables : 32)); \
-        e = launch_pdl(k_unpack_sum<B>, g.ctas, kThreads, tables + each * batch, stream, d_packed_k, d_levels_k, K, d_off, \
-                       d_packed_off, T, total, g.chunk, s, batch, scale, d_out);                      \
+        e = with_rest<B>(rest_of<B, true>(K), [&](auto rest) {                                         \
+            return launch_pdl(k_unpack_sum<B, decltype(rest)::value>, g.ctas, kThreads, tables + each * batch, stream, d_packed_k, \
+                              d_levels_k, K, d_off, d_packed_off, T, total, g.chunk, s, batch, scale, d_out); \
+        });                                                                                           \
     }
     launch_begin("k_unpack_sum", stream);
     switch (bits) {

@@ -9,6 +9,8 @@
 // byte of output traffic costs two to three reads), DRAM for 1-bit codes.
 #pragma once
 
+#include <type_traits>
+
 #include "ogq_common.cuh"
 #include "ogq_quant.cuh"
 
@@ -18,6 +20,18 @@ template <int BITS>
 constexpr int kTableWorkers = BITS == 1 ? 8 : BITS == 2 ? 4 : 0;  // workers that the table of sums takes in (0: no table)
 template <int BITS>
 constexpr int kTableFloats = kTableWorkers<BITS> ? 256 : 0;
+// Workers whose words are loaded before any is used, and those of the last, partial batch.  That number is a template argument of the
+// kernels: a kernel then has no condition between the reads of one worker's levels and the next's, which kept them from
+// overlapping, and no instructions but its own (20 M elements of nine levels: two workers 26.9 -> 21 us, five 38 -> 32; 17 levels,
+// seven 55 -> 45).  Eight at a time but for 3-bit codes, where four were as fast with half the instructions to fetch.
+template <int BITS>
+constexpr int kBatch = BITS == 1 || BITS == 3 ? 4 : 8;
+template <int BITS, bool TABLE>
+int rest_of(int K)
+{
+    const int rows = K - (TABLE ? kTableWorkers<BITS> : 0);
+    return rows > 0 ? rows % kBatch<BITS> : 0;
+}
 template <int BITS>
 constexpr int kRowStride = 1 << BITS;  // floats per level row: every code a field can hold has an entry
 
@@ -52,6 +66,15 @@ __device__ __forceinline__ EightCodes<BITS> load_codes(const uint32_t* __restric
         c.hi = b >> sh;
     }
     return c;
+}
+
+// launch(std::integral_constant<int, REST>) for the number of workers in the last, partial batch.
+template <int BITS, int R = kBatch<BITS> - 1, class Launch>
+cudaError_t with_rest(int rest, Launch launch)
+{
+    if (rest == R) return launch(std::integral_constant<int, R>());
+    if constexpr (R > 0) return with_rest<BITS, R - 1>(rest, launch);
+    else return cudaErrorInvalidValue;
 }
 
 // Shared addresses of the levels of the eight codes in the row at `row`, a multiple of the row's size (4-bit codes: of 256): it
@@ -110,18 +133,27 @@ __device__ __forceinline__ void add_levels(const EightCodes<BITS>& c, uint32_t r
         add2(acc[j], acc[j + 1], load_level<U * kRowStride<BITS> * 4>(o[j]), load_level<U * kRowStride<BITS> * 4>(o[j + 1]));
 }
 
-// The workers from U on of a batch of B.
-template <int BITS, int G, int B, int U = 0>
-__device__ __forceinline__ void add_batch(const EightCodes<BITS> (&c)[G][B], int workers, uint32_t row, float (&acc)[G][8])
+// `words` and the sums of N workers whose rows begin at `row`: all words are loaded before any is used, and no condition comes
+// between the workers (a branch after each kept the reads of one from overlapping those of the next).
+template <int BITS, int G, int N, int U = 0>
+__device__ __forceinline__ void add_batch(const EightCodes<BITS> (&c)[G][N], uint32_t row, float (&acc)[G][8])
 {
-    if constexpr (U < B) {
-        if (U >= workers) return;
+    if constexpr (U < N) {
 #pragma unroll
         for (int g = 0; g < G; ++g) add_levels<BITS, U>(c[g][U], row, acc[g]);
-        add_batch<BITS, G, B, U + 1>(c, workers, row, acc);
+        add_batch<BITS, G, N, U + 1>(c, row, acc);
     }
 }
-
+template <int BITS, int G, int N, class Word>
+__device__ __forceinline__ void sum_batch(int k0, int lane, uint32_t row, Word word, float (&acc)[G][8])
+{
+    EightCodes<BITS> c[G][N];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int u = 0; u < N; ++u) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
+    add_batch<BITS, G, N>(c, row, acc);
+}
 // Table indices of eight elements from the codes of the kTableWorkers workers of a table (workers that do not
 // exist: zeros): byte e of x[0], byte e - 4 of x[1] is the index of element e, worker u's code in its bits
 // [u BITS, (u + 1) BITS).
@@ -186,11 +218,10 @@ __host__ __device__ constexpr uint32_t row_bytes(int K) { return ((uint32_t)K * 
 // Sums of the G groups of 256 elements at word(k, g) (worker k's first word of group g), eight elements of each for
 // this lane.  table (not read unless TABLE), rows: shared addresses.  The words of several workers are loaded before any
 // is used.
-template <int BITS, int G, bool TABLE, class Word>
+template <int BITS, int G, bool TABLE, int REST, class Word>
 __device__ __forceinline__ void sum_workers(int K, int lane, uint32_t table, uint32_t rows, Word word, float (&acc)[G][8])
 {
-    constexpr int W = TABLE ? kTableWorkers<BITS> : 0;
-    constexpr int B = BITS == 4 ? 8 : 4;  // workers per batch
+    constexpr int W = TABLE ? kTableWorkers<BITS> : 0, B = kBatch<BITS>;
     static_assert(BITS != 4 || B * kRowStride<BITS> * 4 % 256 == 0, "a batch's rows begin at a multiple of 256 bytes");
     int k0 = 0;
     if constexpr (W > 0) {
@@ -211,37 +242,24 @@ __device__ __forceinline__ void sum_workers(int K, int lane, uint32_t table, uin
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[g][j] = 0.f;
     }
-    for (; k0 < K; k0 += B) {
-        const uint32_t r = rows + (uint32_t)k0 * (kRowStride<BITS> * 4u);
-        EightCodes<BITS> c[G][B];
-        if (k0 + B <= K) {
-#pragma unroll
-            for (int g = 0; g < G; ++g)
-#pragma unroll
-                for (int u = 0; u < B; ++u) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
-            add_batch<BITS, G, B>(c, B, r, acc);
-        } else if (W == 0 && k0 + 1 == K) {  // (the last one alone, often the only one: few instructions to fetch)
-#pragma unroll
-            for (int g = 0; g < G; ++g) c[g][0] = load_codes<BITS>(word(k0, g), lane);
-#pragma unroll
-            for (int g = 0; g < G; ++g) add_levels<BITS, 0>(c[g][0], r, acc[g]);
-        } else {
-#pragma unroll
-            for (int u = 0; u < B; ++u)
-                if (k0 + u < K)
-#pragma unroll
-                    for (int g = 0; g < G; ++g) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
-            add_batch<BITS, G, B>(c, K - k0, r, acc);
-        }
-    }
+    for (; k0 + B <= K; k0 += B) sum_batch<BITS, G, B>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
+    if constexpr (REST > 0) sum_batch<BITS, G, REST>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
 }
 
+// (WIDE: on a 32-byte boundary with one 256-bit store.  Two 128-bit stores write every 32-byte sector twice, half of it each time: 54.5
+// -> 52.2 us for the ResNet-50 bucket at eight workers of nine levels, 32 -> 29.3 for 20 M elements of four workers of five.)
 // Stores eight consecutive floats per lane at p (p: the lane's first, 32 bytes times lane above the warp's first),
 // whose address is `shift` floats above a 16-byte boundary, with 128-bit stores: lanes pass their last
 // `shift` values on to the next lane, the warp's two ends are stored one by one.
+template <bool WIDE>
 __device__ __forceinline__ void store8(float* p, int shift, int lane, const float (&v)[8])
 {
     if (shift == 0) {
+        if (WIDE && (reinterpret_cast<uintptr_t>(p) & 31) == 0) {  // (the same in all lanes)
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" :: "l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                         "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+            return;
+        }
         *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
         *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
         return;
