@@ -217,28 +217,69 @@ __device__ __forceinline__ uint32_t dense_fraction(uint32_t w)
     else return (uint32_t)(((uint64_t)w * 995507236u + ((w >> 1) + 1u)) >> 32) + w + 1u;
 }
 
-// acc[e] += the level of digit e of w.  row: shared address of the worker's levels.
-template <int S>
+// A worker's row of levels for D digits at a time: D tables of S^D entries, table a that of the a-th of the D digits (the highest
+// first) in the number that the D digits make.  Entries of one table lie in different banks, S^D <= 32.
+template <int S, int D>
+struct DenseRow {
+    static constexpr int kEntries = (int)dense_pow(S, D), kFloats = D * kEntries, kPlain = (D - 1) * kEntries;  // kPlain: the levels themselves
+    static_assert(D == 1 || kEntries <= 32, "no bank conflicts");
+};
+
+// acc[e] += the level of digit e of w.  row: shared address of the worker's row.
+template <int S, int D>
 __device__ __forceinline__ void add_digits(uint32_t w, uint32_t row, float (&acc)[Dense<S>::M])
 {
-    constexpr int M = Dense<S>::M;
+    constexpr int M = Dense<S>::M, E = DenseRow<S, D>::kEntries;
     uint32_t f = dense_fraction<S>(w);
     float v[M];
 #pragma unroll
-    for (int e = M - 1; e >= 0; --e) {
-        asm("{ .reg .b64 p; .reg .b32 d; mul.wide.u32 p, %1, %2; mov.b64 {%1, d}, p; mad.lo.u32 d, d, 4, %3; ld.shared.f32 %0, [d]; }"
-            : "=f"(v[e]), "+r"(f) : "n"(S), "r"(row));
+    for (int e = M - 1; e >= 0; e -= D) {
+        constexpr int kLeft = M % D == 0 ? D : M % D;  // digits of the last step
+        const int r = e + 1 < D ? kLeft : D;
+        uint32_t at;
+        asm("{ .reg .b64 p; .reg .b32 d; mul.wide.u32 p, %1, %2; mov.b64 {%1, d}, p; mad.lo.u32 %0, d, 4, %3; }"
+            : "=r"(at), "+r"(f) : "r"(dense_pow(S, r)), "r"(row));
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+            if (i < r) asm("ld.shared.f32 %0, [%1];" : "=f"(v[e - i >= 0 ? e - i : 0]) : "r"(at + (uint32_t)((D - r + i) * E * 4)));
     }
 #pragma unroll
     for (int e = 0; e + 1 < M; e += 2) add2(acc[e], acc[e + 1], v[e], v[e + 1]);
     if constexpr (M & 1) acc[M - 1] = __fadd_rn(acc[M - 1], v[M - 1]);
 }
 
-// What bounds it: shared-memory reads, one per element and worker, with the instructions for the digits close behind.
-// (One lane per group with divisions by S and stores of its own, each spread over 32 lines: 119 us for 25.6 M
-// elements of 8 workers at s = 5.)  Two digits at a time through a table of pairs were no faster: a 64-bit
+// The rows of K workers for tensor t, by `warps` warps of which this is number w; sync: their barrier.
+template <int S, int D, class Sync>
+__device__ __forceinline__ void dense_rows(float* rows, const float* const* lv, int K, int64_t t, int w, int warps, Sync sync)
+{
+    using Row = DenseRow<S, D>;
+    const int lane = threadIdx.x & 31;
+    for (int i = w * 32 + lane; i < K * S; i += warps * 32) rows[i / S * Row::kFloats + Row::kPlain + i % S] = __ldcg(lv[i / S] + t * S + i % S);
+    sync();
+    if constexpr (D > 1) {
+        // entry `lane` of every table, from the levels themselves, which are the first entries of the last
+        if (lane < Row::kEntries) {
+#pragma unroll 4
+            for (int k = w; k < K; k += warps) {
+                float* row = rows + k * Row::kFloats;
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                    const float x = row[Row::kPlain + (uint32_t)lane / dense_pow(S, D - 1 - a) % S];
+                    if (a + 1 < D || lane >= S) row[a * Row::kEntries + lane] = x;
+                }
+            }
+        }
+        sync();
+    }
+}
+
+// What bounds it: shared-memory reads, one per element and worker, with the instructions for the digits close behind: a wide product
+// holds the multiply pipe for four cycles.  So three digits at a time (S = 3) or two (S = 5) come from one product and one address,
+// each with a read of a table of its own, as long as four CTAs' tables fit an SM (25.6 M elements of eight workers at S = 5, whole
+// step: 204 -> 198 us; 20 M at S = 3: 49 -> 41).  (One lane per group with divisions by S and stores of its own, each spread over 32 lines: 119 us for 25.6 M
+// elements of 8 workers at s = 5.)  Two digits at a time through one table of pairs were no faster: a 64-bit
 // read costs as much as two.
-template <int S>
+template <int S, int D>
 __global__ void __launch_bounds__(kThreads, 4)
 k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
                    const int64_t* __restrict__ off, const int64_t* __restrict__ packed_off, int T, int64_t total,
@@ -247,7 +288,8 @@ k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* co
     constexpr int M = Dense<S>::M, U = 4 * M;  // U: elements of a group here (whole 16-byte lines whatever M)
     constexpr int kTile = 32 * M;              // elements of a tile
     constexpr int kEdgeTiles = 4;              // tensors of no more tiles in this chunk go to one warp each
-    extern __shared__ __align__(16) float sh_sums[];  // [kWarps][kTile] sums, then [kWarps + 2][K][S] level rows
+    constexpr int kRow = DenseRow<S, D>::kFloats;
+    extern __shared__ __align__(16) float sh_sums[];  // [kWarps][kTile] sums, then [kWarps + 2][K][kRow] level rows
     __shared__ const uint32_t* sh_pk[kMaxWorkers];
     __shared__ const float* sh_lv[kMaxWorkers];
     pdl_wait();
@@ -277,17 +319,15 @@ k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* co
         const bool vec = (reinterpret_cast<uintptr_t>(outp + tb) & 15) == 0;
 
         const bool small = tiles <= kEdgeTiles;
-        float* rows = all_rows + (small ? warp : kWarps + set) * K * S;
+        float* rows = all_rows + (small ? warp : kWarps + set) * K * kRow;
         if (small) {
             turn = (turn + 1) & (kWarps - 1);
             if (turn != warp) return;
             __syncwarp();
-            for (int i = lane; i < K * S; i += 32) rows[i] = __ldcg(sh_lv[i / S] + (int64_t)t * S + i % S);
-            __syncwarp();
+            dense_rows<S, D>(rows, sh_lv, K, t, 0, 1, [] { __syncwarp(); });
         } else {
             set ^= 1;
-            for (int i = threadIdx.x; i < K * S; i += kThreads) rows[i] = __ldcg(sh_lv[i / S] + (int64_t)t * S + i % S);
-            __syncthreads();
+            dense_rows<S, D>(rows, sh_lv, K, t, warp, kWarps, [] { __syncthreads(); });
         }
         const uint32_t rows_addr = (uint32_t)__cvta_generic_to_shared(rows);
         const int first = small ? 0 : warp, step = small ? 1 : kWarps;
@@ -313,7 +353,7 @@ k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* co
                     for (int u = 0; u < B; ++u) w[u] = have && k + u < K ? __ldcg(sh_pk[k + u] + at) : 0u;
 #pragma unroll
                     for (int u = 0; u < B; ++u)
-                        if (k + u < K) add_digits<S>(w[u], rows_addr + (k + u) * (S * 4), acc);
+                        if (k + u < K) add_digits<S, D>(w[u], rows_addr + (k + u) * (kRow * 4), acc);
                 }
             } else {
                 int k = 0;
@@ -322,9 +362,9 @@ k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* co
 #pragma unroll
                     for (int u = 0; u < B; ++u) w[u] = have ? __ldcg(sh_pk[k + u] + at) : 0u;
 #pragma unroll
-                    for (int u = 0; u < B; ++u) add_digits<S>(w[u], rows_addr + (k + u) * (S * 4), acc);
+                    for (int u = 0; u < B; ++u) add_digits<S, D>(w[u], rows_addr + (k + u) * (kRow * 4), acc);
                 }
-                for (; k < K; ++k) add_digits<S>(have ? __ldcg(sh_pk[k] + at) : 0u, rows_addr + k * (S * 4), acc);
+                for (; k < K; ++k) add_digits<S, D>(have ? __ldcg(sh_pk[k] + at) : 0u, rows_addr + k * (kRow * 4), acc);
             }
 #pragma unroll
             for (int e = 0; e < M; ++e) acc[e] = __fmul_rn(acc[e], scale);
@@ -388,15 +428,24 @@ cudaError_t launch_unpack_sum_dense(const uint32_t* const* d_packed_k, const flo
     const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas, 4096);
     cudaError_t e = cudaErrorInvalidValue;
     launch_begin("k_unpack_sum_dense", stream);
-#define OGQ_LAUNCH_UD(SS)                                                                                       \
-    e = launch_pdl_smem(k_unpack_sum_dense<SS>, g.ctas, kThreads, \
-                        (kWarps * 32 * Dense<SS>::M + (kWarps + 2) * K * SS) * sizeof(float), stream, d_packed_k, d_levels_k, K, d_off, d_packed_off, T, \
-                   total, g.chunk, scale, d_out)
+    auto bytes = [&](int digits, int row) { return (size_t)(kWarps * 32 * digits + (kWarps + 2) * K * row) * sizeof(float); };
+    // shared memory of which four CTAs fit an SM
+    constexpr size_t kFour = 54 * 1024;
+#define OGQ_LAUNCH_UD(SS, DD)                                                                                   \
+    e = launch_pdl_smem(k_unpack_sum_dense<SS, DD>, g.ctas, kThreads, bytes(Dense<SS>::M, DenseRow<SS, DD>::kFloats), stream, \
+                        d_packed_k, d_levels_k, K, d_off, d_packed_off, T, total, g.chunk, scale, d_out)
     switch (s) {
-        case 3: OGQ_LAUNCH_UD(3); break;
-        case 5: OGQ_LAUNCH_UD(5); break;
-        case 9: OGQ_LAUNCH_UD(9); break;
-        case 17: OGQ_LAUNCH_UD(17); break;
+        case 3:
+            if (bytes(Dense<3>::M, DenseRow<3, 3>::kFloats) <= kFour) OGQ_LAUNCH_UD(3, 3);
+            else if (bytes(Dense<3>::M, DenseRow<3, 2>::kFloats) <= kFour) OGQ_LAUNCH_UD(3, 2);
+            else OGQ_LAUNCH_UD(3, 1);
+            break;
+        case 5:
+            if (bytes(Dense<5>::M, DenseRow<5, 2>::kFloats) <= kFour) OGQ_LAUNCH_UD(5, 2);
+            else OGQ_LAUNCH_UD(5, 1);
+            break;
+        case 9: OGQ_LAUNCH_UD(9, 1); break;
+        case 17: OGQ_LAUNCH_UD(17, 1); break;
         default: return cudaErrorInvalidValue;
     }
 #undef OGQ_LAUNCH_UD
