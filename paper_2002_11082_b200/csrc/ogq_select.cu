@@ -63,12 +63,18 @@ constexpr int kRound1Mag = 256 - kSelW + (kSelW << kSelM);  // round-1 cells per
 constexpr int kRound1Cells = 2 * kRound1Mag;
 static_assert(kRound1Cells <= kCells, "round-1 cells exceed the budget");
 
+// TState::compact_only: what the next pass does with the keys inside the intervals.
+constexpr int kCounted = 0;        // copies them and counts them on finer cells
+constexpr int kCompact = 1;        // copies them: they fit one CTA's index
+constexpr int kOrdered = 2;        // copies them in order of round 1's cells; the second solver launch selects among one cell's at a time
+constexpr int kOrderedLarger = 3;  // the same, with cells so large that round 3 does it, with a cluster of CTAs
+
 struct TState {
     int done, round, m, hi_e;
-    unsigned kmin_inv, kmax, nonfinite, arrive;
+    unsigned kmin_inv, kmax, nonfinite;
+    unsigned arrive;    // slices that have arrived in round 3; of a tensor copied in order of round 1's cells, the keys of the fullest
     unsigned expected;  // CTAs that work on the tensor in round 3; the candidate cells of a tensor copied in their order
-    int compact_only;  // 1: the next pass only copies the keys inside the intervals: they fit one sort.  2: it copies them in order of
-                       // round 1's cells, for k_sel_round3 to select among one cell's at a time
+    int compact_only;
     int overflow;      // the current pass dropped copies that did not fit the tensor's region
     int from_grad;     // the current pass (round >= 3) reads the gradient, not the previous pass's copies
     unsigned long long cursor[2];
@@ -138,6 +144,9 @@ extern __shared__ __align__(16) unsigned char smem[];
 // cells would have their sums, the cursors of the cells where they would have their counts.
 constexpr int kCandCells = 512;  // at most
 constexpr int kCellBits = 23;    // log2 of the keys of the widest cell
+// Most keys of a cell that the second solver launch selects among by itself, and most where round 3 has other tensors to work on anyway (which then
+// takes no longer).  One tensor of 6 M elements, nine levels: 109 -> 90 us; the VGG-19 bucket, with the first limit alone: 496 -> 517.
+constexpr int kCellsAlone = 16384, kCellsBeside = 4096;
 static_assert(kCandCells <= 1 << (32 - kCellBits), "a cell's number fits above its keys");
 struct CandCell {
     double sbefore;      // sum of the elements below it
@@ -2355,7 +2364,7 @@ struct __align__(16) Solve1Shared {
     uint32_t starts[kCandCells / 32];   // which of the sorted candidate cells begin a run of neighbours
     int first[kMaxIv + 1], cells_at[kMaxIv + 1];
     int m, fail, runs;
-    uint32_t cand;
+    uint32_t cand, most;  // candidates, and those of the fullest cell
     int pb_a, pb_b;
 };
 
@@ -2482,7 +2491,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
     uint32_t* raw_cnt = reinterpret_cast<uint32_t*>(smem + kOffRawCnt1);
     {
         if (tid < (kRound1Cells + 31) / 32) Q.marks[tid] = 0u;
-        if (tid == 0) { Q.m = 0; Q.fail = 0; Q.runs = 0; Q.cand = 0u; Q.pb_a = 0; Q.pb_b = 0; }
+        if (tid == 0) { Q.m = 0; Q.fail = 0; Q.runs = 0; Q.cand = 0u; Q.most = 0u; Q.pb_a = 0; Q.pb_b = 0; }
 #pragma unroll
         for (int u = 0; u < kC; ++u)
             if ((tid + u * kSolveThreads) * 4 < ncells) reinterpret_cast<uint4*>(raw_cnt)[tid + u * kSolveThreads] = c[u];
@@ -2584,9 +2593,11 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
         const bool fresh = k && !(atomicOr(&Q.marks[c >> 5], bit) & bit);
         const uint32_t b = __ballot_sync(0xffffffffu, fresh), sum = __reduce_add_sync(0xffffffffu, fresh ? k : 0u);
         int i = 0;
+        const uint32_t most = __reduce_max_sync(0xffffffffu, k);
         if (lane == 0 && b) {
             i = atomicAdd(&Q.m, __popc(b));
             atomicAdd(&Q.cand, sum);
+            atomicMax(&Q.most, most);
         }
         i = __shfl_sync(0xffffffffu, i, 0) + __popc(b & ((1u << lane) - 1u));
         if (fresh && i < kCandCells) Q.list[i] = c;
@@ -2650,7 +2661,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
         runs = m <= kCandCells ? Q.runs : kMaxIv + 1;
     }
     // More candidates than one CTA's index holds, but not more than the copies have room for: round 2 copies them in order of
-    // these cells and k_sel_round3 selects among one cell's at a time.
+    // these cells, and a level is selected among one cell's.
     const bool ordered = !pb && cand > (uint32_t)kSortN && (int64_t)cand + 3 * m <= sel_region(tend) - sel_region(tbeg) && runs <= kMaxIv;
     int r = runs <= kMaxIv && !ordered ? 31 - __clz(kCells / runs) : 0;
     bool fits = runs <= kMaxIv;
@@ -2746,15 +2757,16 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
             reinterpret_cast<CandCell*>(glsum)[my_rank] = x;
             gcnt[tid] = 0u;
         }
-        if (tid == 0) A.ws.items[(size_t)A.T * kMaxSlices - 1 - atomicAdd(A.ws.nitems + 1, 1u)].x = t;
+        if (tid == 0 && Q.most > (uint32_t)kCellsAlone) A.ws.items[(size_t)A.T * kMaxSlices - 1 - atomicAdd(A.ws.nitems + 1, 1u)].x = t;
     } else if (!compact_only) {
         for (int i = tid; i < ncells_next; i += kSolveThreads) { gcnt[i] = 0u; glsum[i] = 0ull; }
     }
     if (tid == 96) {
+        if (ordered) st->arrive = Q.most;
         st->m = runs;
         st->cand = cand;
         if (ordered) st->expected = (unsigned)m;
-        st->compact_only = ordered ? 2 : compact_only ? 1 : 0;
+        st->compact_only = ordered ? (Q.most > (uint32_t)kCellsAlone ? kOrderedLarger : kOrdered) : compact_only ? kCompact : kCounted;
         st->round = 2;
     }
 }
@@ -2779,7 +2791,7 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
         table_from_intervals(tb, st->iv, __ldcg(&st->m));
         __syncthreads();
         build_prefilter(tb, pb);
-        const int mode = __ldcg(&st->compact_only);
+        const int mode = min(__ldcg(&st->compact_only), kOrdered);
         if (mode == 0) zero_hist(hist, tb.ncells);
         if (mode == 2) {
             const CandCell* cells = reinterpret_cast<const CandCell*>(A.ws.glsum + (size_t)t * kCells);
@@ -2796,6 +2808,213 @@ __global__ void __launch_bounds__(kSelThreads, kSelResident) k_sel_round2(SelArg
         __syncthreads();
         if (mode == 0) flush_hist(hist, tb.ncells, A.ws.gcnt + (size_t)t * kCells, A.ws.glsum + (size_t)t * kCells);
     }, down);
+}
+
+// ---------------------------------------------------------------------------
+// ORQ tensors with more candidates than one CTA's index holds: their keys lie in order of round 1's candidate cells, whose
+// exact counts and sums are known.  The exact rank of a level, known when its two brackets are, tells the cell; the level is
+// selected among that cell's keys alone.  Cells of up to kCellsAlone keys: by one CTA, a group of its warps on every level of a depth of Algorithm
+// 1, by counts on some of the keys' bits at a time, the upper ones first.
+//   What bounds it: latency, 6000 cycles a depth for small cells.  A cluster (tensor_from_cells) takes 20,000 for its barriers and for what its CTAs
+// read from one another's shared memory, whatever the number of keys: 1.2 M elements of 17 levels 82 -> 57 us.
+// ---------------------------------------------------------------------------
+constexpr int kGroups = 8;         // levels of a depth
+constexpr int kGroupThreads = 256; // of a level's group, at most, where cells are small
+constexpr int kRest = 32;          // keys that are left to one warp
+
+struct GroupSelect {
+    int cell, open;       // the rank's cell, -1: none has it; whether there is a rank (the brackets differ)
+    uint32_t rank;        // of the level
+    uint32_t bin, below, own;
+    uint32_t listed, list[kRest];
+    uint32_t warp_n[kSolveThreads / 32];
+    unsigned long long warp_sum[kSolveThreads / 32];
+};
+
+struct __align__(16) CellGroups {
+    LvInfo lv[kMaxLv];
+    GroupSelect group[kGroups];
+    uint32_t bins[kGroups * 2 * (kSolveThreads / kGroups)];  // two a thread
+    int fail;
+    CandCell cells[kCandCells];
+};
+static_assert(sizeof(CellGroups) <= kIndexBytes, "fits the solver's shared memory");
+__device__ __forceinline__ CellGroups& cell_groups() { return *reinterpret_cast<CellGroups*>(smem); }
+
+// The cells of tensor t into `cells`, by every thread of the CTA; those beyond the last begin behind everything.  The caller synchronises.
+__device__ __forceinline__ void cells_load(const SelArgs& A, const TState* st, int t, CandCell* cells)
+{
+    static_assert(kCandCells <= kSolveThreads, "a thread per candidate cell");
+    if (threadIdx.x < kCandCells) {
+        CandCell x = reinterpret_cast<const CandCell*>(A.ws.glsum + (size_t)t * kCells)[threadIdx.x];
+        if ((int)threadIdx.x >= (int)__ldcg(&st->expected)) {
+            x.cbefore = 0xffffffffu;
+            x.n = 0u;
+        }
+        cells[threadIdx.x] = x;
+    }
+}
+
+// Level q between levels q - stride and q + stride, by the `threads` threads (a power of two) of group g, which all call this; a barrier
+// of the caller's ends it.  keys: the tensor's copied keys.
+__device__ __noinline__ void level_by_group(int q, int stride, int g, int threads, const uint32_t* keys)
+{
+    CellGroups& Q = cell_groups();
+    GroupSelect& X = Q.group[g];
+    const int gt = (int)threadIdx.x & (threads - 1), lane = gt & 31, warp = gt >> 5, warps = threads >> 5;
+    uint32_t* bins = Q.bins + g * 2 * threads;
+    const int bin_bits = 32 - __clz(threads);
+    auto sync = [&]() { asm volatile("bar.sync %0, %1;" :: "r"(g + 1), "r"(threads) : "memory"); };
+    if (warp == 0) {
+        const LvInfo &L = Q.lv[q - stride], &R = Q.lv[q + stride];
+        const double width = R.val - L.val, nseg = (double)((uint32_t)R.c_le - (uint32_t)L.c_lt);
+        const bool open = width > 0.0;
+        const uint32_t p = open ? (uint32_t)R.c_le - 1u - (uint32_t)fmin(fmax(floor_of_t(R.s_le, L.s_lt, L.val, width, nseg), 0.0), nseg - 1.0) : 0u;
+        // the last cell that begins at or before rank p
+        constexpr int kStep = kCandCells / 32;
+        int c = __popc(__ballot_sync(0xffffffffu, Q.cells[lane * kStep].cbefore <= p)) - 1;
+        if (c >= 0) c = c * kStep + __popc(__ballot_sync(0xffffffffu, lane < kStep && Q.cells[c * kStep + (lane & (kStep - 1))].cbefore <= p)) - 1;
+        const bool in = open && c >= 0 && p - Q.cells[max(c, 0)].cbefore < Q.cells[max(c, 0)].n;
+        if (lane == 0) {
+            X.cell = in ? c : -1;
+            X.open = open ? 1 : 0;
+            X.rank = p;
+            X.listed = 0u;
+        }
+    }
+    reinterpret_cast<uint2*>(bins)[gt] = make_uint2(0u, 0u);
+    sync();
+    if (X.cell < 0) {
+        if (gt == 0) {
+            Q.lv[q] = Q.lv[q - stride];
+            if (X.open) Q.fail = 1;  // no candidate cell holds the rank: an inconsistency
+        }
+        return;
+    }
+    const CandCell& cell = Q.cells[X.cell];
+    const int n = (int)cell.n;
+    const uint4* src = reinterpret_cast<const uint4*>(keys + cell.base);
+    uint32_t k = X.rank - cell.cbefore, prefix = 0u, below = 0u;
+    int rem = cell.sh, own = n;  // bits that are still open; keys that share the others
+    unsigned long long sum = 0ull;
+    auto each = [&](auto f) {
+        constexpr int kCols = 2;  // loads in flight
+#pragma unroll 1
+        for (int i0 = gt; 4 * i0 < n; i0 += kCols * threads) {
+            uint4 x[kCols];
+#pragma unroll
+            for (int u = 0; u < kCols; ++u)
+                if (4 * (i0 + u * threads) < n) x[u] = __ldcg(src + i0 + u * threads);
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) {
+                const int left = n - 4 * (i0 + u * threads);
+                if (left > 0) f(x[u].x);
+                if (left > 1) f(x[u].y);
+                if (left > 2) f(x[u].z);
+                if (left > 3) f(x[u].w);
+            }
+        }
+    };
+#pragma unroll 1
+    while (rem > 0 && own > kRest) {
+        const int bits = min(rem, bin_bits), shift = rem - bits;
+        each([&](uint32_t x) {
+            if (x >> rem == prefix) atomicAdd(bins + ((x >> shift) & ((1u << bits) - 1u)), 1u);
+        });
+        sync();
+        const uint2 c = reinterpret_cast<const uint2*>(bins)[gt];
+        uint32_t inc = c.x + c.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t nb = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += nb;
+        }
+        if (lane == 31) X.warp_n[warp] = inc;
+        reinterpret_cast<uint2*>(bins)[gt] = make_uint2(0u, 0u);  // (for the next bits)
+        sync();
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? X.warp_n[lane] : 0u) + inc - (c.x + c.y);
+        if (before <= k && k - before < c.x + c.y) {
+            const bool second = k - before >= c.x;
+            X.bin = 2u * (uint32_t)gt + (second ? 1u : 0u);
+            X.below = before + (second ? c.x : 0u);
+            X.own = second ? c.y : c.x;
+        }
+        sync();
+        const uint32_t next = prefix << bits | X.bin;
+        own = (int)X.own;
+        below += X.below;
+        k -= X.below;
+        if (stride > 1)
+            each([&](uint32_t x) {
+                if (x >> shift < next && x >> rem == prefix) sum += x;
+            });
+        prefix = next;
+        rem = shift;
+    }
+    if (rem > 0)  // a few keys, for one warp
+        each([&](uint32_t x) {
+            if (x >> rem == prefix) X.list[atomicAdd(&X.listed, 1u)] = x;
+        });
+    sum = (unsigned long long)warp_sum((long long)sum);
+    if (lane == 0) X.warp_sum[warp] = sum;
+    sync();
+    if (warp != 0) return;
+    sum = (unsigned long long)warp_sum(lane < warps ? (long long)X.warp_sum[lane] : 0ll);
+    uint32_t rel = prefix, lt = 0u, eq = (uint32_t)own;
+    if (rem > 0) {  // the k-th of them
+        rel = lane < own ? X.list[lane] : 0xffffffffu;
+        eq = 0u;
+        uint32_t smaller = 0u;
+#pragma unroll 4
+        for (int j = 0; j < own; ++j) {
+            const uint32_t x = X.list[j];
+            if (x < rel) { ++lt; smaller += x; }
+            eq += x == rel ? 1u : 0u;
+        }
+        const int at = (__ffs(__ballot_sync(0xffffffffu, lane < own && lt <= k && k - lt < eq)) - 1) & 31;
+        rel = __shfl_sync(0xffffffffu, rel, at);
+        lt = __shfl_sync(0xffffffffu, lt, at);
+        eq = __shfl_sync(0xffffffffu, eq, at);
+        sum += __shfl_sync(0xffffffffu, smaller, at);
+    }
+    if (lane == 0) {
+        LvInfo& o = Q.lv[q];
+        lt += below;
+        o.val = (double)sel_key_to_float(cell.klo + rel);
+        o.c_lt = (long long)cell.cbefore + lt;
+        o.c_le = o.c_lt + eq;
+        o.s_lt = cell.sbefore + sel_cell_sum(cell.klo, cell.sh, lt, sum);  // (of the last depth's levels nobody asks)
+        o.s_le = o.s_lt + o.val * (double)eq;
+    }
+}
+
+// The levels of tensor t, by one CTA.
+__device__ __forceinline__ void levels_from_cells(const SelArgs& A, TState* st, int t, const uint32_t* keys, int most_threads)
+{
+    CellGroups& Q = cell_groups();
+    const int tid = threadIdx.x, s = A.s;
+    __syncthreads();
+    cells_load(A, st, t, Q.cells);
+    if (tid >= kCandCells && tid - kCandCells < s) {
+        const ExactLv& e = st->lv[tid - kCandCells];
+        LvInfo& l = Q.lv[tid - kCandCells];
+        l.val = (double)sel_key_to_float(e.key);
+        l.c_lt = e.c_lt; l.c_le = e.c_le; l.s_lt = e.s_lt; l.s_le = e.s_le;
+    }
+    if (tid == kSolveThreads - 1) Q.fail = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int stride = (s - 1) >> 1; stride >= 1; stride >>= 1) {
+        const int levels = (s - 1) / (2 * stride), threads = min(kSolveThreads / levels, most_threads), g = tid / threads;
+        if (g < levels) level_by_group(stride * (2 * g + 1), stride, g, threads, keys);
+        __syncthreads();
+    }
+    if (tid < s) A.levels[(int64_t)t * s + tid] = Q.fail ? 0.f : (float)Q.lv[tid].val;
+    if (tid == 0) {
+        if (Q.fail) A.status[t] |= OGQ_ST_INTERNAL;
+        st->done = 1;
+    }
+    __syncthreads();
 }
 
 // What follows round 2, one CTA per tensor: the finish from the copied keys when round 2 only copied, else a solver pass and
@@ -2827,8 +3046,17 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve2(SelArgs A)
     const int done = __ldcg(&st->done), compact_only = __ldcg(&st->compact_only);
     const long long cand = __ldcg(&st->cand), src_cnt = (long long)__ldcg(&st->cursor[0]);
     finish_load(st, A.scheme == OGQ_BINGRAD_PB, A.s, S);  // (all loads in one go, the decision what to do with them after)
-    if (done || compact_only == 2) return;
-    if (compact_only != 0) {
+    if (done || compact_only == kOrderedLarger) return;
+    if (compact_only == kOrdered) {
+        const int most = (int)__ldcg(&st->arrive);
+        if (most > kCellsBeside && __ldcg(A.ws.nitems + 1) > 0u) {
+            if (threadIdx.x == 0) A.ws.items[(size_t)A.T * kMaxSlices - 1 - atomicAdd(A.ws.nitems + 1, 1u)].x = t;
+            return;
+        }
+        levels_from_cells(A, st, t, A.ws.buf[0] + sel_region(tbeg), most > kCellsBeside ? kSolveThreads : kGroupThreads);
+        return;
+    }
+    if (compact_only == kCompact) {
         finish_from_keys(st, t, A.scheme == OGQ_BINGRAD_PB, A.s, A.ws.buf[0] + sel_region(tbeg), (int)min(src_cnt, cand), true,
                          A.levels, A.status);
         return;
