@@ -33,13 +33,13 @@ struct BbArgs {
 
 // Sums of {v < b0} and {v >= b0} of grad[pb, pe) over the CTA; valid in thread 0.  CLIP: every value is first
 // clamped to [-tau, tau].
-template <bool CLIP>
+template <bool CLIP, bool WIDE = false>
 __device__ __forceinline__ PartSum bb_split(const float* __restrict__ grad, int64_t pb, int64_t pe, float b0, float tau,
                                             double* sh_d, long long* sh_l, bool down = false)
 {
     PartSum r = {0.0, 0.0, 0, 0};
     int below = 0;
-    visit_piece(grad, pb, pe, [&](float raw) {
+    visit_piece<WIDE>(grad, pb, pe, [&](float raw) {
         const float v = CLIP ? copysignf(fminf(fabsf(raw), tau), raw) : raw;
         const bool b = v < b0;
         const double d = (double)v;
@@ -109,7 +109,7 @@ __device__ __forceinline__ PartSum cluster_load(const PartSum* p, int rank)
 }
 
 // Grid: the flat CTAs, and in pass 0 after them one CTA per tensor for the tensors of up to kSoloN elements.
-//   Pass bound: DRAM where the bucket exceeds L2 (143.7 M elements: 101 us, 5.7 TB/s); small buckets: the
+//   Pass bound: DRAM where the bucket exceeds L2 (143.7 M elements: 92 us, 6.2 TB/s); small buckets: the
 // latency of one load and one block sum.
 template <bool CLIP>
 __global__ void __launch_bounds__(kThreads) k_bb_pass(BbArgs A, int flat_ctas, int pass)
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kThreads) k_bb_pass(BbArgs A, int flat_ctas, i
     for_each_piece(A.off, A.T, lo, hi, [&](int t, int64_t tb, int64_t te, int64_t pb, int64_t pe) {
         if (te - tb <= kSoloN || (pass > 0 && __ldcg(A.ws.done + t))) return;
         const float b0 = pass == 0 ? -INFINITY : __ldcg(A.thresh + t);
-        const PartSum a = bb_split<CLIP>(A.grad, pb, pe, b0, CLIP ? __ldcg(A.tau + t) : 0.f, sh_d, sh_l, down);
+        const PartSum a = bb_split<CLIP, true>(A.grad, pb, pe, b0, CLIP ? __ldcg(A.tau + t) : 0.f, sh_d, sh_l, down);
         if (threadIdx.x == 0) {
             BbPart p;
             p.s_lo = a.s_lo; p.s_hi = a.s_hi; p.c_lo = a.c_lo; p.c_hi = a.c_hi;
