@@ -530,32 +530,30 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
     f.mn = __int_as_float(0x7f800000); f.mx = __int_as_float(0xff800000); f.nonfinite = 0u;
     f.clipped = 0u;
     if (CLIP && threadIdx.x < 2) sh_clipped[threadIdx.x] = 0u;
-    int64_t a = (pb + 3) & ~(int64_t)3;
+    // the body from the first 32-byte boundary on, whole blocks of eight floats
+    int64_t a = pb + (int64_t)((0u - (uint32_t)(reinterpret_cast<uintptr_t>(grad + pb) >> 2)) & 7u);
     if (a > pe) a = pe;
-    int64_t b = pe & ~(int64_t)3;
-    if (b < a) b = a;
+    const int64_t b = a + ((pe - a) & ~(int64_t)7);
     const int tid = threadIdx.x;
     if (tid < (int)(a - pb)) f.one(__ldg(grad + pb + tid));
     if (tid < (int)(pe - b)) f.one(__ldg(grad + b + tid));
-    const float4* g4 = reinterpret_cast<const float4*>(grad);
-    const int64_t first = a >> 2, e = b >> 2;
-    const int ntrips = (int)((e - first) / (4 * kSelThreads));  // full trips: the same for every thread
+    const int ntrips = (int)((b - a) / (16 * kSelThreads));  // full trips: the same for every thread
     constexpr int kNp = MAG ? kPackedPerSign : kPackedCells;
     // upwards; downwards behind the clipping threshold's pass, which went up
-    constexpr int kStep = CLIP ? -4 * kSelThreads : 4 * kSelThreads;
-    const float4* src = g4 + first + tid + (CLIP ? (ntrips - 1) * 4 * kSelThreads : 0);  // this thread's next load
+    constexpr int kStep = CLIP ? -16 * kSelThreads : 16 * kSelThreads;
+    const float* src = grad + a + 8 * tid + (CLIP ? (int64_t)(ntrips - 1) * 16 * kSelThreads : 0);  // this thread's next load
     int pf_left = ntrips - kPrefetchTrips;
     for (int t0 = 0; t0 < ntrips; t0 += kPackTrips<MAG>) {
         const int nt = min(ntrips - t0, kPackTrips<MAG>);
         if (tid == 0) { sh_coarse = 0u; sh_total = 0u; }
         __syncthreads();
-        const float4* const period = src;
+        const float* const period = src;
         for (int tt = 0; tt < nt; ++tt) {
             if (tid == 0 && pf_left > 0) prefetch_l2(src + kPrefetchTrips * kStep, kTripBytes);
             --pf_left;
             float4 x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = __ldg(src + u * kSelThreads);
+            for (int u = 0; u < 4; u += 2) load8(src + u * 4 * kSelThreads, x[u], x[u + 1]);
             src += kStep;
 #pragma unroll
             for (int u = 0; u < 4; ++u) f.template four<true>(x[u]);
@@ -610,7 +608,7 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
             for (int tt = 0; tt < nt; ++tt) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const float4 x = __ldg(period + tt * kStep + u * kSelThreads);
+                    const float4 x = __ldg(reinterpret_cast<const float4*>(period + tt * kStep + (u >> 1) * 8 * kSelThreads) + (u & 1));
                     const float vv[4] = {f.canon(x.x), f.canon(x.y), f.canon(x.z), f.canon(x.w)};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -624,7 +622,8 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
         __syncthreads();  // everyone has read the totals before they are reset
     }
     __syncthreads();
-    for (int64_t i = first + (int64_t)ntrips * 4 * kSelThreads + tid; i < e; i += kSelThreads) f.template four<false>(__ldg(g4 + i));
+    const float4* rest = reinterpret_cast<const float4*>(grad + a + (int64_t)ntrips * 16 * kSelThreads);
+    for (int i = tid; i < (int)((b - a) / 4) - ntrips * 4 * kSelThreads; i += kSelThreads) f.template four<false>(__ldg(rest + i));
     if constexpr (CLIP) {
         // the clipped values, all of one magnitude: counted aside, because they would wrap the packed count of their cell in every
         // period (three clipped levels of the ResNet-50 bucket: round 1 took 52 us, with every period done again, now 38)
@@ -785,17 +784,16 @@ struct Round2Warp {
     {
         hits = __funnelshift_l(top_is_hit(__float_as_uint(clip(v))), hits, 1);
     }
-    // Parks the elements marked in `hits` (bit 15 = the first of the sixteen elements tested: p[0].x,
-    // ..., p[0].w, p[stride].x, ..., p[3 * stride].w).  The values are read again, from L1: a hit is
+    // Parks the elements marked in `hits` (bit 15 = the first of the sixteen elements tested: p[0], ..., p[7],
+    // p[stride], ..., p[stride + 7]).  The values are read again, from L1: a hit is
     // rare, and a register cannot be picked by a run-time index.
-    __device__ __forceinline__ void park_hits(uint32_t hits, const float4* p, int stride)
+    __device__ __forceinline__ void park_hits(uint32_t hits, const float* p, int stride)
     {
         while (hits) {
             const int b = 31 - __clz(hits);
             hits &= ~(1u << b);
             const int j = 15 - b;
-            const float* src = reinterpret_cast<const float*>(p + (j >> 2) * stride) + (j & 3);
-            park(__float_as_uint(clip(__ldg(src))));
+            park(__float_as_uint(clip(__ldg(p + (j >> 3) * stride + (j & 7)))));
         }
     }
 };
@@ -816,38 +814,38 @@ __device__ __forceinline__ void stream_round2(const float* __restrict__ grad, in
     w.coarse = (uint32_t)__cvta_generic_to_shared(tb.coarse);
     w.stage = (uint32_t)__cvta_generic_to_shared(sel_stage() + warp * kStageCap);
     w.fillp = (uint32_t)__cvta_generic_to_shared(&fills[warp]);
-    int64_t a = (pb + 3) & ~(int64_t)3;
+    // the body from the first 32-byte boundary on, whole blocks of eight floats
+    int64_t a = pb + (int64_t)((0u - (uint32_t)(reinterpret_cast<uintptr_t>(grad + pb) >> 2)) & 7u);
     if (a > pe) a = pe;
-    int64_t b = pe & ~(int64_t)3;
-    if (b < a) b = a;
+    const int64_t b = a + ((pe - a) & ~(int64_t)7);
     if (warp == 0) {  // ragged head and tail, one element per lane
         if (lane < (int)(a - pb)) w.one(__ldg(grad + pb + lane));
-        else if (lane >= 4 && lane - 4 < (int)(pe - b)) w.one(__ldg(grad + b + lane - 4));
+        else if (lane >= 8 && lane - 8 < (int)(pe - b)) w.one(__ldg(grad + b + lane - 8));
         __syncwarp();
     }
-    const float4* g4 = reinterpret_cast<const float4*>(grad);
-    const int64_t e = b >> 2;
-    int64_t i0 = (a >> 2) + warp * 32;  // the trip counts below are warp-uniform
-    // Trips of 4 x NT float4 (one contiguous block of 64 NT bytes per CTA).  One thread asks
+    const float* const body = grad + a + 8 * lane;
+    const int64_t e = (b - a) >> 3;    // blocks
+    int64_t i0 = warp * 32;            // the trip counts below are warp-uniform
+    // Trips of 2 x NT blocks (contiguous, 64 NT bytes per CTA).  One thread asks
     // L2 for the block kPrefetchTrips ahead, so that the loads below find their lines there.
     // A lane tests its sixteen values of a trip without branching; the warp then parks the trip's
     // hits in one go (nearly every trip has a hit in some lane, so the divergent parking code is
     // paid once per trip, not once per few values).  `fill` mirrors the stage's fill counter in a
     // register: it is the same in all lanes, so whether to drain first is a uniform decision.
-    const int64_t rest = e - i0 - 3 * NT - 32;
-    const int64_t trips = rest >= 0 ? rest / (4 * NT) + 1 : 0, after = i0 + trips * 4 * NT;
-    constexpr int64_t step = DOWN ? -4 * NT : 4 * NT;
-    if (DOWN) i0 += (trips - 1) * 4 * NT;
+    const int64_t rest = e - i0 - NT - 32;
+    const int64_t trips = rest >= 0 ? rest / (2 * NT) + 1 : 0, after = i0 + trips * 2 * NT;
+    constexpr int64_t step = DOWN ? -2 * NT : 2 * NT;
+    if (DOWN) i0 += (trips - 1) * 2 * NT;
     // blocks to ask for: thread 0's trips, but for one upwards that the CTA's last warps do not have
     int64_t pf_left = trips - kPrefetchTrips - (!DOWN && after > e ? 1 : 0);
     __syncwarp();
     int fill = *(volatile int*)&fills[warp];
-    auto park = [&](uint32_t hits, const float4* p) {
+    auto park = [&](uint32_t hits, const float* p) {
         for (;;) {  // one turn, unless the stage has to be drained to make room
             const int tot = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(hits));
             if (tot == 0) break;
             if (fill + tot <= kStageCap) {
-                if (hits) w.park_hits(hits, p, NT);
+                if (hits) w.park_hits(hits, p, 8 * NT);
                 fill += tot;
                 break;
             }
@@ -860,36 +858,41 @@ __device__ __forceinline__ void stream_round2(const float* __restrict__ grad, in
             }
             // more hits in one trip than the empty stage holds: the first eight values of every lane now
             const uint32_t first = hits & 0xff00u;
-            if (first) w.park_hits(first, p, NT);
+            if (first) w.park_hits(first, p, 8 * NT);
             fill = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(first));
             hits &= 0xffu;
         }
     };
-    auto last_trip = [&]() {  // the float4 after the whole trips, some of the four
+    auto last_trip = [&]() {  // the blocks after the whole trips
         if (after >= e) return;
+        const float* p = body + 8 * after;
         float4 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = after + lane + u * NT < e ? __ldg(g4 + after + lane + u * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < 4; u += 2) {
+            x[u] = x[u + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (after + lane + (u / 2) * NT < e) load8(p + u * 4 * NT, x[u], x[u + 1]);
+        }
         uint32_t hits = 0u;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             w.test(x[u].x, hits); w.test(x[u].y, hits); w.test(x[u].z, hits); w.test(x[u].w, hits);
-            if (after + lane + u * NT >= e) hits &= ~15u;
+            if (after + lane + (u / 2) * NT >= e) hits &= ~15u;
         }
-        park(hits, g4 + after + lane);
+        park(hits, p);
     };
     if (DOWN) last_trip();
     for (int64_t k = 0; k < trips; ++k, i0 += step) {
-        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(g4 + i0 + kPrefetchTrips * step, 4u * NT * 16u);
+        const float* p = body + 8 * i0;
+        if (threadIdx.x == 0 && k < pf_left) prefetch_l2(p + kPrefetchTrips * 8 * step, 4u * NT * 16u);
         float4 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = __ldg(g4 + i0 + lane + u * NT);
+        for (int u = 0; u < 4; u += 2) load8(p + u * 4 * NT, x[u], x[u + 1]);
         uint32_t hits = 0u;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             w.test(x[u].x, hits); w.test(x[u].y, hits); w.test(x[u].z, hits); w.test(x[u].w, hits);
         }
-        park(hits, g4 + i0 + lane);
+        park(hits, p);
     }
     if (!DOWN) last_trip();
     __syncwarp();
