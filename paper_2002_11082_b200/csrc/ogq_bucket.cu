@@ -68,6 +68,8 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
         int stbits = 0;
         // Element 4 u + c of thread t is value 4 (u nt + t) + c of the bucket: 128-bit loads, all issued
         // before the first use, and the arrangement the quantizer works in.
+        // x / n: of a full bucket, whose length is a power of two, by an exact product
+        auto over_n = [&](double x) -> double { return EXACT ? x * (1.0 / (double)KPT) * (WARP ? 0.03125 : __hiloint2double((1023 - (31 - __clz(nt))) << 20, 0)) : x / (double)n; };
         auto index = [&](int e) -> int { return 4 * ((e >> 2) * nt + t) + (e & 3); };
         auto have = [&](int e) -> bool { return EXACT || index(e) < n; };
         auto load4 = [&](int u) -> float4 {
@@ -103,12 +105,16 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
 #pragma unroll
             for (int e = 0; e < KPT; ++e) {
                 if (have(e)) {
-                    const float v = value(e);
-                    const uint32_t m = __float_as_uint(v) & 0x7fffffffu;
+                    const uint32_t m = __float_as_uint(value(e)) & 0x7fffffffu;
                     maxbits = max(maxbits, m);
                     if (e % 4 == 0) meanbits += m >> 16;
-                    if (A.clip_c > 0.f) {
-                        const double dv = (double)v - v0;
+                }
+            }
+            if (A.clip_c > 0.f) {
+#pragma unroll
+                for (int e = 0; e < KPT; ++e) {
+                    if (have(e)) {
+                        const double dv = (double)value(e) - v0;
                         sums[0] += dv;
                         sums[1] += dv * dv;
                     }
@@ -118,7 +124,7 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
             meanbits = (uint32_t)((float)meanbits / (float)((n + 3) >> 2));  // of every fourth value
             if (A.clip_c > 0.f) {
                 team_sum<WARP>(sums, X.d);
-                double var = (sums[1] - sums[0] * sums[0] / (double)n) / (double)n;
+                double var = over_n(sums[1] - over_n(sums[0] * sums[0]));
                 if (!(var > 0.0)) var = 0.0;  // also a non-finite bucket: everything clips to 0
                 tau = (float)((double)A.clip_c * sqrt(var));
             }
@@ -149,7 +155,7 @@ __device__ __forceinline__ void bkt_encode_one(const BktArgs& A, const PhiloxKey
             for (int e = 0; e < KPT; ++e)
                 if (have(e)) sum[0] += (double)clipped(e);
             team_sum<WARP>(sum, X.d);
-            b0 = (float)(sum[0] / (double)n);
+            b0 = (float)over_n(sum[0]);
             long long prev_lo = -1;
             float l_lo = 0.f, l_hi = 0.f;
             for (int it = 0;; ++it) {
