@@ -111,7 +111,7 @@ cudaError_t launch_bucket_decode_sum(const uint32_t* const* d_packed_k, const fl
 #define OGQ_LAUNCH_BD(B)                                                                                        \
     do {                                                                                                        \
         rows = (size_t)kWarps * 2 * row_bytes<B>(K);                                                            \
-        e = with_rest<B>(rest_of<B, false>(K), [&](auto rest) -> cudaError_t {                                  \
+        e = with_rest<B, false>(rest_of<B, false>(K), [&](auto rest) -> cudaError_t {                                  \
             auto kernel = pairs ? k_bucket_decode_sum<B, decltype(rest)::value, true>                           \
                                 : k_bucket_decode_sum<B, decltype(rest)::value, false>;                         \
             if (rows > 40 * 1024) {                                                                             \

@@ -189,9 +189,9 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
     const int64_t lo = (int64_t)blockIdx.x * chunk;
     const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if ((int)threadIdx.x < K) {
-        sh_pk[threadIdx.x] = packed_k[threadIdx.x];
-        sh_lv[threadIdx.x] = levels_k[threadIdx.x];
+    if ((int)threadIdx.x < (REST < 0 ? 8 : K)) {  // (a table's absent workers read the last one's codes)
+        sh_pk[threadIdx.x] = packed_k[min((int)threadIdx.x, K - 1)];
+        if ((int)threadIdx.x < K) sh_lv[threadIdx.x] = levels_k[threadIdx.x];
     }
     __syncthreads();
     const uint32_t rb = row_bytes<BITS>(K);
@@ -257,7 +257,38 @@ k_unpack_sum(const uint32_t* const* __restrict__ packed_k, const float* const* _
         constexpr int kAhead = 8;  // trips between two prefetch requests
         constexpr int kTrip = G * kWarps;
         int gl = first;
-        for (int trip = 0; gl + kWarps < ng; gl += kTrip, ++trip) {
+        if constexpr (REST < 0) {
+            // 1-bit codes of a few workers: a warp takes four groups in a row, whose codes are one word per lane and worker, and gets a
+            // group's bytes from the lanes that have them.
+            constexpr int N = REST == kTableOnly ? 8 : 4;  // (codes of workers that do not exist mean nothing to the table)
+            const int quads = ng >> 2;
+            uint32_t next[N];
+            auto load = [&](int q) {
+#pragma unroll
+                for (int u = 0; u < N; ++u) next[u] = __ldcg(sh_pk[u] + w0 + (int64_t)q * 32 + lane);
+            };
+            int q = first;
+            if (q < quads) load(q);
+            for (; q < quads; q += kWarps) {
+                uint32_t w[N];
+#pragma unroll
+                for (int u = 0; u < N; ++u) w[u] = next[u];
+                if (q + kWarps < quads) load(q + kWarps);
+#pragma unroll 1
+                for (int g = 0; g < 4; ++g) {
+                    uint32_t c[kTableWorkers<BITS>], x[2];
+#pragma unroll
+                    for (int u = 0; u < kTableWorkers<BITS>; ++u)
+                        c[u] = u < N ? __byte_perm(__shfl_sync(0xffffffffu, w[u < N ? u : 0], 8 * g + (lane >> 2)), 0u, 0x4440 + (lane & 3)) : 0u;
+                    table_indices<BITS>(c, x);
+                    float a[8];
+                    read_table(x, table, a);
+                    write(4 * q + g, a);
+                }
+            }
+            gl = 4 * quads + first;
+        }
+        for (int trip = 0; REST >= 0 && gl + kWarps < ng; gl += kTrip, ++trip) {
             // every kAhead trips K threads ask L2 for the workers' words of the kAhead trips after the next
             // kAhead (no gain at one bit per code)
             if (BITS >= 2 && (trip & (kAhead - 1)) == 0 && (int)threadIdx.x < K && (trip + 2 * kAhead) * kTrip <= ng)
@@ -421,6 +452,9 @@ cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* co
 {
     const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas, 4096);
     const int bits = ogq_bits_for_levels(s);
+    // 1-bit codes, four groups of a tensor at a time, where a CTA has many of one (VGG-19 bucket, eight workers: 180 -> 131 us; 5 M elements
+    // 10.1 -> 8.8): many small tensors want their groups shared out more evenly (3 M in 50, five workers: 9.4 against 10.9).
+    const bool quads = total / (g.ctas + T) >= 8192;
     cudaError_t e = cudaErrorInvalidValue;
 #define OGQ_LAUNCH_U(B)                                                                               \
     if (K == 1) { /* faster at every size and width measured, see the kernel */                       \
@@ -429,7 +463,7 @@ cudaError_t launch_unpack_sum(const uint32_t* const* d_packed_k, const float* co
     } else {                                                                                          \
         const size_t each = row_bytes<B>(K), tables = kTableFloats<B> > 0 ? kMaxTables * 1024 : 0;       \
         const int batch = (int)std::min<size_t>(std::max<size_t>(kRowsBytes / each, 1), (size_t)std::min(T, tables ? kMaxTables : 32)); \
-        e = with_rest<B>(rest_of<B, true>(K), [&](auto rest) {                                         \
+        e = with_rest<B, true>(rest_of<B, true>(K, quads), [&](auto rest) {                                         \
             return launch_pdl(k_unpack_sum<B, decltype(rest)::value>, g.ctas, kThreads, tables + each * batch, stream, d_packed_k, \
                               d_levels_k, K, d_off, d_packed_off, T, total, g.chunk, s, batch, scale, d_out); \
         });                                                                                           \

@@ -26,11 +26,13 @@ constexpr int kTableFloats = kTableWorkers<BITS> ? 256 : 0;
 // seven 55 -> 45).  Eight at a time but for 3-bit codes, where four were as fast with half the instructions to fetch.
 template <int BITS>
 constexpr int kBatch = BITS == 1 || BITS == 3 ? 4 : 8;
+// In place of that number, 1-bit codes: the table of sums takes in all workers, up to eight (kTableOnly) or four of them.
+constexpr int kTableOnly = -1;
 template <int BITS, bool TABLE>
-int rest_of(int K)
+int rest_of(int K, bool quads = false)
 {
     const int rows = K - (TABLE ? kTableWorkers<BITS> : 0);
-    return rows > 0 ? rows % kBatch<BITS> : 0;
+    return rows > 0 ? rows % kBatch<BITS> : TABLE && BITS == 1 && quads ? (K > 4 ? kTableOnly : kTableOnly - 1) : 0;
 }
 template <int BITS>
 constexpr int kRowStride = 1 << BITS;  // floats per level row: every code a field can hold has an entry
@@ -69,11 +71,11 @@ __device__ __forceinline__ EightCodes<BITS> load_codes(const uint32_t* __restric
 }
 
 // launch(std::integral_constant<int, REST>) for the number of workers in the last, partial batch.
-template <int BITS, int R = kBatch<BITS> - 1, class Launch>
+template <int BITS, bool TABLE, int R = kBatch<BITS> - 1, class Launch>
 cudaError_t with_rest(int rest, Launch launch)
 {
     if (rest == R) return launch(std::integral_constant<int, R>());
-    if constexpr (R > 0) return with_rest<BITS, R - 1>(rest, launch);
+    if constexpr (R > (TABLE && BITS == 1 ? kTableOnly - 1 : 0)) return with_rest<BITS, TABLE, R - 1>(rest, launch);
     else return cudaErrorInvalidValue;
 }
 
@@ -242,7 +244,8 @@ __device__ __forceinline__ void sum_workers(int K, int lane, uint32_t table, uin
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[g][j] = 0.f;
     }
-    for (; k0 + B <= K; k0 += B) sum_batch<BITS, G, B>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
+    if constexpr (REST >= 0)
+        for (; k0 + B <= K; k0 += B) sum_batch<BITS, G, B>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
     if constexpr (REST > 0) sum_batch<BITS, G, REST>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
 }
 
