@@ -9,12 +9,12 @@
 // direction, and copies the few percent of elements inside the intervals to scratch.  What follows depends on their
 // number:
 //   up to kSortN            round 2 only copies them; one CTA indexes the copied keys and finishes the tensor.
-//   ORQ, more, and room     round 2 copies them in order of round 1's cells; a cluster of CTAs selects every
-//                           level among the keys of the cell that holds its rank (k_sel_round3).
+//   ORQ, more, and room     round 2 copies them in order of round 1's cells; every level is selected among the keys of the
+//                           cell that holds its rank, by one CTA, or where a cell has many, by a cluster (k_sel_round3).
 //   otherwise               round 2 counts them on a finer grid as well; another launch per tensor solves again, and round
 //                           3 and later work on the copied keys only, until every level's rank falls into a single-key
 //                           cell or one CTA's index holds the rest.
-// Tensors of at most kSmallN elements are not streamed: the first solver launch indexes them in shared memory.  The key
+// Tensors of at most kSmallN elements are not streamed: the second solver launch indexes them in shared memory.  The key
 // buffers hold one eighth of the bucket: a pass whose copies do not fit is repeated on the gradient with
 // the narrower intervals.
 //
@@ -22,9 +22,10 @@
 // values reach their cells: counts are exact, sums of what one cell holds are exact but for values of many
 // binades, and an integer T is recognised within their rounding (floor_of_t).  No kernel waits on another CTA but for the
 // clusters of round 3; the slices of a tensor there are counted off by an atomic, and the last CTA goes on with the solver.
-//   What bounds it: the rounds stream at 4.6 to 5.0 TB/s from DRAM, bound by the integer pipe (with every load pinned to one
-// block in the cache round 1 of 143.7 M elements takes 133 us, with its own loads 125); the solver launches are bound by
-// the latency of one CTA's barriers and of code that runs once (ResNet-50 bucket, nine levels: about 21 and 17 of 147 us).
+//   What bounds it: the rounds stream at 4.7 to 5.1 TB/s from DRAM, bound by the integer pipe and the wait for their loads
+// (60 % of the issue slots); the solver launches are bound by the latency of one CTA's barriers and of code that runs once
+// (ResNet-50 bucket, nine levels: about 13 and 16 of 135 us, 20,000 and 30,000 cycles).  Running them on made-up cells
+// while they wait, so that their instructions are in the cache, gained nothing: the second run takes as long as the first.
 // Solving in the streaming kernels, by the CTA that arrived last, took 89 and 125 us for the two rounds of that bucket
 // instead of 61 and 61.
 #include <math.h>
@@ -2495,7 +2496,7 @@ __device__ __noinline__ void solve1_level(int lo_e, double n, int q, int stride)
 
 // One CTA per streamed tensor: prefix sums over round 1's cells, conservative cell ranges of the levels, every populated cell in
 // them becomes an interval of round 2.
-//   What bounds it: latency, 20,000 cycles of barriers, dependent loads and code that runs once.
+//   What bounds it: latency, 20,000 cycles of barriers, dependent loads and code that runs once (12,000 for BinGrad-pb).
 __global__ void __launch_bounds__(kSolveThreads, 1) k_sel_solve1(SelArgs A)
 {
     SolverShared& S = sel_state();
