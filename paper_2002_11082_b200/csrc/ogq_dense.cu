@@ -254,6 +254,22 @@ __device__ __forceinline__ void dense_rows(float* rows, const float* const* lv, 
 {
     using Row = DenseRow<S, D>;
     const int lane = threadIdx.x & 31;
+    if constexpr (D == 2) {
+        // A warp has a worker or a few to itself: both tables straight from the levels, one wait and one barrier.  (With three
+        // tables, and with one warp for all workers, it is no faster: 1 % and 3 % more for eight workers.)
+        if (warps > 1) {
+            if (lane < Row::kEntries) {
+                for (int k = w; k < K; k += warps) {
+                    const float* l = lv[k] + t * S;
+                    float* row = rows + k * Row::kFloats;
+                    row[lane] = __ldcg(l + lane / S);
+                    row[Row::kEntries + lane] = __ldcg(l + lane % S);
+                }
+            }
+            sync();
+            return;
+        }
+    }
     for (int i = w * 32 + lane; i < K * S; i += warps * 32) rows[i / S * Row::kFloats + Row::kPlain + i % S] = __ldcg(lv[i / S] + t * S + i % S);
     sync();
     if constexpr (D > 1) {
@@ -273,13 +289,20 @@ __device__ __forceinline__ void dense_rows(float* rows, const float* const* lv, 
     }
 }
 
+// Workers whose words the server step asks for before it uses any.
+template <int S> constexpr int kDenseBatch = Dense<S>::M == 20 ? 2 : 4;
+
 // What bounds it: shared-memory reads, one per element and worker, with the instructions for the digits close behind: a wide product
 // holds the multiply pipe for four cycles.  So three digits at a time (S = 3) or two (S = 5) come from one product and one address,
 // each with a read of a table of its own, as long as four CTAs' tables fit an SM (25.6 M elements of eight workers at S = 5, whole
 // step: 204 -> 198 us; 20 M at S = 3: 49 -> 41).  (One lane per group with divisions by S and stores of its own, each spread over 32 lines: 119 us for 25.6 M
 // elements of 8 workers at s = 5.)  Two digits at a time through one table of pairs were no faster: a 64-bit
 // read costs as much as two.
-template <int S, int D>
+// REST: number of workers in the last, partial batch.  They are loaded together as those of a full one, and as a template argument
+// it leaves no condition between them (25 M elements in 161 tensors, two and three workers, one after the other before: S = 5 37 -> 31
+// and 47 -> 35 us, S = 9 46 -> 35 and 58 -> 42; seven workers of nine levels 87 -> 73).  With a loop over the number instead, the full
+// batches of S = 9 get slower (eight workers 76 -> 83 us).
+template <int S, int D, int REST>
 __global__ void __launch_bounds__(kThreads, 4)
 k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* const* __restrict__ levels_k, int K,
                    const int64_t* __restrict__ off, const int64_t* __restrict__ packed_off, int T, int64_t total,
@@ -342,30 +365,17 @@ k_unpack_sum_dense(const uint32_t* const* __restrict__ packed_k, const float* co
             float acc[M];
 #pragma unroll
             for (int e = 0; e < M; ++e) acc[e] = 0.f;
-            constexpr int B = M == 20 ? 2 : 4;  // workers whose words are loaded before any is used
-            if constexpr (S == 17) {
-                // the words of the last, partial batch are loaded together, too (one worker after the other: 131 instead of
-                // 114 us for 25.6 M elements of eleven workers; with the longer words of the other S the conditions cost
-                // more than they save)
-                for (int k = 0; k < K; k += B) {
-                    uint32_t w[B];
+            constexpr int B = kDenseBatch<S>;
+            auto batch = [&](auto count, int k) {
+                constexpr int N = decltype(count)::value;
+                uint32_t w[N];
 #pragma unroll
-                    for (int u = 0; u < B; ++u) w[u] = have && k + u < K ? __ldcg(sh_pk[k + u] + at) : 0u;
+                for (int u = 0; u < N; ++u) w[u] = have ? __ldcg(sh_pk[k + u] + at) : 0u;
 #pragma unroll
-                    for (int u = 0; u < B; ++u)
-                        if (k + u < K) add_digits<S, D>(w[u], rows_addr + (k + u) * (kRow * 4), acc);
-                }
-            } else {
-                int k = 0;
-                for (; k + B <= K; k += B) {
-                    uint32_t w[B];
-#pragma unroll
-                    for (int u = 0; u < B; ++u) w[u] = have ? __ldcg(sh_pk[k + u] + at) : 0u;
-#pragma unroll
-                    for (int u = 0; u < B; ++u) add_digits<S, D>(w[u], rows_addr + (k + u) * (kRow * 4), acc);
-                }
-                for (; k < K; ++k) add_digits<S, D>(have ? __ldcg(sh_pk[k] + at) : 0u, rows_addr + k * (kRow * 4), acc);
-            }
+                for (int u = 0; u < N; ++u) add_digits<S, D>(w[u], rows_addr + (k + u) * (kRow * 4), acc);
+            };
+            for (int k = 0; k + B <= K; k += B) batch(std::integral_constant<int, B>{}, k);
+            if constexpr (REST > 0) batch(std::integral_constant<int, REST>{}, K - REST);
 #pragma unroll
             for (int e = 0; e < M; ++e) acc[e] = __fmul_rn(acc[e], scale);
             float* mine = sum + lane * M;  // no bank conflicts at any of these strides and widths
@@ -431,24 +441,39 @@ cudaError_t launch_unpack_sum_dense(const uint32_t* const* d_packed_k, const flo
     auto bytes = [&](int digits, int row) { return (size_t)(kWarps * 32 * digits + (kWarps + 2) * K * row) * sizeof(float); };
     // shared memory of which four CTAs fit an SM
     constexpr size_t kFour = 54 * 1024;
-#define OGQ_LAUNCH_UD(SS, DD)                                                                                   \
-    e = launch_pdl_smem(k_unpack_sum_dense<SS, DD>, g.ctas, kThreads, bytes(Dense<SS>::M, DenseRow<SS, DD>::kFloats), stream, \
-                        d_packed_k, d_levels_k, K, d_off, d_packed_off, T, total, g.chunk, scale, d_out)
+    auto launch = [&](auto levels, auto digits, auto rest) {
+        constexpr int S = decltype(levels)::value, D = decltype(digits)::value, R = decltype(rest)::value;
+        e = launch_pdl_smem(k_unpack_sum_dense<S, D, R>, g.ctas, kThreads, bytes(Dense<S>::M, DenseRow<S, D>::kFloats), stream,
+                            d_packed_k, d_levels_k, K, d_off, d_packed_off, T, total, g.chunk, scale, d_out);
+    };
+    auto pick = [&](auto levels, auto digits) {
+        constexpr int B = kDenseBatch<decltype(levels)::value>;
+        const int rest = K % B;
+        if (rest == 0) launch(levels, digits, std::integral_constant<int, 0>{});
+        else if (rest == 1) launch(levels, digits, std::integral_constant<int, 1>{});
+        else if constexpr (B > 2) {
+            if (rest == 2) launch(levels, digits, std::integral_constant<int, 2>{});
+            else launch(levels, digits, std::integral_constant<int, 3>{});
+        }
+    };
+    constexpr std::integral_constant<int, 1> one{};
+    constexpr std::integral_constant<int, 2> two{};
+    constexpr std::integral_constant<int, 3> three{};
+    constexpr std::integral_constant<int, 5> five{};
     switch (s) {
         case 3:
-            if (bytes(Dense<3>::M, DenseRow<3, 3>::kFloats) <= kFour) OGQ_LAUNCH_UD(3, 3);
-            else if (bytes(Dense<3>::M, DenseRow<3, 2>::kFloats) <= kFour) OGQ_LAUNCH_UD(3, 2);
-            else OGQ_LAUNCH_UD(3, 1);
+            if (bytes(Dense<3>::M, DenseRow<3, 3>::kFloats) <= kFour) pick(three, three);
+            else if (bytes(Dense<3>::M, DenseRow<3, 2>::kFloats) <= kFour) pick(three, two);
+            else pick(three, one);
             break;
         case 5:
-            if (bytes(Dense<5>::M, DenseRow<5, 2>::kFloats) <= kFour) OGQ_LAUNCH_UD(5, 2);
-            else OGQ_LAUNCH_UD(5, 1);
+            if (bytes(Dense<5>::M, DenseRow<5, 2>::kFloats) <= kFour) pick(five, two);
+            else pick(five, one);
             break;
-        case 9: OGQ_LAUNCH_UD(9, 1); break;
-        case 17: OGQ_LAUNCH_UD(17, 1); break;
+        case 9: pick(std::integral_constant<int, 9>{}, one); break;
+        case 17: pick(std::integral_constant<int, 17>{}, one); break;
         default: return cudaErrorInvalidValue;
     }
-#undef OGQ_LAUNCH_UD
     launch_end(stream);
     return e;
 }

@@ -43,7 +43,8 @@ def test_unpack_sum_partial_batches(s, K):
     assert np.all(np.abs(got.astype(np.float64) - want) <= bound)
 
 
-@pytest.mark.parametrize("s,K", [(3, 10), (3, 11), (3, 48), (3, 49), (5, 1), (5, 20), (5, 21), (9, 6), (17, 7)])
+@pytest.mark.parametrize("s,K", [(3, 10), (3, 11), (3, 48), (3, 49), (5, 1), (5, 20), (5, 21), (9, 6), (17, 7)]
+                         + [(s, K) for s in (3, 5, 9, 17) for K in (2, 3, 4, 5, 8)])
 def test_unpack_sum_dense_tables(s, K):
     off, packed, levels, h_po, bound = workers(s, K, dense=True)
     dev = torch.device("cuda:0")
