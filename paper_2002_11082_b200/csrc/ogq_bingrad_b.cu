@@ -39,14 +39,16 @@ __device__ __forceinline__ PartSum bb_split(const float* __restrict__ grad, int6
 {
     PartSum r = {0.0, 0.0, 0, 0};
     int below = 0;
-    visit_piece<WIDE>(grad, pb, pe, [&](float raw) {
+    auto add = [&](float raw) {
         const float v = CLIP ? copysignf(fminf(fabsf(raw), tau), raw) : raw;
         const bool b = v < b0;
         const double d = (double)v;
         r.s_lo += b ? d : 0.0;
         r.s_hi += b ? 0.0 : d;
         below += b ? 1 : 0;
-    }, down);
+    };
+    if constexpr (WIDE) visit_piece_wide(grad, pb, pe, add, down);
+    else visit_piece(grad, pb, pe, add, down);
     r.s_lo = block_sum(r.s_lo, sh_d);
     r.s_hi = block_sum(r.s_hi, sh_d);
     r.c_lo = block_sum((long long)below, sh_l);
@@ -111,8 +113,11 @@ __device__ __forceinline__ PartSum cluster_load(const PartSum* p, int rank)
 // Grid: the flat CTAs, and in pass 0 after them one CTA per tensor for the tensors of up to kSoloN elements.
 //   Pass bound: DRAM where the bucket exceeds L2 (143.7 M elements: 92 us, 6.2 TB/s); small buckets: the
 // latency of one load and one block sum.
+//   48 registers: an SM takes a fifth CTA beside the grid's four.  With 62 the passes of eight workers on eight streams had no room
+// for one another (ResNet-50 bucket: 411 us, now 377), and neither had the CTAs of small tensors (9000 of 3000 elements: 148, now
+// 139).  The clipped passes, which wait for fp64 as much as for DRAM, had 60 before the wide loads and keep 64.
 template <bool CLIP>
-__global__ void __launch_bounds__(kThreads) k_bb_pass(BbArgs A, int flat_ctas, int pass)
+__global__ void __launch_bounds__(kThreads, CLIP ? 4 : 5) k_bb_pass(BbArgs A, int flat_ctas, int pass)
 {
     __shared__ double sh_d[kWarps];
     __shared__ long long sh_l[kWarps];
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(kThreads) k_bb_pass(BbArgs A, int flat_ctas, i
         BbState st;
         float b0 = -INFINITY;
         for (int p = 0;; ++p) {
-            const PartSum a = bb_split<CLIP>(A.grad, tb, te, b0, tau, sh_d, sh_l);
+            const PartSum a = bb_split<CLIP, true>(A.grad, tb, te, b0, tau, sh_d, sh_l);
             bool end = false;
             if (threadIdx.x == 0) {
                 end = bb_advance(a, p, A.lloyd_iters, st);
@@ -257,6 +262,14 @@ __global__ void __cluster_dims__(kBbCluster, 1, 1) __launch_bounds__(kThreads) k
     cluster_sync();  // a CTA's shared memory stays until the others have read it
 }
 
+// From this size on a pass keeps the fifth place of every SM empty, with shared memory that it does not use.  A pass is launched
+// while the kernel before it drains; SMs that are done early otherwise take five of its CTAs and others three, and the whole
+// waits for the SMs with five (one worker, encode: 143.7 M elements 298 and 280 us, 40 M 89 and 86).  Smaller buckets lose
+// less by it than several streams gain (ResNet-50 bucket, eight streams: 378 us, 409 with the place kept empty; one stream:
+// 67 us either way behind a threshold quantizer that lets a pass be launched late, see there).
+constexpr int64_t kBbAloneN = 32 << 20;
+constexpr size_t kBbAloneBytes = 46 * 1024;  // four CTAs fit an SM, five do not
+
 static FlatGrid bb_grid(int64_t total, int sm_count)
 {
     return make_flat_grid(total, sm_count * 4 < kMaxFlatCtas ? sm_count * 4 : kMaxFlatCtas, 8192);
@@ -277,10 +290,11 @@ static cudaError_t bb_run(const float* d_grad, const int64_t* d_off, int T, int6
     }
     const int flat = total > kSoloN ? g.ctas : 0;  // some tensor may be larger than one CTA solves on its own
     auto kernel = d_tau ? k_bb_pass<true> : k_bb_pass<false>;
+    const size_t unused = total >= kBbAloneN && T <= g.ctas ? kBbAloneBytes : 0;  // (not where CTAs of small tensors want the place)
     cudaError_t e = cudaSuccess;
     for (int pass = 0; pass <= lloyd_iters + 1 && e == cudaSuccess; ++pass) {
         launch_begin("k_bb_pass", stream);
-        e = launch_pdl(kernel, flat + (pass == 0 ? T : 0), kThreads, 0, stream, A, flat, pass);
+        e = launch_pdl(kernel, flat + (pass == 0 ? T : 0), kThreads, unused, stream, A, flat, pass);
         launch_end(stream);
         if (flat == 0 || e != cudaSuccess) break;
         launch_begin("k_bb_combine", stream);

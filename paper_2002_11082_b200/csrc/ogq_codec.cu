@@ -23,12 +23,13 @@ __global__ void __launch_bounds__(kThreads, 4)
 k_quantize_pack(const float* __restrict__ grad, const int64_t* __restrict__ off, int T, int64_t total,
                 int64_t chunk, int s, const float* levels, const float* thresh, const float* tau_arr,
                 const __grid_constant__ PhiloxKeys keys, uint32_t stream_id,
-                const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed, const __grid_constant__ QuantSteps steps)
+                const int64_t* __restrict__ packed_off, uint32_t* __restrict__ packed, const __grid_constant__ QuantSteps steps,
+                int early)
 {
     __shared__ float sh_lv[kMaxLevels];
     __shared__ float2 sh_tab[kMaxLevels];
     pdl_wait();
-    pdl_launch_dependents();
+    if (early) pdl_launch_dependents();
 
     const int64_t lo = (int64_t)blockIdx.x * chunk;
     const int64_t hi = (lo + chunk < total) ? lo + chunk : total;
@@ -418,10 +419,13 @@ cudaError_t launch_quantize_pack(const float* d_grad, const int64_t* d_off, int 
     const FlatGrid g = make_flat_grid(total, sm_count * kStreamCtas * (scheme == OGQ_BINGRAD_B ? 1 : 3), 8192);
     const PhiloxKeys keys = philox_round_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     const int bits = ogq_bits_for_levels(s);
+    // What follows a threshold quantizer of a full wave is launched when its CTAs end: the next worker's first pass would otherwise
+    // share the SMs out unevenly (see kBbAloneN; ResNet-50 bucket in one bit, one worker after the other: 68.1 and 67.1 us each).
+    const int early = scheme != OGQ_BINGRAD_B || g.ctas <= sm_count * (kStreamCtas - 1) ? 1 : 0;
     cudaError_t e = cudaErrorInvalidValue;
 #define OGQ_LAUNCH_QC(B, TH, CL)                                                                        \
     e = launch_pdl(k_quantize_pack<B, TH, CL>, g.ctas, kThreads, 0, stream, d_grad, d_off, T, total, g.chunk, s, \
-                   d_levels, d_thresh, d_tau, keys, stream_id, d_packed_off, d_packed, quant_steps())
+                   d_levels, d_thresh, d_tau, keys, stream_id, d_packed_off, d_packed, quant_steps(), early)
 #define OGQ_LAUNCH_Q(B, TH)                    \
     do {                                       \
         if (d_tau) OGQ_LAUNCH_QC(B, TH, true); \

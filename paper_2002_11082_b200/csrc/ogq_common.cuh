@@ -148,9 +148,7 @@ __device__ __forceinline__ void load8(const float* p, float4& a, float4& b)
 
 // Block-cooperative visit of grad[pb, pe): 128-bit loads on the aligned body,
 // scalar loads on the ragged head and tail; downwards when `down`.  f(float) is called once per element.
-// WIDE: 256-bit loads, two in flight per thread, where the body lies on 32-byte boundaries (BinGrad-b's passes over 143.7 M elements,
-// which wait for DRAM: 98 -> 92 us each; four in flight 101.  The clipping threshold, which waits for fp64, ran slower: 25 -> 27).
-template <bool WIDE = false, class F>
+template <class F>
 __device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int64_t pb, int64_t pe, F f, bool down = false)
 {
     int64_t a = (pb + 3) & ~(int64_t)3;
@@ -161,23 +159,7 @@ __device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int6
     if (tid < (int)(a - pb)) f(__ldg(grad + pb + tid));
     if (tid < (int)(pe - b)) f(__ldg(grad + b + tid));
     const float4* g4 = reinterpret_cast<const float4*>(grad);
-    const int64_t e = b >> 2;
-    int64_t first = (a >> 2) + tid;
-    if constexpr (WIDE) {
-        if ((reinterpret_cast<uintptr_t>(g4 + (a >> 2)) & 31) == 0) {
-            constexpr int kTrip = 4 * kThreads;  // float4s
-            const int64_t trips = (e - (a >> 2)) / kTrip;
-            const float* p = grad + a + 8 * tid + (down ? (trips - 1) * 4 * kTrip : 0);
-            for (int64_t k = 0; k < trips; ++k, p += down ? -4 * kTrip : 4 * kTrip) {
-                float4 x[4];
-                load8(p, x[0], x[1]);
-                load8(p + 8 * kThreads, x[2], x[3]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) { f(x[u].x); f(x[u].y); f(x[u].z); f(x[u].w); }
-            }
-            first += trips * kTrip;
-        }
-    }
+    const int64_t first = (a >> 2) + tid, e = b >> 2;
     const int64_t trips = first + 3 * kThreads < e ? (e - first - 3 * kThreads - 1) / (4 * kThreads) + 1 : 0;
     const int64_t step = down ? -4 * kThreads : 4 * kThreads;
     int64_t i = down ? first + (trips - 1) * 4 * kThreads : first;
@@ -194,6 +176,37 @@ __device__ __forceinline__ void visit_piece(const float* __restrict__ grad, int6
     for (i = first + trips * 4 * kThreads; i < e; i += kThreads) {
         float4 x = __ldg(g4 + i);
         f(x.x); f(x.y); f(x.z); f(x.w);
+    }
+}
+
+// The same with 256-bit loads, two in flight per thread, on a body that begins at the first 32-byte boundary of memory
+// (BinGrad-b's passes over 143.7 M elements, which wait for DRAM: 98 -> 92 us each; four in flight 101.  The clipping
+// threshold, which waits for fp64, ran slower: 25 -> 27).
+template <class F>
+__device__ __forceinline__ void visit_piece_wide(const float* __restrict__ grad, int64_t pb, int64_t pe, F f, bool down)
+{
+    int64_t a = pb + (int64_t)((0u - (uint32_t)(reinterpret_cast<uintptr_t>(grad + pb) >> 2)) & 7u);
+    if (a > pe) a = pe;
+    const int tid = threadIdx.x, blocks = (int)((pe - a) >> 3);  // of eight floats
+    const int64_t b = a + 8 * (int64_t)blocks;
+    if (tid < (int)(a - pb)) f(__ldg(grad + pb + tid));
+    if (tid < (int)(pe - b)) f(__ldg(grad + b + tid));
+    constexpr int kTrip = 2 * kThreads;  // blocks
+    const int trips = blocks / kTrip;
+    const float* body = grad + a + 8 * tid;
+    const float* p = body + (down ? (int64_t)(trips - 1) * 8 * kTrip : 0);
+    for (int k = 0; k < trips; ++k, p += down ? -8 * kTrip : 8 * kTrip) {
+        float4 x[4];
+        load8(p, x[0], x[1]);
+        load8(p + 8 * kThreads, x[2], x[3]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { f(x[u].x); f(x[u].y); f(x[u].z); f(x[u].w); }
+    }
+    for (int i = trips * kTrip + tid; i < blocks; i += kThreads) {
+        float4 x[2];
+        load8(body + 8 * (int64_t)(i - tid), x[0], x[1]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) { f(x[u].x); f(x[u].y); f(x[u].z); f(x[u].w); }
     }
 }
 
