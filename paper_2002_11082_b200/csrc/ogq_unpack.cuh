@@ -22,19 +22,26 @@ template <int BITS>
 constexpr int kTableWorkers = BITS == 1 ? 8 : BITS == 2 ? 4 : 0;  // workers that the table of sums takes in (0: no table)
 template <int BITS>
 constexpr int kTableFloats = kTableWorkers<BITS> ? 256 : 0;
-// Workers whose words are loaded before any is used, and those of the last, partial batch.  That number is a template argument of the
-// kernels: a kernel then has no condition between the reads of one worker's levels and the next's, which kept them from
+// Workers whose words are loaded before any is used, and those of the last batch, which may be a full one.  That number is a template
+// argument of the kernels: a kernel then has no condition between the reads of one worker's levels and the next's, which kept them from
 // overlapping, and no instructions but its own (20 M elements of nine levels: two workers 26.9 -> 21 us, five 38 -> 32; 17 levels,
 // seven 55 -> 45).  Eight at a time but for 3-bit codes, where four were as fast with half the instructions to fetch.
+//   The last full batch outside the loop as well: in the loop its words are waited for batch by batch (VGG-19 bucket, a loop for all full
+// batches and this: nine levels, eight workers 301 and 291 us; 17 levels, eight 370 and 351; 1-bit codes, twelve 277 and 242).
 template <int BITS>
 constexpr int kBatch = BITS == 1 || BITS == 3 ? 4 : 8;
+// Workers of the last batch, at most.  Behind the table of 1-bit codes it is a double one, which takes in up to sixteen workers without a
+// loop (VGG-19 bucket, sixteen: 403 us in the loop, 326 so).
+template <int BITS, bool TABLE>
+constexpr int kLast = TABLE && BITS == 1 ? 2 * kBatch<BITS> : kBatch<BITS>;
 // In place of that number, 1-bit codes: the table of sums takes in all workers, up to eight (kTableOnly) or four of them.
 constexpr int kTableOnly = -1;
 template <int BITS, bool TABLE>
 int rest_of(int K, bool quads = false)
 {
     const int rows = K - (TABLE ? kTableWorkers<BITS> : 0);
-    return rows > 0 ? rows % kBatch<BITS> : TABLE && BITS == 1 && quads ? (K > 4 ? kTableOnly : kTableOnly - 1) : 0;
+    if (rows > kLast<BITS, TABLE>) return kLast<BITS, TABLE> - kBatch<BITS> + 1 + (rows - kLast<BITS, TABLE> - 1) % kBatch<BITS>;
+    return rows > 0 ? rows : TABLE && BITS == 1 && quads ? (K > 4 ? kTableOnly : kTableOnly - 1) : 0;
 }
 template <int BITS>
 constexpr int kRowStride = 1 << BITS;  // floats per level row: every code a field can hold has an entry
@@ -72,12 +79,12 @@ __device__ __forceinline__ EightCodes<BITS> load_codes(const uint32_t* __restric
     return c;
 }
 
-// launch(std::integral_constant<int, REST>) for the number of workers in the last, partial batch.
-template <int BITS, bool TABLE, int R = kBatch<BITS> - 1, class Launch>
+// launch(std::integral_constant<int, REST>) for the number of workers in the last batch.
+template <int BITS, bool TABLE, int R = kLast<BITS, TABLE>, class Launch>
 cudaError_t with_rest(int rest, Launch launch)
 {
     if (rest == R) return launch(std::integral_constant<int, R>());
-    if constexpr (R > (TABLE && BITS == 1 ? kTableOnly - 1 : 0)) return with_rest<BITS, TABLE, R - 1>(rest, launch);
+    if constexpr (R > (TABLE && BITS == 1 ? kTableOnly - 1 : TABLE && kTableWorkers<BITS> ? 0 : 1)) return with_rest<BITS, TABLE, R - 1>(rest, launch);
     else return cudaErrorInvalidValue;
 }
 
@@ -246,8 +253,8 @@ __device__ __forceinline__ void sum_workers(int K, int lane, uint32_t table, uin
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[g][j] = 0.f;
     }
-    if constexpr (REST >= 0)
-        for (; k0 + B <= K; k0 += B) sum_batch<BITS, G, B>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
+    if constexpr (REST > 0)
+        for (; k0 + kLast<BITS, TABLE> < K; k0 += B) sum_batch<BITS, G, B>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
     if constexpr (REST > 0) sum_batch<BITS, G, REST>(k0, lane, rows + (uint32_t)k0 * (kRowStride<BITS> * 4u), word, acc);
 }
 
