@@ -55,7 +55,10 @@ k_bucket_decode_sum(const uint32_t* const* __restrict__ packed_k, const float* c
         auto write = [&](int64_t q, float (&a)[8]) {
 #pragma unroll
             for (int e = 0; e < 8; ++e) a[e] = __fmul_rn(a[e], scale);
-            store8<(BITS > 1)>(outp + (q << 8) + 8 * lane, shift, lane, a);
+            // (256-bit stores for 1-bit codes, too, with two groups at a time: there two 128-bit ones, which write every sector by halves, cost
+            // 31.4 instead of 22.0 us for 25 M elements of one worker at d = 2048.  With one group at a time they are the
+            // faster: 1.7 M elements of sixteen workers 9.1 instead of 9.7.)
+            store8<(BITS > 1 || PAIRS)>(outp + (q << 8) + 8 * lane, shift, lane, a);
         };
         if (PAIRS && at + 512 <= d && g + 1 < g_end && g + 1 < full) {  // two groups of one bucket
             float a[2][8];

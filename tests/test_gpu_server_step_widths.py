@@ -58,7 +58,7 @@ def test_unpack_sum_dense_tables(s, K):
 
 
 @pytest.mark.parametrize("s,d,K,total", [(9, 512, 3, 11_000_077), (3, 640, 2, 10_500_001), (5, 4096, 6, 9_800_000), (2, 1024, 9, 12_345_679),
-                                         (17, 256, 5, 10_000_001), (9, 512, 7, 900_013)])
+                                         (17, 256, 5, 10_000_001), (9, 512, 7, 900_013), (2, 2048, 1, 11_000_077)])
 def test_bucket_decode_sum_runs(s, d, K, total):
     """Equal to ogq_unpack_sum called with offsets j * d, bit for bit: the same additions (any words are codes)."""
     dev, bits = torch.device("cuda:0"), ogq.ogq_bits_for_levels(s)
