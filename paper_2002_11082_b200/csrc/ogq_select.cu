@@ -392,8 +392,9 @@ struct Round1Body {
     uint32_t one24;   // 1 << 24 (the count field of a packed word), kept in a register
     float mn, mx;
     uint32_t nonfinite;
-    float tau;  // clipping threshold (CLIP only)
-    uint32_t clipped;  // values beyond it since the last fold; of those, the negative ones in the upper half (CLIP only)
+    float tau;         // clipping threshold (CLIP only)
+    float tau_mag;     // its magnitude: that of a clipped value, also where a caller's threshold is negative
+    uint32_t clipped;  // values at that magnitude since the last fold; of those, the negative ones in the upper half (CLIP only)
 
     // clip to [-tau, tau] (CLIP), magnitude for BinGrad-pb, and fold -0 into +0
     __device__ __forceinline__ float canon(float v) const
@@ -435,8 +436,9 @@ struct Round1Body {
         if constexpr (CLIP) {
             uint32_t count = 1u;
             if (!MAG) asm("mad.lo.u32 %0, %1, 65536, %2;" : "=r"(count) : "r"(bits >> 31), "r"(one24 >> 24));
-            asm volatile("{ .reg .pred p; setp.lt.f32 p, %3, %4; @p red.shared.add.u32 [%1], %2; @!p add.u32 %0, %0, %5; }"
-                         : "+r"(clipped) : "r"(addr), "r"(word), "f"(fabsf(__uint_as_float(bits))), "f"(tau), "r"(count) : "memory");
+            // (unordered: a threshold that is not a number clips nothing, see canon)
+            asm volatile("{ .reg .pred p; setp.ltu.f32 p, %3, %4; @p red.shared.add.u32 [%1], %2; @!p add.u32 %0, %0, %5; }"
+                         : "+r"(clipped) : "r"(addr), "r"(word), "f"(fabsf(__uint_as_float(bits))), "f"(tau_mag), "r"(count) : "memory");
         } else {
             red_shared_add(addr, word);
         }
@@ -521,6 +523,7 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
     uint32_t *hist = sel_hist(), *packed = sel_stage();
     Round1Body<MAG, CLIP> f;
     f.tau = tau;
+    f.tau_mag = fabsf(tau);
     f.lo23 = (uint32_t)lo_e << 23;
     f.neg_lo23x2 = 0u - (f.lo23 << 1);
     f.one24 = 0x01000000u;
@@ -615,7 +618,7 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
                     for (int j = 0; j < 4; ++j) {
                         const uint32_t bits = __float_as_uint(vv[j]);
                         const uint32_t rel = (bits & 0x7fffffffu) - f.lo23;
-                        if (rel < ((uint32_t)kSelW << 23) && !(CLIP && fabsf(vv[j]) >= tau)) f.fine_wide(bits, rel);
+                        if (rel < ((uint32_t)kSelW << 23) && !(CLIP && fabsf(vv[j]) >= f.tau_mag)) f.fine_wide(bits, rel);
                     }
                 }
             }
@@ -630,17 +633,15 @@ __device__ __noinline__ Round1Out stream_round1(const float* __restrict__ grad, 
         // period (three clipped levels of the ResNet-50 bucket: round 1 took 52 us, with every period done again, now 38)
         __syncthreads();
         if (threadIdx.x < 2 && sh_clipped[threadIdx.x]) {
+            // (only values inside the fine window are counted aside, so the threshold lies in it)
             const bool neg = threadIdx.x == 1;
-            const uint32_t mag = __float_as_uint(tau), rel = mag - f.lo23, n = sh_clipped[threadIdx.x];
-            const bool fine = rel < ((uint32_t)kSelW << 23);
-            const int e = (int)(mag >> 23), mi = fine ? lo_e + (int)(rel >> (23 - kSelM)) : e < lo_e ? e : e - kSelW + (kSelW << kSelM);
-            const uint32_t mask = fine ? (1u << (23 - kSelM)) - 1u : 0x7fffffu, low = (neg ? ~mag : mag) & mask;
-            const int cell = (MAG ? 0 : kRound1Mag) + (neg ? ~mi : mi);
+            const uint32_t mag = __float_as_uint(f.tau_mag), rel = mag - f.lo23, n = sh_clipped[threadIdx.x];
+            const int mi = lo_e + (int)(rel >> (23 - kSelM)), cell = (MAG ? 0 : kRound1Mag) + (neg ? ~mi : mi);
+            const uint32_t low = (neg ? ~mag : mag) & ((1u << (23 - kSelM)) - 1u);
             const unsigned long long sum = ((unsigned long long)hist[2 * kCells + cell] << 32 | hist[kCells + cell]) + (unsigned long long)n * low;
             hist[cell] += n;
             hist[kCells + cell] = (uint32_t)sum;
             hist[2 * kCells + cell] = (uint32_t)(sum >> 32);
-            if (e == 255) f.nonfinite = 1u;
         }
     }
     return Round1Out{f.mn, f.mx, f.nonfinite};
