@@ -13,13 +13,22 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kChunkAlign = 1024;   // flat chunk boundaries are multiples of this many elements
 
 // ---------------------------------------------------------------------------
-// Programmatic dependent launch: a kernel of this library is put on the device while the kernel before it
-// in the stream is still running and waits, before its first access to global memory, until that one has
-// finished and its writes are visible.  The launch latency of every kernel of a chain so overlaps with the
-// kernel before it.  Every kernel launched with launch_pdl calls pdl_wait() in all its threads, so
-// completion passes from kernel to kernel, and only then allows its own successor to be launched: at most
-// two kernels of a chain are on the device.  What one kernel of a chain writes and a later one reads is
-// loaded plainly or from L2 (__ldcg), never through the read-only path, whose loads the compiler may move.
+// Programmatic dependent launch: a kernel of this library may be put on the device while the kernel before it
+// in the stream is still running; pdl_wait() returns when that one has finished and its writes are visible, and
+// pdl_launch_dependents() (or the end) of every CTA lets the next kernel be launched.  The launch latency of every
+// kernel of a chain so overlaps with the kernel before it.  The rules:
+//   1. The first kernel of a call waits in every CTA before it touches global memory and before it lets its successor go.  Whatever
+//      the call's later kernels do before their own wait, everything earlier in the stream has then finished.
+//   2. Before its wait a later kernel reads nothing but the call's input (gradient, offsets, thresholds) and writes nothing but
+//      outputs that no kernel of the call before it touches.
+//   3. At least one CTA of every kernel waits before it ends, and every CTA that uses what the kernel before it wrote: completion
+//      so passes from kernel to kernel, to the next call as well.
+// Nearly every kernel simply waits first, in all its threads.  The exceptions are those of the exact selection: round 1 streams the
+// gradient while k_sel_prepare clears its cells, and lets the first solver launch go before it waits; in the solver launches the CTAs
+// of small tensors need nothing of the rounds, and of those only tensor 0's waits.  All of them rest on rule 1 in
+// k_sel_prepare.  (A bucket without rounds begins with the second solver launch, which then waits in every CTA.)
+//   What one kernel of a chain writes and a later one reads is loaded plainly or from L2 (__ldcg), never through the
+// read-only path, whose loads the compiler may move.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -165,8 +165,8 @@ __device__ __forceinline__ void sum_batch(int k0, int lane, uint32_t row, Word w
         for (int u = 0; u < N; ++u) c[g][u] = load_codes<BITS>(word(k0 + u, g), lane);
     add_batch<BITS, G, N>(c, row, acc);
 }
-// Table indices of eight elements from the codes of the kTableWorkers workers of a table (workers that do not
-// exist: zeros): byte e of x[0], byte e - 4 of x[1] is the index of element e, worker u's code in its bits
+// Table indices of eight elements from the codes of the kTableWorkers workers of a table (of workers that do not exist any
+// code: the table's entries do not depend on it): byte e of x[0], byte e - 4 of x[1] is the index of element e, worker u's code in its bits
 // [u BITS, (u + 1) BITS).
 template <int BITS>
 __device__ __forceinline__ void table_indices(const uint32_t (&c)[kTableWorkers<BITS>], uint32_t (&x)[2])

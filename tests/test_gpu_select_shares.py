@@ -33,4 +33,6 @@ def test_levels_of_shares(bucket):
     for k in got:
         (lv, st), (w_lv, w_st) = got[k], want[k]
         assert np.array_equal(st, w_st)
+        if k == "orq":  # order statistics
+            assert np.array_equal(lv, w_lv.astype(np.float32))
         assert np.all(np.abs(lv.astype(np.float64) - w_lv) <= 1e-5 * np.max(np.abs(w_lv), axis=1, keepdims=True)), k
