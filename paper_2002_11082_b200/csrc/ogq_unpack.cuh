@@ -5,10 +5,9 @@
 // conflicts, a row is at most 32 words).  1- and 2-bit codes have a table besides: the codes of the first eight
 // (four) workers are transposed, in registers, into one index per element, and a table of 256 sums, built
 // once per tensor in worker order, gives the sum of all of them in one read.
-//   What bounds it: for the wider codes shared-memory reads (two thirds of the load/store pipe for eight workers of nine
-// levels), the instructions that turn codes into addresses, and the wait for the words from L2, of which more in flight would
-// not fit the registers (asked for a trip ahead in registers: 57 instead of 52 us for the ResNet-50 bucket); for 1-bit
-// codes DRAM.
+//   What bounds it: for the wider codes a shared-memory read and the instructions for its address per element and worker, and the
+// wait for the words from L2, of which more in flight would not fit the registers (asked for a trip ahead in registers: 57
+// instead of 52 us for the ResNet-50 bucket, eight workers of nine levels); for 1-bit codes DRAM.
 #pragma once
 
 #include <type_traits>
